@@ -367,9 +367,9 @@ int hmg_assemble_trace(hmg_ctx *c) {
   if (!c) return HMG_ERR_INVALID_ARG;
   HMG_CUDA(c, cudaSetDevice(c->device));
   const bool need_fp32 = c->opt.precision == HMG_PRECISION_MIXED;
+  if (!c->have_mesh || !c->have_coeffs) return fail(c, HMG_ERR_NOT_READY, "mesh or coefficients not set");
   if (c->have_fp32 && need_fp32) c->have_fp32 = false;  // rebuild copies from fresh FP64 data
-  int st = assemble_all(c);
-  if (st) return st;
+  int st;
   const Level &f = c->lv[0];
   const int64_t T = f.ntrace, C = f.ncell;
   const int64_t T1 = c->opt.degree >= 1 ? ho_trace_size(c, c->opt.degree) : 0;
@@ -399,6 +399,7 @@ int hmg_assemble_trace(hmg_ctx *c) {
     c->work_cap = nwork;
     drop_graph(c);
   }
+  if ((st = assemble_all(c))) return st;   // its per-cell data passes through the Krylov vectors
   if (!c->cb) {
     double *tmp;
     if ((st = dev_alloc(c, &tmp, (size_t)C))) return st;

@@ -20,7 +20,7 @@ constexpr int kRedBlocks = 1216;  // blocks of the grid-stride vector reductions
 constexpr int kMaxRedBlocks = 1 << 18;  // partial-sum slots per reduction (one row per thread)
 constexpr int kRedThreads = 256;
 
-// Per-cell record written by the geometry kernel on every multigrid level.
+// Per-cell record of the finest level that configuration 1's 2x2 system is built from.
 // Offsets into a [ncell][kCellData] array.
 struct CellRec {
   static constexpr int M = 0;      // 21 entries: upper triangle of M_K, row-major (f <= g)
@@ -60,6 +60,7 @@ struct Level {
   double *corners = nullptr;        // [ncol][4][3]
   double *z = nullptr;              // [nlev+1]
   double *theta_lev = nullptr, *exner_lev = nullptr, *exner = nullptr;
+  double *ctab = nullptr, *ltab = nullptr;   // geometry sums per column and per level (assembly)
   // assembled pressure operator (device)
   double *H = nullptr;              // [7][ncell]
   // Thomas factors of H_z with the relaxation mg_omega folded in (pivot p_k): omega / p_k,
@@ -128,6 +129,7 @@ struct Ctx {
   double *Ainv = nullptr;     // [49][ncell] A_K^-1, entry (i, j) at (7 i + j) * ncell + K
   double *kth = nullptr;      // [6][ncell] diagonal of K_K (k theta on each local face)
   double *gamma = nullptr;    // [ncell]
+  int *asm_flag = nullptr;    // set by the assembly when a cell matrix is singular
   float *S32 = nullptr, *Sz_w32 = nullptr, *Sz_l32 = nullptr, *Sz_cp32 = nullptr, *Sh_w32 = nullptr,
         *gamma32 = nullptr;
   // Krylov workspace (FP64, [ntrace] each)
