@@ -7,19 +7,11 @@
 // m3^rho, m3^Pi); Eq. 2x2system (B = Q32 + M3^rho M3^-1 D); Sec. 2.4 Eqs. hybrid-A,
 // hybrid-K, hybrid-S (S = C^T A^-1 K); Sec. 2.3 Eq. elliptic_pressure_system
 // (H = -B Mlump^-1 G + M3^Pi); Sec. 2.5 Eq. scaling_matrix (Gamma).
+#include "assemble.cuh"
 #include "device_common.cuh"
 #include "hmg_internal.cuh"
 
 namespace hmg {
-
-struct CellArgs {
-  int geometry, ncol, L;
-  int64_t ncell;
-  double radius;
-  const double *corners, *z, *theta_lev, *exner_lev, *exner;
-  const int32_t *col_nbr;
-  hmg_scalars sc;
-};
 
 // ---- the geometry of an extruded column, factorised -----------------------------------------
 // A vertex at height z over corner c is c (R + z) on the sphere and (c_x, c_y, z) on the plane, so
@@ -57,9 +49,9 @@ struct Col {   // per-column sums [ncol][N]; face pairs f <= g in row-major orde
   static constexpr int RJ = 35;    // 3: (r . C_xi), (r . C_eta), |C| at the centre
   static constexpr int C = 38;     // 30: C at the nine points and the centre
   static constexpr int CD = 68;    // 18: C_xi at the three eta, C_eta at the three xi
-  // 36: sum over xi of h s_f C at the three eta for faces 1 and 3, over eta at the three xi for 0 and 2
+  // 36 floats: sum over xi of h s_f C at the three eta for faces 1 and 3, over eta at the three xi for 0, 2
   static constexpr int K = 86;
-  static constexpr int N = 122;
+  static constexpr int N = 104;
 };
 struct Lev {   // per-level sums [L][N]
   static constexpr int V1 = 0;     // 2: bottom, top
@@ -70,13 +62,14 @@ struct Lev {   // per-level sums [L][N]
   static constexpr int DZ = 9, IDZ = 10; // the layer's depth in the map (s1 - s0) and its inverse
   static constexpr int IZ = 11;    // 1 / (z1 - z0), of the background's vertical differences
   static constexpr int SQ = 12;    // 3: s at the Gauss points
-  static constexpr int WQ = 15;    // 6: w (zeta - 1) / s^2 and w zeta / s^2 there
-  static constexpr int N = 21;
+  static constexpr int WQ = 15;    // 6 floats: w (zeta - 1) / s^2 and w zeta / s^2 there
+  static constexpr int N = 18;
 };
 
 // the three Gauss points and weights on [0, 1]: 1/2 -+ sqrt(15) / 10
 constexpr double kGq = 0.3872983346207417, kG0 = 0.5 - kGq, kG2 = 0.5 + kGq, kW0 = 5.0 / 18.0, kW1 = 8.0 / 18.0;
 __constant__ double c_gx[3] = {kG0, 0.5, kG2}, c_gw[3] = {kW0, kW1, kW0};
+__constant__ float c_gxf[3] = {(float)kG0, 0.5f, (float)kG2}, c_gwf[3] = {(float)kW0, (float)kW1, (float)kW0};
 // bilinear weights of the corners (0,0), (1,0), (0,1), (1,1) at the nine points and the centre
 #define HMG_BILINEAR(x, y) {(1.0 - x) * (1.0 - y), x * (1.0 - y), (1.0 - x) * y, x * y}
 __constant__ double c_bilinear[10][4] = {
@@ -108,8 +101,9 @@ __global__ void __launch_bounds__(64) column_kernel(const CellArgs a, double *__
       s2 = fma(w * s, s, s2);
       double *o = ltab + (int64_t)k * Lev::N;
       o[Lev::SQ + q] = s;
-      o[Lev::WQ + 2 * q] = w * m * is;
-      o[Lev::WQ + 2 * q + 1] = w * p * is;
+      float *of = reinterpret_cast<float *>(o + Lev::WQ) + 2 * q;
+      of[0] = (float)(w * m * is);
+      of[1] = (float)(w * p * is);
     }
     const double sc = sph ? fma(0.5, dz, s0) : 1.0;
     double *o = ltab + (int64_t)k * Lev::N;
@@ -146,6 +140,7 @@ __global__ void __launch_bounds__(64) column_kernel(const CellArgs a, double *__
   for (int i = 0; i < 10; ++i) A[i] = B[i] = 0.0;
 #pragma unroll
   for (int i = 0; i < 4; ++i) U[i] = XU[i] = X[i] = 0.0;
+  float *kf = reinterpret_cast<float *>(o + Col::K);
 #pragma unroll 1
   for (int q = 0; q < 3; ++q)
 #pragma unroll
@@ -153,7 +148,7 @@ __global__ void __launch_bounds__(64) column_kernel(const CellArgs a, double *__
       o[Col::CD + 3 * q + i] = fma(gx[q], p3[i], p1[i]);
       o[Col::CD + 9 + 3 * q + i] = fma(gx[q], p3[i], p2[i]);
 #pragma unroll
-      for (int j = 0; j < 4; ++j) o[Col::K + 3 * (q + 3 * j) + i] = 0.0;
+      for (int j = 0; j < 4; ++j) kf[3 * (q + 3 * j) + i] = 0.f;
     }
   auto at = [&](double xi, double eta, double (&C)[3], double (&Cx)[3], double (&Ce)[3]) {
 #pragma unroll
@@ -205,7 +200,7 @@ __global__ void __launch_bounds__(64) column_kernel(const CellArgs a, double *__
 #pragma unroll
       for (int j = 0; j < 4; ++j)
 #pragma unroll
-        for (int i = 0; i < 3; ++i) o[Col::K + 3 * ((j < 2 ? q / 3 : q % 3) + 3 * j) + i] += h * s[face[j]] * C[i];
+        for (int i = 0; i < 3; ++i) kf[3 * ((j < 2 ? q / 3 : q % 3) + 3 * j) + i] += (float)(h * s[face[j]] * C[i]);
     } else {
       W += h;
     }
@@ -336,7 +331,7 @@ __device__ __forceinline__ void cell_geometry(const CellArgs &a, const double *_
   float C[3], Cx[3], Ce[3], n[3], e[3];
 #pragma unroll 1
   for (int q = 0; q < 9; ++q) {
-    const float xi = (float)c_gx[q % 3], eta = (float)c_gx[q / 3], w = (float)(c_gw[q % 3] * c_gw[q / 3]);
+    const float xi = c_gxf[q % 3], eta = c_gxf[q / 3], w = c_gwf[q % 3] * c_gwf[q / 3];
     rounding(q, e);
     at(xi, eta, C, Cx, Ce, n);
     const float D = dot(n, C), h = w / D, cc = dot(C, C), ic = 1.f / cc, ne = dot(n, e), tau = ne / D, ce = dot(C, e);
@@ -378,8 +373,6 @@ __device__ __forceinline__ void cell_geometry(const CellArgs &a, const double *_
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       o.xx[i] = fma((double)dx[i], idz, o.xx[i]);
-      o.us[i][0] = fma((double)du[i], l[Lev::V1], o.us[i][0]);
-      o.us[i][1] = fma((double)du[i], l[Lev::V1 + 1], o.us[i][1]);
       o.px[i] += (double)dp[i];
     }
     // e_xi at (eta, zeta) for faces 1 and 3, e_eta at (xi, zeta) for faces 0 and 2
@@ -390,7 +383,8 @@ __device__ __forceinline__ void cell_geometry(const CellArgs &a, const double *_
     for (int q = 0; q < 9; ++q) {
       const int hq = q % 3, vq = q / 3;
       const double sv = l[Lev::SQ + vq];
-      const float w0 = (float)l[Lev::WQ + 2 * vq], w1 = (float)l[Lev::WQ + 2 * vq + 1];
+      const float *wq = reinterpret_cast<const float *>(l + Lev::WQ) + 2 * vq;
+      const float w0 = wq[0], w1 = wq[1];
       const double *bw = c_bilinear[q];
 #pragma unroll
       for (int d = 0; d < 2; ++d) {
@@ -408,8 +402,8 @@ __device__ __forceinline__ void cell_geometry(const CellArgs &a, const double *_
         }
 #pragma unroll
         for (int j = 0; j < 2; ++j) {
-          const double *kk = t + Col::K + 3 * (hq + 3 * (2 * d + j));
-          const float m = fmaf(ed[2], (float)kk[2], fmaf(ed[1], (float)kk[1], ed[0] * (float)kk[0]));
+          const float *kk = reinterpret_cast<const float *>(t + Col::K) + 3 * (hq + 3 * (2 * d + j));
+          const float m = fmaf(ed[2], kk[2], fmaf(ed[1], kk[1], ed[0] * kk[0]));
           const int f = d == 0 ? 1 + 2 * j : 2 * j;
           dz1[f][0] = fmaf(w0, m, dz1[f][0]);
           dz1[f][1] = fmaf(w1, m, dz1[f][1]);
@@ -418,8 +412,8 @@ __device__ __forceinline__ void cell_geometry(const CellArgs &a, const double *_
     }
 #pragma unroll
     for (int f = 0; f < 4; ++f) {
-      o.us[f][0] = fma(kap, (double)dz1[f][0], o.us[f][0]);
-      o.us[f][1] = fma(kap, (double)dz1[f][1], o.us[f][1]);
+      o.us[f][0] += (double)fmaf(fkap, dz1[f][0], du[f] * (float)l[Lev::V1]);
+      o.us[f][1] += (double)fmaf(fkap, dz1[f][1], du[f] * (float)l[Lev::V1 + 1]);
     }
   }
   o.wz = fma(kap * dz, (double)dw, o.wz);
@@ -430,12 +424,6 @@ __device__ __forceinline__ void cell_geometry(const CellArgs &a, const double *_
   o.vol1 = fma(o.vol1, (double)tc, o.vol1);
   o.rj[2] = fma(o.rj[2], (double)rc, o.rj[2]);
 }
-
-// The coefficients of one cell: the diagonal of K_K, the pressure-row couplings, M3^Pi and this
-// cell's share |M(f,f)| + |M(f, opposite f)| of the lumped mass of each face.
-struct CellCo {
-  double kth[6], b[6], m, lump[6];
-};
 
 template <bool XPART>
 __device__ __forceinline__ void cell_coefficients(const CellArgs &a, const double *__restrict__ t,
@@ -484,23 +472,6 @@ __device__ __forceinline__ void cell_coefficients(const CellArgs &a, const doubl
 
 __device__ __forceinline__ double coriolis(const CellArgs &a) {   // tau_u dt 2 Omega (Eq. gh-u)
   return a.sc.preset == 1 ? 0.0 : a.sc.tau_u * a.sc.dt * 2.0 * a.sc.omega;
-}
-
-// What the pressure operator needs of each cell, face-major [f][ncell] (level 0: written by
-// condense_kernel). Pointers may lie in different buffers.
-struct CellOut {
-  double *b[2], *lump[2];   // faces 0-2 and 3-5
-  double *kth, *m;
-};
-
-__device__ __forceinline__ void store_cell(const CellOut &q, const CellCo &o, int64_t C, int64_t K) {
-#pragma unroll
-  for (int f = 0; f < 6; ++f) {
-    q.b[f / 3][(f % 3) * C + K] = o.b[f];
-    q.lump[f / 3][(f % 3) * C + K] = o.lump[f];
-    q.kth[f * C + K] = o.kth[f];
-  }
-  q.m[K] = o.m;
 }
 
 __global__ void __launch_bounds__(128) cell_kernel(const CellArgs a, const double *__restrict__ ctab,
@@ -705,7 +676,9 @@ __global__ void trace_rows_kernel(const RowArgs a, const double *__restrict__ Ai
   if (row >= a.NT) return;
   const int64_t C = a.ncell, T = a.NT;
   double v[kSlots];
-  auto sk = [&](int64_t K, int i, int j) { return Ainv[(int64_t)(7 * i + j) * C + K] * kth[(int64_t)j * C + K]; };
+  auto sk = [&](int64_t K, int i, int j) {   // (rounded before any sum: a contracted sum would depend on the row)
+    return __dmul_rn(Ainv[(int64_t)(7 * i + j) * C + K], kth[(int64_t)j * C + K]);
+  };
   if (row < a.NH) {
     const int e = (int)((unsigned)row / (unsigned)a.L), k = (int)((unsigned)row - (unsigned)e * (unsigned)a.L);
     const int c1 = a.stencil[8 * (int64_t)e], c2 = a.stencil[8 * (int64_t)e + 1];
@@ -849,7 +822,7 @@ __global__ void gamma_kernel(const RowArgs a, const double *__restrict__ Ainv, c
   if (K >= a.ncell) return;
   const int c = (int)((unsigned)K / (unsigned)a.L), k = (int)((unsigned)K - (unsigned)c * (unsigned)a.L);
   const int64_t C = a.ncell;
-  auto sk1 = [&](int f, int64_t cell) { return m[cell] * Ainv[(int64_t)(7 * f + 6) * C + cell]; };
+  auto sk1 = [&](int f, int64_t cell) { return __dmul_rn(m[cell], Ainv[(int64_t)(7 * f + 6) * C + cell]); };
   double ps1 = 0.0;
 #pragma unroll
   for (int f = 0; f < 4; ++f) {
@@ -960,7 +933,7 @@ static CellOut cell_buffers(Ctx *c, int l) {
   return q;
 }
 
-int assemble_all(Ctx *c) {
+static int assemble_levels(Ctx *c, double *rec) {
   Level &f = c->lv[0];
   const int64_t C = f.ncell, T = f.ntrace;
   int st;
@@ -978,9 +951,14 @@ int assemble_all(Ctx *c) {
   HMG_CUDA(c, cudaMemsetAsync(c->asm_flag, 0, sizeof(int), c->stream));
   for (int l = 0; l < c->nmg; ++l) {
     Level &lv = c->lv[l];
-    if (!lv.ctab) {
-      if ((st = dev_alloc(c, &lv.ctab, (size_t)Col::N * lv.ncol))) return st;
-      if ((st = dev_alloc(c, &lv.ltab, (size_t)Lev::N * lv.nlev))) return st;
+    const CellArgs a{lv.geometry, lv.ncol, lv.nlev, lv.ncell, lv.radius, lv.corners, lv.z,
+                     lv.theta_lev, lv.exner_lev, lv.exner, lv.col_nbr, c->sc};
+    if (!lv.geo_ready) {   // the sums depend on the mesh only, which a context keeps
+      if (!lv.ctab && (st = dev_alloc(c, &lv.ctab, (size_t)Col::N * lv.ncol))) return st;
+      if (!lv.ltab && (st = dev_alloc(c, &lv.ltab, (size_t)Lev::N * lv.nlev))) return st;
+      column_kernel<<<grid_for(lv.ncol, 64) + grid_for(lv.nlev, 64), 64, 0, c->stream>>>(a, lv.ctab, lv.ltab);
+      HMG_CUDA(c, cudaGetLastError());
+      lv.geo_ready = true;
     }
     if (!lv.H) {
       if ((st = dev_alloc(c, &lv.H, (size_t)kHCoef * lv.ncell))) return st;
@@ -988,11 +966,10 @@ int assemble_all(Ctx *c) {
       if ((st = dev_alloc(c, &lv.Hz_l, (size_t)lv.ncell))) return st;
       if ((st = dev_alloc(c, &lv.Hz_cp, (size_t)lv.ncell))) return st;
     }
-    const CellArgs a{lv.geometry, lv.ncol, lv.nlev, lv.ncell, lv.radius, lv.corners, lv.z,
-                     lv.theta_lev, lv.exner_lev, lv.exner, lv.col_nbr, c->sc};
     const CellOut q = cell_buffers(c, l);
-    column_kernel<<<grid_for(lv.ncol, 64) + grid_for(lv.nlev, 64), 64, 0, c->stream>>>(a, lv.ctab, lv.ltab);
-    if (l == 0) condense_kernel<<<grid_for(C, 128), 128, 0, c->stream>>>(a, lv.ctab, lv.ltab, c->Ainv, q, c->asm_flag);
+    if (rec) {
+      if ((st = gauss_cells(c, a, q, rec, l == 0 ? c->Ainv : nullptr))) return st;
+    } else if (l == 0) condense_kernel<<<grid_for(C, 128), 128, 0, c->stream>>>(a, lv.ctab, lv.ltab, c->Ainv, q, c->asm_flag);
     else cell_kernel<<<grid_for(lv.ncell, 128), 128, 0, c->stream>>>(a, lv.ctab, lv.ltab, q);
     const HArgs ha{lv.nlev, lv.ncol, lv.ncell, lv.col_nbr, lv.col_nbr_face};
     pressure_rows_kernel<<<grid_for(lv.ncell, 256), 256, 0, c->stream>>>(ha, q, lv.H);
@@ -1002,13 +979,13 @@ int assemble_all(Ctx *c) {
       trace_rows_kernel<<<grid_for(T, 256), 256, 0, c->stream>>>(ra, c->Ainv, c->kth, c->S);
       gamma_kernel<<<grid_for(C, 256), 256, 0, c->stream>>>(ra, c->Ainv, q.m, c->gamma);
       HMG_CUDA(c, cudaGetLastError());
-      if (c->opt.precond == HMG_PRECOND_SCHUR) {   // configuration 1 needs M_K itself
-        double *rec = nullptr;
-        HMG_CUDA(c, cudaMalloc(&rec, (size_t)C * kCellData * sizeof(double)));
-        record_kernel<<<grid_for(C, 128), 128, 0, c->stream>>>(a, lv.ctab, lv.ltab, rec);
-        st = build_mixed(c, rec);
+      if (c->opt.precond == HMG_PRECOND_SCHUR) {   // configuration 1 (FP64) needs M_K itself
+        double *mk = nullptr;
+        HMG_CUDA(c, cudaMalloc(&mk, (size_t)C * kCellData * sizeof(double)));
+        record_kernel<<<grid_for(C, 128), 128, 0, c->stream>>>(a, lv.ctab, lv.ltab, mk);
+        st = build_mixed(c, mk);
         const cudaError_t e = cudaStreamSynchronize(c->stream);
-        cudaFree(rec);
+        cudaFree(mk);
         if (st) return st;
         HMG_CUDA(c, e);
       }
@@ -1029,6 +1006,19 @@ int assemble_all(Ctx *c) {
   HMG_CUDA(c, cudaStreamSynchronize(c->stream));
   if (sing) return fail(c, HMG_ERR_INVALID_ARG, "a velocity mass block M_K is not positive definite or A_K is singular");
   return HMG_OK;
+}
+
+int assemble_all(Ctx *c) {
+  if (c->opt.precision != HMG_PRECISION_MIXED) return assemble_levels(c, nullptr);
+  // contexts with the FP32 preconditioner: direct Gauss sums (gauss_cells.cu says why)
+  double *rec = nullptr;
+  int st = gauss_setup(c, c->lv[0].ncell, &rec);
+  if (!st) st = assemble_levels(c, rec);
+  if (rec) {
+    cudaStreamSynchronize(c->stream);   // (an error return may leave kernels that use it in flight)
+    cudaFree(rec);
+  }
+  return st;
 }
 
 }  // namespace hmg

@@ -18,238 +18,12 @@
 // interface k) at NH + NB (c (L + 1) + k), node (s, t) at + NT s + t; on a vertical facet s
 // counts along the edge in the traversal of its owner column (the other column's local s is
 // p - s).
-#include <cmath>
-#include <vector>
-
 #include "device_common.cuh"
 #include "hmg_internal.cuh"
+#include "ho_common.cuh"
 #include "precond.cuh"
 
 namespace hmg {
-
-template <int P>
-struct Ho {
-  static constexpr int NT = P + 1;                    // Gauss-Legendre nodes per direction
-  static constexpr int NB = NT * NT;                  // nodes (trace rows) per facet
-  static constexpr int NF = 6 * NB;                   // facet dofs: the hybridised cell matrix is NF x NF
-  static constexpr int NU = 3 * NT * NT * (P + 2);    // RT_p dofs
-  static constexpr int NP = NT * NT * NT;             // DG_p dofs
-  static constexpr int N = NU + NP;                   // the mixed cell matrix
-  static constexpr int NQ1 = P + 3;                   // volume Gauss points per direction
-  static constexpr int Q = NQ1 * NQ1 * NQ1;
-  static constexpr int SLOTS = 2 * NF;                // S coefficients stored per trace row
-  static constexpr int NINT = P * NT * NT;            // interior dofs per component
-  // reference tables: velocity values, pressure values, weights, points, G, facet weights
-  static constexpr int TV = 0, TPHI = TV + Q * NU, TW = TPHI + Q * NP, TX = TW + Q, TG = TX + 3 * Q,
-                       TC = TG + NU * NP, TAB = TC + NB;
-  // the sweep's line part: lanes per column (a group of LPC >= NB lanes of one warp; lane n < NB
-  // computes component n of each block product) and columns per warp (p = 2: three groups of
-  // nine, five lanes idle)
-  static constexpr int LPC = P == 1 ? 4 : (P == 2 ? 9 : 16);
-  static constexpr int CPW = 32 / LPC;
-};
-
-// ---- reference tables, formed on the host ---------------------------------------------------
-// n-point Gauss-Legendre rule on [0, 1]: Newton's method on the Legendre polynomial P_n from the
-// initial guesses cos(pi (i + 3/4) / (n + 1/2)), weights 2 / ((1 - x^2) P_n'(x)^2) on [-1, 1],
-// halved
-static void gauss_legendre01(int n, double *x, double *w) {
-  for (int i = 0; i < n; ++i) {
-    double z = std::cos(M_PI * (i + 0.75) / (n + 0.5)), dp = 1.0;
-    for (int it = 0; it < 100; ++it) {
-      double p0 = 1.0, p1 = z;
-      for (int k = 2; k <= n; ++k) {
-        const double p2 = ((2.0 * k - 1.0) * z * p1 - (k - 1.0) * p0) / k;
-        p0 = p1;
-        p1 = p2;
-      }
-      // p1 = P_n(z), p0 = P_{n-1}(z) (n = 1: P_1 = z, P_0 = 1)
-      dp = n * (z * p1 - p0) / (z * z - 1.0);
-      const double dz = p1 / dp;
-      z -= dz;
-      if (std::fabs(dz) < 1e-16) break;
-    }
-    x[n - 1 - i] = 0.5 * (z + 1.0);   // ascending
-    w[n - 1 - i] = 1.0 / ((1.0 - z * z) * dp * dp);
-  }
-}
-
-// n = 2 .. 5 Gauss-Lobatto points on [0, 1]: the end points and the roots of P'_{n-1}
-static void gauss_lobatto01(int n, double *x) {
-  x[0] = 0.0;
-  x[n - 1] = 1.0;
-  if (n == 3) x[1] = 0.5;
-  if (n == 4) {
-    const double r = 1.0 / std::sqrt(5.0);
-    x[1] = 0.5 * (1.0 - r);
-    x[2] = 0.5 * (1.0 + r);
-  }
-  if (n == 5) {
-    const double r = std::sqrt(3.0 / 7.0);
-    x[1] = 0.5 * (1.0 - r);
-    x[2] = 0.5;
-    x[3] = 0.5 * (1.0 + r);
-  }
-}
-
-static void lagrange1d(const double *nodes, int n, double x, double *val, double *der) {
-  for (int i = 0; i < n; ++i) {
-    double v = 1.0, d = 0.0;
-    for (int j = 0; j < n; ++j)
-      if (j != i) v *= (x - nodes[j]) / (nodes[i] - nodes[j]);
-    for (int m = 0; m < n; ++m) {
-      if (m == i) continue;
-      double t = 1.0 / (nodes[i] - nodes[m]);
-      for (int j = 0; j < n; ++j)
-        if (j != i && j != m) t *= (x - nodes[j]) / (nodes[i] - nodes[j]);
-      d += t;
-    }
-    val[i] = v;
-    der[i] = d;
-  }
-}
-
-// face f: the component normal to it, whether it is the far end (xi, eta or zeta = 1), the sign
-// of the outward normal
-static const int kFaceComp[6] = {1, 0, 1, 0, 2, 2};
-static const int kFaceFar[6] = {0, 1, 1, 0, 0, 1};
-static const double kFaceSign[6] = {-1.0, 1.0, 1.0, -1.0, -1.0, 1.0};
-
-// a velocity dof: its component d, its node a along d (Gauss-Lobatto), its nodes (b, c) across d
-// (Gauss-Legendre, the other two coordinates in increasing order), its sign
-struct HoDof { int d, a, b, c; double sign; };
-
-template <int P>
-static std::vector<HoDof> ho_dofs() {
-  using H = Ho<P>;
-  std::vector<HoDof> v;
-  for (int f = 0; f < 6; ++f)
-    for (int s = 0; s < H::NT; ++s)
-      for (int t = 0; t < H::NT; ++t) {
-        const int b = (f == 2 || f == 3) ? P - s : s;   // e2, e3 traverse their edge backwards
-        v.push_back({kFaceComp[f], kFaceFar[f] ? P + 1 : 0, b, t, kFaceSign[f]});
-      }
-  for (int d = 0; d < 3; ++d)
-    for (int a = 1; a <= P; ++a)
-      for (int b = 0; b < H::NT; ++b)
-        for (int c = 0; c < H::NT; ++c) v.push_back({d, a, b, c, 1.0});
-  return v;
-}
-
-// the RT_p basis (value of its one nonzero component and its divergence) and the DG_p basis at
-// the Q Gauss points, G(f, j) = -int phi_j div v_f, and the facet weights of C_K
-template <int P>
-static void ho_tables(std::vector<double> &tab) {
-  using H = Ho<P>;
-  tab.assign(H::TAB, 0.0);
-  double gl[H::NT], glw[H::NT], gll[P + 2], qx[H::NQ1], qw[H::NQ1];
-  gauss_legendre01(H::NT, gl, glw);
-  gauss_lobatto01(P + 2, gll);
-  gauss_legendre01(H::NQ1, qx, qw);
-  const std::vector<HoDof> dofs = ho_dofs<P>();
-  for (int a = 0; a < H::NQ1; ++a)
-    for (int b = 0; b < H::NQ1; ++b)
-      for (int c = 0; c < H::NQ1; ++c) {
-        const int q = (a * H::NQ1 + b) * H::NQ1 + c;
-        const double x[3] = {qx[a], qx[b], qx[c]};
-        double tv[3][H::NT], td[3][H::NT], nv[3][P + 2], nd[3][P + 2];
-        for (int k = 0; k < 3; ++k) {
-          lagrange1d(gl, H::NT, x[k], tv[k], td[k]);
-          lagrange1d(gll, P + 2, x[k], nv[k], nd[k]);
-        }
-        const double wq = qw[a] * qw[b] * qw[c];
-        tab[H::TW + q] = wq;
-        for (int k = 0; k < 3; ++k) tab[H::TX + 3 * q + k] = x[k];
-        double phi[H::NP];
-        for (int ii = 0; ii < H::NT; ++ii)
-          for (int jj = 0; jj < H::NT; ++jj)
-            for (int kk = 0; kk < H::NT; ++kk) phi[(ii * H::NT + jj) * H::NT + kk] = tv[0][ii] * tv[1][jj] * tv[2][kk];
-        for (int j = 0; j < H::NP; ++j) tab[H::TPHI + q * H::NP + j] = phi[j];
-        for (int i = 0; i < H::NU; ++i) {
-          const HoDof &o = dofs[i];
-          const int t1 = o.d == 0 ? 1 : 0, t2 = o.d == 2 ? 1 : 2;
-          const double tan = tv[t1][o.b] * tv[t2][o.c];
-          tab[H::TV + q * H::NU + i] = o.sign * nv[o.d][o.a] * tan;
-          // divergence: the derivative of the one nonzero component along its own coordinate
-          const double dv = o.sign * nd[o.d][o.a] * tan;
-          for (int j = 0; j < H::NP; ++j) tab[H::TG + i * H::NP + j] -= wq * dv * phi[j];
-        }
-      }
-  for (int s = 0; s < H::NT; ++s)
-    for (int t = 0; t < H::NT; ++t) tab[H::TC + s * H::NT + t] = glw[s] * glw[t];
-}
-
-template <int P>
-__device__ __forceinline__ int ho_comp(int i) {   // the nonzero component of velocity dof i
-  using H = Ho<P>;
-  if (i < H::NF) {
-    const int f = i / H::NB;
-    return f == 0 || f == 2 ? 1 : (f == 1 || f == 3 ? 0 : 2);
-  }
-  return (i - H::NF) / H::NINT;
-}
-
-// ---- mesh access ------------------------------------------------------------------------------
-struct HoGeo {
-  int L, ncol;
-  int64_t NH;                 // rows of the vertical facets (NB nedge L)
-  int64_t nhf, nzf;           // vertical and horizontal facets
-  const int32_t *col_edges, *stencil, *edge_fc;
-  const int8_t *own;          // [ncol][4] 1 if the column owns the edge of that face
-};
-
-// trace row of local facet dof q of cell (c, k)
-template <int P>
-__device__ __forceinline__ int64_t ho_gid(const HoGeo &g, int c, int k, int q) {
-  using H = Ho<P>;
-  const int f = q / H::NB, r = q - f * H::NB, s = r / H::NT, t = r - s * H::NT;
-  if (f < 4) {
-    const int64_t e = g.col_edges[4 * (int64_t)c + f];
-    const int sg = g.own[4 * (int64_t)c + f] ? s : P - s;
-    return H::NB * (e * g.L + k) + H::NT * sg + t;
-  }
-  const int kk = k + (f == 5 ? 1 : 0);
-  return g.NH + H::NB * ((int64_t)c * (g.L + 1) + kk) + H::NT * s + t;
-}
-
-// The one or two cells of facet F: A (and B), their local faces, and whether a node's local s is
-// reversed in B (vertical facets: B traverses the edge backwards).
-struct HoFacet {
-  int cA, kA, fA, cB, kB, fB;   // cB < 0: a ground or lid facet (one cell)
-  bool flipB;
-};
-
-__device__ __forceinline__ HoFacet ho_facet(const HoGeo &g, int64_t F) {
-  HoFacet r;
-  if (F < g.nhf) {
-    const int e = (int)(F / g.L), k = (int)(F - (int64_t)e * g.L);
-    r.cA = g.stencil[8 * (int64_t)e];
-    r.cB = g.stencil[8 * (int64_t)e + 1];
-    r.fA = g.edge_fc[2 * (int64_t)e];
-    r.fB = g.edge_fc[2 * (int64_t)e + 1];
-    r.kA = r.kB = k;
-    r.flipB = true;
-  } else {
-    const int64_t zf = F - g.nhf;
-    const int c = (int)(zf / (g.L + 1)), k = (int)(zf - (int64_t)c * (g.L + 1));
-    r.cA = c;
-    r.flipB = false;
-    if (k < g.L) {
-      r.kA = k;
-      r.fA = 4;                                  // the facet is the bottom of the cell above
-      r.cB = k > 0 ? c : -1;
-      r.kB = k - 1;
-      r.fB = 5;
-    } else {
-      r.kA = g.L - 1;
-      r.fA = 5;                                  // the lid: the top of the last cell
-      r.cB = -1;
-      r.kB = 0;
-      r.fB = 0;
-    }
-  }
-  return r;
-}
 
 // NB consecutive coefficients of one slot (the facet's rows) times x into acc: FP64 coefficients
 // as double2 pairs, FP32 ones (the FP32 preconditioner's copy) as float4 quads where NB allows
@@ -305,197 +79,6 @@ __device__ __forceinline__ void ho_rows(const TS *__restrict__ S, const TX *__re
     if (q / H::NB == fc.fB || (OFFD && !vert && q / H::NB >= 4)) continue;
     const TA xv = (TA)__ldg(x + ho_gid<P>(g, fc.cB, fc.kB, q));
     ho_slot<H::NB, NEG>(Sr + (int64_t)(H::NF + q) * T, xv, acc);
-  }
-}
-
-// ---- assembly -------------------------------------------------------------------------------
-struct HoCellArgs {
-  int geometry, ncol, L;
-  int64_t ncell;
-  double radius, sigma;
-  const double *corners, *z;
-};
-
-// Shared memory of the cell kernel: the mixed matrix when it fits (p <= 2), then the per-point
-// metric terms and the elimination's vectors.
-template <int P>
-struct HoCellSmem {
-  static constexpr bool IN_SMEM = P <= 2;
-  static constexpr size_t MAT = IN_SMEM ? sizeof(double) * Ho<P>::N * Ho<P>::N : 0;
-  static constexpr size_t BYTES =
-      MAT + sizeof(double) * (Ho<P>::Q * 7 + 3 * Ho<P>::N + 24) + sizeof(int) * (Ho<P>::N + 8);
-};
-
-// A_K = [[M, G], [-G^T, Mp]] by the (p+3)^3 Gauss rule (M with the contravariant Piola map,
-// Mp = sigma int phi_i phi_j), then A_K^-1 by in-place Gauss-Jordan elimination with partial
-// pivoting of the symmetrically equilibrated D A_K D, D = |diag A_K|^-1/2: A^-1 = D (D A D)^-1 D.
-// The row interchanges are undone at the end as column interchanges in reverse order. One cell
-// per block; the matrix lives in shared memory for p <= 2 and in its output slot (global memory)
-// at p = 3. m[K] = sigma |K|_1 (the one-point volume), H 1 of the coarse operator.
-template <int P>
-__global__ void __launch_bounds__(256)
-    ho_cell_kernel(const HoCellArgs a, const double *__restrict__ tab, double *__restrict__ Ainv,
-                   double *__restrict__ mK, int *singular) {
-  using H = Ho<P>;
-  using SM = HoCellSmem<P>;
-  constexpr int N = H::N;
-  extern __shared__ __align__(16) unsigned char ho_smem[];
-  const int64_t K = blockIdx.x;
-  double *Ag = SM::IN_SMEM ? reinterpret_cast<double *>(ho_smem) : Ainv + K * (int64_t)(N * N);
-  double *Kq = reinterpret_cast<double *>(ho_smem + SM::MAT);   // [Q][6] (w / det) J^T J
-  double *wd = Kq + 6 * H::Q;                                     // [Q] sigma w det
-  double *dsc = wd + H::Q, *fac = dsc + N, *rowk = fac + N;
-  double *X = rowk + N;                                           // [8][3] corners
-  int *perm = reinterpret_cast<int *>(X + 24);
-  int *piv = perm + N;
-  __shared__ double bestv[8];
-  __shared__ int besti[8];
-  const int tid = threadIdx.x, nthr = blockDim.x;
-  const int c = (int)(K / a.L), k = (int)(K - (int64_t)c * a.L);
-  if (tid < 8) {
-    const int va = tid & 1, vb = (tid >> 1) & 1, vc = (tid >> 2) & 1;
-    const int corner = va == 0 ? (vb == 0 ? 0 : 3) : (vb == 0 ? 1 : 2);
-    const double *cp = a.corners + (4 * (int64_t)c + corner) * 3;
-    const double h = a.z[k + vc];
-    if (a.geometry == 1) {
-      for (int i = 0; i < 3; ++i) X[3 * tid + i] = cp[i] * (a.radius + h);
-    } else {
-      X[3 * tid] = cp[0];
-      X[3 * tid + 1] = cp[1];
-      X[3 * tid + 2] = h;
-    }
-  }
-  __syncthreads();
-  auto jacobian = [&](double xi, double eta, double zeta, double J[3][3]) {
-    for (int i = 0; i < 3; ++i) J[i][0] = J[i][1] = J[i][2] = 0.0;
-    for (int v = 0; v < 8; ++v) {
-      const int va = v & 1, vb = (v >> 1) & 1, vc = (v >> 2) & 1;
-      const double fx = va ? xi : 1.0 - xi, fy = vb ? eta : 1.0 - eta, fz = vc ? zeta : 1.0 - zeta;
-      const double gx = va ? 1.0 : -1.0, gy = vb ? 1.0 : -1.0, gz = vc ? 1.0 : -1.0;
-      const double dn[3] = {gx * fy * fz, fx * gy * fz, fx * fy * gz};
-      for (int i = 0; i < 3; ++i)
-        for (int d = 0; d < 3; ++d) J[i][d] += X[3 * v + i] * dn[d];
-    }
-  };
-  auto det3 = [](const double J[3][3]) {
-    return J[0][0] * (J[1][1] * J[2][2] - J[1][2] * J[2][1]) - J[0][1] * (J[1][0] * J[2][2] - J[1][2] * J[2][0]) +
-           J[0][2] * (J[1][0] * J[2][1] - J[1][1] * J[2][0]);
-  };
-  for (int q = tid; q <= H::Q; q += nthr) {
-    if (q < H::Q) {
-      const double *xq = tab + H::TX + 3 * q;
-      double J[3][3];
-      jacobian(xq[0], xq[1], xq[2], J);
-      const double det = det3(J), w = tab[H::TW + q];
-      double G[3][3];
-      for (int p = 0; p < 3; ++p)
-        for (int r = 0; r < 3; ++r) G[p][r] = J[0][p] * J[0][r] + J[1][p] * J[1][r] + J[2][p] * J[2][r];
-      const double s = w / det;
-      Kq[6 * q] = s * G[0][0];
-      Kq[6 * q + 1] = s * G[1][1];
-      Kq[6 * q + 2] = s * G[2][2];
-      Kq[6 * q + 3] = s * G[0][1];
-      Kq[6 * q + 4] = s * G[0][2];
-      Kq[6 * q + 5] = s * G[1][2];
-      wd[q] = a.sigma * w * det;
-    } else {
-      double J[3][3];
-      jacobian(0.5, 0.5, 0.5, J);
-      mK[K] = a.sigma * det3(J);
-    }
-  }
-  __syncthreads();
-  const double *tv = tab + H::TV, *tp = tab + H::TPHI, *tg = tab + H::TG;
-  for (int idx = tid; idx < N * N; idx += nthr) {
-    const int i = idx / N, j = idx - i * N;
-    double v = 0.0;
-    if (i < H::NU && j < H::NU) {
-      const int di = ho_comp<P>(i), dj = ho_comp<P>(j);
-      const int kk = di == dj ? di : (di + dj == 1 ? 3 : (di + dj == 2 ? 4 : 5));
-      for (int q = 0; q < H::Q; ++q)
-        v = fma(__ldg(tv + q * H::NU + i) * __ldg(tv + q * H::NU + j), Kq[6 * q + kk], v);
-    } else if (i < H::NU) {
-      v = __ldg(tg + i * H::NP + (j - H::NU));
-    } else if (j < H::NU) {
-      v = -__ldg(tg + j * H::NP + (i - H::NU));
-    } else {
-      for (int q = 0; q < H::Q; ++q)
-        v = fma(wd[q] * __ldg(tp + q * H::NP + (i - H::NU)), __ldg(tp + q * H::NP + (j - H::NU)), v);
-    }
-    Ag[idx] = v;
-  }
-  __syncthreads();
-  for (int i = tid; i < N; i += nthr) dsc[i] = 1.0 / sqrt(fabs(Ag[(int64_t)i * N + i]));
-  __syncthreads();
-  for (int idx = tid; idx < N * N; idx += nthr) {
-    const int i = idx / N, j = idx - i * N;
-    Ag[idx] *= dsc[i] * dsc[j];
-  }
-  __syncthreads();
-  const int warp = tid >> 5, lane = tid & 31, nwarp = nthr >> 5;
-  for (int col = 0; col < N; ++col) {
-    // pivot: the largest |A[r][col]|, r >= col (the first such row on ties)
-    double bv = -1.0;
-    int bi = col;
-    for (int r = col + tid; r < N; r += nthr) {
-      const double v = fabs(Ag[(int64_t)r * N + col]);
-      if (v > bv) { bv = v; bi = r; }
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const double ov = __shfl_xor_sync(0xffffffffu, bv, o);
-      const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-      if (ov > bv || (ov == bv && oi < bi)) { bv = ov; bi = oi; }
-    }
-    if (lane == 0) { bestv[warp] = bv; besti[warp] = bi; }
-    __syncthreads();
-    if (tid == 0) {
-      double v = bestv[0];
-      int p = besti[0];
-      for (int w = 1; w < nwarp; ++w)
-        if (bestv[w] > v || (bestv[w] == v && besti[w] < p)) { v = bestv[w]; p = besti[w]; }
-      if (!(v > 0.0)) atomicExch(singular, 1);
-      piv[0] = p;
-      perm[col] = p;
-    }
-    __syncthreads();
-    const int p = piv[0];
-    if (p != col)
-      for (int j = tid; j < N; j += nthr) {
-        const double t = Ag[(int64_t)col * N + j];
-        Ag[(int64_t)col * N + j] = Ag[(int64_t)p * N + j];
-        Ag[(int64_t)p * N + j] = t;
-      }
-    __syncthreads();
-    for (int r = tid; r < N; r += nthr) fac[r] = Ag[(int64_t)r * N + col];
-    __syncthreads();
-    const double pinv = 1.0 / fac[col];
-    for (int j = tid; j < N; j += nthr) {
-      const double v = (j == col ? 1.0 : Ag[(int64_t)col * N + j]) * pinv;
-      Ag[(int64_t)col * N + j] = v;
-      rowk[j] = v;
-    }
-    __syncthreads();
-    for (int idx = tid; idx < N * N; idx += nthr) {
-      const int r = idx / N, j = idx - r * N;
-      if (r != col) Ag[idx] = fma(-fac[r], rowk[j], j == col ? 0.0 : Ag[idx]);
-    }
-    __syncthreads();
-  }
-  for (int col = N - 1; col >= 0; --col) {   // undo the row interchanges: columns, in reverse
-    const int p = perm[col];
-    if (p != col)
-      for (int r = tid; r < N; r += nthr) {
-        const double t = Ag[(int64_t)r * N + col];
-        Ag[(int64_t)r * N + col] = Ag[(int64_t)r * N + p];
-        Ag[(int64_t)r * N + p] = t;
-      }
-    __syncthreads();
-  }
-  double *out = Ainv + K * (int64_t)(N * N);
-  for (int idx = tid; idx < N * N; idx += nthr) {
-    const int i = idx / N, j = idx - i * N;
-    out[idx] = dsc[i] * Ag[idx] * dsc[j];
   }
 }
 
@@ -949,12 +532,30 @@ __global__ void ho_convert_kernel(const Ta *__restrict__ x, Tb *__restrict__ y, 
   if (i < n) y[i] = (Tb)x[i];
 }
 
+// Gamma = (H 1) / (P^T S P 1) (Eq. scaling_matrix): P^T sums a facet's nodes with weight 1/2 (1 on
+// ground and lid facets), S 1 on a facet is the sum over its cells of S_K 1 (sk1 [6][ncell], summed over
+// the facet's nodes).
+__global__ void ho_gamma_kernel(int64_t ncell, int L, const int32_t *__restrict__ nbr,
+                                const int32_t *__restrict__ nbr_face, const double *__restrict__ m,
+                                const double *__restrict__ sk1, double *__restrict__ gamma) {
+  const int64_t K = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (K >= ncell) return;
+  const int c = (int)(K / L), k = (int)(K - (int64_t)c * L);
+  double s = 0.0;
+#pragma unroll
+  for (int f = 0; f < 4; ++f)
+    s += 0.5 * (sk1[f * ncell + K] + sk1[nbr_face[4 * (int64_t)c + f] * ncell + (int64_t)nbr[4 * (int64_t)c + f] * L + k]);
+  s += k == 0 ? sk1[4 * ncell + K] : 0.5 * (sk1[4 * ncell + K] + sk1[5 * ncell + K - 1]);
+  s += k == L - 1 ? sk1[5 * ncell + K] : 0.5 * (sk1[5 * ncell + K] + sk1[4 * ncell + K + 1]);
+  gamma[K] = m[K] / s;
+}
+
 __global__ void ho_fill_kernel(double *__restrict__ x, int64_t n, double v) {
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i < n) x[i] = v;
 }
 
-__global__ void ho_gamma_kernel(int64_t ncell, const double *__restrict__ m, double *__restrict__ gamma) {
+__global__ void ho_gamma_div_kernel(int64_t ncell, const double *__restrict__ m, double *__restrict__ gamma) {
   const int64_t K = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (K < ncell) gamma[K] = m[K] / gamma[K];   // gamma holds P^T S P 1 on entry
 }
@@ -1033,11 +634,13 @@ static int ho_build_fp32(Ctx *c) {
 
 void ho_free(Ctx *c) {
   HoData &h = c->ho;
-  double **bufs[] = {&h.tab, &h.S, &h.Ainv, &h.hw, &h.zf, &h.gamma, &h.m};
+  double **bufs[] = {&h.tab, &h.gtab, &h.ctab, &h.ltab, &h.S, &h.Ainv, &h.hw, &h.zf, &h.gamma, &h.m};
   for (double **b : bufs) {
     dev_free(c, *b);
     *b = nullptr;
   }
+  dev_free(c, h.itab);
+  h.itab = nullptr;
   dev_free(c, h.own);
   h.own = nullptr;
   dev_free(c, h.flag);
@@ -1053,6 +656,9 @@ void ho_free(Ctx *c) {
 }
 
 template <int P>
+static int ho_launch_spmv_p(Ctx *c, const double *x, double *y, int mode, const double *w, int slot0, int slot1);
+
+template <int P>
 static int ho_assemble_p(Ctx *c) {
   using H = Ho<P>;
   const Level &f = c->lv[0];
@@ -1062,10 +668,7 @@ static int ho_assemble_p(Ctx *c) {
   if (C > 0x7fffffff) return fail(c, HMG_ERR_INVALID_ARG, "too many cells for one launch");
   if (h.degree != P || h.ncell != C || h.T != ho_trace_size(c, P)) {   // (re)allocate for this degree and mesh
     ho_free(c);
-    std::vector<double> tab;
-    ho_tables<P>(tab);
-    if ((st = dev_alloc(c, &h.tab, tab.size()))) return st;
-    HMG_CUDA(c, cudaMemcpy(h.tab, tab.data(), sizeof(double) * tab.size(), cudaMemcpyHostToDevice));
+    if ((st = ho_make_tables<P>(c))) return st;
     const int64_t T = ho_trace_size(c, P);
     if ((st = dev_alloc(c, &h.S, (size_t)H::SLOTS * T))) return st;
     if ((st = dev_alloc(c, &h.Ainv, (size_t)H::N * H::N * C))) return st;
@@ -1074,7 +677,6 @@ static int ho_assemble_p(Ctx *c) {
     if ((st = dev_alloc(c, &h.gamma, (size_t)C))) return st;
     if ((st = dev_alloc(c, &h.m, (size_t)C))) return st;
     if ((st = dev_alloc(c, &h.own, (size_t)4 * f.ncol))) return st;
-    if ((st = dev_alloc(c, &h.flag, 1))) return st;
     h.degree = P;
     h.ncell = C;
     h.T = T;
@@ -1083,11 +685,9 @@ static int ho_assemble_p(Ctx *c) {
   HMG_CUDA(c, cudaMemsetAsync(h.own, 0, 4 * (size_t)f.ncol, c->stream));
   ho_own_kernel<<<grid_for(f.nedge, 256), 256, 0, c->stream>>>(f.edge_stencil, f.edge_fc, f.nedge, h.own);
   HMG_CUDA(c, cudaMemsetAsync(h.flag, 0, sizeof(int), c->stream));
-  HoCellArgs a{f.geometry, f.ncol, f.nlev, C, f.radius, c->sc.sigma, f.corners, f.z};
-  const size_t smem = HoCellSmem<P>::BYTES;
-  HMG_CUDA(c, cudaFuncSetAttribute(ho_cell_kernel<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  ho_cell_kernel<P><<<(unsigned)C, 256, smem, c->stream>>>(a, h.tab, h.Ainv, h.m, h.flag);
-  HMG_CUDA(c, cudaGetLastError());
+  double *sk1 = static_cast<double *>(c->w1);   // 6 C doubles of at least NB (3 C + ncol)
+  const bool gauss = c->opt.precision == HMG_PRECISION_MIXED;   // (gauss_cells.cu says why)
+  if ((st = gauss ? ho_gauss_cell_matrices<P>(c) : ho_cell_matrices<P>(c, sk1))) return st;
   int sing = 0;
   HMG_CUDA(c, cudaMemcpyAsync(&sing, h.flag, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
   HMG_CUDA(c, cudaStreamSynchronize(c->stream));
@@ -1095,13 +695,15 @@ static int ho_assemble_p(Ctx *c) {
   const HoGeo g = ho_geo<P>(c);
   ho_rows_kernel<P><<<grid_for(h.T, 256), 256, 0, c->stream>>>(g, h.T, h.tab, h.Ainv, h.S);
   HMG_CUDA(c, cudaGetLastError());
-  // Gamma = (H 1) / (P^T S P 1): S applied to the ones vector (P 1 = 1), then P^T
-  double *ones = static_cast<double *>(c->w1), *s1 = static_cast<double *>(c->w2);
-  ho_fill_kernel<<<grid_for(h.T, 256), 256, 0, c->stream>>>(ones, h.T, 1.0);
-  ho_spmv_kernel<P, 0><<<grid_for(g.nhf + g.nzf, kRedThreads), kRedThreads, 0, c->stream>>>(
-      g, h.T, h.S, ones, s1, nullptr, c->part, 0, 0);
-  ho_restrict_kernel<P, double><<<grid_for(C, 256), 256, 0, c->stream>>>(g, C, s1, nullptr, h.gamma);
-  ho_gamma_kernel<<<grid_for(C, 256), 256, 0, c->stream>>>(C, h.m, h.gamma);
+  if (gauss) {   // P^T S P 1 by the operator itself (P 1 = 1)
+    double *ones = sk1, *s1 = static_cast<double *>(c->w2);
+    ho_fill_kernel<<<grid_for(h.T, 256), 256, 0, c->stream>>>(ones, h.T, 1.0);
+    if ((st = ho_launch_spmv_p<P>(c, ones, s1, 0, nullptr, 0, 0))) return st;
+    ho_restrict_kernel<P, double><<<grid_for(C, 256), 256, 0, c->stream>>>(g, C, s1, nullptr, h.gamma);
+    ho_gamma_div_kernel<<<grid_for(C, 256), 256, 0, c->stream>>>(C, h.m, h.gamma);
+  } else {
+    ho_gamma_kernel<<<grid_for(C, 256), 256, 0, c->stream>>>(C, f.nlev, f.col_nbr, f.col_nbr_face, h.m, sk1, h.gamma);
+  }
   HMG_CUDA(c, cudaGetLastError());
   if ((st = ho_build_factors<P>(c))) return st;
   if (c->opt.precision == HMG_PRECISION_MIXED) return ho_build_fp32<P>(c);

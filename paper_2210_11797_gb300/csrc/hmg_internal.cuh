@@ -61,6 +61,7 @@ struct Level {
   double *z = nullptr;              // [nlev+1]
   double *theta_lev = nullptr, *exner_lev = nullptr, *exner = nullptr;
   double *ctab = nullptr, *ltab = nullptr;   // geometry sums per column and per level (assembly)
+  bool geo_ready = false;                    // they have been made (they depend on the mesh only)
   // assembled pressure operator (device)
   double *H = nullptr;              // [7][ncell]
   // Thomas factors of H_z with the relaxation mg_omega folded in (pivot p_k): omega / p_k,
@@ -99,6 +100,9 @@ struct HoData {
   double *m = nullptr;         // [ncell] sigma |K|_1 = (H 1)_K
   int8_t *own = nullptr;       // [ncol][4] 1 where the column owns the edge of its face
   double *tab = nullptr;       // reference-element tables
+  int *itab = nullptr;         // and their integer part
+  double *gtab = nullptr;      // tables of the direct Gauss sums (contexts with the FP32 preconditioner)
+  double *ctab = nullptr, *ltab = nullptr;   // geometry sums per column and per level
   int *flag = nullptr;         // singular-matrix flag of the assembly
   double factor_omega = 0.0;   // the omega the smoother factors hold
   // FP32 copies for the FP32 preconditioner (precision mixed): S, the smoother factors, Gamma
