@@ -25,63 +25,64 @@
 
 namespace hmg {
 
-// NB consecutive coefficients of one slot (the facet's rows) times x into acc: FP64 coefficients
-// as double2 pairs, FP32 ones (the FP32 preconditioner's copy) as float4 quads where NB allows
-template <int NB, bool NEG, typename TS, typename TA>
-__device__ __forceinline__ void ho_slot(const TS *__restrict__ s, TA xv, TA acc[NB]) {
-  if constexpr (sizeof(TS) == 8 && NB % 2 == 0) {
-#pragma unroll
-    for (int n = 0; n < NB; n += 2) {
-      const double2 v = __ldcs(reinterpret_cast<const double2 *>(s + n));
-      acc[n] = fma(NEG ? -(TA)v.x : (TA)v.x, xv, acc[n]);
-      acc[n + 1] = fma(NEG ? -(TA)v.y : (TA)v.y, xv, acc[n + 1]);
-    }
-  } else if constexpr (sizeof(TS) == 4 && NB % 4 == 0) {
-#pragma unroll
-    for (int n = 0; n < NB; n += 4) {
-      const float4 v = __ldcs(reinterpret_cast<const float4 *>(s + n));
-      acc[n] = fma(NEG ? -(TA)v.x : (TA)v.x, xv, acc[n]);
-      acc[n + 1] = fma(NEG ? -(TA)v.y : (TA)v.y, xv, acc[n + 1]);
-      acc[n + 2] = fma(NEG ? -(TA)v.z : (TA)v.z, xv, acc[n + 2]);
-      acc[n + 3] = fma(NEG ? -(TA)v.w : (TA)v.w, xv, acc[n + 3]);
-    }
-  } else {
-#pragma unroll
-    for (int n = 0; n < NB; ++n) {
-      const TA v = (TA)__ldcs(s + n);
-      acc[n] = fma(NEG ? -v : v, xv, acc[n]);
-    }
-  }
-}
+// Threads of the row kernels: one thread per trace row, whole facets per block (p = 2: 28 facets of nine
+// rows). A row's S coefficients are one value per slot, so the lanes of a warp read consecutive
+// addresses, and the NB rows of a facet read the same x value. One thread per facet with NB
+// accumulators instead spread a warp's loads over 32 lines and left most of the GPU idle on small
+// meshes (16 x 16 x 16 cells at p = 3: 49 blocks on 152 SMs, S apply 266 us).
+constexpr int kHoRowThreads = 256;
+template <int P>
+constexpr int kHoFacets = kHoRowThreads / Ho<P>::NB;   // facets per block
+template <int P>
+constexpr int kHoRows = kHoFacets<P> * Ho<P>::NB;      // rows per block
 
-// acc[n] (+/-)= sum over the stored slots of row NB F + n times x: cell A's NF facet dofs, then
-// cell B's without the shared facet (merged into A's slots when S was assembled). OFFD leaves out
+// acc (+/-)= sum over the stored slots of row NB F + n times x, in slot order: cell A's NF facet dofs,
+// then cell B's without the shared facet (merged into A's slots when S was assembled). OFFD leaves out
 // the couplings inside the smoother's diagonal block D of Algorithm 1 (acc - (S - D) x): on a
 // vertical facet its own nodes, on a horizontal facet the horizontal facets of its column (A's
 // bottom and top, B's bottom).
-template <int P, bool NEG, bool OFFD = false, typename TS = double, typename TX = double, typename TA = double>
-__device__ __forceinline__ void ho_rows(const TS *__restrict__ S, const TX *__restrict__ x, const HoGeo &g,
-                                        int64_t T, int64_t F, TA acc[Ho<P>::NB]) {
+template <int P, bool NEG, bool OFFD, typename TS, typename TX, typename TA>
+__device__ __forceinline__ TA ho_row(const TS *__restrict__ S, const TX *__restrict__ x, const HoGeo &g, int64_t T,
+                                     int64_t F, int n, TA acc) {
   using H = Ho<P>;
+  constexpr int NB = H::NB, NT = H::NT;
   const HoFacet fc = ho_facet(g, F);
-  const TS *Sr = S + (int64_t)H::NB * F;
   const bool vert = F < g.nhf;
-  constexpr int U = P == 1 ? 4 : 2;
-#pragma unroll U
-  for (int q = 0; q < H::NF; ++q) {
-    if (OFFD && (vert ? q / H::NB == fc.fA : q / H::NB >= 4)) continue;
-    const TA xv = (TA)__ldg(x + ho_gid<P>(g, fc.cA, fc.kA, q));
-    ho_slot<H::NB, NEG>(Sr + (int64_t)q * T, xv, acc);
-  }
-  if (fc.cB < 0) return;
-#pragma unroll U
-  for (int q = 0; q < H::NF; ++q) {
-    if (q / H::NB == fc.fB || (OFFD && !vert && q / H::NB >= 4)) continue;
-    const TA xv = (TA)__ldg(x + ho_gid<P>(g, fc.cB, fc.kB, q));
-    ho_slot<H::NB, NEG>(Sr + (int64_t)(H::NF + q) * T, xv, acc);
-  }
+  const TS *s = S + (int64_t)NB * F + n;
+  auto cell = [&](int c, int k, int shared, bool skip_shared) {
+#pragma unroll(P == 1 ? 3 : 1)
+    for (int f = 0; f < 6; ++f, s += (int64_t)NB * T) {
+      if ((skip_shared && f == shared) || (OFFD && !vert && f >= 4)) continue;
+      const TX *xf;      // the facet's first value in the cell's traversal, step per s
+      int ds = NT;
+      if (f < 4) {
+        const int64_t e = __ldg(g.col_edges + 4 * (int64_t)c + f);
+        xf = x + NB * (e * g.L + k);
+        if (!g.own[4 * (int64_t)c + f]) {
+          xf += NT * P;
+          ds = -NT;
+        }
+      } else {
+        xf = x + g.NH + NB * ((int64_t)c * (g.L + 1) + k + (f == 5 ? 1 : 0));
+      }
+      TS a[NB];
+      TX v[NB];
+#pragma unroll
+      for (int q = 0; q < NB; ++q) a[q] = __ldcs(s + (int64_t)q * T);
+#pragma unroll
+      for (int q = 0; q < NT; ++q)
+#pragma unroll
+        for (int t = 0; t < NT; ++t) v[q * NT + t] = __ldg(xf + q * ds + t);
+#pragma unroll
+      for (int q = 0; q < NB; ++q) acc = fma(NEG ? -(TA)a[q] : (TA)a[q], (TA)v[q], acc);
+    }
+  };
+  cell(fc.cA, fc.kA, fc.fA, OFFD && vert);
+  if (fc.cB >= 0) cell(fc.cB, fc.kB, fc.fB, true);
+  return acc;
 }
 
+// ---- assembly -------------------------------------------------------------------------------
 // own[c][f] = 1 where column c owns the edge of its face f (each entry written by one edge)
 __global__ void ho_own_kernel(const int32_t *__restrict__ stencil, const int32_t *__restrict__ edge_fc, int nedge,
                               int8_t *__restrict__ own) {
@@ -171,8 +172,9 @@ __device__ bool warp_gauss_jordan(double *W, int lane) {
 constexpr int kHoFacWarps = 4;   // warps per block of the factor kernels
 
 // omega times the inverse of each vertical facet's NB x NB block of S (the Jacobi part of
-// Algorithm 1), entry (n, m) at hw[(NB n + m) nhf + F]; one warp per facet. The facet block lives
-// in the slots of cell A's face (A owns the edge, so its local nodes are the facet's).
+// Algorithm 1), entry (n, m) at hw[NB^2 F + NB m + n] (the rows of a facet, one lane each, read one run
+// per m); one warp per facet. The facet block lives in the slots of cell A's face (A owns the edge, so
+// its local nodes are the facet's).
 template <int P>
 __global__ void __launch_bounds__(32 * kHoFacWarps)
     ho_hfactor_kernel(const HoGeo g, int64_t T, const double *__restrict__ S, double omega,
@@ -193,7 +195,7 @@ __global__ void __launch_bounds__(32 * kHoFacWarps)
   if (!warp_gauss_jordan<NB>(W, lane) && lane == 0) atomicExch(singular, 1);
   for (int e = lane; e < NB * NB; e += 32) {
     const int n = e / NB, m = e - n * NB;
-    hw[(int64_t)(NB * n + m) * g.nhf + F] = omega * W[n * W2 + NB + m];
+    hw[(int64_t)NB * NB * F + NB * m + n] = omega * W[n * W2 + NB + m];
   }
 }
 
@@ -264,54 +266,184 @@ __global__ void __launch_bounds__(32 * kHoFacWarps)
 }
 
 // ---- the operator, the right-hand side and the recovery --------------------------------------
-// y = S x, one thread per facet (its NB rows share the gathered values); MODE 1, 2, 3 fuse the
-// inner products of the Krylov loop as the lowest-order S apply does (3: (b - S x, b - S x), no y).
+// y = S x, one thread per row; MODE 1, 2, 3 fuse the inner products of the Krylov loop as the
+// lowest-order S apply does (3: (b - S x, b - S x), no y): a facet's products are summed in row order by
+// one thread into fs[F] (and fs[nF + F]), which ho_reduce_kernel adds up.
 template <int P, int MODE>
-__global__ void __launch_bounds__(kRedThreads)
+__global__ void __launch_bounds__(kHoRowThreads)
     ho_spmv_kernel(const HoGeo g, int64_t T, const double *__restrict__ S, const double *__restrict__ x,
-                   double *__restrict__ y, const double *__restrict__ w, double *part, int slot0, int slot1) {
-  constexpr int NB = Ho<P>::NB;
-  const int64_t F = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  double a0 = 0.0, a1 = 0.0;
-  if (F < g.nhf + g.nzf) {
-    double acc[NB];
-    const int64_t r0 = (int64_t)NB * F;
-    if (MODE == 3) {
-#pragma unroll
-      for (int n = 0; n < NB; ++n) acc[n] = __ldg(w + r0 + n);
-      ho_rows<P, true>(S, x, g, T, F, acc);
-#pragma unroll
-      for (int n = 0; n < NB; ++n) a0 = fma(acc[n], acc[n], a0);
-    } else {
-#pragma unroll
-      for (int n = 0; n < NB; ++n) acc[n] = 0.0;
-      ho_rows<P, false>(S, x, g, T, F, acc);
+                   double *__restrict__ y, const double *__restrict__ w, double *__restrict__ fs) {
+  constexpr int NB = Ho<P>::NB, FB = kHoFacets<P>;
+  __shared__ double sv[MODE ? kHoRows<P> : 1], sw[MODE == 1 || MODE == 2 ? kHoRows<P> : 1];
+  const int i = threadIdx.x;
+  const int64_t row = (int64_t)blockIdx.x * kHoRows<P> + i, F = (int64_t)blockIdx.x * FB + i / NB;
+  if (i < kHoRows<P> && row < T) {
+    const double v = MODE == 3 ? ho_row<P, true, false>(S, x, g, T, F, i % NB, __ldg(w + row))
+                               : ho_row<P, false, false>(S, x, g, T, F, i % NB, 0.0);
+    if (MODE != 3) y[row] = v;
+    if (MODE) sv[i] = v;
+    if (MODE == 1 || MODE == 2) sw[i] = __ldg(w + row);
+  }
+  if (MODE) {
+    __syncthreads();
+    const int64_t f = (int64_t)blockIdx.x * FB + i, nF = g.nhf + g.nzf;
+    if (i < FB && f < nF) {
+      double a0 = 0.0, a1 = 0.0;
 #pragma unroll
       for (int n = 0; n < NB; ++n) {
-        y[r0 + n] = acc[n];
-        if (MODE == 1) a0 = fma(__ldg(w + r0 + n), acc[n], a0);
-        if (MODE == 2) { a0 = fma(acc[n], __ldg(w + r0 + n), a0); a1 = fma(acc[n], acc[n], a1); }
+        const double v = sv[i * NB + n];
+        if (MODE == 1) a0 = fma(sw[i * NB + n], v, a0);
+        if (MODE == 2) a0 = fma(v, sw[i * NB + n], a0);
+        if (MODE == 2) a1 = fma(v, v, a1);
+        if (MODE == 3) a0 = fma(v, v, a0);
       }
+      fs[f] = a0;
+      if (MODE == 2) fs[nF + f] = a1;
     }
   }
-  if (MODE == 1 || MODE == 3) {
-    const double val[1] = {a0};
-    const int sl[1] = {slot0};
-    block_partials<1>(val, sl, part);
-  } else if (MODE == 2) {
-    const double val[2] = {a0, a1};
-    const int sl[2] = {slot0, slot1};
-    block_partials<2>(val, sl, part);
+}
+
+// The sums of the facets' partial products: a warp adds 256 facets (eight per lane, then a shuffle
+// tree) into part[slot][group]; the last block adds the groups into scal. Fixed order, and the order of
+// block_sum and finalize_kernel over blocks of 256 facets.
+template <int NV>
+__global__ void __launch_bounds__(256)
+    ho_reduce_kernel(const double *__restrict__ fs, int64_t nF, int slot0, int slot1, double *part,
+                     unsigned int *counter, double *scal) {
+  __shared__ double sh[NV][32];
+  __shared__ bool is_last;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int ng = (int)((nF + 255) / 256), grp = blockIdx.x * 8 + warp;
+  if (grp < ng) {
+#pragma unroll
+    for (int q = 0; q < NV; ++q) {
+      double f[8];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const int64_t F = (int64_t)grp * 256 + lane + 32 * j;
+        f[j] = F < nF ? fs[q * nF + F] : 0.0;
+      }
+      double v = f[0];
+#pragma unroll
+      for (int j = 1; j < 8; ++j) v += f[j];
+      v = warp_sum(v);
+      if (lane == 0) part[(int64_t)(q ? slot1 : slot0) * kMaxRedBlocks + grp] = v;
+    }
   }
+  __threadfence();   // every warp's partials before the block's ticket
+  __syncthreads();
+  if (threadIdx.x == 0) is_last = atomicAdd(&counter[slot0], 1u) == gridDim.x - 1;
+  __syncthreads();
+  if (!is_last) return;
+  __threadfence();
+#pragma unroll
+  for (int q = 0; q < NV; ++q) {
+    const double *p = part + (int64_t)(q ? slot1 : slot0) * kMaxRedBlocks;
+    for (int j = 0; j < 4; ++j) {   // the 1024 threads of finalize_kernel
+      double acc[4] = {0.0, 0.0, 0.0, 0.0};
+      int b = threadIdx.x + 256 * j;
+      for (; b + 3 * 1024 < ng; b += 4 * 1024) {
+        acc[0] += __ldcg(p + b);
+        acc[1] += __ldcg(p + b + 1024);
+        acc[2] += __ldcg(p + b + 2048);
+        acc[3] += __ldcg(p + b + 3072);
+      }
+      for (; b < ng; b += 1024) acc[0] += __ldcg(p + b);
+      const double v = warp_sum((acc[0] + acc[1]) + (acc[2] + acc[3]));
+      if (lane == 0) sh[q][warp + 8 * j] = v;
+    }
+  }
+  __syncthreads();
+  if (threadIdx.x < NV) {
+    double s = 0.0;
+    for (int i = 0; i < 32; ++i) s += sh[threadIdx.x][i];
+    scal[threadIdx.x ? slot1 : slot0] = s;
+  }
+  if (threadIdx.x == 0) counter[slot0] = 0u;
+}
+
+// ---- products with A_K^-1 ----------------------------------------------------------------------
+// One block per cell, one thread per row, each row's dot product in column order. A warp stages its 32
+// rows 16 columns at a time through shared memory (cp.async, two tiles in flight), so that the loads are
+// runs along the rows; one thread per row straight from global memory touched 32 lines per load (p = 3,
+// 4,096 cells: recovery 1,402 us, 0.3 of HBM bandwidth).
+constexpr int kHoTile = 16;
+
+__device__ __forceinline__ void cp_async8(double *smem, const double *gmem) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((unsigned)__cvta_generic_to_shared(smem)), "l"(gmem));
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int NLEFT>
+__device__ __forceinline__ void cp_async_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(NLEFT) : "memory");
+}
+
+// sum_j I[row][j] r[j] for this thread's row (rows past `rows` give 0); r in shared memory, tile: this
+// warp's 2 x 32 x (kHoTile + 1) doubles
+template <int N>
+__device__ __forceinline__ double ho_row_dot(const double *__restrict__ I, int rows, const double *r, double *tile) {
+  constexpr int LD = kHoTile + 1, NTILE = (N + kHoTile - 1) / kHoTile;
+  const int lane = threadIdx.x & 31, row0 = threadIdx.x & ~31;
+  auto stage = [&](int j) {
+    double *t = tile + (j & 1) * 32 * LD;
+    const int col = j * kHoTile + (lane & (kHoTile - 1));
+#pragma unroll
+    for (int q = 0; q < 32; q += 2) {
+      const int rr = q + (lane >> 4);
+      if (row0 + rr < rows && col < N) cp_async8(t + rr * LD + (lane & (kHoTile - 1)), I + (int64_t)(row0 + rr) * N + col);
+    }
+    cp_async_commit();
+  };
+  static_assert(kHoTile == 16, "two rows per warp load");
+  stage(0);
+  double v = 0.0;
+  for (int j = 0; j < NTILE; ++j) {
+    if (j + 1 < NTILE) {
+      stage(j + 1);
+      cp_async_wait<1>();
+    } else {
+      cp_async_wait<0>();
+    }
+    __syncwarp();
+    const double *t = tile + (j & 1) * 32 * LD + lane * LD, *rj = r + j * kHoTile;
+    const int m = N - j * kHoTile < kHoTile ? N - j * kHoTile : kHoTile;
+    if (row0 + lane < rows) {
+      if (m == kHoTile) {
+#pragma unroll
+        for (int q = 0; q < kHoTile; ++q) v = fma(t[q], rj[q], v);
+      } else {
+        for (int q = 0; q < m; ++q) v = fma(t[q], rj[q], v);
+      }
+    }
+    __syncwarp();   // the tile is staged again two steps on
+  }
+  return v;
+}
+
+// d[q] = (A_K^-1 R_K)_q on the facet dofs q < NF of cell K, in two halves of NF / 2 per cell
+template <int P>
+__global__ void __launch_bounds__(((Ho<P>::NF + 31) / 32) * 32)
+    ho_cell_rhs_kernel(const double *__restrict__ Ainv, const double *__restrict__ Ru, const double *__restrict__ Rp,
+                       double *__restrict__ d0, double *__restrict__ d1) {
+  using H = Ho<P>;
+  constexpr int N = H::N, NW = (H::NF + 31) / 32;
+  __shared__ double r[N], tile[NW][2 * 32 * (kHoTile + 1)];
+  const int64_t K = blockIdx.x;
+  for (int j = threadIdx.x; j < N; j += 32 * NW) r[j] = j < H::NU ? Ru[K * H::NU + j] : Rp[K * H::NP + (j - H::NU)];
+  __syncthreads();
+  const double v = ho_row_dot<N>(Ainv + K * (int64_t)(N * N), H::NF, r, tile[threadIdx.x >> 5]);
+  const int q = threadIdx.x;
+  constexpr int HF = H::NF / 2;
+  if (q < HF) d0[K * HF + q] = v;
+  else if (q < H::NF) d1[K * HF + q - HF] = v;
 }
 
 // B_lambda row NB F + n: the sum over the facet's cells of C_K (A_K^-1 R_K) at the node's local dof
 template <int P>
-__global__ void ho_rhs_kernel(const HoGeo g, int64_t T, const double *__restrict__ tab,
-                              const double *__restrict__ Ainv, const double *__restrict__ Ru,
-                              const double *__restrict__ Rp, double *__restrict__ B) {
+__global__ void ho_rhs_kernel(const HoGeo g, int64_t T, const double *__restrict__ tab, const double *__restrict__ d0,
+                              const double *__restrict__ d1, double *__restrict__ B) {
   using H = Ho<P>;
-  constexpr int N = H::N;
+  constexpr int HF = H::NF / 2;
   const int64_t row = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (row >= T) return;
   const int64_t F = row / H::NB;
@@ -319,48 +451,43 @@ __global__ void ho_rhs_kernel(const HoGeo g, int64_t T, const double *__restrict
   const HoFacet fc = ho_facet(g, F);
   auto cell = [&](int cc, int kk, int q) {
     const int64_t K = (int64_t)cc * g.L + kk;
-    const double *I = Ainv + K * (int64_t)(N * N) + (int64_t)q * N;
-    double v = 0.0;
-    for (int j = 0; j < H::NU; ++j) v = fma(I[j], Ru[K * H::NU + j], v);
-    for (int j = 0; j < H::NP; ++j) v = fma(I[H::NU + j], Rp[K * H::NP + j], v);
-    return v;
+    return q < HF ? d0[K * HF + q] : d1[K * HF + q - HF];
   };
   double v = cell(fc.cA, fc.kA, H::NB * fc.fA + n);
   if (fc.cB >= 0) v += cell(fc.cB, fc.kB, H::NB * fc.fB + H::NT * (fc.flipB ? P - s : s) + t);
   B[row] = tab[H::TC + n] * v;
 }
 
-// X_K = A_K^-1 (R_K - C_K lambda_K): u [ncell][NU], pi [ncell][NP]; one thread per (cell, dof)
+// X_K = A_K^-1 (R_K - C_K lambda_K): u [ncell][NU], pi [ncell][NP]
 template <int P>
-__global__ void ho_reconstruct_kernel(const HoGeo g, int64_t ncell, const double *__restrict__ tab,
-                                      const double *__restrict__ Ainv, const double *__restrict__ lam,
-                                      const double *__restrict__ Ru, const double *__restrict__ Rp,
-                                      double *__restrict__ u, double *__restrict__ pi) {
+__global__ void __launch_bounds__(((Ho<P>::N + 31) / 32) * 32)
+    ho_reconstruct_kernel(const HoGeo g, const double *__restrict__ tab, const double *__restrict__ Ainv,
+                          const double *__restrict__ lam, const double *__restrict__ Ru, const double *__restrict__ Rp,
+                          double *__restrict__ u, double *__restrict__ pi) {
   using H = Ho<P>;
-  constexpr int N = H::N;
-  const int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (idx >= ncell * N) return;
-  const int64_t K = idx / N;
-  const int i = (int)(idx - K * N);
+  constexpr int N = H::N, NW = (N + 31) / 32;
+  extern __shared__ __align__(16) double hr_smem[];   // r [N], then the warps' tiles
+  const int64_t K = blockIdx.x;
   const int c = (int)(K / g.L), k = (int)(K - (int64_t)c * g.L);
-  const double *I = Ainv + K * (int64_t)(N * N) + (int64_t)i * N;
-  double v = 0.0;
-  for (int j = 0; j < H::NU; ++j) {
-    double r = Ru[K * H::NU + j];
-    if (j < H::NF) r = fma(-tab[H::TC + j % H::NB], lam[ho_gid<P>(g, c, k, j)], r);
-    v = fma(I[j], r, v);
+  double *r = hr_smem, *tile = r + N + (threadIdx.x >> 5) * (2 * 32 * (kHoTile + 1));
+  for (int j = threadIdx.x; j < N; j += 32 * NW) {
+    double v = j < H::NU ? Ru[K * H::NU + j] : Rp[K * H::NP + (j - H::NU)];
+    if (j < H::NF) v = fma(-tab[H::TC + j % H::NB], lam[ho_gid<P>(g, c, k, j)], v);
+    r[j] = v;
   }
-  for (int j = 0; j < H::NP; ++j) v = fma(I[H::NU + j], Rp[K * H::NP + j], v);
+  __syncthreads();
+  const double v = ho_row_dot<N>(Ainv + K * (int64_t)(N * N), N, r, tile);
+  const int i = threadIdx.x;
   if (i < H::NU) u[K * H::NU + i] = v;
-  else pi[K * H::NP + (i - H::NU)] = v;
+  else if (i < N) pi[K * H::NP + (i - H::NU)] = v;
 }
 
 // ---- Algorithm 1 at p >= 1 ------------------------------------------------------------------------
 // lam_out = lam_in + omega D^-1 (b - S lam_in) (ZERO: lam_in = 0), evaluated as
 // (1 - omega) lam_in + omega D^-1 (b - (S - D) lam_in): equal in exact arithmetic, without the
-// couplings of a row inside D. Two launches per sweep. Part 1, one thread per facet (all facets,
-// as parallel as the S apply): the residual rows r = b - (S - D) lam_in; on a vertical facet the
-// NB x NB block Jacobi step lam_out = keep lam_in + (omega D_F^-1) r at once, on a horizontal
+// couplings of a row inside D. Two launches per sweep. Part 1, one thread per row (as parallel as the
+// S apply): the residual rows r = b - (S - D) lam_in; on a vertical facet the NB x NB block Jacobi step
+// lam_out = keep lam_in + (omega D_F^-1) r at once (the facet's r in shared memory), on a horizontal
 // facet r is parked in lam_out's rows (ZERO: vertical facets only, r = b). Part 2, the line
 // solves: each column's r staged in shared memory, the block Thomas recurrences with LPC lanes
 // per column (lane n < NB computes component n of each NB x NB product from its rows of the
@@ -369,28 +496,31 @@ __global__ void ho_reconstruct_kernel(const HoGeo g, int64_t ncell, const double
 // type (double, or float in the FP32 preconditioner, whose b is the FP64 Krylov residual and
 // whose last sweep writes FP64).
 template <int P, bool ZERO, typename T = double, typename Tb = double, typename Tin = double, typename Tout = double>
-__global__ void __launch_bounds__(kRedThreads)
+__global__ void __launch_bounds__(kHoRowThreads)
     ho_sweep_rows_kernel(const HoGeo g, int64_t TT, const T *__restrict__ S, const T *__restrict__ hw,
                          const Tb *__restrict__ b, const Tin *__restrict__ lam_in,
                          Tout *__restrict__ lam_out, double keep) {
   constexpr int NB = Ho<P>::NB;
-  const int64_t F = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (F >= (ZERO ? g.nhf : g.nhf + g.nzf)) return;
-  const int64_t r0 = (int64_t)NB * F;
-  T acc[NB];
-#pragma unroll
-  for (int n = 0; n < NB; ++n) acc[n] = (T)__ldg(b + r0 + n);
-  if (!ZERO) ho_rows<P, true, true>(S, lam_in, g, TT, F, acc);
+  __shared__ T sr[kHoRows<P>];
+  const int i = threadIdx.x, n = i % NB;
+  const int64_t row = (int64_t)blockIdx.x * kHoRows<P> + i, F = (int64_t)blockIdx.x * kHoFacets<P> + i / NB;
+  const bool act = i < kHoRows<P> && row < (ZERO ? g.NH : TT);
+  T r = (T)0;
+  if (act) {
+    r = (T)__ldg(b + row);
+    if (!ZERO) r = ho_row<P, true, true>(S, lam_in, g, TT, F, n, r);
+    sr[i] = r;
+  }
+  __syncthreads();
+  if (!act) return;
   if (F < g.nhf) {
-    for (int n = 0; n < NB; ++n) {
-      T v = ZERO ? (T)0 : (T)keep * (T)lam_in[r0 + n];
+    const T *f = hw + (int64_t)NB * NB * F + n, *rf = sr + (i - n);
+    T v = ZERO ? (T)0 : (T)keep * (T)lam_in[row];
 #pragma unroll
-      for (int m = 0; m < NB; ++m) v = fma(hw[(int64_t)(NB * n + m) * g.nhf + F], acc[m], v);
-      lam_out[r0 + n] = (Tout)v;
-    }
+    for (int m = 0; m < NB; ++m) v = fma(__ldg(f + NB * m), rf[m], v);
+    lam_out[row] = (Tout)v;
   } else {
-#pragma unroll
-    for (int n = 0; n < NB; ++n) lam_out[r0 + n] = (Tout)acc[n];
+    lam_out[row] = (Tout)r;
   }
 }
 
@@ -474,24 +604,18 @@ __global__ void __launch_bounds__(128)
     lam_out[base + i] = (Tout)(ZERO ? sr[i] : fma((T)keep, (T)lam_in[base + i], sr[i]));
 }
 
-// R = b - S lam (Algorithm 2 line 3), one thread per facet. ZSWEEP: lam is one sweep from zero,
+// R = b - S lam (Algorithm 2 line 3), one thread per row. ZSWEEP: lam is one sweep from zero,
 // lam = omega D^-1 b, so R = (1 - omega) b - (S - D) lam (equal in exact arithmetic).
 template <int P, bool ZSWEEP, typename T = double>
-__global__ void ho_residual_kernel(const HoGeo g, int64_t TT, const T *__restrict__ S,
-                                   const double *__restrict__ b, const T *__restrict__ lam,
-                                   T *__restrict__ R, double keep) {
+__global__ void __launch_bounds__(kHoRowThreads)
+    ho_residual_kernel(const HoGeo g, int64_t TT, const T *__restrict__ S, const double *__restrict__ b,
+                       const T *__restrict__ lam, T *__restrict__ R, double keep) {
   constexpr int NB = Ho<P>::NB;
-  const int64_t F = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (F >= g.nhf + g.nzf) return;
-  T acc[NB];
-#pragma unroll
-  for (int n = 0; n < NB; ++n) {
-    const T bv = (T)__ldg(b + (int64_t)NB * F + n);
-    acc[n] = ZSWEEP ? (T)keep * bv : bv;
-  }
-  ho_rows<P, true, ZSWEEP>(S, lam, g, TT, F, acc);
-#pragma unroll
-  for (int n = 0; n < NB; ++n) R[(int64_t)NB * F + n] = acc[n];
+  const int i = threadIdx.x;
+  const int64_t row = (int64_t)blockIdx.x * kHoRows<P> + i, F = (int64_t)blockIdx.x * kHoFacets<P> + i / NB;
+  if (i >= kHoRows<P> || row >= TT) return;
+  const T bv = (T)__ldg(b + row);
+  R[row] = ho_row<P, true, ZSWEEP>(S, lam, g, TT, F, i % NB, ZSWEEP ? (T)keep * bv : bv);
 }
 
 // bbar_K = Gamma_K (P^T R)_K (Algorithm 2 lines 4-5): P is constant on a facet (all its nodes)
@@ -634,7 +758,7 @@ static int ho_build_fp32(Ctx *c) {
 
 void ho_free(Ctx *c) {
   HoData &h = c->ho;
-  double **bufs[] = {&h.tab, &h.gtab, &h.ctab, &h.ltab, &h.S, &h.Ainv, &h.hw, &h.zf, &h.gamma, &h.m};
+  double **bufs[] = {&h.tab, &h.gtab, &h.ctab, &h.ltab, &h.S, &h.Ainv, &h.hw, &h.zf, &h.gamma, &h.m, &h.fs};
   for (double **b : bufs) {
     dev_free(c, *b);
     *b = nullptr;
@@ -677,6 +801,7 @@ static int ho_assemble_p(Ctx *c) {
     if ((st = dev_alloc(c, &h.gamma, (size_t)C))) return st;
     if ((st = dev_alloc(c, &h.m, (size_t)C))) return st;
     if ((st = dev_alloc(c, &h.own, (size_t)4 * f.ncol))) return st;
+    if ((st = dev_alloc(c, &h.fs, (size_t)2 * (T / H::NB)))) return st;
     h.degree = P;
     h.ncell = C;
     h.T = T;
@@ -714,17 +839,21 @@ template <int P>
 static int ho_launch_spmv_p(Ctx *c, const double *x, double *y, int mode, const double *w, int slot0, int slot1) {
   const HoData &h = c->ho;
   const HoGeo g = ho_geo<P>(c);
-  const unsigned grid = grid_for(g.nhf + g.nzf, kRedThreads);
-  if (grid > (unsigned)kMaxRedBlocks) return fail(c, HMG_ERR_INVALID_ARG, "too many facets for one reduction");
+  const int64_t nF = g.nhf + g.nzf;
+  if (grid_for(nF, 256) > (unsigned)kMaxRedBlocks)
+    return fail(c, HMG_ERR_INVALID_ARG, "too many facets for one reduction");
+  const unsigned grid = grid_for(h.T, kHoRows<P>);
   Prof prof(c, kCompApply);
   switch (mode) {
-    case 0: ho_spmv_kernel<P, 0><<<grid, kRedThreads, 0, c->stream>>>(g, h.T, h.S, x, y, w, c->part, slot0, slot1); break;
-    case 1: ho_spmv_kernel<P, 1><<<grid, kRedThreads, 0, c->stream>>>(g, h.T, h.S, x, y, w, c->part, slot0, slot1); break;
-    case 2: ho_spmv_kernel<P, 2><<<grid, kRedThreads, 0, c->stream>>>(g, h.T, h.S, x, y, w, c->part, slot0, slot1); break;
-    default: ho_spmv_kernel<P, 3><<<grid, kRedThreads, 0, c->stream>>>(g, h.T, h.S, x, y, w, c->part, slot0, slot1); break;
+    case 0: ho_spmv_kernel<P, 0><<<grid, kHoRowThreads, 0, c->stream>>>(g, h.T, h.S, x, y, w, h.fs); break;
+    case 1: ho_spmv_kernel<P, 1><<<grid, kHoRowThreads, 0, c->stream>>>(g, h.T, h.S, x, y, w, h.fs); break;
+    case 2: ho_spmv_kernel<P, 2><<<grid, kHoRowThreads, 0, c->stream>>>(g, h.T, h.S, x, y, w, h.fs); break;
+    default: ho_spmv_kernel<P, 3><<<grid, kHoRowThreads, 0, c->stream>>>(g, h.T, h.S, x, y, w, h.fs); break;
   }
+  const unsigned rg = grid_for(nF, 2048);
+  if (mode == 2) ho_reduce_kernel<2><<<rg, 256, 0, c->stream>>>(h.fs, nF, slot0, slot1, c->part, c->counter, c->scal);
+  else if (mode) ho_reduce_kernel<1><<<rg, 256, 0, c->stream>>>(h.fs, nF, slot0, 0, c->part, c->counter, c->scal);
   HMG_CUDA(c, cudaGetLastError());
-  if (mode != 0) return launch_finalize(c, (int)grid, slot0, mode == 2 ? slot1 : -1);
   return HMG_OK;
 }
 
@@ -732,16 +861,21 @@ template <int P>
 static int ho_trace_rhs_p(Ctx *c, const double *Ru, const double *Rp, double *B) {
   const HoData &h = c->ho;
   Prof prof(c, kCompRhs);
-  ho_rhs_kernel<P><<<grid_for(h.T, 128), 128, 0, c->stream>>>(ho_geo<P>(c), h.T, h.tab, h.Ainv, Ru, Rp, B);
+  // the cells' products pass through the preconditioner's work vectors (T >= 3 NB C = NF / 2 C doubles each)
+  double *d0 = static_cast<double *>(c->w1), *d1 = static_cast<double *>(c->w2);
+  ho_cell_rhs_kernel<P><<<(unsigned)c->lv[0].ncell, ((Ho<P>::NF + 31) / 32) * 32, 0, c->stream>>>(h.Ainv, Ru, Rp, d0, d1);
+  ho_rhs_kernel<P><<<grid_for(h.T, 256), 256, 0, c->stream>>>(ho_geo<P>(c), h.T, h.tab, d0, d1, B);
   HMG_CUDA(c, cudaGetLastError());
   return HMG_OK;
 }
 
 template <int P>
 static int ho_reconstruct_p(Ctx *c, const double *lam, const double *Ru, const double *Rp, double *u, double *pi) {
-  const int64_t C = c->lv[0].ncell;
-  ho_reconstruct_kernel<P><<<grid_for(C * Ho<P>::N, 128), 128, 0, c->stream>>>(ho_geo<P>(c), C, c->ho.tab,
-                                                                              c->ho.Ainv, lam, Ru, Rp, u, pi);
+  constexpr int NW = (Ho<P>::N + 31) / 32;
+  const int smem = (int)sizeof(double) * (Ho<P>::N + NW * 2 * 32 * (kHoTile + 1));
+  HMG_CUDA(c, cudaFuncSetAttribute(ho_reconstruct_kernel<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+  ho_reconstruct_kernel<P><<<(unsigned)c->lv[0].ncell, 32 * NW, smem, c->stream>>>(ho_geo<P>(c), c->ho.tab, c->ho.Ainv,
+                                                                                 lam, Ru, Rp, u, pi);
   HMG_CUDA(c, cudaGetLastError());
   return HMG_OK;
 }
@@ -778,7 +912,7 @@ static int ho_sweep(Ctx *c, const double *b, const Tin *lam_in, Tout *lam_out) {
   const double keep = 1.0 - h.factor_omega;
   Prof prof(c, ZERO ? kCompPresmooth : kCompSweep, 2);
   ho_sweep_rows_kernel<P, ZERO, T, double, Tin, Tout>
-      <<<grid_for(ZERO ? g.nhf : g.nhf + g.nzf, kRedThreads), kRedThreads, 0, c->stream>>>(
+      <<<grid_for(ZERO ? g.NH : h.T, kHoRows<P>), kHoRowThreads, 0, c->stream>>>(
           g, h.T, HoPrec<T>::S(h), HoPrec<T>::hw(h), b, lam_in, lam_out, keep);
   if constexpr (ZERO)
     ho_sweep_lines_kernel<P, ZERO, T, double, Tin, Tout><<<nzb, 128, smem, c->stream>>>(g, cpb, HoPrec<T>::zf(h), b,
@@ -852,10 +986,10 @@ static int ho_precond_p(Ctx *c, const double *r, double *z) {
   {
     Prof pr(c, kCompResidual, 2);
     if (c->opt.n_pre == 1)   // w1 is one sweep from zero                                       // line 3
-      ho_residual_kernel<P, true, T><<<grid_for(g.nhf + g.nzf, 128), 128, 0, c->stream>>>(
+      ho_residual_kernel<P, true, T><<<grid_for(TT, kHoRows<P>), kHoRowThreads, 0, c->stream>>>(
           g, TT, HoPrec<T>::S(h), r, w1, w2, 1.0 - h.factor_omega);
     else
-      ho_residual_kernel<P, false, T><<<grid_for(g.nhf + g.nzf, 128), 128, 0, c->stream>>>(
+      ho_residual_kernel<P, false, T><<<grid_for(TT, kHoRows<P>), kHoRowThreads, 0, c->stream>>>(
           g, TT, HoPrec<T>::S(h), r, w1, w2, 0.0);
     ho_restrict_kernel<P, T><<<grid_for(C, 256), 256, 0, c->stream>>>(g, C, w2, HoPrec<T>::gamma(h), cb);   // lines 4-5
     HMG_CUDA(c, cudaGetLastError());

@@ -94,10 +94,11 @@ struct HoData {
   int64_t T = 0;               // trace rows: NB per facet
   double *S = nullptr;         // [2 NF][T] two cells x NF facet-dof coefficients per row
   double *Ainv = nullptr;      // [ncell][N][N] A_K^-1
-  double *hw = nullptr;        // [NB^2][vertical facets] omega (facet block of S)^-1
+  double *hw = nullptr;        // [vertical facets][NB][NB] omega (facet block of S)^-1 (transposed)
   double *zf = nullptr;        // [horizontal facets][3][NB][NB] block Thomas factors of S^zz (transposed)
   double *gamma = nullptr;     // [ncell] Gamma of Eq. scaling_matrix
   double *m = nullptr;         // [ncell] sigma |K|_1 = (H 1)_K
+  double *fs = nullptr;        // [2][facets] partial products of the S apply's reductions
   int8_t *own = nullptr;       // [ncol][4] 1 where the column owns the edge of its face
   double *tab = nullptr;       // reference-element tables
   int *itab = nullptr;         // and their integer part

@@ -75,8 +75,9 @@ struct HoFacet {
 
 __device__ __forceinline__ HoFacet ho_facet(const HoGeo &g, int64_t F) {
   HoFacet r;
-  if (F < g.nhf) {
-    const int e = (int)(F / g.L), k = (int)(F - (int64_t)e * g.L);
+  if (F < g.nhf) {   // (facets number less than 2^31: 32-bit index arithmetic)
+    const unsigned Fu = (unsigned)F, Lu = (unsigned)g.L;
+    const int e = (int)(Fu / Lu), k = (int)(Fu - (unsigned)e * Lu);
     r.cA = g.stencil[8 * (int64_t)e];
     r.cB = g.stencil[8 * (int64_t)e + 1];
     r.fA = g.edge_fc[2 * (int64_t)e];
@@ -84,8 +85,8 @@ __device__ __forceinline__ HoFacet ho_facet(const HoGeo &g, int64_t F) {
     r.kA = r.kB = k;
     r.flipB = true;
   } else {
-    const int64_t zf = F - g.nhf;
-    const int c = (int)(zf / (g.L + 1)), k = (int)(zf - (int64_t)c * (g.L + 1));
+    const unsigned zf = (unsigned)(F - g.nhf), L1 = (unsigned)g.L + 1u;
+    const int c = (int)(zf / L1), k = (int)(zf - (unsigned)c * L1);
     r.cA = c;
     r.flipB = false;
     if (k < g.L) {
