@@ -362,41 +362,99 @@ __global__ void __launch_bounds__(256)
   if (threadIdx.x == 0) counter[slot0] = 0u;
 }
 
-// ---- products with A_K^-1 ----------------------------------------------------------------------
-// One block per cell, one thread per row, each row's dot product in column order. A warp stages its 32
-// rows 16 columns at a time through shared memory (cp.async, two tiles in flight), so that the loads are
-// runs along the rows; one thread per row straight from global memory touched 32 lines per load (p = 3,
-// 4,096 cells: recovery 1,402 us, 0.3 of HBM bandwidth).
-constexpr int kHoTile = 16;
-
-__device__ __forceinline__ void cp_async8(double *smem, const double *gmem) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((unsigned)__cvta_generic_to_shared(smem)), "l"(gmem));
+template <int P>
+static HoGeo ho_geo(const Ctx *c) {
+  const Level &f = c->lv[0];
+  HoGeo g;
+  g.L = f.nlev;
+  g.ncol = f.ncol;
+  g.nhf = (int64_t)f.nedge * f.nlev;
+  g.nzf = (int64_t)f.ncol * (f.nlev + 1);
+  g.NH = (int64_t)Ho<P>::NB * g.nhf;
+  g.col_edges = f.col_edges;
+  g.stencil = f.edge_stencil;
+  g.edge_fc = f.edge_fc;
+  g.own = c->ho.own;
+  return g;
 }
+
+// ---- products with A_K^-1 ----------------------------------------------------------------------
+// One thread per row of A_K^-1, each row's dot product in column order; the rows of all cells in one
+// index space, so that no lane idles (p = 1: 44 rows per cell, 24 for the right-hand side). A warp stages
+// its 32 rows 16 columns at a time through shared memory (cp.async, two tiles in flight): one thread per
+// row straight from global memory touched 32 lines per load (p = 3, 4,096 cells: recovery 1,402 us, 0.3
+// of HBM bandwidth; now bound by the FP64 rate of its 378 M FMAs).
+constexpr int kHoTile = 16, kHoDotThreads = 256;
+
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int NLEFT>
 __device__ __forceinline__ void cp_async_wait() {
   asm volatile("cp.async.wait_group %0;" ::"n"(NLEFT) : "memory");
 }
+template <int BYTES>   // 4, 8 or 16, both addresses aligned to it
+__device__ __forceinline__ void cp_async(void *smem, const void *gmem) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"((unsigned)__cvta_generic_to_shared(smem)), "l"(gmem),
+               "n"(BYTES)
+               : "memory");
+}
 
-// sum_j I[row][j] r[j] for this thread's row (rows past `rows` give 0); r in shared memory, tile: this
-// warp's 2 x 32 x (kHoTile + 1) doubles
-template <int N>
-__device__ __forceinline__ double ho_row_dot(const double *__restrict__ I, int rows, const double *r, double *tile) {
-  constexpr int LD = kHoTile + 1, NTILE = (N + kHoTile - 1) / kHoTile;
-  const int lane = threadIdx.x & 31, row0 = threadIdx.x & ~31;
+// The rows of cell K that a product takes (all N, or the NF facet dofs) and its shared memory: the
+// block's cells' vectors, then per warp the row addresses and two tiles.
+template <int P, bool REC>
+struct HoDot {
+  using H = Ho<P>;
+  static constexpr int ROWS = REC ? H::N : H::NF, CELLS = (kHoDotThreads - 1) / ROWS + 2, LD = kHoTile + 1;
+  static constexpr int WARP = 32 + 2 * 32 * LD;   // doubles per warp
+  static constexpr int SMEM = (int)sizeof(double) * (CELLS * H::N + (kHoDotThreads / 32) * WARP);
+};
+
+// REC: X_K = A_K^-1 (R_K - C_K lambda_K) into o0 = u [ncell][NU], o1 = pi [ncell][NP]. Otherwise
+// (A_K^-1 R_K)_q on the facet dofs q < NF, into o0 (q < NF / 2) and o1, NF / 2 per cell each.
+template <int P, bool REC>
+__global__ void __launch_bounds__(kHoDotThreads)
+    ho_dot_kernel(const HoGeo g, int64_t ncell, const double *__restrict__ tab, const double *__restrict__ Ainv,
+                  const double *__restrict__ lam, const double *__restrict__ Ru, const double *__restrict__ Rp,
+                  double *__restrict__ o0, double *__restrict__ o1) {
+  using H = Ho<P>;
+  using D = HoDot<P, REC>;
+  constexpr int N = H::N, LD = D::LD, NTILE = (N + kHoTile - 1) / kHoTile, HF = H::NF / 2;
+  extern __shared__ __align__(16) double hd_smem[];
+  const int lane = threadIdx.x & 31;
+  const int64_t first = (int64_t)blockIdx.x * kHoDotThreads, total = ncell * D::ROWS, idx = first + threadIdx.x;
+  const int64_t K0 = first / D::ROWS;
+  double *r = hd_smem;
+  double *wsm = r + D::CELLS * N + (threadIdx.x >> 5) * D::WARP, *tile = wsm + 32;
+  const double **rows = reinterpret_cast<const double **>(wsm);
+  for (int e = threadIdx.x; e < D::CELLS * N; e += kHoDotThreads) {
+    const int64_t K = K0 + e / N;
+    const int j = e % N;
+    if (K >= ncell) break;
+    double v = j < H::NU ? Ru[K * H::NU + j] : Rp[K * H::NP + (j - H::NU)];
+    if (REC && j < H::NF) {
+      const int c = (int)((unsigned)K / (unsigned)g.L), k = (int)((unsigned)K - (unsigned)c * (unsigned)g.L);
+      v = fma(-tab[H::TC + j % H::NB], lam[ho_gid<P>(g, c, k, j)], v);
+    }
+    r[e] = v;
+  }
+  const int64_t K = idx / D::ROWS;
+  const int q = (int)(idx - K * D::ROWS);
+  rows[lane] = idx < total ? Ainv + K * (int64_t)(N * N) + (int64_t)q * N : nullptr;
+  __syncthreads();
+  static_assert(kHoTile == 16, "two rows per warp load");
   auto stage = [&](int j) {
     double *t = tile + (j & 1) * 32 * LD;
-    const int col = j * kHoTile + (lane & (kHoTile - 1));
+    const int sub = lane & (kHoTile - 1), col = j * kHoTile + sub;
 #pragma unroll
-    for (int q = 0; q < 32; q += 2) {
-      const int rr = q + (lane >> 4);
-      if (row0 + rr < rows && col < N) cp_async8(t + rr * LD + (lane & (kHoTile - 1)), I + (int64_t)(row0 + rr) * N + col);
+    for (int s = 0; s < 32; s += 2) {
+      const int rr = s + (lane >> 4);
+      const double *row = rows[rr];
+      if (row && col < N) cp_async<8>(t + rr * LD + sub, row + col);
     }
     cp_async_commit();
   };
-  static_assert(kHoTile == 16, "two rows per warp load");
   stage(0);
   double v = 0.0;
+  const double *rk = r + (int)(K - K0) * N;
   for (int j = 0; j < NTILE; ++j) {
     if (j + 1 < NTILE) {
       stage(j + 1);
@@ -405,37 +463,37 @@ __device__ __forceinline__ double ho_row_dot(const double *__restrict__ I, int r
       cp_async_wait<0>();
     }
     __syncwarp();
-    const double *t = tile + (j & 1) * 32 * LD + lane * LD, *rj = r + j * kHoTile;
+    const double *t = tile + (j & 1) * 32 * LD + lane * LD, *rj = rk + j * kHoTile;
     const int m = N - j * kHoTile < kHoTile ? N - j * kHoTile : kHoTile;
-    if (row0 + lane < rows) {
+    if (idx < total) {
       if (m == kHoTile) {
 #pragma unroll
-        for (int q = 0; q < kHoTile; ++q) v = fma(t[q], rj[q], v);
+        for (int s = 0; s < kHoTile; ++s) v = fma(t[s], rj[s], v);
       } else {
-        for (int q = 0; q < m; ++q) v = fma(t[q], rj[q], v);
+        for (int s = 0; s < m; ++s) v = fma(t[s], rj[s], v);
       }
     }
     __syncwarp();   // the tile is staged again two steps on
   }
-  return v;
+  if (idx >= total) return;
+  if (REC) {
+    if (q < H::NU) o0[K * H::NU + q] = v;
+    else o1[K * H::NP + (q - H::NU)] = v;
+  } else {
+    if (q < HF) o0[K * HF + q] = v;
+    else o1[K * HF + q - HF] = v;
+  }
 }
 
-// d[q] = (A_K^-1 R_K)_q on the facet dofs q < NF of cell K, in two halves of NF / 2 per cell
-template <int P>
-__global__ void __launch_bounds__(((Ho<P>::NF + 31) / 32) * 32)
-    ho_cell_rhs_kernel(const double *__restrict__ Ainv, const double *__restrict__ Ru, const double *__restrict__ Rp,
-                       double *__restrict__ d0, double *__restrict__ d1) {
-  using H = Ho<P>;
-  constexpr int N = H::N, NW = (H::NF + 31) / 32;
-  __shared__ double r[N], tile[NW][2 * 32 * (kHoTile + 1)];
-  const int64_t K = blockIdx.x;
-  for (int j = threadIdx.x; j < N; j += 32 * NW) r[j] = j < H::NU ? Ru[K * H::NU + j] : Rp[K * H::NP + (j - H::NU)];
-  __syncthreads();
-  const double v = ho_row_dot<N>(Ainv + K * (int64_t)(N * N), H::NF, r, tile[threadIdx.x >> 5]);
-  const int q = threadIdx.x;
-  constexpr int HF = H::NF / 2;
-  if (q < HF) d0[K * HF + q] = v;
-  else if (q < H::NF) d1[K * HF + q - HF] = v;
+template <int P, bool REC>
+static int ho_launch_dot(Ctx *c, const double *lam, const double *Ru, const double *Rp, double *o0, double *o1) {
+  using D = HoDot<P, REC>;
+  const int64_t C = c->lv[0].ncell;
+  HMG_CUDA(c, cudaFuncSetAttribute(ho_dot_kernel<P, REC>, cudaFuncAttributeMaxDynamicSharedMemorySize, D::SMEM));
+  ho_dot_kernel<P, REC><<<grid_for(C * D::ROWS, kHoDotThreads), kHoDotThreads, D::SMEM, c->stream>>>(
+      ho_geo<P>(c), C, c->ho.tab, c->ho.Ainv, lam, Ru, Rp, o0, o1);
+  HMG_CUDA(c, cudaGetLastError());
+  return HMG_OK;
 }
 
 // B_lambda row NB F + n: the sum over the facet's cells of C_K (A_K^-1 R_K) at the node's local dof
@@ -456,30 +514,6 @@ __global__ void ho_rhs_kernel(const HoGeo g, int64_t T, const double *__restrict
   double v = cell(fc.cA, fc.kA, H::NB * fc.fA + n);
   if (fc.cB >= 0) v += cell(fc.cB, fc.kB, H::NB * fc.fB + H::NT * (fc.flipB ? P - s : s) + t);
   B[row] = tab[H::TC + n] * v;
-}
-
-// X_K = A_K^-1 (R_K - C_K lambda_K): u [ncell][NU], pi [ncell][NP]
-template <int P>
-__global__ void __launch_bounds__(((Ho<P>::N + 31) / 32) * 32)
-    ho_reconstruct_kernel(const HoGeo g, const double *__restrict__ tab, const double *__restrict__ Ainv,
-                          const double *__restrict__ lam, const double *__restrict__ Ru, const double *__restrict__ Rp,
-                          double *__restrict__ u, double *__restrict__ pi) {
-  using H = Ho<P>;
-  constexpr int N = H::N, NW = (N + 31) / 32;
-  extern __shared__ __align__(16) double hr_smem[];   // r [N], then the warps' tiles
-  const int64_t K = blockIdx.x;
-  const int c = (int)(K / g.L), k = (int)(K - (int64_t)c * g.L);
-  double *r = hr_smem, *tile = r + N + (threadIdx.x >> 5) * (2 * 32 * (kHoTile + 1));
-  for (int j = threadIdx.x; j < N; j += 32 * NW) {
-    double v = j < H::NU ? Ru[K * H::NU + j] : Rp[K * H::NP + (j - H::NU)];
-    if (j < H::NF) v = fma(-tab[H::TC + j % H::NB], lam[ho_gid<P>(g, c, k, j)], v);
-    r[j] = v;
-  }
-  __syncthreads();
-  const double v = ho_row_dot<N>(Ainv + K * (int64_t)(N * N), N, r, tile);
-  const int i = threadIdx.x;
-  if (i < H::NU) u[K * H::NU + i] = v;
-  else if (i < N) pi[K * H::NP + (i - H::NU)] = v;
 }
 
 // ---- Algorithm 1 at p >= 1 ------------------------------------------------------------------------
@@ -524,83 +558,99 @@ __global__ void __launch_bounds__(kHoRowThreads)
   }
 }
 
+// Part 2's ring of factor blocks: levels in flight and values per column of a slot (padded by NB, so that
+// the columns of a warp meet different banks).
+template <int P>
+struct HoLines {
+  static constexpr int DEPTH = P == 1 ? 8 : (P == 2 ? 6 : 4);
+  static constexpr int NB2 = Ho<P>::NB * Ho<P>::NB, STRIDE = 2 * NB2 + Ho<P>::NB;
+};
+
+// One warp per block of CPW columns. The recurrences are serial over the levels (2 L + 1 steps of
+// NB-term dot products), so a step must not wait for its factors: they stream through shared memory by
+// cp.async, DEPTH - 1 steps ahead. Loaded one step ahead into registers, four warps per block, the
+// kernel took 1.1 us per step, one memory latency (37 us per sweep at p = 1 on 64 x 64 x 16 cells, 40 us
+// at p = 3 in FP32 on 16 x 16 x 16).
 // Part 2; r is read from src (lam_out after part 1, b for a sweep from zero)
 template <int P, bool ZERO, typename T = double, typename Ts = double, typename Tin = double, typename Tout = double>
-__global__ void __launch_bounds__(128)
+__global__ void __launch_bounds__(32)
     ho_sweep_lines_kernel(const HoGeo g, int cpb, const T *__restrict__ zf, const Ts *src,
                           const Tin *__restrict__ lam_in, Tout *lam_out, double keep) {
   using H = Ho<P>;
-  constexpr int NB = H::NB, NB2 = NB * NB, LPC = H::LPC;
+  using W = HoLines<P>;
+  constexpr int NB = H::NB, NB2 = NB * NB, LPC = H::LPC, D = W::DEPTH, CS = W::STRIDE;
+  // the widest copy that every matrix of every facet is aligned to
+  constexpr int VB = (NB2 * sizeof(T)) % 16 == 0 ? 16 : (int)sizeof(T), VN = VB / (int)sizeof(T);
   extern __shared__ __align__(16) unsigned char ho_lines_smem[];
-  T *sr = reinterpret_cast<T *>(ho_lines_smem);   // [cpb][L+1][NB]
-  const int L1 = g.L + 1;
+  T *ring = reinterpret_cast<T *>(ho_lines_smem);   // [D][CPW][CS]
+  T *sr = ring + D * H::CPW * CS;                   // [cpb][L+1][NB]
+  const int L1 = g.L + 1, lane = threadIdx.x;
   const int c0 = blockIdx.x * cpb, nc = min(cpb, g.ncol - c0);
   const int64_t base = g.NH + (int64_t)NB * c0 * L1;
-  for (int i = threadIdx.x; i < nc * L1 * NB; i += blockDim.x) sr[i] = (T)src[base + i];
-  __syncthreads();
-  const int lane = threadIdx.x & 31, gw = lane / LPC;   // the lane's group within its warp
-  const int cc = gw < H::CPW ? (threadIdx.x >> 5) * H::CPW + gw : cpb, n = lane - gw * LPC;
-  const unsigned grp = ((1u << LPC) - 1u) << (gw * LPC);   // this column's lanes
-  if (cc < nc) {
-    T *r = sr + NB * cc * L1;
-    const T *f0 = zf + 3 * NB2 * ((int64_t)(c0 + cc) * L1) + n;   // this lane's rows (transposed)
-    const bool act = n < NB;
-    // forward: y_k = (omega G_k^-1) r_k - (G_k^-1 L_k) y_{k-1}, y written over r; the next level's
-    // factor rows are loaded one step ahead (the serial recurrence waits on nothing else)
-    T fa[NB], fb[NB];
-    if (act) {
-#pragma unroll
-      for (int m = 0; m < NB; ++m) { fa[m] = __ldg(f0 + NB * m); fb[m] = __ldg(f0 + NB2 + NB * m); }
+  // step s of the two passes: the forward step of level s, then the backward step of level 2 L1 - 2 - s
+  const int steps = 2 * L1 - 1;
+  auto stage = [&](int s) {
+    if (s < steps) {
+      T *slot = ring + (s % D) * (H::CPW * CS);
+      const bool fwd = s < L1;
+      const T *f = zf + 3 * NB2 * ((int64_t)c0 * L1 + (fwd ? s : 2 * L1 - 2 - s)) + (fwd ? 0 : 2 * NB2);
+      const int per = (fwd ? 2 * NB2 : NB2) / VN;
+      for (int cc = 0; cc < nc; ++cc, f += 3 * NB2 * (int64_t)L1)
+        for (int e = lane; e < per; e += 32) cp_async<VB>(slot + cc * CS + e * VN, f + e * VN);
     }
-    for (int k = 0; k < L1; ++k) {
-      T na[NB], nb[NB];
-      if (act && k + 1 < L1) {
-        const T *f = f0 + 3 * NB2 * (k + 1);
+    cp_async_commit();
+  };
 #pragma unroll
-        for (int m = 0; m < NB; ++m) { na[m] = __ldg(f + NB * m); nb[m] = __ldg(f + NB2 + NB * m); }
-      }
-      T v = (T)0, u = (T)0;
-      if (act) {
+  for (int s = 0; s < D; ++s) stage(s);
+  for (int i = lane; i < nc * L1 * NB; i += 32) sr[i] = (T)src[base + i];
+  const int cc = lane / LPC, n = lane - cc * LPC;
+  const bool act = cc < nc && n < NB;
+  T *r = sr + NB * (act ? cc : 0) * L1;
+  // a step's factors and what does not depend on the step before it are taken one step ahead:
+  // forward v = (omega G_k^-1) r_k, backward v = y_k
+  T f[NB], v = (T)0;
+  auto load = [&](int s) {
+    const T *q = ring + (s % D) * (H::CPW * CS) + (act ? cc * CS + n : 0);   // this lane's rows (transposed)
+    if (s < L1) {
+      const T *rk = r + NB * s;
+      v = (T)0;
 #pragma unroll
-        for (int m = 0; m < NB; ++m) v = fma(fa[m], r[NB * k + m], v);
-        if (k > 0) {
-#pragma unroll
-          for (int m = 0; m < NB; ++m) u = fma(-fb[m], r[NB * (k - 1) + m], u);
-        }
-      }
-      __syncwarp(grp);
-      if (act) r[NB * k + n] = v + u;
-      __syncwarp(grp);
-#pragma unroll
-      for (int m = 0; m < NB; ++m) { fa[m] = na[m]; fb[m] = nb[m]; }
+      for (int m = 0; m < NB; ++m) v = fma(q[NB * m], rk[m], v);
+      q += NB2;
+    } else {
+      v = r[NB * (2 * L1 - 2 - s) + (act ? n : 0)];
     }
-    // backward: x_k = y_k - (G_k^-1 U_k) x_{k+1}, x written over y (row k + 1 is not written in
-    // this step, row k only by its own lane); G_k^-1 U_k one step ahead as well
-    if (act && L1 >= 2) {
-      const T *f = f0 + 3 * NB2 * (L1 - 2) + 2 * NB2;
 #pragma unroll
-      for (int m = 0; m < NB; ++m) fa[m] = __ldg(f + NB * m);
-    }
-    for (int k = L1 - 2; k >= 0; --k) {
-      T na[NB];
-      if (act && k > 0) {
-        const T *f = f0 + 3 * NB2 * (k - 1) + 2 * NB2;
+    for (int m = 0; m < NB; ++m) f[m] = q[NB * m];
+  };
+  cp_async_wait<D - 1>();
+  __syncwarp();
+  load(0);
+  for (int s = 0; s < steps; ++s) {
+    if (s < L1) {
+      // forward: y_k = (omega G_k^-1) r_k - (G_k^-1 L_k) y_{k-1}, y written over r
+      T u = (T)0;
+      if (s > 0) {
+        const T *y = r + NB * (s - 1);
 #pragma unroll
-        for (int m = 0; m < NB; ++m) na[m] = __ldg(f + NB * m);
+        for (int m = 0; m < NB; ++m) u = fma(-f[m], y[m], u);
       }
-      if (act) {
-        T v = r[NB * k + n];
+      if (act) r[NB * s + n] = v + u;
+    } else {
+      // backward: x_k = y_k - (G_k^-1 U_k) x_{k+1}, x written over y
+      const int k = 2 * L1 - 2 - s;
+      const T *x = r + NB * (k + 1);
+      T u = v;
 #pragma unroll
-        for (int m = 0; m < NB; ++m) v = fma(-fa[m], r[NB * (k + 1) + m], v);
-        r[NB * k + n] = v;
-      }
-      __syncwarp(grp);
-#pragma unroll
-      for (int m = 0; m < NB; ++m) fa[m] = na[m];
+      for (int m = 0; m < NB; ++m) u = fma(-f[m], x[m], u);
+      if (act) r[NB * k + n] = u;
     }
+    cp_async_wait<D - 2>();   // the next step's factors
+    __syncwarp();
+    if (s + 1 < steps) load(s + 1);
+    stage(s + D);             // (its slot was read before this step)
   }
-  __syncthreads();
-  for (int i = threadIdx.x; i < nc * L1 * NB; i += blockDim.x)
+  for (int i = lane; i < nc * L1 * NB; i += 32)
     lam_out[base + i] = (Tout)(ZERO ? sr[i] : fma((T)keep, (T)lam_in[base + i], sr[i]));
 }
 
@@ -685,22 +735,6 @@ __global__ void ho_gamma_div_kernel(int64_t ncell, const double *__restrict__ m,
 }
 
 // ---- host side ------------------------------------------------------------------------------------
-template <int P>
-static HoGeo ho_geo(const Ctx *c) {
-  const Level &f = c->lv[0];
-  HoGeo g;
-  g.L = f.nlev;
-  g.ncol = f.ncol;
-  g.nhf = (int64_t)f.nedge * f.nlev;
-  g.nzf = (int64_t)f.ncol * (f.nlev + 1);
-  g.NH = (int64_t)Ho<P>::NB * g.nhf;
-  g.col_edges = f.col_edges;
-  g.stencil = f.edge_stencil;
-  g.edge_fc = f.edge_fc;
-  g.own = c->ho.own;
-  return g;
-}
-
 int64_t ho_trace_size(const Ctx *c, int p) {
   const Level &f = c->lv[0];
   return (int64_t)(p + 1) * (p + 1) * ((int64_t)f.nedge * f.nlev + (int64_t)f.ncol * (f.nlev + 1));
@@ -824,7 +858,7 @@ static int ho_assemble_p(Ctx *c) {
     double *ones = sk1, *s1 = static_cast<double *>(c->w2);
     ho_fill_kernel<<<grid_for(h.T, 256), 256, 0, c->stream>>>(ones, h.T, 1.0);
     if ((st = ho_launch_spmv_p<P>(c, ones, s1, 0, nullptr, 0, 0))) return st;
-    ho_restrict_kernel<P, double><<<grid_for(C, 256), 256, 0, c->stream>>>(g, C, s1, nullptr, h.gamma);
+    ho_restrict_kernel<P, double><<<grid_for(C, 64), 64, 0, c->stream>>>(g, C, s1, nullptr, h.gamma);
     ho_gamma_div_kernel<<<grid_for(C, 256), 256, 0, c->stream>>>(C, h.m, h.gamma);
   } else {
     ho_gamma_kernel<<<grid_for(C, 256), 256, 0, c->stream>>>(C, f.nlev, f.col_nbr, f.col_nbr_face, h.m, sk1, h.gamma);
@@ -863,7 +897,8 @@ static int ho_trace_rhs_p(Ctx *c, const double *Ru, const double *Rp, double *B)
   Prof prof(c, kCompRhs);
   // the cells' products pass through the preconditioner's work vectors (T >= 3 NB C = NF / 2 C doubles each)
   double *d0 = static_cast<double *>(c->w1), *d1 = static_cast<double *>(c->w2);
-  ho_cell_rhs_kernel<P><<<(unsigned)c->lv[0].ncell, ((Ho<P>::NF + 31) / 32) * 32, 0, c->stream>>>(h.Ainv, Ru, Rp, d0, d1);
+  int st;
+  if ((st = ho_launch_dot<P, false>(c, nullptr, Ru, Rp, d0, d1))) return st;
   ho_rhs_kernel<P><<<grid_for(h.T, 256), 256, 0, c->stream>>>(ho_geo<P>(c), h.T, h.tab, d0, d1, B);
   HMG_CUDA(c, cudaGetLastError());
   return HMG_OK;
@@ -871,13 +906,7 @@ static int ho_trace_rhs_p(Ctx *c, const double *Ru, const double *Rp, double *B)
 
 template <int P>
 static int ho_reconstruct_p(Ctx *c, const double *lam, const double *Ru, const double *Rp, double *u, double *pi) {
-  constexpr int NW = (Ho<P>::N + 31) / 32;
-  const int smem = (int)sizeof(double) * (Ho<P>::N + NW * 2 * 32 * (kHoTile + 1));
-  HMG_CUDA(c, cudaFuncSetAttribute(ho_reconstruct_kernel<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-  ho_reconstruct_kernel<P><<<(unsigned)c->lv[0].ncell, 32 * NW, smem, c->stream>>>(ho_geo<P>(c), c->ho.tab, c->ho.Ainv,
-                                                                                 lam, Ru, Rp, u, pi);
-  HMG_CUDA(c, cudaGetLastError());
-  return HMG_OK;
+  return ho_launch_dot<P, true>(c, lam, Ru, Rp, u, pi);
 }
 
 // The FP64 operator or the FP32 preconditioner's copies
@@ -902,24 +931,26 @@ static int ho_sweep(Ctx *c, const double *b, const Tin *lam_in, Tout *lam_out) {
   using H = Ho<P>;
   const HoData &h = c->ho;
   const HoGeo g = ho_geo<P>(c);
-  // columns per block of the line part: 4 warps of CPW columns, and the block's rows
-  // (NB (L + 1) values per column) within 48 KB
+  // columns per block of the line part: one warp of CPW columns, and the block's rows (NB (L + 1)
+  // values per column) within 48 KB beside the ring
   const int cap = (int)((48 * 1024) / (sizeof(T) * H::NB * (g.L + 1)));
   if (cap < 1) return fail(c, HMG_ERR_INVALID_ARG, "too many layers for the degree-p line smoother");
-  const int cpb = cap < 4 * H::CPW ? cap : 4 * H::CPW;
+  const int cpb = cap < H::CPW ? cap : H::CPW;
   const unsigned nzb = (unsigned)((g.ncol + cpb - 1) / cpb);
-  const size_t smem = sizeof(T) * H::NB * cpb * (g.L + 1);
+  const size_t smem = sizeof(T) * (HoLines<P>::DEPTH * H::CPW * HoLines<P>::STRIDE + (size_t)H::NB * cpb * (g.L + 1));
   const double keep = 1.0 - h.factor_omega;
   Prof prof(c, ZERO ? kCompPresmooth : kCompSweep, 2);
   ho_sweep_rows_kernel<P, ZERO, T, double, Tin, Tout>
       <<<grid_for(ZERO ? g.NH : h.T, kHoRows<P>), kHoRowThreads, 0, c->stream>>>(
           g, h.T, HoPrec<T>::S(h), HoPrec<T>::hw(h), b, lam_in, lam_out, keep);
-  if constexpr (ZERO)
-    ho_sweep_lines_kernel<P, ZERO, T, double, Tin, Tout><<<nzb, 128, smem, c->stream>>>(g, cpb, HoPrec<T>::zf(h), b,
-                                                                                      lam_in, lam_out, keep);
-  else
-    ho_sweep_lines_kernel<P, ZERO, T, Tout, Tin, Tout><<<nzb, 128, smem, c->stream>>>(
-        g, cpb, HoPrec<T>::zf(h), lam_out, lam_in, lam_out, keep);
+  auto lines = [&](auto kern, const auto *src) {
+    const cudaError_t e = smem > 48 * 1024 ? cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)
+                                           : cudaSuccess;
+    if (e == cudaSuccess) kern<<<nzb, 32, smem, c->stream>>>(g, cpb, HoPrec<T>::zf(h), src, lam_in, lam_out, keep);
+    return e;
+  };
+  if constexpr (ZERO) HMG_CUDA(c, lines(ho_sweep_lines_kernel<P, ZERO, T, double, Tin, Tout>, b));
+  else HMG_CUDA(c, lines(ho_sweep_lines_kernel<P, ZERO, T, Tout, Tin, Tout>, lam_out));
   HMG_CUDA(c, cudaGetLastError());
   return HMG_OK;
 }
@@ -991,7 +1022,7 @@ static int ho_precond_p(Ctx *c, const double *r, double *z) {
     else
       ho_residual_kernel<P, false, T><<<grid_for(TT, kHoRows<P>), kHoRowThreads, 0, c->stream>>>(
           g, TT, HoPrec<T>::S(h), r, w1, w2, 0.0);
-    ho_restrict_kernel<P, T><<<grid_for(C, 256), 256, 0, c->stream>>>(g, C, w2, HoPrec<T>::gamma(h), cb);   // lines 4-5
+    ho_restrict_kernel<P, T><<<grid_for(C, 64), 64, 0, c->stream>>>(g, C, w2, HoPrec<T>::gamma(h), cb);   // lines 4-5
     HMG_CUDA(c, cudaGetLastError());
   }
   T *dpi = nullptr;

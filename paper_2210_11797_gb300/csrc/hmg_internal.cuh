@@ -403,6 +403,17 @@ int time_vcycle(Ctx *c, int fp32, float *ms);
 // (3 x ((L + 1) | 1) doubles) stay within the default 48 KB of dynamic shared memory
 constexpr int kMaxLayers = 2045;
 
+// Columns per block of a column kernel that no shape was given for: 32 (a lane per column of the serial
+// phase, which occupies the FP64 pipe per warp), fewer where that would leave SMs without a block: a
+// level of few columns waits on latency, and a small block takes its cells in one pass. C12 x 30 (864
+// columns, FP64): a smoothing sweep 13.7 us at 32 columns (27 blocks), 5.0 us at 4; its fused
+// restriction and sweep 31 and 7 us.
+inline int default_columns(const Ctx *c, int ncol, int limit) {
+  int n = limit < 32 ? limit : 32;
+  while (n > 1 && (int64_t)n * c->num_sms > ncol) n >>= 1;
+  return n;
+}
+
 inline int mg_cpb_limit(int nlev) {
   const int m = 2048 / (nlev | 1);
   return m < 1 ? 1 : (m > 64 ? 64 : m);
