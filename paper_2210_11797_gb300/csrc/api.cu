@@ -179,6 +179,7 @@ int hmg_create(hmg_ctx **out, const hmg_options *opt, void *cuda_stream) {
   if (!st) st = dev_alloc(c, &c->part, (size_t)Scal::N * kMaxRedBlocks);
   if (!st) st = dev_alloc(c, &c->counter, Scal::N);
   if (!st) st = dev_alloc(c, &c->mg_bar, 64);
+  if (!st) st = dev_alloc(c, &c->x_slot, 1);
   if (!st && cudaDeviceGetAttribute(&c->num_sms, cudaDevAttrMultiProcessorCount, c->device) != cudaSuccess)
     st = HMG_ERR_CUDA;
   if (!st && cudaMemset(c->counter, 0, sizeof(unsigned int) * Scal::N) != cudaSuccess) st = HMG_ERR_CUDA;

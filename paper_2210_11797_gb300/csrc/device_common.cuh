@@ -56,10 +56,10 @@ __device__ __forceinline__ void block_sum(const double (&val)[NV], double (&out)
 // Deterministic reduction of NV per-thread values over the whole grid (gridDim.x <=
 // kMaxRedBlocks, blockDim.x a multiple of 32, <= 1024). Each block writes its partial sums to
 // part[slot][blockIdx.x]; the block that takes the last ticket sums the partials in block
-// order and writes scal[slot]. The summation order depends only on the launch shape, so
-// repeated runs give bit-identical results. No block waits on another.
+// order and writes scal[slot] (thread 0), and is told so. The summation order depends only on the
+// launch shape, so repeated runs give bit-identical results. No block waits on another.
 template <int NV>
-__device__ __forceinline__ void grid_reduce(const double (&val)[NV], const int (&slot)[NV],
+__device__ __forceinline__ bool grid_reduce(const double (&val)[NV], const int (&slot)[NV],
                                             double *part, unsigned int *counter, double *scal) {
   __shared__ double sh[NV][32];
   __shared__ bool is_last;
@@ -77,7 +77,7 @@ __device__ __forceinline__ void grid_reduce(const double (&val)[NV], const int (
     is_last = (ticket == gridDim.x - 1);
   }
   __syncthreads();
-  if (!is_last) return;
+  if (!is_last) return false;
   __threadfence();
 #pragma unroll
   for (int i = 0; i < NV; ++i) {
@@ -95,6 +95,28 @@ __device__ __forceinline__ void grid_reduce(const double (&val)[NV], const int (
     }
   }
   if (threadIdx.x == 0) counter[slot[0]] = 0u;
+  return true;
+}
+
+// Sum of the per-block partials of one slot by 1024 threads, in a fixed order; valid in thread 0.
+// sh: 32 doubles of shared memory.
+__device__ __forceinline__ double sum_partials(const double *p, int nblocks, double *sh) {
+  double acc[4] = {0.0, 0.0, 0.0, 0.0};
+  int b = threadIdx.x;
+  for (; b + 3 * 1024 < nblocks; b += 4 * 1024) {
+    acc[0] += __ldcg(p + b);
+    acc[1] += __ldcg(p + b + 1024);
+    acc[2] += __ldcg(p + b + 2048);
+    acc[3] += __ldcg(p + b + 3072);
+  }
+  for (; b < nblocks; b += 1024) acc[0] += __ldcg(p + b);
+  const double v = warp_sum((acc[0] + acc[1]) + (acc[2] + acc[3]));
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
+  __syncthreads();
+  double s = 0.0;
+  if (threadIdx.x == 0)
+    for (int i = 0; i < 32; ++i) s += sh[i];
+  return s;
 }
 
 // Block-level sums of NV per-thread values written to part[slot][blockIdx.x] (no atomics, no

@@ -40,6 +40,7 @@ struct Scal {
   static constexpr int BB = 6;              // (B, B)
   static constexpr int ALPHA = 7, OMEGA = 8;
   static constexpr int AUX = 9;             // scratch for tests / true residual
+  static constexpr int BETA = 10;           // (rho_i / rho_{i-1}) (alpha / omega) of the next iteration
   static constexpr int N = 16;
 };
 
@@ -165,10 +166,8 @@ struct Ctx {
   cudaStream_t cap_stream = nullptr;
   cudaGraphExec_t graph_exec = nullptr;
   cudaGraph_t graph = nullptr;
-  struct GraphKey {
-    const void *Rub, *Rpi, *lam;
-    hmg_options opt;
-  } graph_key{};
+  hmg_options graph_opt{};     // what it was captured for
+  double **x_slot = nullptr;   // device: the iterate the graph's kernels update (written per solve)
   uint64_t graph_gen = next_graph_gen();
   // the batched-solve graph this context holds as the first context of a batch, and what it
   // was captured for: each member's address, generation, vectors and options
@@ -298,13 +297,24 @@ int make_fp32(Ctx *c);   // FP32 copies of the assembled operators and factors (
 // ---- trace-space kernels (trace_ops.cu) -----------------------------------------------
 // y = S x (FP64). mode 0: plain; 1: also (w, y) -> scal[slot0]; 2: also (y, w) -> slot0 and
 // (y, y) -> slot1; 3: y is not stored, (b - S x, b - S x) -> slot0 with w = b.
+// alpha: mode 1 also leaves BiCGStab's alpha = rho_i / (w, y) in scal[ALPHA].
 int launch_spmv(Ctx *c, const double *x, double *y, int mode, const double *w, int slot0,
-                int slot1);
+                int slot1, bool alpha = false);
 int launch_trace_rhs(Ctx *c, const double *Rub, const double *Rpi, double *B);
 int launch_reconstruct(Ctx *c, const double *lam, const double *Rub, const double *Rpi,
                        double *ub, double *pi);
-// preconditioners: z = M^-1 r, r and z FP64 Krylov vectors
-int precond_apply(Ctx *c, const double *r, double *z);
+// A Krylov vector that the preconditioner's first, zero-start sweep forms as it reads it (and stores):
+// kind 1: out = r + beta (out - omega v), BiCGStab's p; kind 2: out = r - alpha v, its s. The scalars
+// are in scal.
+struct FusedVector {
+  int kind = 0;
+  const double *r = nullptr, *v = nullptr, *scal = nullptr;
+  double *out = nullptr;
+};
+// whether precond_apply can form its input so
+bool precond_fuses(const Ctx *c);
+// preconditioners: z = M^-1 r, r and z FP64 Krylov vectors (fv: r = fv->out is formed on the way)
+int precond_apply(Ctx *c, const double *r, double *z, const FusedVector *fv = nullptr);
 int line_smooth_fp64(Ctx *c, const double *b, double *lam, int nsweeps);
 // looks up the device address of the allocation-free sweep's scratch array (set-up)
 int noalloc_setup(Ctx *c);

@@ -124,6 +124,7 @@ __global__ void bicg_start_kernel(double *scal, int *state, double *hist, LoopPa
   scal[Scal::RHO1] = 1.0;
   scal[Scal::ALPHA] = 1.0;
   scal[Scal::OMEGA] = 1.0;
+  scal[Scal::BETA] = rr0;   // (rr0 / 1) (1 / 1)
   const double rel0 = bb > 0.0 ? sqrt(rr0 / bb) : 0.0;
   int status = isfinite(bb) && isfinite(rr0) ? HMG_OK : HMG_ERR_NONFINITE;
   const bool work = status == HMG_OK && bb > 0.0 && rel0 > lp.tol;
@@ -139,7 +140,8 @@ __global__ void bicg_start_kernel(double *scal, int *state, double *hist, LoopPa
 // Vector updates take kVecUnroll grid-stride elements per pass, loads first, so that each
 // thread keeps several independent loads in flight (HBM latency x bandwidth).
 constexpr int kVecUnroll = 4;
-constexpr int kXrUnroll = 2;   // six input vectors: 2 keeps bicg_xr_kernel at 8 blocks per SM
+constexpr int kXrUnroll = 2;   // six input vectors
+constexpr int kXrBlocks = 6;   // bicg_xr_kernel's blocks per SM, all resident (a constant: the sums depend on it)
 
 // p = r + beta (p - omega v), beta = (rho_i / rho_{i-1}) (alpha / omega)
 __global__ void bicg_p_kernel(const double *__restrict__ r, double *__restrict__ p,
@@ -197,12 +199,17 @@ __global__ void bicg_s_kernel(const double *__restrict__ r, const double *__rest
 }
 
 // omega = (t, s) / (t, t); x += alpha phat + omega shat; r = s - omega t;
-// (rhat, r) -> scal[1 - par] (rho_{i+1}), (r, r) -> scal[RR]
-__global__ void __launch_bounds__(kRedThreads)
-    bicg_xr_kernel(double *__restrict__ x, double *__restrict__ r, const double *__restrict__ s,
+// (rhat, r) -> scal[1 - par] (rho_{i+1}), (r, r) -> scal[RR]. x_slot (may be null): where x is. The block
+// that finishes the sums also ends the iteration: it records ||r_i|| / ||B||, decides the status and
+// whether to go on, and forms the next beta.
+template <bool GRAPH>
+__global__ void __launch_bounds__(kRedThreads, kXrBlocks)
+    bicg_xr_kernel(double *x_direct, double *const *x_slot, double *__restrict__ r, const double *__restrict__ s,
                    const double *__restrict__ t, const double *__restrict__ phat,
                    const double *__restrict__ shat, const double *__restrict__ rhat, double *scal,
-                   double *part, unsigned int *counter, const int *__restrict__ state, int64_t n) {
+                   double *part, unsigned int *counter, int *state, double *hist, LoopParams lp,
+                   cudaGraphConditionalHandle handle, int64_t n) {
+  double *__restrict__ x = x_slot ? *x_slot : x_direct;
   const int par = state[kIt] & 1;
   const double alpha = scal[Scal::ALPHA];
   __shared__ double coef;
@@ -243,47 +250,41 @@ __global__ void __launch_bounds__(kRedThreads)
   if (blockIdx.x == 0 && threadIdx.x == 0) scal[Scal::OMEGA] = omega;
   const double val[2] = {a0, a1};
   const int sl[2] = {1 - par, Scal::RR};
-  grid_reduce<2>(val, sl, part, counter, scal);
-}
-
-// End of an iteration: record ||r_i|| / ||B||, decide the status, continue or stop.
-template <bool GRAPH>
-__global__ void bicg_check_kernel(const double *scal, int *state, double *hist, LoopParams lp,
-                                  cudaGraphConditionalHandle handle) {
+  if (!grid_reduce<2>(val, sl, part, counter, scal) || threadIdx.x != 0) return;
   const int it = state[kIt] + 1;        // iterations completed after this one
-  const int par_next = it & 1;          // slot holding rho_{i+1}
-  const double bnorm = sqrt(scal[Scal::BB]);
+  const double rho_next = scal[1 - par], bnorm = sqrt(scal[Scal::BB]);
   const double rel = sqrt(scal[Scal::RR]) / bnorm;
   hist[it < HMG_MAX_HISTORY ? it : HMG_MAX_HISTORY - 1] = rel;
   int status = HMG_OK, cont = 0;
-  if (!isfinite(rel) || !isfinite(scal[Scal::ALPHA]) || !isfinite(scal[Scal::OMEGA])) {
+  if (!isfinite(rel) || !isfinite(alpha) || !isfinite(omega)) {
     status = HMG_ERR_NONFINITE;
   } else if (rel <= lp.tol) {
     status = HMG_OK;
-  } else if (scal[Scal::RV] == 0.0 || scal[Scal::TT] == 0.0 || scal[par_next] == 0.0) {
+  } else if (scal[Scal::RV] == 0.0 || scal[Scal::TT] == 0.0 || rho_next == 0.0) {
     status = HMG_ERR_BREAKDOWN;
   } else if (rel > lp.divergence || it >= lp.max_iter) {
     status = HMG_ERR_NOT_CONVERGED;
   } else {
     cont = 1;
   }
+  scal[Scal::BETA] = (rho_next / scal[par]) * (alpha / omega);
   state[kIt] = it;
   state[kStatus] = status;
   state[kContinue] = cont;
   if (GRAPH) cudaGraphSetConditional(handle, cont);
 }
 
+
 static LoopParams loop_params(const Ctx *c) {
   return LoopParams{c->opt.tol, c->opt.divergence, c->opt.max_iter, c->opt.warm_start ? 1 : 0};
 }
 
-// B_lambda, (B, B), x = 0, r = rhat = B, loop state
-static int solve_head(Ctx *c, const double *Rub, const double *Rpi, double *x, bool graph,
-                      cudaGraphConditionalHandle h) {
+// B_lambda, (B, B), x = 0, r = rhat = B
+static int solve_head(Ctx *c, const double *Rub, const double *Rpi, double *x) {
   const int64_t n = sys_n(c);
   int s;
   if ((s = sys_rhs(c, Rub, Rpi, c->B))) return s;
-  Prof pk(c, kCompKrylov, 3);
+  Prof pk(c, kCompKrylov, 2);
   if ((s = launch_dot(c, c->B, c->B, n, Scal::BB))) return s;
   if (c->opt.warm_start) {
     if ((s = sys_apply(c, x, c->r, 0, nullptr, 0, 0))) return s;
@@ -292,11 +293,20 @@ static int solve_head(Ctx *c, const double *Rub, const double *Rpi, double *x, b
   } else {
     bicg_init_kernel<<<red_grid(n), kRedThreads, 0, c->stream>>>(c->B, x, c->r, c->rhat, c->p, c->v, n);
   }
+  HMG_CUDA(c, cudaGetLastError());
+  return HMG_OK;
+}
+
+// the loop's state and scalars
+static int solve_start(Ctx *c, bool graph, cudaGraphConditionalHandle h) {
+  Prof pk(c, kCompKrylov);
   if (graph) bicg_start_kernel<true><<<1, 1, 0, c->stream>>>(c->scal, c->state, c->hist, loop_params(c), h);
   else bicg_start_kernel<false><<<1, 1, 0, c->stream>>>(c->scal, c->state, c->hist, loop_params(c), h);
   HMG_CUDA(c, cudaGetLastError());
   return HMG_OK;
 }
+
+__global__ void set_slot_kernel(double **slot, double *x) { *slot = x; }
 
 // Blocks of a grid-stride vector kernel: one wave of resident blocks (no partial second
 // wave), at most one row per thread; fixed per device, so the reductions stay deterministic.
@@ -310,34 +320,46 @@ static int wave_grid(Ctx *c, int which, const void *kernel, int64_t n, unsigned 
   return HMG_OK;
 }
 
-// one BiCGStab iteration and its check
-static int solve_body(Ctx *c, double *x, bool graph, cudaGraphConditionalHandle h) {
+// One BiCGStab iteration and its check; slot: x comes from c->x_slot. p and s are formed in the
+// preconditioner's first sweep where it can (a profiled solve keeps them as kernels of their own, so
+// that the component times stay apart).
+static int solve_body(Ctx *c, double *x, bool graph, bool slot, cudaGraphConditionalHandle h) {
   const int64_t n = sys_n(c);
+  const bool fuse = precond_fuses(c) && !c->opt.profile;
   unsigned gp, gs, gx;
   int s;
-  if ((s = wave_grid(c, 0, (const void *)bicg_p_kernel, n, &gp))) return s;
-  if ((s = wave_grid(c, 1, (const void *)bicg_s_kernel, n, &gs))) return s;
-  if ((s = wave_grid(c, 2, (const void *)bicg_xr_kernel, n, &gx))) return s;
-  {
-    Prof pk(c, kCompKrylov);
-    bicg_p_kernel<<<gp, kRedThreads, 0, c->stream>>>(c->r, c->p, c->v, c->scal, c->state, n);
-    HMG_CUDA(c, cudaGetLastError());
+  gx = (unsigned)std::min<int64_t>((int64_t)kXrBlocks * c->num_sms, grid_for(n, kRedThreads));
+  if (fuse) {
+    const FusedVector fp{1, c->r, c->v, c->scal, c->p}, fs{2, c->r, c->v, c->scal, c->s};
+    if ((s = precond_apply(c, c->p, c->phat, &fp))) return s;
+    if ((s = launch_spmv(c, c->phat, c->v, 1, c->rhat, Scal::RV, 0, true))) return s;
+    if ((s = precond_apply(c, c->s, c->shat, &fs))) return s;
+  } else {
+    if ((s = wave_grid(c, 0, (const void *)bicg_p_kernel, n, &gp))) return s;
+    if ((s = wave_grid(c, 1, (const void *)bicg_s_kernel, n, &gs))) return s;
+    {
+      Prof pk(c, kCompKrylov);
+      bicg_p_kernel<<<gp, kRedThreads, 0, c->stream>>>(c->r, c->p, c->v, c->scal, c->state, n);
+      HMG_CUDA(c, cudaGetLastError());
+    }
+    if ((s = precond_apply(c, c->p, c->phat))) return s;
+    if ((s = sys_apply(c, c->phat, c->v, 1, c->rhat, Scal::RV, 0))) return s;
+    {
+      Prof pk(c, kCompKrylov);
+      bicg_s_kernel<<<gs, kRedThreads, 0, c->stream>>>(c->r, c->v, c->s, c->scal, c->state, n);
+      HMG_CUDA(c, cudaGetLastError());
+    }
+    if ((s = precond_apply(c, c->s, c->shat))) return s;
   }
-  if ((s = precond_apply(c, c->p, c->phat))) return s;
-  if ((s = sys_apply(c, c->phat, c->v, 1, c->rhat, Scal::RV, 0))) return s;
-  {
-    Prof pk(c, kCompKrylov);
-    bicg_s_kernel<<<gs, kRedThreads, 0, c->stream>>>(c->r, c->v, c->s, c->scal, c->state, n);
-    HMG_CUDA(c, cudaGetLastError());
-  }
-  if ((s = precond_apply(c, c->s, c->shat))) return s;
   if ((s = sys_apply(c, c->shat, c->t, 2, c->s, Scal::TS, Scal::TT))) return s;
   {
-    Prof pk(c, kCompKrylov, 2);
-    bicg_xr_kernel<<<gx, kRedThreads, 0, c->stream>>>(x, c->r, c->s, c->t, c->phat, c->shat, c->rhat,
-                                                      c->scal, c->part, c->counter, c->state, n);
-    if (graph) bicg_check_kernel<true><<<1, 1, 0, c->stream>>>(c->scal, c->state, c->hist, loop_params(c), h);
-    else bicg_check_kernel<false><<<1, 1, 0, c->stream>>>(c->scal, c->state, c->hist, loop_params(c), h);
+    Prof pk(c, kCompKrylov);
+    auto go = [&](auto kern) {
+      kern<<<gx, kRedThreads, 0, c->stream>>>(x, slot ? c->x_slot : nullptr, c->r, c->s, c->t, c->phat, c->shat, c->rhat,
+                                              c->scal, c->part, c->counter, c->state, c->hist, loop_params(c), h, n);
+    };
+    if (graph) go(bicg_xr_kernel<true>);
+    else go(bicg_xr_kernel<false>);
     HMG_CUDA(c, cudaGetLastError());
   }
   return HMG_OK;
@@ -347,11 +369,12 @@ static int solve_body(Ctx *c, double *x, bool graph, cudaGraphConditionalHandle 
 static int solve_tail(Ctx *c, const double *x) { return sys_apply(c, x, nullptr, 3, c->B, Scal::AUX, 0); }
 
 // ---- graph construction ------------------------------------------------------------------
-// Adds one solve (head -> WHILE(body) -> tail) to graph g, without dependencies on other
+// Adds one solve (head -> start -> WHILE(body) -> tail) to graph g, without dependencies on other
 // nodes of g: the head is captured into g, the WHILE node is added after the head's last
 // nodes, the body is captured into the WHILE node's graph on a second stream, and the tail
-// is captured after the WHILE node.
-static int add_solve_branch(Ctx *c, cudaGraph_t g, const double *Rub, const double *Rpi, double *x) {
+// is captured after the WHILE node. loop_only: start and loop alone, on the iterate that c->x_slot names
+// (head and tail are launched around the graph, so that it holds no pointer of the caller's).
+static int add_solve_branch(Ctx *c, cudaGraph_t g, bool loop_only, const double *Rub, const double *Rpi, double *x) {
   if (!c->cap_stream) HMG_CUDA(c, cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking));
   cudaGraphConditionalHandle h;
   HMG_CUDA(c, cudaGraphConditionalHandleCreate(&h, g, 0, cudaGraphCondAssignDefault));
@@ -359,7 +382,8 @@ static int add_solve_branch(Ctx *c, cudaGraph_t g, const double *Rub, const doub
   HMG_CUDA(c, cudaStreamBeginCaptureToGraph(c->cap_stream, g, nullptr, nullptr, 0,
                                             cudaStreamCaptureModeThreadLocal));
   c->stream = c->cap_stream;
-  int st = solve_head(c, Rub, Rpi, x, true, h);
+  int st = loop_only ? HMG_OK : solve_head(c, Rub, Rpi, x);
+  if (!st) st = solve_start(c, true, h);
   if (!st) {
     cudaStreamCaptureStatus cs;
     const cudaGraphNode_t *deps = nullptr;
@@ -385,19 +409,14 @@ static int add_solve_branch(Ctx *c, cudaGraph_t g, const double *Rub, const doub
         st = cuda_fail(c, e, "capture of the iteration body");
       } else {
         c->stream = s2;
-        st = solve_body(c, x, true, h);
+        st = solve_body(c, x, true, loop_only, h);
         cudaGraph_t tmp;
         e = cudaStreamEndCapture(s2, &tmp);
         if (!st && e != cudaSuccess) st = cuda_fail(c, e, "end of the body capture");
       }
       if (s2) cudaStreamDestroy(s2);
       c->stream = c->cap_stream;
-      // an event node after the loop: a copy of lambda to the host can overlap the tail
-      if (!st) {
-        e = cudaEventRecordWithFlags(c->loop_done, c->cap_stream, cudaEventRecordExternal);
-        if (e != cudaSuccess) st = cuda_fail(c, e, "loop-end event node");
-      }
-      if (!st) st = solve_tail(c, x);
+      if (!st && !loop_only) st = solve_tail(c, x);
     }
   }
   c->stream = saved;
@@ -406,11 +425,6 @@ static int add_solve_branch(Ctx *c, cudaGraph_t g, const double *Rub, const doub
   if (st) return st;
   HMG_CUDA(c, e);
   return HMG_OK;
-}
-
-static bool same_key(const Ctx::GraphKey &k, const double *Rub, const double *Rpi, const double *lam,
-                     const hmg_options &o) {
-  return k.Rub == Rub && k.Rpi == Rpi && k.lam == lam && std::memcmp(&k.opt, &o, sizeof(o)) == 0;
 }
 
 uint64_t next_graph_gen() {
@@ -439,16 +453,31 @@ void drop_graph(Ctx *c) {
   drop_batch_graph(c);
 }
 
-static int ensure_solve_graph(Ctx *c, const double *Rub, const double *Rpi, double *x) {
-  if (c->graph_exec && same_key(c->graph_key, Rub, Rpi, x, c->opt)) return HMG_OK;
+// The graph of the loop depends on the options only: a caller's new vectors do not rebuild it (capturing
+// and instantiating it again took 0.18 ms, a fifth of a small solve).
+static int ensure_solve_graph(Ctx *c) {
+  if (c->graph_exec && std::memcmp(&c->graph_opt, &c->opt, sizeof(c->opt)) == 0) return HMG_OK;
   drop_graph(c);
   HMG_CUDA(c, cudaGraphCreate(&c->graph, 0));
-  int st = add_solve_branch(c, c->graph, Rub, Rpi, x);
+  int st = add_solve_branch(c, c->graph, true, nullptr, nullptr, nullptr);
   if (st) { drop_graph(c); return st; }
   cudaError_t e = cudaGraphInstantiate(&c->graph_exec, c->graph, 0);
   if (e != cudaSuccess) { drop_graph(c); return cuda_fail(c, e, "cudaGraphInstantiate"); }
-  c->graph_key = Ctx::GraphKey{Rub, Rpi, x, c->opt};
+  c->graph_opt = c->opt;
   return HMG_OK;
+}
+
+// The whole solve, enqueued: head, loop graph, tail (loop_done is recorded between the last two: a copy
+// of lambda to the host can overlap the tail).
+static int enqueue_solve(Ctx *c, const double *Rub, const double *Rpi, double *x) {
+  int s;
+  if ((s = ensure_solve_graph(c))) return s;
+  if ((s = solve_head(c, Rub, Rpi, x))) return s;
+  set_slot_kernel<<<1, 1, 0, c->stream>>>(c->x_slot, x);
+  HMG_CUDA(c, cudaGetLastError());
+  HMG_CUDA(c, cudaGraphLaunch(c->graph_exec, c->stream));
+  HMG_CUDA(c, cudaEventRecord(c->loop_done, c->stream));
+  return solve_tail(c, x);
 }
 
 // ---- results --------------------------------------------------------------------------------
@@ -556,11 +585,10 @@ int krylov_solve(Ctx *c, const double *Rub, const double *Rpi, double *lambda, h
   const bool host_coarse = c->opt.precond == HMG_PRECOND_NONNESTED &&
                            (c->opt.coarse == HMG_COARSE_KRYLOV_EXACT || c->opt.coarse == HMG_COARSE_KRYLOV_APPROX);
   if (c->opt.graph && !c->opt.profile && !c->collect_x && !host_coarse) {
-    if ((s = ensure_solve_graph(c, Rub, Rpi, lambda))) return s;
     if (allow_async && c->opt.async_stats) {
       // enqueue only: the results travel to the pinned buffers behind the solve
       HMG_CUDA(c, cudaEventRecord(c->as_e0, c->stream));
-      HMG_CUDA(c, cudaGraphLaunch(c->graph_exec, c->stream));
+      if ((s = enqueue_solve(c, Rub, Rpi, lambda))) return s;
       if ((s = enqueue_results(c))) return s;
       // the end event follows the copies: once it completes, the host buffers hold this solve's
       // results (solve_ms includes the few-microsecond copies)
@@ -569,7 +597,7 @@ int krylov_solve(Ctx *c, const double *Rub, const double *Rpi, double *lambda, h
       if (st) st->status = HMG_ERR_NOT_READY;   // the stats come from hmg_solve_stats_get
       return HMG_OK;
     }
-    HMG_CUDA(c, cudaGraphLaunch(c->graph_exec, c->stream));
+    if ((s = enqueue_solve(c, Rub, Rpi, lambda))) return s;
     // one synchronisation: the solve's end, the copy of lambda to the host (on its own stream,
     // from the end of the Krylov loop, so it overlaps the final residual), the results
     HMG_CUDA(c, cudaEventRecord(timer.e1, c->stream));
@@ -589,12 +617,13 @@ int krylov_solve(Ctx *c, const double *Rub, const double *Rpi, double *lambda, h
     return fill_stats(c, st, ms);
   } else {
     cudaGraphConditionalHandle none = 0;
-    if ((s = solve_head(c, Rub, Rpi, lambda, false, none))) return s;
+    if ((s = solve_head(c, Rub, Rpi, lambda))) return s;
+    if ((s = solve_start(c, false, none))) return s;
     for (;;) {
       HMG_CUDA(c, cudaMemcpyAsync(c->state_host, c->state, sizeof(int) * 3, cudaMemcpyDeviceToHost, c->stream));
       HMG_CUDA(c, cudaStreamSynchronize(c->stream));
       if (!c->state_host[kContinue]) break;
-      if ((s = solve_body(c, lambda, false, none))) return s;
+      if ((s = solve_body(c, lambda, false, false, none))) return s;
     }
     if ((s = solve_tail(c, lambda))) return s;
   }
@@ -647,7 +676,7 @@ int krylov_solve_batched(hmg_ctx *const *ctxs, int n, const double *const *Rub,
     HMG_CUDA(c0, cudaGraphCreate(&g, 0));
     for (int i = 0; i < n && !s; ++i) {
       Ctx *c = ctxs[i];
-      s = add_solve_branch(c, g, Rub[i], Rpi[i], lambda[i]);
+      s = add_solve_branch(c, g, false, Rub[i], Rpi[i], lambda[i]);
       if (s && c != c0) c0->err = c->err;
     }
     if (!s) {

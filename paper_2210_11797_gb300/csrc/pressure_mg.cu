@@ -728,7 +728,7 @@ int vcycle_launches(const Ctx *c) {
   if (nmg == 1) return c->opt.mg_ncoarse;
   // finest level: pre-sweeps, restriction, injection and post-sweeps; the coarse levels one launch
   if (c->opt.mg_fused) return npre + 1 + 1 + 1 + npost;
-  int n = npre + 1 + npost;   // finest level: pre-sweeps, injection, post-sweeps
+  int n = npre + (fuse_level(c, 0) ? 0 : 1) + npost;   // finest level: pre-sweeps, (injection,) post-sweeps
   for (int l = 1; l < nmg; ++l) {
     const bool f = fuse_level(c, l);
     n += (l == nmg - 1 ? c->opt.mg_ncoarse : npre) + (f ? 0 : 1);   // sweeps (+ restriction)
@@ -799,9 +799,9 @@ static int vcycle_impl(Ctx *c, const T *b0, T **x_out, const T *x0, const T *R, 
     Level &lv = c->lv[l];
     T *other = x[l] == static_cast<T *>(lv.vx) ? static_cast<T *>(lv.vy) : static_cast<T *>(lv.vx);
     int done = 0;
-    if (l >= 1 && fuse_level(c, l)) {
-      // the injection rides in the first post-sweep (on the finest level it would add 7 FP64
-      // adds per cell to an FP64-bound sweep)
+    if (fuse_level(c, l)) {
+      // the injection rides in the first post-sweep (on larger levels its 7 FP64 adds per cell would
+      // cost an FP64-bound sweep more than the launch saves: 3 us at 2^18 cells)
       if ((st = inject_smooth<T>(c, l, b[l], x[l], x[l + 1], other))) return st;
       done = 1;
     } else {

@@ -54,48 +54,116 @@ __global__ void __launch_bounds__(kRedThreads)
   }
 }
 
-// Sum of the per-block partials of slots s0 (and s1) into scal, in a fixed order.
+// Sum of the per-block partials of slots s0 (and s1) into scal, in a fixed order. alpha: the loop's
+// state, for scal[ALPHA] = rho_i / scal[s0] (null: not wanted).
 __global__ void __launch_bounds__(1024)
-    finalize_kernel(const double *__restrict__ part, int nblocks, int s0, int s1, double *scal) {
+    finalize_kernel(const double *__restrict__ part, int nblocks, int s0, int s1, double *scal, const int *alpha) {
   __shared__ double sh[2][32];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   for (int q = 0; q < 2; ++q) {
     const int slot = q == 0 ? s0 : s1;
     if (slot < 0) break;
-    const double *p = part + (int64_t)slot * kMaxRedBlocks;
-    double acc[4] = {0.0, 0.0, 0.0, 0.0};
-    int b = threadIdx.x;
-    for (; b + 3 * 1024 < nblocks; b += 4 * 1024) {
-      acc[0] += p[b];
-      acc[1] += p[b + 1024];
-      acc[2] += p[b + 2048];
-      acc[3] += p[b + 3072];
-    }
-    for (; b < nblocks; b += 1024) acc[0] += p[b];
-    double v = warp_sum((acc[0] + acc[1]) + (acc[2] + acc[3]));
-    if (lane == 0) sh[q][warp] = v;
-    __syncthreads();
+    const double s = sum_partials(part + (int64_t)slot * kMaxRedBlocks, nblocks, sh[q]);
     if (threadIdx.x == 0) {
-      double s = 0.0;
-      for (int i = 0; i < 32; ++i) s += sh[q][i];
       scal[slot] = s;
+      if (q == 0 && alpha) scal[Scal::ALPHA] = scal[alpha[0] & 1] / s;
     }
   }
 }
 
 int launch_finalize(Ctx *c, int nblocks, int s0, int s1) {
-  finalize_kernel<<<1, 1024, 0, c->stream>>>(c->part, nblocks, s0, s1, c->scal);
+  finalize_kernel<<<1, 1024, 0, c->stream>>>(c->part, nblocks, s0, s1, c->scal, nullptr);
   HMG_CUDA(c, cudaGetLastError());
   return HMG_OK;
 }
 
+// The same S apply for meshes of few rows: one row per thread (1024 per block, so the blocks and the order
+// of every sum are those of spmv_kernel and finalize_kernel), and the last block adds the partials,
+// one launch instead of two. At 6,400 rows spmv_kernel's seven blocks took their four rows per thread one
+// after another: 18 us and 8 us for the sum (serialised); this form 8 us.
+template <int MODE>
+__global__ void __launch_bounds__(1024)
+    spmv_small_kernel(const double *__restrict__ S, const double *__restrict__ x, double *__restrict__ y,
+                      const double *__restrict__ w, const TraceDims d, const int32_t *__restrict__ stencil,
+                      const int32_t *__restrict__ col_edges, double *part, int slot0, int slot1,
+                      unsigned int *counter, double *scal, const int *alpha) {
+  constexpr int NV = MODE == 2 ? 2 : 1;
+  static_assert(kSpmvRows * kRedThreads == 1024, "the block's rows");
+  __shared__ double sv[1024], sw[1024], sh[NV][kRedThreads];
+  __shared__ bool is_last;
+  const int t = threadIdx.x;
+  const int64_t row = (int64_t)blockIdx.x * 1024 + t;
+  if (row < d.NT) {
+    const double v = MODE == 3 ? s_row<double, double, double, true>(S, x, stencil, col_edges, d, row, __ldg(w + row))
+                               : s_row<double, double, double, false>(S, x, stencil, col_edges, d, row, 0.0);
+    if (MODE != 3) y[row] = v;
+    sv[t] = v;
+    if (MODE != 3) sw[t] = __ldg(w + row);
+  }
+  __syncthreads();
+  if (t < kRedThreads) {
+    double a0 = 0.0, a1 = 0.0;
+#pragma unroll
+    for (int j = 0; j < kSpmvRows; ++j) {
+      const int q = t + j * kRedThreads;
+      if ((int64_t)blockIdx.x * 1024 + q < d.NT) {
+        const double v = sv[q];
+        if (MODE == 3) a0 = fma(v, v, a0);
+        if (MODE == 1) a0 = fma(sw[q], v, a0);
+        if (MODE == 2) { a0 = fma(v, sw[q], a0); a1 = fma(v, v, a1); }
+      }
+    }
+    sh[0][t] = a0;
+    if (NV == 2) sh[NV - 1][t] = a1;
+  }
+  __syncthreads();
+  if (t < 32) {
+#pragma unroll
+    for (int i = 0; i < NV; ++i) {
+      double v = sh[i][t];
+      for (int j = t + 32; j < kRedThreads; j += 32) v += sh[i][j];
+      v = warp_sum(v);
+      if (t == 0) part[(int64_t)(i == 0 ? slot0 : slot1) * kMaxRedBlocks + blockIdx.x] = v;
+    }
+  }
+  if (t == 0) {
+    __threadfence();
+    is_last = atomicAdd(&counter[slot0], 1u) == gridDim.x - 1;
+  }
+  __syncthreads();
+  if (!is_last) return;
+  __threadfence();
+#pragma unroll
+  for (int i = 0; i < NV; ++i) {
+    const int slot = i == 0 ? slot0 : slot1;
+    const double s = sum_partials(part + (int64_t)slot * kMaxRedBlocks, (int)gridDim.x, sh[i]);
+    if (t == 0) {
+      scal[slot] = s;
+      if (i == 0 && alpha) scal[Scal::ALPHA] = scal[alpha[0] & 1] / s;
+    }
+  }
+  if (t == 0) counter[slot0] = 0u;
+}
+
 int launch_spmv(Ctx *c, const double *x, double *y, int mode, const double *w, int slot0,
-                int slot1) {
+                int slot1, bool alpha) {
   const Level &f = c->lv[0];
   const TraceDims d = dims_of(f);
   const unsigned g = grid_for(f.ntrace, kRedThreads * kSpmvRows);
   if (g > (unsigned)kMaxRedBlocks) return fail(c, HMG_ERR_INVALID_ARG, "too many rows for one reduction");
   Prof prof(c, kCompApply);
+  const int *as = alpha && mode == 1 ? c->state : nullptr;
+  // few rows (at most a block per SM): one row per thread and one launch, bitwise the same
+  if (mode != 0 && g <= (unsigned)c->num_sms) {
+    auto go = [&](auto kern) {
+      kern<<<g, 1024, 0, c->stream>>>(c->S, x, y, w, d, f.edge_stencil, f.col_edges, c->part, slot0, slot1, c->counter,
+                                      c->scal, as);
+    };
+    if (mode == 1) go(spmv_small_kernel<1>);
+    else if (mode == 2) go(spmv_small_kernel<2>);
+    else go(spmv_small_kernel<3>);
+    HMG_CUDA(c, cudaGetLastError());
+    return HMG_OK;
+  }
   switch (mode) {
     case 0: spmv_kernel<0><<<g, kRedThreads, 0, c->stream>>>(c->S, x, y, w, d, f.edge_stencil, f.col_edges, c->part, slot0, slot1); break;
     case 1: spmv_kernel<1><<<g, kRedThreads, 0, c->stream>>>(c->S, x, y, w, d, f.edge_stencil, f.col_edges, c->part, slot0, slot1); break;
@@ -103,7 +171,7 @@ int launch_spmv(Ctx *c, const double *x, double *y, int mode, const double *w, i
     default: spmv_kernel<3><<<g, kRedThreads, 0, c->stream>>>(c->S, x, y, w, d, f.edge_stencil, f.col_edges, c->part, slot0, slot1); break;
   }
   if (mode != 0)
-    finalize_kernel<<<1, 1024, 0, c->stream>>>(c->part, (int)g, slot0, mode == 2 ? slot1 : -1, c->scal);
+    finalize_kernel<<<1, 1024, 0, c->stream>>>(c->part, (int)g, slot0, mode == 2 ? slot1 : -1, c->scal, as);
   HMG_CUDA(c, cudaGetLastError());
   return HMG_OK;
 }
@@ -208,9 +276,27 @@ struct SweepArgs {
   int ncol, cpb, nzb;
   const int32_t *stencil, *col_edges;
   double keep;   // 1 - omega
+  FusedVector fv;
 };
 
-template <typename T, typename Tb, typename Tout, bool ZERO>
+// b of one row; FUSE: formed from other Krylov vectors and stored (a zero-start sweep reads every row of
+// b once, so BiCGStab's p and s need no kernel of their own: one pass over the vector and one launch less)
+template <int FUSE, typename Tb>
+__device__ __forceinline__ Tb sweep_b(const SweepArgs &a, const Tb *__restrict__ b, int64_t row) {
+  if constexpr (FUSE == 1) {
+    const double p = fma(a.fv.scal[Scal::BETA], fma(-a.fv.scal[Scal::OMEGA], a.fv.v[row], a.fv.out[row]), a.fv.r[row]);
+    a.fv.out[row] = p;
+    return p;
+  } else if constexpr (FUSE == 2) {
+    const double s = fma(-a.fv.scal[Scal::ALPHA], a.fv.v[row], a.fv.r[row]);
+    a.fv.out[row] = s;
+    return s;
+  } else {
+    return __ldg(b + row);
+  }
+}
+
+template <typename T, typename Tb, typename Tout, bool ZERO, int FUSE = 0>
 __global__ void __launch_bounds__(256)
     sweep_kernel(const SweepArgs a, const T *__restrict__ S, const T *__restrict__ zw,
                  const T *__restrict__ zl, const T *__restrict__ zcp, const T *__restrict__ hw,
@@ -232,7 +318,7 @@ __global__ void __launch_bounds__(256)
 #pragma unroll 2
     for (int i = threadIdx.x; i < nrow; i += blockDim.x) {
       const int64_t row = base + i;
-      T r = (T)__ldg(b + row);
+      T r = (T)sweep_b<FUSE>(a, b, row);
       if (!ZERO) r = s_row_z_off<T, T, T>(S, lam_in, a.col_edges, d, row, r);
       const int j = (i / L1) * ld + i % L1;
       sr[j] = r * __ldg(zw + (row - d.NH));
@@ -254,7 +340,7 @@ __global__ void __launch_bounds__(256)
     for (int j = 0; j < HR; ++j) {
       const int64_t row = base + (int64_t)j * blockDim.x;
       if (row < d.NH) {
-        T r = (T)__ldg(b + row);
+        T r = (T)sweep_b<FUSE>(a, b, row);
         if (!ZERO) r = s_row_h<T, T, T, true>(S, lam_in, a.stencil, d, row, r);
         lam_out[row] = (Tout)(ZERO ? r * __ldg(hw + row) : fma(r, __ldg(hw + row), lam_in[row]));
       }
@@ -266,7 +352,7 @@ __global__ void __launch_bounds__(256)
 // block -1; L + 1 <= 32 M rows): lane j holds rows j M .. j M + M - 1, whose residuals it
 // computes, and the Thomas recurrences run as a warp scan (warp_thomas); 8 columns per block of
 // 256 threads. The remaining blocks take lambda^h rows as in sweep_kernel.
-template <typename T, typename Tb, typename Tout, bool ZERO, int M>
+template <typename T, typename Tb, typename Tout, bool ZERO, int M, int FUSE = 0>
 __global__ void __launch_bounds__(256)
     sweep_warp_kernel(const SweepArgs a, const T *__restrict__ S, const T *__restrict__ zw,
                       const T *__restrict__ zl, const T *__restrict__ zcp, const T *__restrict__ hw,
@@ -284,7 +370,7 @@ __global__ void __launch_bounds__(256)
       s[i] = lo[i] = up[i] = (T)0;
       if (k < L1) {
         const int64_t row = base + k;
-        T r = (T)__ldg(b + row);
+        T r = (T)sweep_b<FUSE>(a, b, row);
         if (!ZERO) r = s_row_z_off<T, T, T>(S, lam_in, a.col_edges, d, row, r);
         s[i] = r * __ldg(zw + (row - d.NH));
         if (k > 0) lo[i] = __ldg(zl + (row - d.NH));
@@ -307,7 +393,7 @@ __global__ void __launch_bounds__(256)
     for (int j = 0; j < HR; ++j) {
       const int64_t row = base + (int64_t)j * blockDim.x;
       if (row < d.NH) {
-        T r = (T)__ldg(b + row);
+        T r = (T)sweep_b<FUSE>(a, b, row);
         if (!ZERO) r = s_row_h<T, T, T, true>(S, lam_in, a.stencil, d, row, r);
         lam_out[row] = (Tout)(ZERO ? r * __ldg(hw + row) : fma(r, __ldg(hw + row), lam_in[row]));
       }
@@ -322,11 +408,12 @@ static int sweep_cpb_limit(int nlev) {
   return m < 1 ? 1 : (m > 64 ? 64 : m);
 }
 
-template <typename T, typename Tb, typename Tout, bool ZERO>
+template <typename T, typename Tb, typename Tout, bool ZERO, int FUSE = 0>
 static int launch_sweep(Ctx *c, const Tb *b, const T *lam_in, Tout *lam_out, int cpb_override = 0,
-                        int threads_override = 0) {
+                        int threads_override = 0, const FusedVector *fv = nullptr) {
   const Level &f = c->lv[0];
   SweepArgs a;
+  if (FUSE) a.fv = *fv;
   a.d = dims_of(f);
   a.ncol = f.ncol;
   const int cpb_max = sweep_cpb_limit(f.nlev);
@@ -347,9 +434,9 @@ static int launch_sweep(Ctx *c, const Tb *b, const T *lam_in, Tout *lam_out, int
         kern<<<a.nzb + nhb, 256, 0, c->stream>>>(a, Prec<T>::S(c), Prec<T>::Sz_w(c), Prec<T>::Sz_l(c),
                                                  Prec<T>::Sz_cp(c), Prec<T>::Sh_w(c), b, lam_in, lam_out);
       };
-      if (L1 <= 32) go(sweep_warp_kernel<T, Tb, Tout, ZERO, 1>);
-      else if (L1 <= 64) go(sweep_warp_kernel<T, Tb, Tout, ZERO, 2>);
-      else go(sweep_warp_kernel<T, Tb, Tout, ZERO, 4>);
+      if (L1 <= 32) go(sweep_warp_kernel<T, Tb, Tout, ZERO, 1, FUSE>);
+      else if (L1 <= 64) go(sweep_warp_kernel<T, Tb, Tout, ZERO, 2, FUSE>);
+      else go(sweep_warp_kernel<T, Tb, Tout, ZERO, 4, FUSE>);
       HMG_CUDA(c, cudaGetLastError());
       return HMG_OK;
     }
@@ -368,7 +455,7 @@ static int launch_sweep(Ctx *c, const Tb *b, const T *lam_in, Tout *lam_out, int
   const unsigned nhb = grid_for(f.nth, (int64_t)threads * kSweepHRows<T, ZERO>);
   const size_t smem = (size_t)3 * a.cpb * ((f.nlev + 1) | 1) * sizeof(T);
   Prof prof(c, ZERO ? kCompPresmooth : kCompSweep);
-  sweep_kernel<T, Tb, Tout, ZERO><<<a.nzb + nhb, threads, smem, c->stream>>>(
+  sweep_kernel<T, Tb, Tout, ZERO, FUSE><<<a.nzb + nhb, threads, smem, c->stream>>>(
       a, Prec<T>::S(c), Prec<T>::Sz_w(c), Prec<T>::Sz_l(c), Prec<T>::Sz_cp(c), Prec<T>::Sh_w(c), b,
       lam_in, lam_out);
   HMG_CUDA(c, cudaGetLastError());
@@ -409,17 +496,15 @@ __global__ void restrict_kernel(const T *__restrict__ R, const T *__restrict__ g
 }
 
 // ---- lam_out = lam_in + P dPi (Algorithm 2 line 7) ---------------------------------------
-constexpr int kProlongRows = 4;
-
-template <typename T>
+template <typename T, int ROWS>
 __global__ void prolong_kernel(const T *__restrict__ lam_in, const T *__restrict__ dpi,
                                T *__restrict__ lam_out, const TraceDims d,
                                const int32_t *__restrict__ stencil) {
-  // kProlongRows rows per thread, block-strided: few operations per row, so the kernel waits on
-  // its loads and more rows per thread keep more of them in flight
-  const int64_t base = blockIdx.x * (int64_t)blockDim.x * kProlongRows + threadIdx.x;
+  // ROWS rows per thread, block-strided: few operations per row, so the kernel waits on its loads and
+  // more rows per thread keep more of them in flight
+  const int64_t base = blockIdx.x * (int64_t)blockDim.x * ROWS + threadIdx.x;
 #pragma unroll
-  for (int j = 0; j < kProlongRows; ++j) {
+  for (int j = 0; j < ROWS; ++j) {
     const int64_t row = base + (int64_t)j * blockDim.x;
     if (row >= d.NT) break;
     // lam_in + (1/2)(a + b) as one FMA: the halving is exact, so it rounds as the add did
@@ -449,14 +534,23 @@ __global__ void convert_kernel(const Tin *__restrict__ in, Tout *__restrict__ ou
 }
 
 // ---- preconditioners -----------------------------------------------------------------------
+// The first sweep, from zero; with fv it forms r on the way.
+template <typename T, typename Tout>
+static int first_sweep(Ctx *c, const double *r, Tout *out, const FusedVector *fv) {
+  const T *none = nullptr;
+  if (!fv) return launch_sweep<T, double, Tout, true>(c, r, none, out);
+  if (fv->kind == 1) return launch_sweep<T, double, Tout, true, 1>(c, r, none, out, 0, 0, fv);
+  return launch_sweep<T, double, Tout, true, 2>(c, r, none, out, 0, 0, fv);
+}
+
 // Configuration 2: n_smooth sweeps of Algorithm 1 from zero.
 template <typename T>
-static int line_precond(Ctx *c, const double *r, double *z) {
+static int line_precond(Ctx *c, const double *r, double *z, const FusedVector *fv) {
   const int n = c->opt.n_smooth;
   T *a = static_cast<T *>(c->w1), *b2 = static_cast<T *>(c->w2);
   int st;
-  if (n == 1) return launch_sweep<T, double, double, true>(c, r, nullptr, z);
-  if ((st = launch_sweep<T, double, T, true>(c, r, nullptr, a))) return st;
+  if (n == 1) return first_sweep<T>(c, r, z, fv);
+  if ((st = first_sweep<T>(c, r, a, fv))) return st;
   for (int i = 1; i < n - 1; ++i) {
     if ((st = launch_sweep<T, double, T, false>(c, r, a, b2))) return st;
     T *t = a; a = b2; b2 = t;
@@ -466,14 +560,14 @@ static int line_precond(Ctx *c, const double *r, double *z) {
 
 // Configuration 3c: Algorithm 2 with one pressure V-cycle as the coarse solve.
 template <typename T>
-static int two_level(Ctx *c, const double *r, double *z) {
+static int two_level(Ctx *c, const double *r, double *z, const FusedVector *fv) {
   const Level &f = c->lv[0];
   const TraceDims d = dims_of(f);
   T *w1 = static_cast<T *>(c->w1), *w2 = static_cast<T *>(c->w2), *w3 = static_cast<T *>(c->w3);
   int st;
   // line 1-2: lambda = 0, presmooth
   if (c->opt.n_pre >= 1) {
-    if ((st = launch_sweep<T, double, T, true>(c, r, nullptr, w1))) return st;
+    if ((st = first_sweep<T>(c, r, w1, fv))) return st;
     for (int i = 1; i < c->opt.n_pre; ++i) {
       if ((st = launch_sweep<T, double, T, false>(c, r, w1, w2))) return st;
       T *t = w1; w1 = w2; w2 = t;
@@ -530,7 +624,11 @@ static int two_level(Ctx *c, const double *r, double *z) {
   // line 7: lambda += P dPi
   {
     Prof pp(c, kCompProlong);
-    prolong_kernel<T><<<grid_for(f.ntrace, 256 * kProlongRows), 256, 0, c->stream>>>(w1, dpi, w2, d, f.edge_stencil);
+    // four rows per thread where that still gives every SM two blocks of 256
+    if (f.ntrace >= (int64_t)4 * 256 * 2 * c->num_sms)
+      prolong_kernel<T, 4><<<grid_for(f.ntrace, 256 * 4), 256, 0, c->stream>>>(w1, dpi, w2, d, f.edge_stencil);
+    else
+      prolong_kernel<T, 1><<<grid_for(f.ntrace, 128), 128, 0, c->stream>>>(w1, dpi, w2, d, f.edge_stencil);
   }
   HMG_CUDA(c, cudaGetLastError());
   // line 8: postsmooth
@@ -548,7 +646,12 @@ static int two_level(Ctx *c, const double *r, double *z) {
   return launch_sweep<T, double, double, false>(c, r, cur, z);
 }
 
-int precond_apply(Ctx *c, const double *r, double *z) {
+bool precond_fuses(const Ctx *c) {
+  return c->degree == 0 && (c->opt.precond == HMG_PRECOND_LINESMOOTH ||
+                            (c->opt.precond == HMG_PRECOND_NONNESTED && c->opt.n_pre >= 1));
+}
+
+int precond_apply(Ctx *c, const double *r, double *z, const FusedVector *fv) {
   if (c->degree >= 1) return ho_precond(c, r, z);
   const bool mixed = c->opt.precision == HMG_PRECISION_MIXED;
   switch (c->opt.precond) {
@@ -559,9 +662,9 @@ int precond_apply(Ctx *c, const double *r, double *z) {
                                   c->stream));
       return HMG_OK;
     case HMG_PRECOND_LINESMOOTH:
-      return mixed ? line_precond<float>(c, r, z) : line_precond<double>(c, r, z);
+      return mixed ? line_precond<float>(c, r, z, fv) : line_precond<double>(c, r, z, fv);
     default:
-      return mixed ? two_level<float>(c, r, z) : two_level<double>(c, r, z);
+      return mixed ? two_level<float>(c, r, z, fv) : two_level<double>(c, r, z, fv);
   }
 }
 
