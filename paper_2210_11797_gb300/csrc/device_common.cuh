@@ -98,24 +98,36 @@ __device__ __forceinline__ bool grid_reduce(const double (&val)[NV], const int (
   return true;
 }
 
-// Sum of the per-block partials of one slot by 1024 threads, in a fixed order; valid in thread 0.
-// sh: 32 doubles of shared memory.
+// Sum of the per-block partials of one slot, in a fixed order that does not depend on the block's THREADS:
+// that of 1024 threads, thread t taking partials t, t + 1024, ..., a shuffle tree per 32 of them and the
+// 32 trees' sums in turn. Valid in thread 0. Trees without partials are left out (their sums are +0): the
+// FP64 pipe is occupied per warp, and 32 idle trees took 3 us. sh: 32 doubles of shared memory.
+template <int THREADS>
 __device__ __forceinline__ double sum_partials(const double *p, int nblocks, double *sh) {
-  double acc[4] = {0.0, 0.0, 0.0, 0.0};
-  int b = threadIdx.x;
-  for (; b + 3 * 1024 < nblocks; b += 4 * 1024) {
-    acc[0] += __ldcg(p + b);
-    acc[1] += __ldcg(p + b + 1024);
-    acc[2] += __ldcg(p + b + 2048);
-    acc[3] += __ldcg(p + b + 3072);
+  const int lane = threadIdx.x & 31, ntree = min(32, (nblocks + 31) >> 5);
+  for (int w = threadIdx.x >> 5; w < ntree; w += THREADS / 32) {
+    int b = w * 32 + lane;
+    double v;
+    if (nblocks <= 1024) {
+      v = b < nblocks ? __ldcg(p + b) : 0.0;
+    } else {
+      double acc[4] = {0.0, 0.0, 0.0, 0.0};
+      for (; b + 3 * 1024 < nblocks; b += 4 * 1024) {
+        acc[0] += __ldcg(p + b);
+        acc[1] += __ldcg(p + b + 1024);
+        acc[2] += __ldcg(p + b + 2048);
+        acc[3] += __ldcg(p + b + 3072);
+      }
+      for (; b < nblocks; b += 1024) acc[0] += __ldcg(p + b);
+      v = (acc[0] + acc[1]) + (acc[2] + acc[3]);
+    }
+    v = warp_sum(v);
+    if (lane == 0) sh[w] = v;
   }
-  for (; b < nblocks; b += 1024) acc[0] += __ldcg(p + b);
-  const double v = warp_sum((acc[0] + acc[1]) + (acc[2] + acc[3]));
-  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
   __syncthreads();
   double s = 0.0;
   if (threadIdx.x == 0)
-    for (int i = 0; i < 32; ++i) s += sh[i];
+    for (int i = 0; i < ntree; ++i) s += sh[i];
   return s;
 }
 

@@ -338,26 +338,9 @@ __global__ void __launch_bounds__(256)
   __threadfence();
 #pragma unroll
   for (int q = 0; q < NV; ++q) {
-    const double *p = part + (int64_t)(q ? slot1 : slot0) * kMaxRedBlocks;
-    for (int j = 0; j < 4; ++j) {   // the 1024 threads of finalize_kernel
-      double acc[4] = {0.0, 0.0, 0.0, 0.0};
-      int b = threadIdx.x + 256 * j;
-      for (; b + 3 * 1024 < ng; b += 4 * 1024) {
-        acc[0] += __ldcg(p + b);
-        acc[1] += __ldcg(p + b + 1024);
-        acc[2] += __ldcg(p + b + 2048);
-        acc[3] += __ldcg(p + b + 3072);
-      }
-      for (; b < ng; b += 1024) acc[0] += __ldcg(p + b);
-      const double v = warp_sum((acc[0] + acc[1]) + (acc[2] + acc[3]));
-      if (lane == 0) sh[q][warp + 8 * j] = v;
-    }
-  }
-  __syncthreads();
-  if (threadIdx.x < NV) {
-    double s = 0.0;
-    for (int i = 0; i < 32; ++i) s += sh[threadIdx.x][i];
-    scal[threadIdx.x ? slot1 : slot0] = s;
+    const int slot = q ? slot1 : slot0;
+    const double s = sum_partials<256>(part + (int64_t)slot * kMaxRedBlocks, ng, sh[q]);
+    if (threadIdx.x == 0) scal[slot] = s;
   }
   if (threadIdx.x == 0) counter[slot0] = 0u;
 }

@@ -62,7 +62,7 @@ __global__ void __launch_bounds__(1024)
   for (int q = 0; q < 2; ++q) {
     const int slot = q == 0 ? s0 : s1;
     if (slot < 0) break;
-    const double s = sum_partials(part + (int64_t)slot * kMaxRedBlocks, nblocks, sh[q]);
+    const double s = sum_partials<1024>(part + (int64_t)slot * kMaxRedBlocks, nblocks, sh[q]);
     if (threadIdx.x == 0) {
       scal[slot] = s;
       if (q == 0 && alpha) scal[Scal::ALPHA] = scal[alpha[0] & 1] / s;
@@ -76,72 +76,67 @@ int launch_finalize(Ctx *c, int nblocks, int s0, int s1) {
   return HMG_OK;
 }
 
-// The same S apply for meshes of few rows: one row per thread (1024 per block, so the blocks and the order
-// of every sum are those of spmv_kernel and finalize_kernel), and the last block adds the partials,
-// one launch instead of two. At 6,400 rows spmv_kernel's seven blocks took their four rows per thread one
-// after another: 18 us and 8 us for the sum (serialised); this form 8 us.
+// The same S apply for meshes of few rows, in two launches: the rows, one per thread in small blocks over
+// all SMs, then the inner products from y and w with spmv_kernel's blocks and order, the last block adding
+// the partials in finalize_kernel's order (bitwise the same sums). spmv_kernel leaves most SMs idle there,
+// with its FP64 work four rows deep on a few: at 6,400 rows seven blocks, 12-17 us for the apply and 8 us
+// for the partials.
+template <bool NEG>   // NEG: y = w - S x
+__global__ void __launch_bounds__(128)
+    spmv_rows_kernel(const double *__restrict__ S, const double *__restrict__ x, double *__restrict__ y,
+                     const double *__restrict__ w, const TraceDims d, const int32_t *__restrict__ stencil,
+                     const int32_t *__restrict__ col_edges) {
+  const int64_t row = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (row >= d.NT) return;
+  y[row] = s_row<double, double, double, NEG>(S, x, stencil, col_edges, d, row, NEG ? __ldg(w + row) : 0.0);
+}
+
 template <int MODE>
-__global__ void __launch_bounds__(1024)
-    spmv_small_kernel(const double *__restrict__ S, const double *__restrict__ x, double *__restrict__ y,
-                      const double *__restrict__ w, const TraceDims d, const int32_t *__restrict__ stencil,
-                      const int32_t *__restrict__ col_edges, double *part, int slot0, int slot1,
-                      unsigned int *counter, double *scal, const int *alpha) {
+__global__ void __launch_bounds__(kRedThreads)
+    spmv_dots_kernel(const double *__restrict__ y, const double *__restrict__ w, int64_t n, double *part, int slot0,
+                     int slot1, unsigned int *counter, double *scal, const int *alpha) {
   constexpr int NV = MODE == 2 ? 2 : 1;
-  static_assert(kSpmvRows * kRedThreads == 1024, "the block's rows");
-  __shared__ double sv[1024], sw[1024], sh[NV][kRedThreads];
+  __shared__ double sh[32];
   __shared__ bool is_last;
-  const int t = threadIdx.x;
-  const int64_t row = (int64_t)blockIdx.x * 1024 + t;
-  if (row < d.NT) {
-    const double v = MODE == 3 ? s_row<double, double, double, true>(S, x, stencil, col_edges, d, row, __ldg(w + row))
-                               : s_row<double, double, double, false>(S, x, stencil, col_edges, d, row, 0.0);
-    if (MODE != 3) y[row] = v;
-    sv[t] = v;
-    if (MODE != 3) sw[t] = __ldg(w + row);
-  }
-  __syncthreads();
-  if (t < kRedThreads) {
-    double a0 = 0.0, a1 = 0.0;
+  const int64_t base = (int64_t)blockIdx.x * (kRedThreads * kSpmvRows) + threadIdx.x;
+  double val[NV] = {};
+  double v[kSpmvRows], u[kSpmvRows];
 #pragma unroll
-    for (int j = 0; j < kSpmvRows; ++j) {
-      const int q = t + j * kRedThreads;
-      if ((int64_t)blockIdx.x * 1024 + q < d.NT) {
-        const double v = sv[q];
-        if (MODE == 3) a0 = fma(v, v, a0);
-        if (MODE == 1) a0 = fma(sw[q], v, a0);
-        if (MODE == 2) { a0 = fma(v, sw[q], a0); a1 = fma(v, v, a1); }
-      }
-    }
-    sh[0][t] = a0;
-    if (NV == 2) sh[NV - 1][t] = a1;
+  for (int j = 0; j < kSpmvRows; ++j) {
+    const int64_t row = base + j * kRedThreads;
+    v[j] = row < n ? y[row] : 0.0;
+    u[j] = MODE != 3 && row < n ? __ldg(w + row) : 0.0;
   }
-  __syncthreads();
-  if (t < 32) {
 #pragma unroll
-    for (int i = 0; i < NV; ++i) {
-      double v = sh[i][t];
-      for (int j = t + 32; j < kRedThreads; j += 32) v += sh[i][j];
-      v = warp_sum(v);
-      if (t == 0) part[(int64_t)(i == 0 ? slot0 : slot1) * kMaxRedBlocks + blockIdx.x] = v;
+  for (int j = 0; j < kSpmvRows; ++j) {
+    if (base + j * kRedThreads >= n) break;
+    if (MODE == 3) val[0] = fma(v[j], v[j], val[0]);
+    if (MODE == 1) val[0] = fma(u[j], v[j], val[0]);
+    if (MODE == 2) {
+      val[0] = fma(v[j], u[j], val[0]);
+      val[NV - 1] = fma(v[j], v[j], val[NV - 1]);
     }
   }
-  if (t == 0) {
+  int sl[NV];
+  sl[0] = slot0;
+  if (NV == 2) sl[NV - 1] = slot1;
+  block_partials<NV>(val, sl, part);
+  if (threadIdx.x == 0) {
     __threadfence();
     is_last = atomicAdd(&counter[slot0], 1u) == gridDim.x - 1;
   }
   __syncthreads();
   if (!is_last) return;
   __threadfence();
-#pragma unroll
   for (int i = 0; i < NV; ++i) {
-    const int slot = i == 0 ? slot0 : slot1;
-    const double s = sum_partials(part + (int64_t)slot * kMaxRedBlocks, (int)gridDim.x, sh[i]);
-    if (t == 0) {
-      scal[slot] = s;
+    const double s = sum_partials<kRedThreads>(part + (int64_t)sl[i] * kMaxRedBlocks, (int)gridDim.x, sh);
+    if (threadIdx.x == 0) {
+      scal[sl[i]] = s;
       if (i == 0 && alpha) scal[Scal::ALPHA] = scal[alpha[0] & 1] / s;
     }
+    __syncthreads();   // sh is used again
   }
-  if (t == 0) counter[slot0] = 0u;
+  if (threadIdx.x == 0) counter[slot0] = 0u;
 }
 
 int launch_spmv(Ctx *c, const double *x, double *y, int mode, const double *w, int slot0,
@@ -152,15 +147,13 @@ int launch_spmv(Ctx *c, const double *x, double *y, int mode, const double *w, i
   if (g > (unsigned)kMaxRedBlocks) return fail(c, HMG_ERR_INVALID_ARG, "too many rows for one reduction");
   Prof prof(c, kCompApply);
   const int *as = alpha && mode == 1 ? c->state : nullptr;
-  // few rows (at most a block per SM): one row per thread and one launch, bitwise the same
-  if (mode != 0 && g <= (unsigned)c->num_sms) {
-    auto go = [&](auto kern) {
-      kern<<<g, 1024, 0, c->stream>>>(c->S, x, y, w, d, f.edge_stencil, f.col_edges, c->part, slot0, slot1, c->counter,
-                                      c->scal, as);
-    };
-    if (mode == 1) go(spmv_small_kernel<1>);
-    else if (mode == 2) go(spmv_small_kernel<2>);
-    else go(spmv_small_kernel<3>);
+  // up to four of spmv_kernel's blocks per SM (its last wave of them is uneven: 308 blocks at C24 x 30)
+  if (mode != 0 && g <= 4u * (unsigned)c->num_sms) {
+    if (mode == 3) y = static_cast<double *>(c->w1);   // (a place for the residual: the preconditioner is idle)
+    auto rows = mode == 3 ? spmv_rows_kernel<true> : spmv_rows_kernel<false>;
+    rows<<<grid_for(f.ntrace, 128), 128, 0, c->stream>>>(c->S, x, y, w, d, f.edge_stencil, f.col_edges);
+    auto dots = mode == 1 ? spmv_dots_kernel<1> : (mode == 2 ? spmv_dots_kernel<2> : spmv_dots_kernel<3>);
+    dots<<<g, kRedThreads, 0, c->stream>>>(y, w, f.ntrace, c->part, slot0, slot1, c->counter, c->scal, as);
     HMG_CUDA(c, cudaGetLastError());
     return HMG_OK;
   }
