@@ -76,8 +76,8 @@ struct Level {
 // Work buffers of the coarse-model training (learned.cu), grown on demand and reused.
 struct TrainBufs {
   int64_t cap_cells = 0, cap_blocks = 0;
-  void *h1 = nullptr, *h2 = nullptr, *h3 = nullptr;   // activations (BF16 or FP32)
-  float *ga3 = nullptr, *ga2 = nullptr, *gy = nullptr;
+  void *h1 = nullptr, *h2 = nullptr;   // activations (BF16 or FP32)
+  float *ga3 = nullptr, *ga2 = nullptr;
   double *loss_part = nullptr, *loss = nullptr;
   float *part3 = nullptr, *partM = nullptr, *part2 = nullptr, *part1 = nullptr;
   float *grad = nullptr, *m = nullptr, *v = nullptr;

@@ -440,25 +440,37 @@ __global__ void __launch_bounds__(512)
   if (act && q == 0) out[(int64_t)c0 * L + j] = (Tout)(y * dsc);
 }
 
+__host__ __device__ constexpr int back_stride(int L) { return (L + 2) | 1; }   // words per row of h3
+
 // ---- forward, horizontal mix and output layer: h2 -> h3 -> y ---------------------------------
 // mesh: out[K] = y * yscale(K) (yscale = 1/sqrt(diag H)) written as Tout.
-// training: also stores h3 and, for the loss, gy = 2 (y - t) / (||t_s||^2 B) and the per-block
-// sums of (y - t)^2 / ||t_s||^2 (sample s of the block's columns).
-template <typename A, typename Tout>
+// training (TRAIN): gy = 2 (y - t) / (||t_s||^2 B) and the per-block sums of (y - t)^2 / ||t_s||^2
+// (sample s of the block's columns), then the output layer's backward while h3 and gy are in shared
+// memory: gh3 = conv^T(W3, gy), ga3 = gh3 [h3 > 0], partial gW3[ch][d] = sum gy[k] h3[ch][k+d-1] to
+// part[block][96].
+// One thread per (column, level) with the channels in a loop: its nine cells' offsets are formed once,
+// where a thread per element formed them, with two divisions, for every channel. Rows of h3 are an odd
+// number of words apart, so that the 32 channels of one level lie in 32 banks. 64 patches of
+// 16 x 16 x 30 in BF16: 82 us; with a thread per element, h3 stored and a second kernel for the
+// backward, 141 + 91 us.
+template <typename A, typename Tout, bool TRAIN>
 __global__ void __launch_bounds__(128)
     nn_back_kernel(const float *__restrict__ wts, const A *__restrict__ h2, Nbrs nb, int ncol, int L,
                    int cpb, const double *__restrict__ diagH, const float *__restrict__ diagH32,
-                   Tout *__restrict__ out, A *__restrict__ h3_out, const float *__restrict__ target,
+                   Tout *__restrict__ out, const float *__restrict__ target,
                    const float *__restrict__ tnorm2, int patch_cols, float inv_batch,
-                   float *__restrict__ gy_out, double *__restrict__ loss_part) {
-  extern __shared__ float sm[];
-  float *Mw = sm, *W3 = Mw + 96;
-  float *h3 = W3 + 96;                          // [cpb][32][L+2]
+                   double *__restrict__ loss_part, float *__restrict__ ga3, float *__restrict__ part) {
+  extern __shared__ __align__(16) float back_sm[];
+  const int Lp = back_stride(L);
+  float4 *Mw = reinterpret_cast<float4 *>(back_sm), *W3 = Mw + kCh;   // a channel's three weights: one load
+  float *h3 = back_sm + 8 * kCh;                          // [cpb][32][Lp], zero beyond the column ends
+  float *gys = h3 + cpb * kCh * Lp;             // gy [cpb][L+2], likewise (training)
   __shared__ double red[4];
   __shared__ int snb[kMaxNnCpb][8];             // edge and corner neighbours of the block's columns
-  for (int i = threadIdx.x; i < 96; i += blockDim.x) {
-    Mw[i] = rnd<A>(wts[kOffM + i]);
-    W3[i] = rnd<A>(wts[kOffW3 + i]);
+  for (int i = threadIdx.x; i < kCh; i += blockDim.x) {
+    const float *a = wts + kOffM + 3 * i, *b = wts + kOffW3 + 3 * i;
+    Mw[i] = make_float4(rnd<A>(a[0]), rnd<A>(a[1]), rnd<A>(a[2]), 0.f);
+    W3[i] = make_float4(rnd<A>(b[0]), rnd<A>(b[1]), rnd<A>(b[2]), 0.f);
   }
   const int c0 = blockIdx.x * cpb, nc = min(cpb, ncol - c0);
   const int64_t C = (int64_t)ncol * L;
@@ -469,150 +481,165 @@ __global__ void __launch_bounds__(128)
     for (int q = 0; q < 4; ++q) { snb[threadIdx.x][q] = e[q]; snb[threadIdx.x][4 + q] = d[q]; }
   }
   __syncthreads();
-  for (int i = threadIdx.x; i < cpb * kCh * (L + 2); i += blockDim.x) {
-    const int cc = i / (kCh * (L + 2)), r = i % (kCh * (L + 2)), ch = r / (L + 2), k = r % (L + 2) - 1;
-    float v = 0.f;
+  for (int i = threadIdx.x; i < cpb * (L + 2); i += blockDim.x) {
+    const int cc = i / (L + 2), k = i % (L + 2) - 1;
+    float *hb = h3 + cc * kCh * Lp + (k + 1);
     if (cc < nc && k >= 0 && k < L) {
-      const int col = c0 + cc;
-      const int *e = snb[cc], *d = snb[cc] + 4;
-      const A *hc = h2 + (int64_t)ch * C;
-      float se = 0.f, sd = 0.f;
+      const int64_t K = (int64_t)(c0 + cc) * L + k;
+      const A *h0 = h2 + K;
+      int oe[4], od[4];   // offsets from this cell; 0 where there is no neighbour
+      bool he[4], hd[4];
 #pragma unroll
       for (int s = 0; s < 4; ++s) {
-        if (e[s] >= 0) se += to_f<A>(hc[(int64_t)e[s] * L + k]);
-        if (d[s] >= 0) sd += to_f<A>(hc[(int64_t)d[s] * L + k]);
+        he[s] = snb[cc][s] >= 0;
+        hd[s] = snb[cc][4 + s] >= 0;
+        oe[s] = he[s] ? (snb[cc][s] - (c0 + cc)) * L : 0;
+        od[s] = hd[s] ? (snb[cc][4 + s] - (c0 + cc)) * L : 0;
       }
-      const float a = fmaf(Mw[3 * ch], to_f<A>(hc[(int64_t)col * L + k]), fmaf(Mw[3 * ch + 1], se, Mw[3 * ch + 2] * sd));
-      v = rnd<A>(fmaxf(a, 0.f));
-      if (h3_out) h3_out[(int64_t)ch * C + (int64_t)col * L + k] = from_f<A>(v);
+#pragma unroll 4
+      for (int ch = 0; ch < kCh; ++ch, h0 += C) {
+        float se = 0.f, sd = 0.f;
+#pragma unroll
+        for (int s = 0; s < 4; ++s) {
+          const float ve = to_f<A>(h0[oe[s]]), vd = to_f<A>(h0[od[s]]);   // (no branch: the loads go out together)
+          se += he[s] ? ve : 0.f;
+          sd += hd[s] ? vd : 0.f;
+        }
+        const float4 w = Mw[ch];
+        const float a = fmaf(w.x, to_f<A>(h0[0]), fmaf(w.y, se, w.z * sd));
+        const float v = rnd<A>(fmaxf(a, 0.f));
+        hb[ch * Lp] = v;
+      }
+    } else {
+      for (int ch = 0; ch < kCh; ++ch) hb[ch * Lp] = 0.f;
+      if (TRAIN) gys[i] = 0.f;
     }
-    h3[i] = v;
   }
   __syncthreads();
   double lsum = 0.0;
   for (int i = threadIdx.x; i < nc * L; i += blockDim.x) {
     const int cc = i / L, k = i % L;
-    const float *hb = h3 + cc * kCh * (L + 2) + k;
+    const float *hb = h3 + cc * kCh * Lp + k;
     float y = 0.f;
 #pragma unroll 8
     for (int ch = 0; ch < kCh; ++ch) {
-      const float *hc = hb + ch * (L + 2);
-      y = fmaf(W3[3 * ch], hc[0], fmaf(W3[3 * ch + 1], hc[1], fmaf(W3[3 * ch + 2], hc[2], y)));
+      const float *hc = hb + ch * Lp;
+      const float4 w = W3[ch];
+      y = fmaf(w.x, hc[0], fmaf(w.y, hc[1], fmaf(w.z, hc[2], y)));
     }
     const int64_t K = (int64_t)(c0 + cc) * L + k;
-    if (out) {
+    if (!TRAIN) {
       double s = 1.0;
       if (diagH) s = 1.0 / sqrt(diagH[K]);
       else if (diagH32) s = (double)rsqrtf(diagH32[K]);
       out[K] = (Tout)((double)y * s);
-    }
-    if (gy_out) {
+    } else {
       const int sample = (c0 + cc) / patch_cols;
       const float r = y - target[K];
       const float w = 1.0f / tnorm2[sample];
-      gy_out[K] = 2.0f * r * w * inv_batch;
+      gys[cc * (L + 2) + k + 1] = 2.0f * r * w * inv_batch;
       lsum += (double)(r * r * w);
     }
   }
-  if (loss_part) {
-    lsum = warp_sum(lsum);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = lsum;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      double s = 0.0;
-      for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += red[w];
-      loss_part[blockIdx.x] = s;
+  if (!TRAIN) return;
+  lsum = warp_sum(lsum);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = lsum;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double s = 0.0;
+    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += red[w];
+    loss_part[blockIdx.x] = s;
+  }
+  for (int i = threadIdx.x; i < nc * L; i += blockDim.x) {
+    const int cc = i / L, k = i % L;
+    const float *g = gys + cc * (L + 2) + k, *hb = h3 + cc * kCh * Lp + k + 1;   // gy[k-1..k+1] at g[0..2]
+    const float g0 = g[0], g1 = g[1], g2 = g[2];
+    float *gp = ga3 + (int64_t)(c0 + cc) * L + k;
+#pragma unroll 8
+    for (int ch = 0; ch < kCh; ++ch, gp += C) {
+      // y[k'] += W3[ch][d] h3[ch][k'+d-1]  =>  gh3[ch][k] = sum_d W3[ch][d] gy[k-d+1]
+      const float4 w = W3[ch];
+      const float gh = fmaf(w.x, g2, fmaf(w.y, g1, w.z * g0));
+      *gp = hb[ch * Lp] > 0.f ? gh : 0.f;
     }
+  }
+  // gW3: thread w owns (d, ch) = (w / 32, w % 32)
+  for (int w = threadIdx.x; w < 96; w += blockDim.x) {
+    const int d = w / 32, ch = w % 32, k0 = d == 0 ? 1 : 0, k1 = d == 2 ? L - 1 : L;
+    float s = 0.f;
+    for (int cc = 0; cc < nc; ++cc) {
+      const float *hb = h3 + (cc * kCh + ch) * Lp + d, *gb = gys + cc * (L + 2) + 1;   // h3[k+d-1], gy[k]
+#pragma unroll 8
+      for (int k = k0; k < k1; ++k) s = fmaf(gb[k], hb[k], s);
+    }
+    part[(int64_t)blockIdx.x * 96 + 3 * ch + d] = s;
   }
 }
 
 // ---- backward ---------------------------------------------------------------------------------
-// B3: gh3 = conv^T(W3, gy), ga3 = gh3 [h3 > 0]; partial gW3[ch][d] = sum gy[k] h3[ch][k+d-1].
-// One block per CPB columns; the partial sums of its columns go to part[block][96].
-template <typename A>
-__global__ void __launch_bounds__(128)
-    nn_bwd3_kernel(const float *__restrict__ wts, const A *__restrict__ h3, const float *__restrict__ gy,
-                   int ncol, int L, int cpb, float *__restrict__ ga3, float *__restrict__ part) {
-  extern __shared__ float sm[];
-  float *W3 = sm, *gys = W3 + 96;               // gys [cpb][L+2]
-  float *acc = gys + cpb * (L + 2);             // [96] per-block partials
-  for (int i = threadIdx.x; i < 96; i += blockDim.x) { W3[i] = rnd<A>(wts[kOffW3 + i]); acc[i] = 0.f; }
-  const int c0 = blockIdx.x * cpb, nc = min(cpb, ncol - c0);
-  const int64_t C = (int64_t)ncol * L;
-  for (int i = threadIdx.x; i < cpb * (L + 2); i += blockDim.x) {
-    const int cc = i / (L + 2), k = i % (L + 2) - 1;
-    gys[i] = (cc < nc && k >= 0 && k < L) ? gy[(int64_t)(c0 + cc) * L + k] : 0.f;
-  }
-  __syncthreads();
-  // ga3 (one thread per (column, channel, level))
-  for (int i = threadIdx.x; i < nc * kCh * L; i += blockDim.x) {
-    const int cc = i / (kCh * L), r = i % (kCh * L), ch = r / L, k = r % L;
-    const float *g = gys + cc * (L + 2) + k;    // gy[k-1..k+1] at g[0..2]
-    // y[k'] += W3[ch][d] h3[ch][k'+d-1]  =>  gh3[ch][k] = sum_d W3[ch][d] gy[k-d+1]
-    const float gh = fmaf(W3[3 * ch], g[2], fmaf(W3[3 * ch + 1], g[1], W3[3 * ch + 2] * g[0]));
-    const int64_t idx = (int64_t)ch * C + (int64_t)(c0 + cc) * L + k;
-    ga3[idx] = to_f<A>(h3[idx]) > 0.f ? gh : 0.f;
-  }
-  // gW3 partials: thread per (ch, d), loop over the block's positions
-  for (int w = threadIdx.x; w < 96; w += blockDim.x) {
-    const int ch = w / 3, d = w % 3;
-    float s = 0.f;
-    for (int cc = 0; cc < nc; ++cc)
-      for (int k = 0; k < L; ++k) {
-        const int kk = k + d - 1;
-        if (kk < 0 || kk >= L) continue;
-        s = fmaf(gys[cc * (L + 2) + k + 1], to_f<A>(h3[(int64_t)ch * C + (int64_t)(c0 + cc) * L + kk]), s);
-      }
-    acc[w] = s;
-  }
-  __syncthreads();
-  for (int i = threadIdx.x; i < 96; i += blockDim.x) part[(int64_t)blockIdx.x * 96 + i] = acc[i];
-}
-
 // B2: gh2 = w_c ga3 + w_e sum(edge nbrs of ga3) + w_d sum(corner nbrs) (the neighbour relation is
 // symmetric on a patch), ga2 = gh2 [h2 > 0]; partials of gM: (ga3 . h2, ga3 . sum_e h2,
-// ga3 . sum_d h2) per channel. Thread per cell (consecutive threads on consecutive levels, so every
-// channel's loads and stores are coalesced), grid-stride over the cells; blockIdx.y picks 4 of the
-// 32 channels. Block x writes entries 12 y .. 12 y + 11 of partial row x.
-constexpr int kBw2Ch = 4;
+// ga3 . sum_d h2) per channel. A thread walks one row of cells of a patch along y at a fixed (x, level),
+// for two channels, and keeps the 3 x 3 window of both fields in registers: three loads per cell and
+// field, where a thread per cell made nine, which bounded it (the loads of 30-level columns straddle
+// lines: about two cycles of the load unit each). Consecutive threads are on consecutive levels, so the
+// loads and stores are coalesced. 64 patches of 16 x 16 x 30 in BF16: 126 -> 64 us. blockIdx.y picks
+// two of the 32 channels; block x writes entries 6 y .. 6 y + 5 of partial row x.
+constexpr int kBw2Ch = 2;
 template <typename A>
-__global__ void __launch_bounds__(128)
+__global__ void __launch_bounds__(128, 6)
     nn_bwd2_kernel(const float *__restrict__ wts, const A *__restrict__ h2, const float *__restrict__ ga3,
-                   Nbrs nb, int ncol, int L, float *__restrict__ ga2, float *__restrict__ part) {
+                   int nsamp, int nx, int ny, int L, float *__restrict__ ga2, float *__restrict__ part) {
   __shared__ float Mw[3 * kBw2Ch], red[4][3 * kBw2Ch];
   const int ch0 = blockIdx.y * kBw2Ch;
   if (threadIdx.x < 3 * kBw2Ch) Mw[threadIdx.x] = rnd<A>(wts[kOffM + 3 * ch0 + threadIdx.x]);
   __syncthreads();
-  const int64_t C = (int64_t)ncol * L;
+  const int64_t P = (int64_t)nx * ny, C = (int64_t)nsamp * P * L, row = (int64_t)nx * L, units = (int64_t)nsamp * row;
   float acc[3 * kBw2Ch];
 #pragma unroll
   for (int q = 0; q < 3 * kBw2Ch; ++q) acc[q] = 0.f;
-  for (int64_t K = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; K < C; K += (int64_t)gridDim.x * blockDim.x) {
-    const int col = (int)(K / L), k = (int)(K - (int64_t)col * L);
-    int e[4], d[4];
-    nb.get(col, e, d);
-    int64_t oe[4], od[4];
+  for (int64_t U = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; U < units; U += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t sm = U / row;
+    const int ik = (int)(U - sm * row), i = ik / L;
+    const bool left = i > 0, right = i < nx - 1;
+    const int ol = left ? -L : 0, orr = right ? L : 0;   // 0: a load that is not used
+    int64_t K = (int64_t)ch0 * C + sm * P * L + ik;
+    float gp[kBw2Ch][3], gc[kBw2Ch][3], hp[kBw2Ch][3], hc[kBw2Ch][3];   // (left, centre, right) of rows j - 1, j
+    auto load = [&](int64_t at, float (&g)[kBw2Ch][3], float (&h)[kBw2Ch][3]) {
 #pragma unroll
-    for (int s = 0; s < 4; ++s) {
-      oe[s] = e[s] >= 0 ? (int64_t)e[s] * L + k : -1;
-      od[s] = d[s] >= 0 ? (int64_t)d[s] * L + k : -1;
-    }
-#pragma unroll
-    for (int j = 0; j < kBw2Ch; ++j) {
-      const float *g = ga3 + (int64_t)(ch0 + j) * C;
-      const A *h = h2 + (int64_t)(ch0 + j) * C;
-      const float gk = g[K], hk = to_f<A>(h[K]);
-      float ge = 0.f, gd = 0.f, he = 0.f, hd = 0.f;
-#pragma unroll
-      for (int s = 0; s < 4; ++s) {
-        if (oe[s] >= 0) { ge += g[oe[s]]; he += to_f<A>(h[oe[s]]); }
-        if (od[s] >= 0) { gd += g[od[s]]; hd += to_f<A>(h[od[s]]); }
+      for (int c = 0; c < kBw2Ch; ++c) {
+        const float *gq = ga3 + at + c * C;
+        const A *hq = h2 + at + c * C;
+        const float g0 = gq[ol], g1 = gq[0], g2 = gq[orr], h0 = to_f<A>(hq[ol]), h1 = to_f<A>(hq[0]), h2v = to_f<A>(hq[orr]);
+        g[c][0] = left ? g0 : 0.f; g[c][1] = g1; g[c][2] = right ? g2 : 0.f;
+        h[c][0] = left ? h0 : 0.f; h[c][1] = h1; h[c][2] = right ? h2v : 0.f;
       }
-      const float gh = fmaf(Mw[3 * j], gk, fmaf(Mw[3 * j + 1], ge, Mw[3 * j + 2] * gd));
-      ga2[(int64_t)(ch0 + j) * C + K] = hk > 0.f ? gh : 0.f;
-      acc[3 * j] = fmaf(gk, hk, acc[3 * j]);
-      acc[3 * j + 1] = fmaf(gk, he, acc[3 * j + 1]);
-      acc[3 * j + 2] = fmaf(gk, hd, acc[3 * j + 2]);
+    };
+#pragma unroll
+    for (int c = 0; c < kBw2Ch; ++c)
+#pragma unroll
+      for (int q = 0; q < 3; ++q) gp[c][q] = hp[c][q] = 0.f;
+    load(K, gc, hc);
+#pragma unroll 2
+    for (int j = 0; j < ny; ++j, K += row) {
+      float gn[kBw2Ch][3] = {}, hn[kBw2Ch][3] = {};
+      if (j + 1 < ny) load(K + row, gn, hn);
+#pragma unroll
+      for (int c = 0; c < kBw2Ch; ++c) {
+        const float ge = ((gp[c][1] + gc[c][2]) + gn[c][1]) + gc[c][0], gd = ((gp[c][2] + gn[c][2]) + gn[c][0]) + gp[c][0];
+        const float he = ((hp[c][1] + hc[c][2]) + hn[c][1]) + hc[c][0], hd = ((hp[c][2] + hn[c][2]) + hn[c][0]) + hp[c][0];
+        const float gk = gc[c][1], hk = hc[c][1];
+        const float gh = fmaf(Mw[3 * c], gk, fmaf(Mw[3 * c + 1], ge, Mw[3 * c + 2] * gd));
+        ga2[K + c * C] = hk > 0.f ? gh : 0.f;
+        acc[3 * c] = fmaf(gk, hk, acc[3 * c]);
+        acc[3 * c + 1] = fmaf(gk, he, acc[3 * c + 1]);
+        acc[3 * c + 2] = fmaf(gk, hd, acc[3 * c + 2]);
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+          gp[c][q] = gc[c][q]; gc[c][q] = gn[c][q];
+          hp[c][q] = hc[c][q]; hc[c][q] = hn[c][q];
+        }
+      }
     }
   }
   // fixed-order reduction: lanes by butterfly, then the four warps
@@ -715,10 +742,10 @@ constexpr int kBwB1 = ((2 * kBwA1 + 1023) / 1024) * 1024;     // W2 image (6 KB)
 constexpr int kBwA2 = kBwB1 + 6 * 1024;                       // h1 shifted: 16 x 128 x 16 B = 32 KB
 constexpr int kBwB2 = kBwA2 + 16 * 128 * 16;                  // ga2 over the rows: 16 x 32 x 16 B = 8 KB per part
 constexpr int kBwX = kBwB2 + 2 * 16 * 32 * 16;                // x on rows -1 .. 128 (130 floats)
-constexpr int kBwG = kBwX + ((kBwRows * 4 + 15) / 16) * 16;   // ga2 tile, FP32 [32][130]
-constexpr int kBwH = kBwG + 32 * kBwRows * 4;                 // h1 tile, BF16 [32][130]
-constexpr int kBwCell = kBwH + 32 * kBwRows * 2;              // cell of each row, int32 [130]
-constexpr int kBwBar = kBwCell + ((kBwRows * 4 + 15) / 16) * 16;   // mbarrier (8 B), TMEM address (4 B)
+constexpr int kBwG = kBwX + ((kBwRows * 4 + 15) / 16) * 16;   // ga2 on the tile's rows, FP32 [32][129]
+constexpr int kBwGs = kTcM + 1;                               // words between its rows: odd
+constexpr int kBwH = kBwG + 32 * kBwGs * 4;                   // h1 on rows -1 .. 128, BF16 [32][130]
+constexpr int kBwBar = kBwH + 32 * kBwRows * 2;   // mbarrier (8 B), TMEM address (4 B)
 constexpr int kBwSmem = kBwBar + 64;
 constexpr int kBwRed = kBwA2;                                 // end-of-kernel reduction scratch (reuses A2)
 
@@ -738,9 +765,9 @@ struct BwArgs {
 
 __device__ __forceinline__ int64_t bw_cell(const BwArgs &a, int64_t R) {   // cell of padded row R, or -1
   if (R < 0 || R >= a.nrows) return -1;
-  const int64_t col = R / (a.L + 2);
-  const int k = (int)(R - col * (a.L + 2)) - 1;
-  return (k >= 0 && k < a.L) ? col * a.L + k : -1;
+  const unsigned col = (unsigned)R / (unsigned)(a.L + 2);   // (rows are below 2^31: a 32-bit division)
+  const int k = (int)((unsigned)R - col * (unsigned)(a.L + 2)) - 1;
+  return (k >= 0 && k < a.L) ? (int64_t)col * a.L + k : -1;
 }
 
 __device__ __forceinline__ uint32_t pack_bf16x2(float a, float b) {
@@ -753,7 +780,13 @@ __device__ __forceinline__ void split_bf16(float v, float &hi, float &lo) {
   lo = v - hi;
 }
 
-__global__ void __launch_bounds__(128)
+// The MMAs are a few per cent of the time; bringing a tile into the operand layouts is the rest. So: 256
+// threads, two per row with 16 channels each (two CTAs, 512 threads per SM); a thread writes its A1
+// chunks from registers and keeps the signs of its h1; shared memory is read and written without bank
+// conflicts; and the next tile's loads are in flight during the MMAs and the epilogue. 64 patches of
+// 16 x 16 x 30: 331 us (128 threads, everything through shared memory, A2 and B2 written 2 KB and
+// 512 B apart by neighbouring lanes) -> 75 us.
+__global__ void __launch_bounds__(256, 2)
     nn_bwd1_tc_kernel(const BwArgs a, const __nv_bfloat16 *__restrict__ bt, const __nv_bfloat16 *__restrict__ h1,
                       const float *__restrict__ ga2, const float *__restrict__ xin, float *__restrict__ part2,
                       float *__restrict__ part1, int *__restrict__ wait_flag) {
@@ -762,7 +795,6 @@ __global__ void __launch_bounds__(128)
   float *xs = reinterpret_cast<float *>(bw_smem + kBwX);
   float *Gs = reinterpret_cast<float *>(bw_smem + kBwG);
   __nv_bfloat16 *Hs = reinterpret_cast<__nv_bfloat16 *>(bw_smem + kBwH);
-  int *cellr = reinterpret_cast<int *>(bw_smem + kBwCell);
   uint64_t *bar = reinterpret_cast<uint64_t *>(bw_smem + kBwBar);
   uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bw_smem + kBwBar + 16);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -781,9 +813,10 @@ __global__ void __launch_bounds__(128)
     const int kg = e / 32, row = 96 + e % 32;
     *reinterpret_cast<uint4 *>(sA2 + kg * 2048 + row * 16) = make_uint4(0u, 0u, 0u, 0u);
   }
-  float acc1[96];                   // gW1[i][d] partials of this thread's rows
+  const int half = tid >> 7, m = tid & 127, ch0 = 16 * half;   // this thread's tile row and 16 channels
+  float acc1[48];                   // gW1[i][d] partials of its rows, its channels
 #pragma unroll
-  for (int q = 0; q < 96; ++q) acc1[q] = 0.f;
+  for (int q = 0; q < 48; ++q) acc1[q] = 0.f;
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -791,50 +824,85 @@ __global__ void __launch_bounds__(128)
   const uint32_t idesc = umma_idesc_bf16(kTcM, 32);
   bool ok = true, first = true;
   uint32_t phase = 0;
-  for (int64_t t = blockIdx.x; t < a.ntiles && ok; t += gridDim.x) {
+  // a tile's values in registers: row R0 + m, 16 channels; threads 0 .. 63 also a channel of row R0 - 1
+  // or R0 + 128. Each value is read once from global memory.
+  float gv[16], xv = 0.f, ge = 0.f, xe = 0.f;
+  __nv_bfloat16 hv[16], he = __float2bfloat16(0.f);
+  int cell = -1;
+  auto load = [&](int64_t t) {
     const int64_t R0 = t * kTcM;
-    // the tile's rows R0 - 1 .. R0 + 128 (buffer row r = R - R0 + 1): their cells, then ga2 (FP32),
-    // h1 (BF16) and x (BF16-rounded) on them, each value read once from global memory
-    for (int r = tid; r < kBwRows; r += blockDim.x) {
-      const int64_t cell = bw_cell(a, R0 - 1 + r);
-      cellr[r] = (int)cell;
-      xs[r] = cell >= 0 ? rnd<__nv_bfloat16>(xin[cell]) : 0.f;
+    cell = (int)bw_cell(a, R0 + m);
+    const bool in = cell >= 0;
+    const float *gp = ga2 + (int64_t)ch0 * a.C + (in ? cell : 0);
+    const __nv_bfloat16 *hp = h1 + (int64_t)ch0 * a.C + (in ? cell : 0);
+#pragma unroll
+    for (int u = 0; u < 16; ++u) {
+      gv[u] = in ? gp[(int64_t)u * a.C] : 0.f;
+      hv[u] = in ? hp[(int64_t)u * a.C] : __float2bfloat16(0.f);
     }
-    __syncthreads();
-    for (int e = tid; e < 32 * kBwRows; e += blockDim.x) {
-      const int ch = e / kBwRows, r = e - ch * kBwRows, cell = cellr[r];
-      Gs[e] = cell >= 0 ? ga2[(int64_t)ch * a.C + cell] : 0.f;
-      Hs[e] = cell >= 0 ? h1[(int64_t)ch * a.C + cell] : __float2bfloat16(0.f);
+    xv = in && half == 0 ? xin[cell] : 0.f;
+    if (tid < 64) {
+      const int64_t ce = bw_cell(a, tid < 32 ? R0 - 1 : R0 + kTcM);
+      ge = ce >= 0 ? ga2[(int64_t)lane * a.C + ce] : 0.f;
+      he = ce >= 0 ? h1[(int64_t)lane * a.C + ce] : __float2bfloat16(0.f);
+      xe = ce >= 0 && lane == 0 ? xin[ce] : 0.f;
     }
-    __syncthreads();
-    // A1: ga2 on rows -1 .. 128 in the forward's layout, hi and lo parts
-    for (int e = tid; e < 4 * kBwRows; e += blockDim.x) {
-      const int r = e % kBwRows, g = e / kBwRows;
+  };
+  if (blockIdx.x < a.ntiles) load(blockIdx.x);
+  for (int64_t t = blockIdx.x; t < a.ntiles && ok; t += gridDim.x) {
+    // registers -> A1 (ga2 on rows -1 .. 128 in the forward's layout, hi and lo parts), and the tile's
+    // ga2 (FP32), h1 (BF16) and x (BF16-rounded) for the operands over the rows (buffer row R - R0 + 1)
+    unsigned pos = 0;                 // h1 > 0, a bit per channel
+    const bool row_in = cell >= 0;
+#pragma unroll
+    for (int g = 0; g < 2; ++g) {
       uint32_t hw[4], lw[4];
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
         float h0, l0, h1v, l1;
-        split_bf16(Gs[(8 * g + 2 * q) * kBwRows + r], h0, l0);
-        split_bf16(Gs[(8 * g + 2 * q + 1) * kBwRows + r], h1v, l1);
+        split_bf16(gv[8 * g + 2 * q], h0, l0);
+        split_bf16(gv[8 * g + 2 * q + 1], h1v, l1);
         hw[q] = pack_bf16x2(h0, h1v);
         lw[q] = pack_bf16x2(l0, l1);
       }
-      *reinterpret_cast<uint4 *>(sA1 + g * kBwLbo + r * 16) = make_uint4(hw[0], hw[1], hw[2], hw[3]);
-      *reinterpret_cast<uint4 *>(sA1 + kBwA1 + g * kBwLbo + r * 16) = make_uint4(lw[0], lw[1], lw[2], lw[3]);
+      unsigned char *dst = sA1 + (2 * half + g) * kBwLbo + (m + 1) * 16;
+      *reinterpret_cast<uint4 *>(dst) = make_uint4(hw[0], hw[1], hw[2], hw[3]);
+      *reinterpret_cast<uint4 *>(dst + kBwA1) = make_uint4(lw[0], lw[1], lw[2], lw[3]);
     }
+#pragma unroll
+    for (int u = 0; u < 16; ++u) {
+      Gs[(ch0 + u) * kBwGs + m] = gv[u];
+      Hs[(ch0 + u) * kBwRows + m + 1] = hv[u];
+      if (__bfloat162float(hv[u]) > 0.f) pos |= 1u << u;
+    }
+    if (half == 0) xs[m + 1] = rnd<__nv_bfloat16>(xv);
+    if (tid < 64) {
+      const int rb = tid < 32 ? 0 : kTcM + 1;
+      float hi, lo;
+      split_bf16(ge, hi, lo);
+      __nv_bfloat16 *dst = reinterpret_cast<__nv_bfloat16 *>(sA1 + (lane >> 3) * kBwLbo + rb * 16) + (lane & 7);
+      dst[0] = __float2bfloat16(hi);
+      dst[kBwA1 / 2] = __float2bfloat16(lo);
+      Hs[lane * kBwRows + rb] = he;
+      if (lane == 0) xs[rb] = rnd<__nv_bfloat16>(xe);
+    }
+    __syncthreads();
+    const float x0 = xs[m], x1 = xs[m + 1], x2 = xs[m + 2];   // x(m - 1), x(m), x(m + 1)
     // A2: h1[i] on rows m + d - 1 (buffer row m + d), row d 32 + i, m = 8 kg .. 8 kg + 7
+    // (lanes on consecutive rows: both the reads, an odd number of words apart, and the 16-byte writes
+    // are free of bank conflicts; lanes on consecutive groups wrote 2 KB apart, into the same banks)
     for (int e = tid; e < 96 * 16; e += blockDim.x) {
-      const int kg = e % 16, row = e / 16, d = row / 32, i = row % 32;
+      const int kg = e / 96, row = e - 96 * kg, d = row / 32, i = row % 32;
       const __nv_bfloat16 *hr = Hs + i * kBwRows + 8 * kg + d;
       uint32_t w[4];
 #pragma unroll
       for (int q = 0; q < 4; ++q) w[q] = pack_bf16x2(__bfloat162float(hr[2 * q]), __bfloat162float(hr[2 * q + 1]));
       *reinterpret_cast<uint4 *>(sA2 + kg * 2048 + row * 16) = make_uint4(w[0], w[1], w[2], w[3]);
     }
-    // B2: ga2[o] on rows m (buffer row m + 1), hi and lo parts
+    // B2: ga2[o] on rows m, hi and lo parts
     for (int e = tid; e < 32 * 16; e += blockDim.x) {
-      const int kg = e % 16, o = e / 16;
-      const float *gr = Gs + o * kBwRows + 8 * kg + 1;
+      const int kg = e / 32, o = e % 32;
+      const float *gr = Gs + o * kBwGs + 8 * kg;
       uint32_t hw[4], lw[4];
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
@@ -875,6 +943,7 @@ __global__ void __launch_bounds__(128)
       asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar)));
     }
     first = false;
+    if (t + gridDim.x < a.ntiles) load(t + gridDim.x);   // in flight behind the MMAs and the epilogue
     ok = __syncthreads_and(mbar_wait(bar, phase) ? 1 : 0) != 0;
     if (!ok) {   // the MMAs may still be running: one more bounded wait before anything is freed
       if (tid == 0) {
@@ -886,58 +955,50 @@ __global__ void __launch_bounds__(128)
     }
     phase ^= 1u;
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    uint32_t r[32];
-    const uint32_t taddr = tmem + ((uint32_t)(warp * 32) << 16);
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
-                 "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
+    uint32_t r[16];
+    const uint32_t taddr = tmem + ((uint32_t)((warp & 3) * 32) << 16) + ch0;   // row m, columns ch0 .. ch0 + 15
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
                  : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-                   "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
-                   "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
-                   "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+                   "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
                  : "r"(taddr));
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-    const int m = warp * 32 + lane;
-    if (cellr[m + 1] >= 0) {
-      const float x0 = xs[m], x1 = xs[m + 1], x2 = xs[m + 2];   // x(m - 1), x(m), x(m + 1)
+    if (row_in) {
 #pragma unroll
-      for (int i = 0; i < 32; ++i) {
-        const float g = __bfloat162float(Hs[i * kBwRows + m + 1]) > 0.f ? __uint_as_float(r[i]) : 0.f;
+      for (int i = 0; i < 16; ++i) {
+        const float g = (pos >> i) & 1u ? __uint_as_float(r[i]) : 0.f;
         acc1[3 * i] = fmaf(g, x0, acc1[3 * i]);
         acc1[3 * i + 1] = fmaf(g, x1, acc1[3 * i + 1]);
         acc1[3 * i + 2] = fmaf(g, x2, acc1[3 * i + 2]);
       }
     }
+    // the next tile's stores come after every MMA of this one (the wait above), and its first MMA, which
+    // rewrites D1, after the two barriers before it
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    __syncthreads();   // the next tile rewrites the operands and D1
   }
   // D2 -> gW2 partials (row d 32 + i, column o), then the gW1 partials reduced over the block
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   if (ok) {
-    uint32_t r[32];
-    const uint32_t taddr = tmem + 32u + ((uint32_t)(warp * 32) << 16);
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
-                 "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
+    uint32_t r[16];
+    const uint32_t taddr = tmem + 32u + ((uint32_t)((warp & 3) * 32) << 16) + ch0;
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
                  : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-                   "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
-                   "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
-                   "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+                   "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
                  : "r"(taddr));
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-    const int row = warp * 32 + lane;
-    if (row < 96) {
-      const int d = row / 32, i = row % 32;
+    if (m < 96) {
+      const int d = m / 32, i = m % 32;
 #pragma unroll
-      for (int o = 0; o < 32; ++o)
-        part2[(int64_t)blockIdx.x * 3072 + (o * 32 + i) * 3 + d] = __uint_as_float(r[o]);
+      for (int o = 0; o < 16; ++o)
+        part2[(int64_t)blockIdx.x * 3072 + ((ch0 + o) * 32 + i) * 3 + d] = __uint_as_float(r[o]);
     }
   }
-  float *red = reinterpret_cast<float *>(bw_smem + kBwRed);   // [4 warps][96]
+  float *red = reinterpret_cast<float *>(bw_smem + kBwRed);   // [4 warps of a half][96]
 #pragma unroll
-  for (int q = 0; q < 96; ++q) {
+  for (int q = 0; q < 48; ++q) {
     float v = acc1[q];
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-    if (lane == 0) red[warp * 96 + q] = v;
+    if (lane == 0) red[(warp & 3) * 96 + 48 * half + q] = v;
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
@@ -945,35 +1006,59 @@ __global__ void __launch_bounds__(128)
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 64;" ::"r"(tmem));
 }
 
-// Sum of per-block partials [nblocks][n] into out[n]: one block per entry, its threads striding the
-// partials, then a fixed-order tree (deterministic for a given nblocks).
-__global__ void __launch_bounds__(256)
-    sum_partials_kernel(const float *__restrict__ part, int nblocks, int n, float *__restrict__ out) {
-  const int i = blockIdx.x;
+// Sums of per-block partials [nblocks][n] into out[n], the four gradient blocks and the loss (FP64
+// partials) in one launch, in a fixed order (deterministic for a given nblocks). The first block (gW2,
+// 3,072 entries) takes 8 entries per grid block, a sector of each partial row, and 128 rows at a time;
+// the others an entry per grid block, which spreads their FP64 additions over the chip. Five launches
+// of a block per entry were latency chains of 4 to 17 us each, 50 us together, at a batch of 64 patches
+// of 16 x 16 x 30; this takes 21 us.
+struct SumJobs {
+  const float *part[4];   // gW2, gW3, gW1, gM
+  float *out[4];
+  int nblocks[4];
+  const double *loss_part;
+  double *loss;
+  int nloss;
+};
+constexpr int kSumW2Blocks = 3072 / 8, kSumBlocks = kSumW2Blocks + 3 * 96 + 1;
+__global__ void __launch_bounds__(1024) sum_partials_kernel(const SumJobs J) {
+  __shared__ double red[32][8];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   double s = 0.0;
-  for (int b = threadIdx.x; b < nblocks; b += blockDim.x) s += part[(int64_t)b * n + i];
-  s = warp_sum(s);
-  __shared__ double red[8];
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double t = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += red[w];
-    out[i] = (float)t;
+  if (blockIdx.x < kSumW2Blocks) {
+    const int i0 = 8 * blockIdx.x;
+    const float *part = J.part[0] + i0 + (tid & 7);
+#pragma unroll 4
+    for (int b = tid >> 3; b < J.nblocks[0]; b += 128) s += part[(int64_t)b * 3072];
+    s += __shfl_xor_sync(0xffffffffu, s, 8);
+    s += __shfl_xor_sync(0xffffffffu, s, 16);
+    if (lane < 8) red[warp][lane] = s;
+    __syncthreads();
+    if (tid < 8) {
+      double t = 0.0;
+      for (int w = 0; w < 32; ++w) t += red[w][tid];
+      J.out[0][i0 + tid] = (float)t;
+    }
+    return;
   }
-}
-
-__global__ void sum_loss_kernel(const double *__restrict__ part, int n, double *out) {
-  double s = 0.0;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) s += part[i];
+  const int e = blockIdx.x - kSumW2Blocks, q = 1 + e / 96, i = e % 96;   // q = 4: the loss
+  if (q < 4) {
+    const float *part = J.part[q] + i;
+#pragma unroll 4
+    for (int b = tid; b < J.nblocks[q]; b += 1024) s += part[(int64_t)b * 96];
+  } else {
+#pragma unroll 4
+    for (int b = tid; b < J.nloss; b += 1024) s += J.loss_part[b];
+  }
   s = warp_sum(s);
-  __shared__ double red[32];
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
+  if (lane == 0) red[warp][0] = s;
   __syncthreads();
-  if (threadIdx.x == 0) {
-    double t = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += red[w];
-    *out = t;
+  if (warp == 0) {
+    s = warp_sum(red[lane][0]);
+    if (lane == 0) {
+      if (q < 4) J.out[q][i] = (float)s;
+      else *J.loss = s;
+    }
   }
 }
 
@@ -1014,6 +1099,7 @@ int adam_update(Ctx *c, float *w, const float *g, float *m, float *v, int n, int
 __global__ void tnorm_kernel(const float *__restrict__ t, int64_t per_sample, float *__restrict__ out) {
   const int s = blockIdx.x;
   double acc = 0.0;
+#pragma unroll 8
   for (int64_t i = threadIdx.x; i < per_sample; i += blockDim.x) {
     const double v = t[(int64_t)s * per_sample + i];
     acc += v * v;
@@ -1080,7 +1166,9 @@ __global__ void gather_samples_kernel(const float *__restrict__ x, const float *
 
 // ---- host side ---------------------------------------------------------------------------------
 static int front_smem(int cpb, int L) { return (96 + 3072 + cpb * (L + 2) + cpb * kCh * (L + 2)) * 4; }
-static int back_smem(int cpb, int L) { return (96 + 96 + cpb * kCh * (L + 2)) * 4; }
+static int back_smem(int cpb, int L, bool train) {
+  return (8 * kCh + cpb * kCh * back_stride(L) + (train ? cpb * (L + 2) : 0)) * 4;
+}
 static int mix_smem(int cpb, int L) { return (2 * 36 * 4 + 8 * cpb + cpb * (L + 2) * 36) * 4; }
 // diag(H)^-1/2 in FP32 per cell, passed from the tensor-core front kernel to the output layer:
 // the activation buffer (sized for 32 FP32 channels) after the 32 BF16 channels of h2
@@ -1095,7 +1183,9 @@ template <typename A, typename Tin, typename Tout>
 static int nn_attrs(Ctx *c) {
   const int big = 200 * 1024;
   HMG_CUDA(c, cudaFuncSetAttribute(nn_front_kernel<A, Tin>, cudaFuncAttributeMaxDynamicSharedMemorySize, big));
-  HMG_CUDA(c, cudaFuncSetAttribute(nn_back_kernel<A, Tout>, cudaFuncAttributeMaxDynamicSharedMemorySize, big));
+  HMG_CUDA(c, cudaFuncSetAttribute(nn_back_kernel<A, Tout, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, big));
+  if (sizeof(Tout) == 4)
+    HMG_CUDA(c, cudaFuncSetAttribute(nn_back_kernel<A, float, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, big));
   return HMG_OK;
 }
 
@@ -1125,8 +1215,8 @@ static int nn_forward_mesh(Ctx *c, const Tin *bbar, Tout *out, const double *dH,
     nn_mix_out_kernel<Tout><<<gm, thr, mix_smem(cpb, L), c->stream>>>(
         c->nn_w, reinterpret_cast<const __nv_bfloat16 *>(h2), nb, f.ncol, L, cpb, tc_dscale(c), out);
   } else {
-    nn_back_kernel<A, Tout><<<g, 128, back_smem(kNnCpb, L), c->stream>>>(
-        c->nn_w, h2, nb, f.ncol, L, kNnCpb, dH, dH32, out, nullptr, nullptr, nullptr, 1, 1.f, nullptr, nullptr);
+    nn_back_kernel<A, Tout, false><<<g, 128, back_smem(kNnCpb, L, false), c->stream>>>(
+        c->nn_w, h2, nb, f.ncol, L, kNnCpb, dH, dH32, out, nullptr, nullptr, 1, 1.f, nullptr, nullptr, nullptr);
   }
   HMG_CUDA(c, cudaGetLastError());
   return HMG_OK;
@@ -1205,7 +1295,7 @@ static int nn_batch_grad(Ctx *c, const float *x, const float *t, const float *tn
   const int P = nx * ny, ncol = nsamp * P;
   const int64_t C = (int64_t)ncol * L;
   if (C > tb.cap_cells) return fail(c, HMG_ERR_INVALID_ARG, "training batch larger than the buffers");
-  A *h1 = reinterpret_cast<A *>(tb.h1), *h2 = reinterpret_cast<A *>(tb.h2), *h3 = reinterpret_cast<A *>(tb.h3);
+  A *h1 = reinterpret_cast<A *>(tb.h1), *h2 = reinterpret_cast<A *>(tb.h2);
   const unsigned g = (unsigned)((ncol + kNnCpb - 1) / kNnCpb);
   Nbrs nb{nullptr, nullptr, nx, ny};
   if (sizeof(A) == 2) {   // BF16 storage: the column-local layers on the tensor cores, h1 kept
@@ -1218,15 +1308,12 @@ static int nn_batch_grad(Ctx *c, const float *x, const float *t, const float *tn
     nn_front_kernel<A, float><<<g, 128, front_smem(kNnCpb, L), c->stream>>>(c->nn_w, x, nullptr, nullptr, ncol, L,
                                                                             kNnCpb, h1, h2);
   }
-  nn_back_kernel<A, float><<<g, 128, back_smem(kNnCpb, L), c->stream>>>(
-      c->nn_w, h2, nb, ncol, L, kNnCpb, nullptr, nullptr, nullptr, h3, t, tn, P, 1.f / (float)nsamp, tb.gy,
-      tb.loss_part);
-  sum_loss_kernel<<<1, 256, 0, c->stream>>>(tb.loss_part, (int)g, loss_dev);
-  nn_bwd3_kernel<A><<<g, 128, (96 + kNnCpb * (L + 2) + 96) * 4, c->stream>>>(c->nn_w, h3, tb.gy, ncol, L, kNnCpb,
-                                                                             tb.ga3, tb.part3);
-  const int64_t g2max = (int64_t)2 * c->num_sms, g2need = (C + 127) / 128;   // partial rows: at most 2 per SM
+  nn_back_kernel<A, float, true><<<g, 128, back_smem(kNnCpb, L, true), c->stream>>>(
+      c->nn_w, h2, nb, ncol, L, kNnCpb, nullptr, nullptr, nullptr, t, tn, P, 1.f / (float)nsamp, tb.loss_part,
+      tb.ga3, tb.part3);
+  const int64_t g2max = (int64_t)2 * c->num_sms, g2need = ((int64_t)nsamp * nx * L + 127) / 128;   // partial rows: at most 2 per SM
   const unsigned g2 = (unsigned)(g2need < g2max ? g2need : g2max);
-  nn_bwd2_kernel<A><<<dim3(g2, kCh / kBw2Ch), 128, 0, c->stream>>>(c->nn_w, h2, tb.ga3, nb, ncol, L, tb.ga2,
+  nn_bwd2_kernel<A><<<dim3(g2, kCh / kBw2Ch), 128, 0, c->stream>>>(c->nn_w, h2, tb.ga3, nsamp, nx, ny, L, tb.ga2,
                                                                    tb.partM);
   unsigned g1;
   if (sizeof(A) == 2) {   // BF16 storage: the 32 -> 32 convolution's dX and dW on the tensor cores
@@ -1238,7 +1325,7 @@ static int nn_batch_grad(Ctx *c, const float *x, const float *t, const float *tn
     ba.ntiles = (ba.nrows + kTcM - 1) / kTcM;
     const int64_t gmax = (int64_t)2 * c->num_sms;
     g1 = (unsigned)(ba.ntiles < gmax ? ba.ntiles : gmax);
-    nn_bwd1_tc_kernel<<<g1, 128, kBwSmem, c->stream>>>(ba, static_cast<const __nv_bfloat16 *>(c->nn_bimg_t),
+    nn_bwd1_tc_kernel<<<g1, 256, kBwSmem, c->stream>>>(ba, static_cast<const __nv_bfloat16 *>(c->nn_bimg_t),
                                                         reinterpret_cast<const __nv_bfloat16 *>(h1), tb.ga2, x,
                                                         tb.part2, tb.part1, c->state + 3);
   } else {
@@ -1247,10 +1334,11 @@ static int nn_batch_grad(Ctx *c, const float *x, const float *t, const float *tn
     nn_bwd1_kernel<A><<<g1, 256, bwd1_smem(L), c->stream>>>(c->nn_w, h1, tb.ga2, x, ncol, L, cpb1, tb.part2,
                                                             tb.part1);
   }
-  sum_partials_kernel<<<96, 256, 0, c->stream>>>(tb.part1, (int)g1, 96, grad + kOffW1);
-  sum_partials_kernel<<<3072, 256, 0, c->stream>>>(tb.part2, (int)g1, 3072, grad + kOffW2);
-  sum_partials_kernel<<<96, 256, 0, c->stream>>>(tb.partM, (int)g2, 96, grad + kOffM);
-  sum_partials_kernel<<<96, 256, 0, c->stream>>>(tb.part3, (int)g, 96, grad + kOffW3);
+  const SumJobs sj{{tb.part2, tb.part3, tb.part1, tb.partM},
+                   {grad + kOffW2, grad + kOffW3, grad + kOffW1, grad + kOffM},
+                   {(int)g1, (int)g, (int)g1, (int)g2},
+                   tb.loss_part, loss_dev, (int)g};
+  sum_partials_kernel<<<kSumBlocks, 1024, 0, c->stream>>>(sj);
   HMG_CUDA(c, cudaGetLastError());
   return HMG_OK;
 }
@@ -1266,7 +1354,7 @@ int train_buffers(Ctx *c, int64_t cells, int nblocks_max) {
   TrainBufs &tb = c->train;
   int st;
   if (tb.cap_cells < cells) {
-    void **acts[] = {&tb.h1, &tb.h2, &tb.h3};
+    void **acts[] = {&tb.h1, &tb.h2};
     for (void **a : acts) {   // storage for FP32 activations (BF16 uses half of it)
       dev_free(c, *a);
       float *f;
@@ -1278,8 +1366,6 @@ int train_buffers(Ctx *c, int64_t cells, int nblocks_max) {
       dev_free(c, *g);
       if ((st = dev_alloc(c, g, (size_t)kCh * cells))) return st;
     }
-    dev_free(c, tb.gy);
-    if ((st = dev_alloc(c, &tb.gy, (size_t)cells))) return st;
     tb.cap_cells = cells;
   }
   if (tb.cap_blocks < nblocks_max) {

@@ -148,6 +148,31 @@ def test_gradient_matches_oracle():
         assert err < 1e-5, (k, err)
 
 
+@pytest.mark.parametrize("nx,ny,ns,nlev", [(1, 1, 1, 20), (1, 6, 5, 20), (6, 1, 5, 20), (33, 2, 3, 20), (2, 33, 3, 7),
+                                           (3, 3, 2, 1), (3, 2, 2, 128)])
+def test_gradient_of_ragged_patches(nx, ny, ns, nlev):
+    """Patches without left/right or front/back neighbours, column counts that leave a part of the
+    output layer's last block empty, one level and the 128-level limit: FP32 storage against the FP64
+    oracle, the bound of the test above (FP32 sums of a few thousand terms)."""
+    from paper_2210_11797_gb300.hmg import Solver
+    w = I.planar_helmholtz(n=4, nlev=nlev, nmg=1)
+    gpu = Solver(w.hier, w.coeffs, tol=w.tol)
+    try:
+        params = I.coarse_model_init(9)
+        gpu.set_coarse_model(I.flatten_coarse_model(params))
+        p = _rounded(params)
+        x, t = _patch_batch(nx, ny, ns, nlev, 71)
+        loss_ref, g_ref = _oracle_batch_grad(p, x, t, nx, ny)
+        loss, g = gpu.coarse_model_grad(_cuda(x, np.float32), _cuda(t, np.float32), nx, ny, fp32=True)
+        assert abs(loss - loss_ref) / loss_ref < 1e-5
+        gd = I.unflatten_coarse_model(g)
+        for k in g_ref:
+            err = np.abs(gd[k] - g_ref[k]).max() / max(np.abs(g_ref[k]).max(), 1e-300)
+            assert err < 1e-5, (k, err)
+    finally:
+        gpu.close()
+
+
 @pytest.mark.parametrize("nx,ny,ns", [(5, 4, 3), (8, 8, 4)])
 def test_bf16_gradient_matches_the_oracle_with_bf16_storage(nx, ny, ns):
     """The gradient the training uses (BF16 weights and activations, FP32 accumulation; the
