@@ -36,49 +36,94 @@ constexpr int kHoFacets = kHoRowThreads / Ho<P>::NB;   // facets per block
 template <int P>
 constexpr int kHoRows = kHoFacets<P> * Ho<P>::NB;      // rows per block
 
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int NLEFT>
+__device__ __forceinline__ void cp_async_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(NLEFT) : "memory");
+}
+template <int BYTES>   // 4, 8 or 16, both addresses aligned to it
+__device__ __forceinline__ void cp_async(void *smem, const void *gmem) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"((unsigned)__cvta_generic_to_shared(smem)), "l"(gmem),
+               "n"(BYTES)
+               : "memory");
+}
+
 // acc (+/-)= sum over the stored slots of row NB F + n times x, in slot order: cell A's NF facet dofs,
 // then cell B's without the shared facet (merged into A's slots when S was assembled). OFFD leaves out
 // the couplings inside the smoother's diagonal block D of Algorithm 1 (acc - (S - D) x): on a
 // vertical facet its own nodes, on a horizontal facet the horizontal facets of its column (A's
 // bottom and top, B's bottom).
-template <int P, bool NEG, bool OFFD, typename TS, typename TX, typename TA>
-__device__ __forceinline__ TA ho_row(const TS *__restrict__ S, const TX *__restrict__ x, const HoGeo &g, int64_t T,
-                                     int64_t F, int n, TA acc) {
+// A facet's NB coefficients come through shared memory by cp.async, one facet ahead of the products, into
+// this thread's column of buf ([NB][kHoRowThreads]; no barrier, a thread reads what it copied). With plain
+// loads the compiler keeps 32 or 40 registers, four to eight loads in flight per thread, and a mesh of one
+// wave pays eleven times their latency: at p = 3 on 16 x 16 x 16 cells the FP32 sweep's rows took 46 to 54
+// us and take 32 (118 MB), the FP32 residual's 33 and 31, the FP64 S apply 83 and 79 (FP64 issue alone:
+// 64). In FP32 x is an internal work vector (256-byte aligned), read NT values at a time.
+template <int P, bool NEG, bool OFFD, typename TS>
+__device__ __forceinline__ TS ho_row(const TS *__restrict__ S, const TS *__restrict__ x, const HoGeo &g, int64_t T,
+                                     int64_t F, int n, TS acc, TS *buf) {
   using H = Ho<P>;
   constexpr int NB = H::NB, NT = H::NT;
   const HoFacet fc = ho_facet(g, F);
   const bool vert = F < g.nhf;
-  const TS *s = S + (int64_t)NB * F + n;
-  auto cell = [&](int c, int k, int shared, bool skip_shared) {
-#pragma unroll(P == 1 ? 3 : 1)
-    for (int f = 0; f < 6; ++f, s += (int64_t)NB * T) {
-      if ((skip_shared && f == shared) || (OFFD && !vert && f >= 4)) continue;
-      const TX *xf;      // the facet's first value in the cell's traversal, step per s
-      int ds = NT;
-      if (f < 4) {
-        const int64_t e = __ldg(g.col_edges + 4 * (int64_t)c + f);
-        xf = x + NB * (e * g.L + k);
-        if (!g.own[4 * (int64_t)c + f]) {
-          xf += NT * P;
-          ds = -NT;
-        }
-      } else {
-        xf = x + g.NH + NB * ((int64_t)c * (g.L + 1) + k + (f == 5 ? 1 : 0));
-      }
-      TS a[NB];
-      TX v[NB];
-#pragma unroll
-      for (int q = 0; q < NB; ++q) a[q] = __ldcs(s + (int64_t)q * T);
-#pragma unroll
-      for (int q = 0; q < NT; ++q)
-#pragma unroll
-        for (int t = 0; t < NT; ++t) v[q * NT + t] = __ldg(xf + q * ds + t);
-#pragma unroll
-      for (int q = 0; q < NB; ++q) acc = fma(NEG ? -(TA)a[q] : (TA)a[q], (TA)v[q], acc);
+  const TS *s0 = S + (int64_t)NB * F + n;
+  auto next = [&](int j) {   // the first facet from slot group j on that the row takes, or 12
+    for (; j < 12; ++j) {
+      const int f = j < 6 ? j : j - 6;
+      if (OFFD && !vert && f >= 4) continue;
+      if (j < 6 ? !(OFFD && vert && f == fc.fA) : fc.cB >= 0 && f != fc.fB) break;
     }
+    return j;
   };
-  cell(fc.cA, fc.kA, fc.fA, OFFD && vert);
-  if (fc.cB >= 0) cell(fc.cB, fc.kB, fc.fB, true);
+  auto stage = [&](int j) {
+    const TS *s = s0 + (int64_t)j * NB * T;
+#pragma unroll
+    for (int q = 0; q < NB; ++q) cp_async<sizeof(TS)>(buf + q * kHoRowThreads, s + (int64_t)q * T);
+  };
+  int nj = next(0);
+  stage(nj);   // (every row takes a facet of its first cell)
+#pragma unroll 1
+  for (int j = 0; j < 12; ++j) {
+    if (j != nj) continue;
+    const int f = j < 6 ? j : j - 6;
+    const int64_t c = j < 6 ? fc.cA : fc.cB;
+    const int k = j < 6 ? fc.kA : fc.kB;
+    const TS *xf;         // the facet's first value in the cell's traversal, step per s
+    int ds = NT;
+    if (f < 4) {
+      const int64_t e = __ldg(g.col_edges + 4 * c + f);
+      xf = x + NB * (e * g.L + k);
+      if (!__ldg(g.own + 4 * c + f)) {
+        xf += NT * P;
+        ds = -NT;
+      }
+    } else {
+      xf = x + g.NH + NB * (c * (g.L + 1) + k + (f == 5 ? 1 : 0));
+    }
+    TS a[NB], v[NB];
+#pragma unroll
+    for (int q = 0; q < NT; ++q) {
+      const TS *xq = xf + q * ds;
+      if constexpr (NT == 4 && sizeof(TS) == 4) {
+        const float4 u = __ldg(reinterpret_cast<const float4 *>(xq));
+        v[4 * q] = u.x; v[4 * q + 1] = u.y; v[4 * q + 2] = u.z; v[4 * q + 3] = u.w;
+      } else if constexpr (NT == 2 && sizeof(TS) == 4) {
+        const float2 u = __ldg(reinterpret_cast<const float2 *>(xq));
+        v[2 * q] = u.x; v[2 * q + 1] = u.y;
+      } else {
+#pragma unroll
+        for (int t = 0; t < NT; ++t) v[q * NT + t] = __ldg(xq + t);
+      }
+    }
+    cp_async_commit();
+    cp_async_wait<0>();
+#pragma unroll
+    for (int q = 0; q < NB; ++q) a[q] = buf[q * kHoRowThreads];
+    nj = next(j + 1);
+    if (nj < 12) stage(nj);
+#pragma unroll
+    for (int q = 0; q < NB; ++q) acc = fma(NEG ? -a[q] : a[q], v[q], acc);
+  }
   return acc;
 }
 
@@ -274,12 +319,12 @@ __global__ void __launch_bounds__(kHoRowThreads)
     ho_spmv_kernel(const HoGeo g, int64_t T, const double *__restrict__ S, const double *__restrict__ x,
                    double *__restrict__ y, const double *__restrict__ w, double *__restrict__ fs) {
   constexpr int NB = Ho<P>::NB, FB = kHoFacets<P>;
+  __shared__ double ss[NB * kHoRowThreads];
   __shared__ double sv[MODE ? kHoRows<P> : 1], sw[MODE == 1 || MODE == 2 ? kHoRows<P> : 1];
   const int i = threadIdx.x;
   const int64_t row = (int64_t)blockIdx.x * kHoRows<P> + i, F = (int64_t)blockIdx.x * FB + i / NB;
   if (i < kHoRows<P> && row < T) {
-    const double v = MODE == 3 ? ho_row<P, true, false>(S, x, g, T, F, i % NB, __ldg(w + row))
-                               : ho_row<P, false, false>(S, x, g, T, F, i % NB, 0.0);
+    const double v = ho_row<P, MODE == 3, false>(S, x, g, T, F, i % NB, MODE == 3 ? __ldg(w + row) : 0.0, ss + i);
     if (MODE != 3) y[row] = v;
     if (MODE) sv[i] = v;
     if (MODE == 1 || MODE == 2) sw[i] = __ldg(w + row);
@@ -368,18 +413,6 @@ static HoGeo ho_geo(const Ctx *c) {
 // row straight from global memory touched 32 lines per load (p = 3, 4,096 cells: recovery 1,402 us, 0.3
 // of HBM bandwidth; now bound by the FP64 rate of its 378 M FMAs).
 constexpr int kHoTile = 16, kHoDotThreads = 256;
-
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int NLEFT>
-__device__ __forceinline__ void cp_async_wait() {
-  asm volatile("cp.async.wait_group %0;" ::"n"(NLEFT) : "memory");
-}
-template <int BYTES>   // 4, 8 or 16, both addresses aligned to it
-__device__ __forceinline__ void cp_async(void *smem, const void *gmem) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"((unsigned)__cvta_generic_to_shared(smem)), "l"(gmem),
-               "n"(BYTES)
-               : "memory");
-}
 
 // The rows of cell K that a product takes (all N, or the NF facet dofs) and its shared memory: the
 // block's cells' vectors, then per warp the row addresses and two tiles.
@@ -518,14 +551,22 @@ __global__ void __launch_bounds__(kHoRowThreads)
                          const Tb *__restrict__ b, const Tin *__restrict__ lam_in,
                          Tout *__restrict__ lam_out, double keep) {
   constexpr int NB = Ho<P>::NB;
+  constexpr bool AHEAD = !ZERO && sizeof(T) == 4;   // (FP64 is bound by its issue rate)
   __shared__ T sr[kHoRows<P>];
+  __shared__ T sf[AHEAD ? NB * kHoRowThreads : 1];       // the rows of omega D_F^-1, copied behind the products
+  __shared__ T ss[ZERO ? 1 : NB * kHoRowThreads];
   const int i = threadIdx.x, n = i % NB;
   const int64_t row = (int64_t)blockIdx.x * kHoRows<P> + i, F = (int64_t)blockIdx.x * kHoFacets<P> + i / NB;
   const bool act = i < kHoRows<P> && row < (ZERO ? g.NH : TT);
   T r = (T)0;
   if (act) {
+    if (AHEAD && F < g.nhf) {
+      const T *f = hw + (int64_t)NB * NB * F + n;
+#pragma unroll
+      for (int m = 0; m < NB; ++m) cp_async<sizeof(T)>(sf + m * kHoRowThreads + i, f + NB * m);
+    }
     r = (T)__ldg(b + row);
-    if (!ZERO) r = ho_row<P, true, true>(S, lam_in, g, TT, F, n, r);
+    if constexpr (!ZERO) r = ho_row<P, true, true>(S, lam_in, g, TT, F, n, r, ss + i);
     sr[i] = r;
   }
   __syncthreads();
@@ -533,8 +574,12 @@ __global__ void __launch_bounds__(kHoRowThreads)
   if (F < g.nhf) {
     const T *f = hw + (int64_t)NB * NB * F + n, *rf = sr + (i - n);
     T v = ZERO ? (T)0 : (T)keep * (T)lam_in[row];
+    if (AHEAD) {
+      cp_async_commit();
+      cp_async_wait<0>();
+    }
 #pragma unroll
-    for (int m = 0; m < NB; ++m) v = fma(__ldg(f + NB * m), rf[m], v);
+    for (int m = 0; m < NB; ++m) v = fma(AHEAD ? sf[m * kHoRowThreads + i] : __ldg(f + NB * m), rf[m], v);
     lam_out[row] = (Tout)v;
   } else {
     lam_out[row] = (Tout)r;
@@ -549,14 +594,32 @@ struct HoLines {
   static constexpr int NB2 = Ho<P>::NB * Ho<P>::NB, STRIDE = 2 * NB2 + Ho<P>::NB;
 };
 
-// One warp per block of CPW columns. The recurrences are serial over the levels (2 L + 1 steps of
-// NB-term dot products), so a step must not wait for its factors: they stream through shared memory by
-// cp.async, DEPTH - 1 steps ahead. Loaded one step ahead into registers, four warps per block, the
-// kernel took 1.1 us per step, one memory latency (37 us per sweep at p = 1 on 64 x 64 x 16 cells, 40 us
-// at p = 3 in FP32 on 16 x 16 x 16).
+// v = p[0 .. NB - 1] in shared memory, in 16-byte reads where a block is a multiple of them
+template <int NB, typename T>
+__device__ __forceinline__ void ho_block(T (&v)[NB], const T *p) {
+  constexpr int W = 16 / (int)sizeof(T);
+  if constexpr (NB % W == 0) {
+#pragma unroll
+    for (int q = 0; q < NB; q += W) {
+      const int4 u = *reinterpret_cast<const int4 *>(p + q);
+      memcpy(v + q, &u, 16);
+    }
+  } else {
+#pragma unroll
+    for (int q = 0; q < NB; ++q) v[q] = p[q];
+  }
+}
+
+// One warp of recurrences per block of CPW columns, and a second one that feeds it. The recurrences are
+// serial over the levels (2 L + 1 steps of NB-term dot products), so a step must not wait for its factors:
+// they stream through shared memory by cp.async, DEPTH - 1 steps ahead, and the copies' instructions are
+// the other warp's. Loaded one step ahead into registers, four warps per block, the kernel took 1.1 us per
+// step, one memory latency (37 us per sweep at p = 1 on 64 x 64 x 16 cells, 40 us at p = 3 in FP32 on
+// 16 x 16 x 16); with the copies issued by the same warp 22 and 19 us;
+// now 20 and 16.5 (at p = 1 the FP64 pipe's twelve FMAs per step and warp, 3.4 warps per SM, are half of it).
 // Part 2; r is read from src (lam_out after part 1, b for a sweep from zero)
 template <int P, bool ZERO, typename T = double, typename Ts = double, typename Tin = double, typename Tout = double>
-__global__ void __launch_bounds__(32)
+__global__ void __launch_bounds__(64)
     ho_sweep_lines_kernel(const HoGeo g, int cpb, const T *__restrict__ zf, const Ts *src,
                           const Tin *__restrict__ lam_in, Tout *lam_out, double keep) {
   using H = Ho<P>;
@@ -567,7 +630,8 @@ __global__ void __launch_bounds__(32)
   extern __shared__ __align__(16) unsigned char ho_lines_smem[];
   T *ring = reinterpret_cast<T *>(ho_lines_smem);   // [D][CPW][CS]
   T *sr = ring + D * H::CPW * CS;                   // [cpb][L+1][NB]
-  const int L1 = g.L + 1, lane = threadIdx.x;
+  const int L1 = g.L + 1, lane = threadIdx.x & 31;
+  const bool feeds = threadIdx.x >= 32;
   const int c0 = blockIdx.x * cpb, nc = min(cpb, g.ncol - c0);
   const int64_t base = g.NH + (int64_t)NB * c0 * L1;
   // step s of the two passes: the forward step of level s, then the backward step of level 2 L1 - 2 - s
@@ -583,9 +647,10 @@ __global__ void __launch_bounds__(32)
     }
     cp_async_commit();
   };
+  if (feeds)
 #pragma unroll
-  for (int s = 0; s < D; ++s) stage(s);
-  for (int i = lane; i < nc * L1 * NB; i += 32) sr[i] = (T)src[base + i];
+    for (int s = 0; s < D; ++s) stage(s);
+  for (int i = threadIdx.x; i < nc * L1 * NB; i += 64) sr[i] = (T)src[base + i];
   const int cc = lane / LPC, n = lane - cc * LPC;
   const bool act = cc < nc && n < NB;
   T *r = sr + NB * (act ? cc : 0) * L1;
@@ -595,7 +660,8 @@ __global__ void __launch_bounds__(32)
   auto load = [&](int s) {
     const T *q = ring + (s % D) * (H::CPW * CS) + (act ? cc * CS + n : 0);   // this lane's rows (transposed)
     if (s < L1) {
-      const T *rk = r + NB * s;
+      T rk[NB];
+      ho_block<NB>(rk, r + NB * s);
       v = (T)0;
 #pragma unroll
       for (int m = 0; m < NB; ++m) v = fma(q[NB * m], rk[m], v);
@@ -607,33 +673,36 @@ __global__ void __launch_bounds__(32)
     for (int m = 0; m < NB; ++m) f[m] = q[NB * m];
   };
   cp_async_wait<D - 1>();
-  __syncwarp();
-  load(0);
+  __syncthreads();
+  if (!feeds) load(0);
   for (int s = 0; s < steps; ++s) {
-    if (s < L1) {
-      // forward: y_k = (omega G_k^-1) r_k - (G_k^-1 L_k) y_{k-1}, y written over r
-      T u = (T)0;
-      if (s > 0) {
-        const T *y = r + NB * (s - 1);
+    if (!feeds) {
+      if (s < L1) {
+        // forward: y_k = (omega G_k^-1) r_k - (G_k^-1 L_k) y_{k-1}, y written over r
+        T u = (T)0;
+        if (s > 0) {
+          T y[NB];
+          ho_block<NB>(y, r + NB * (s - 1));
 #pragma unroll
-        for (int m = 0; m < NB; ++m) u = fma(-f[m], y[m], u);
+          for (int m = 0; m < NB; ++m) u = fma(-f[m], y[m], u);
+        }
+        if (act) r[NB * s + n] = v + u;
+      } else {
+        // backward: x_k = y_k - (G_k^-1 U_k) x_{k+1}, x written over y
+        const int k = 2 * L1 - 2 - s;
+        T x[NB], u = v;
+        ho_block<NB>(x, r + NB * (k + 1));
+#pragma unroll
+        for (int m = 0; m < NB; ++m) u = fma(-f[m], x[m], u);
+        if (act) r[NB * k + n] = u;
       }
-      if (act) r[NB * s + n] = v + u;
-    } else {
-      // backward: x_k = y_k - (G_k^-1 U_k) x_{k+1}, x written over y
-      const int k = 2 * L1 - 2 - s;
-      const T *x = r + NB * (k + 1);
-      T u = v;
-#pragma unroll
-      for (int m = 0; m < NB; ++m) u = fma(-f[m], x[m], u);
-      if (act) r[NB * k + n] = u;
     }
-    cp_async_wait<D - 2>();   // the next step's factors
-    __syncwarp();
-    if (s + 1 < steps) load(s + 1);
-    stage(s + D);             // (its slot was read before this step)
+    cp_async_wait<D - 2>();   // the next step's factors (the feeding warp's copies)
+    __syncthreads();
+    if (feeds) stage(s + D);  // (its slot was read before this barrier)
+    else if (s + 1 < steps) load(s + 1);
   }
-  for (int i = lane; i < nc * L1 * NB; i += 32)
+  for (int i = threadIdx.x; i < nc * L1 * NB; i += 64)
     lam_out[base + i] = (Tout)(ZERO ? sr[i] : fma((T)keep, (T)lam_in[base + i], sr[i]));
 }
 
@@ -644,11 +713,12 @@ __global__ void __launch_bounds__(kHoRowThreads)
     ho_residual_kernel(const HoGeo g, int64_t TT, const T *__restrict__ S, const double *__restrict__ b,
                        const T *__restrict__ lam, T *__restrict__ R, double keep) {
   constexpr int NB = Ho<P>::NB;
+  __shared__ T ss[NB * kHoRowThreads];
   const int i = threadIdx.x;
   const int64_t row = (int64_t)blockIdx.x * kHoRows<P> + i, F = (int64_t)blockIdx.x * kHoFacets<P> + i / NB;
   if (i >= kHoRows<P> || row >= TT) return;
   const T bv = (T)__ldg(b + row);
-  R[row] = ho_row<P, true, ZSWEEP>(S, lam, g, TT, F, i % NB, ZSWEEP ? (T)keep * bv : bv);
+  R[row] = ho_row<P, true, ZSWEEP>(S, lam, g, TT, F, i % NB, ZSWEEP ? (T)keep * bv : bv, ss + i);
 }
 
 // bbar_K = Gamma_K (P^T R)_K (Algorithm 2 lines 4-5): P is constant on a facet (all its nodes)
@@ -929,7 +999,7 @@ static int ho_sweep(Ctx *c, const double *b, const Tin *lam_in, Tout *lam_out) {
   auto lines = [&](auto kern, const auto *src) {
     const cudaError_t e = smem > 48 * 1024 ? cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)
                                            : cudaSuccess;
-    if (e == cudaSuccess) kern<<<nzb, 32, smem, c->stream>>>(g, cpb, HoPrec<T>::zf(h), src, lam_in, lam_out, keep);
+    if (e == cudaSuccess) kern<<<nzb, 64, smem, c->stream>>>(g, cpb, HoPrec<T>::zf(h), src, lam_in, lam_out, keep);
     return e;
   };
   if constexpr (ZERO) HMG_CUDA(c, lines(ho_sweep_lines_kernel<P, ZERO, T, double, Tin, Tout>, b));
