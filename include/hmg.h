@@ -114,8 +114,10 @@ typedef struct {
                            ||B|| on its way to convergence) */
   int32_t profile;      /* 1: time every solver component with CUDA events (see
                            hmg_solve_stats.comp_ms); 0: no events (default) */
-  int32_t graph;        /* 1 (default): the whole solve is one CUDA graph whose BiCGStab loop
-                           is a device-side WHILE node (no host round trip per iteration);
+  int32_t graph;        /* 1 (default): the BiCGStab loop is one CUDA graph launch with a
+                           device-side WHILE node (no host round trip per iteration; the
+                           right-hand side before it and the stats after it are launched beside
+                           it, so the graph is kept while the options stay);
                            0: the host drives the loop (always so when profile = 1) */
   int32_t coarse;       /* coarse solve of Algorithm 2 line 6: HMG_COARSE_* */
   int32_t krylov;       /* HMG_KRYLOV_BICGSTAB (default) or HMG_KRYLOV_FGMRES */
@@ -133,9 +135,10 @@ typedef struct {
                            internal copy of the last solution) passed in, r_0 = B - S lambda_0
                            (resuming a solve, or a previous time step's solution) */
   int32_t mg_fuse_cells; /* coarse levels of at most this many cells (default 262144) run the
-                           restriction inside their first sweep and the injection inside their
-                           first post-sweep, one launch instead of two (same arithmetic,
-                           bitwise the same result); 0: never. Must be >= 0 */
+                           restriction inside their first sweep, and every level of at most this
+                           many the injection inside its first post-sweep, one launch instead
+                           of two (same arithmetic, bitwise the same result); 0: never. Must be
+                           >= 0 */
   int32_t async_stats;  /* 0 (default): hmg_solve synchronises once, to fill its stats.
                            1: a graph-launched BiCGStab solve (graph = 1, profile = 0, no
                            Krylov coarse solve) is only enqueued on the context's stream;
@@ -211,10 +214,12 @@ int hmg_default_options(hmg_options *opt);
  * cuda_stream: a cudaStream_t owned by the caller (NULL = the legacy default stream). */
 int hmg_create(hmg_ctx **out, const hmg_options *opt, void *cuda_stream);
 
-/* Replace the options (e.g. the tolerance or precision) without reassembling. On an assembled
- * context, switching to HMG_PRECISION_MIXED makes the FP32 copies of the operators and factors
- * from the assembled FP64 ones (device memory for them is allocated here, once; synchronises);
- * a change of degree needs hmg_assemble_trace. */
+/* Replace the options (e.g. the tolerance or a relaxation weight). On an assembled context, the first
+ * switch to HMG_PRECISION_MIXED forms the operators again, by the direct Gauss sums that contexts
+ * created with this precision use (equal to rounding, which the FP32 preconditioner amplifies), and
+ * makes their FP32 copies (device memory for them is allocated here, once; synchronises; where the
+ * sums' scratch does not fit, the copies are made from the operators there are). A change of degree
+ * needs hmg_assemble_trace. */
 int hmg_set_options(hmg_ctx *ctx, const hmg_options *opt);
 
 /* Set the mesh hierarchy: levels[0] finest ... levels[nmg-1] coarsest; every level has
@@ -280,8 +285,8 @@ int hmg_autotune(hmg_ctx *ctx);
 
 /* Read / set the launch shapes of a context (host int32 arrays): sweep[2] = {columns per
  * block, threads per block} of the line sweep; mg[2 * nmg] = the same for the pressure
- * smoother on each level. 0 means the default (32 columns, 256 threads, within the shared
- * memory limit); columns -1 selects one warp per column (Thomas recurrences as a warp scan:
+ * smoother on each level. 0 means the default (32 columns, fewer on levels of few columns, 256
+ * threads, within the shared memory limit); columns -1 selects one warp per column (Thomas recurrences as a warp scan:
  * the same iterate up to rounding order): for a smoother level of at most 128 layers in both
  * precisions, for the sweep (at most 127 layers) in the FP32 preconditioner's kernels only, the
  * FP64 sweep taking the default. hmg_get_launch_shapes reports the shapes of the kernels the

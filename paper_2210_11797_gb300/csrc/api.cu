@@ -200,6 +200,12 @@ int hmg_set_options(hmg_ctx *c, const hmg_options *opt) {
   if (st) return st;
   c->opt = *opt;
   if (c->assembled && c->opt.degree != c->degree) c->assembled = false;   // a new discretisation
+  if (c->assembled && c->opt.precision == HMG_PRECISION_MIXED && !c->direct_sums) {
+    // the operators in the form that contexts created with this precision have (gauss_cells.cu says why);
+    // where their scratch does not fit any more, the FP32 copies of the operators there are
+    st = hmg_assemble_trace(c);
+    if (st != HMG_ERR_OUT_OF_MEMORY || c->degree != c->opt.degree) return st;
+  }
   if (c->assembled && c->opt.precision == HMG_PRECISION_MIXED && !c->have_fp32) {
     // the FP32 copies from the assembled FP64 operators (the degree-p ones below)
     HMG_CUDA(c, cudaSetDevice(c->device));
@@ -420,6 +426,7 @@ int hmg_assemble_trace(hmg_ctx *c) {
   }
   if (c->degree == 0 && c->ho.degree != 0) ho_free(c);   // the degree-p system is no longer in use
   if (!c->noalloc_scratch && (st = noalloc_setup(c))) return st;
+  c->direct_sums = need_fp32;
   c->assembled = true;
   return HMG_OK;
 }

@@ -39,9 +39,10 @@ namespace hmg {
 // form by up to 1e-10 of an entry, with it by 1e-14 of the row's scale.
 //
 // Evaluating the 27 points in every cell cost about 6,700 FP64 operations per cell (22.2 ms for the
-// 1.66M cells of C96 x 30 with rotation, all FP64 issue); here a column costs about 1,000 and a cell
-// of the finest level about 900, most of them for the chains (coarser levels, which need neither
-// M(f, z) nor its correction: 350).
+// 1.66M cells of C96 x 30 with rotation, and 3.0 ms for the condensation; all FP64 issue); here a column
+// costs about 1,000 and a cell of the finest level about 1,000, most of them for the chains (coarser
+// levels, which need neither M(f, z) nor its correction: 480), and the finest level's geometry and
+// condensation together take 4.5 ms, at the FP64 issue rate.
 struct Col {   // per-column sums [ncol][N]; face pairs f <= g in row-major order (10 of them)
   static constexpr int A = 0, B = 10, U = 20, XU = 24;   // XU: (C x C_d) . z part of M(f, z) per cz
   static constexpr int X = 28;     // 4: Coriolis pairs (0,1) (0,3) (1,2) (2,3) per cz / dz
@@ -723,7 +724,7 @@ __global__ void trace_rows_kernel(const RowArgs a, const double *__restrict__ Ai
 // coalesced loads, one lane per column on the serial chain of divides (whole warps on it, as the
 // FP64 pipe is occupied per warp), the factors stored coalesced. A launch per system with one thread
 // per column straight from global memory took 0.24 ms for the five systems of C96 x 30, four of them
-// waiting on the strided loads of a few warps.
+// waiting on the strided loads of a few warps; this takes 0.09 ms.
 struct FactorJob {
   const double *sub, *diag, *sup;   // [ncol][n], sub ignored at k = 0
   double *w, *l, *cp;

@@ -358,7 +358,11 @@ __global__ void gauss_out_kernel(int64_t ncell, const double *__restrict__ rec, 
 int gauss_setup(Ctx *c, int64_t ncell, double **rec) {
   int st;
   if ((st = upload_shape_functions(c))) return st;
-  HMG_CUDA(c, cudaMalloc(rec, (size_t)ncell * kCellData * sizeof(double)));
+  if (cudaMalloc(rec, (size_t)ncell * kCellData * sizeof(double)) != cudaSuccess) {
+    *rec = nullptr;
+    cudaGetLastError();
+    return fail(c, HMG_ERR_OUT_OF_MEMORY, "device allocation of the cell records failed");
+  }
   return HMG_OK;
 }
 

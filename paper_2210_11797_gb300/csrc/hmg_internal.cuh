@@ -124,6 +124,7 @@ struct Ctx {
   int nmg = 0;
   Level lv[kMaxLevels];
   bool have_mesh = false, have_coeffs = false, assembled = false, have_fp32 = false;
+  bool direct_sums = false;   // the operators come from direct Gauss sums (gauss_cells.cu)
   int degree = 0;              // polynomial degree of the assembled system (0 .. 3)
   HoData ho;
   // finest-level trace system (device)
@@ -206,7 +207,7 @@ struct Ctx {
   // looked up once by hmg_assemble_trace
   double *noalloc_scratch = nullptr;
   int num_sms = 0;
-  int wave_blocks[3] = {0, 0, 0};   // resident blocks (all SMs) of the BiCGStab vector kernels
+  int wave_blocks[2] = {0, 0};   // resident blocks (all SMs) of the BiCGStab vector kernels
   // configuration 1 (mixed.cu): the 2x2 operator (velocity block in the 11-slot layout of S,
   // G couplings [2][ntrace], B couplings and M3^Pi [7][ncell]), 1 / lumped mass [ntrace], the
   // solution [ntrace + ncell] and the Step-1 right-hand side [ncell]
@@ -416,8 +417,8 @@ constexpr int kMaxLayers = 2045;
 // Columns per block of a column kernel that no shape was given for: 32 (a lane per column of the serial
 // phase, which occupies the FP64 pipe per warp), fewer where that would leave SMs without a block: a
 // level of few columns waits on latency, and a small block takes its cells in one pass. C12 x 30 (864
-// columns, FP64): a smoothing sweep 13.7 us at 32 columns (27 blocks), 5.0 us at 4; its fused
-// restriction and sweep 31 and 7 us.
+// columns, FP64, cold caches): a smoothing sweep 13.7 us at 32 columns (27 blocks), 8 us at 4 (216); its
+// fused restriction and sweep 31 and 13 us.
 inline int default_columns(const Ctx *c, int ncol, int limit) {
   int n = limit < 32 ? limit : 32;
   while (n > 1 && (int64_t)n * c->num_sms > ncol) n >>= 1;

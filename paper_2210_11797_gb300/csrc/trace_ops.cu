@@ -79,8 +79,9 @@ int launch_finalize(Ctx *c, int nblocks, int s0, int s1) {
 // The same S apply for meshes of few rows, in two launches: the rows, one per thread in small blocks over
 // all SMs, then the inner products from y and w with spmv_kernel's blocks and order, the last block adding
 // the partials in finalize_kernel's order (bitwise the same sums). spmv_kernel leaves most SMs idle there,
-// with its FP64 work four rows deep on a few: at 6,400 rows seven blocks, 12-17 us for the apply and 8 us
-// for the partials.
+// with its FP64 work four rows deep on a few: at 6,400 rows (seven blocks) 17-19 us for the apply and 8 us
+// for the partials, now 7 + 7 us (cold caches). The line lies at four of spmv_kernel's blocks per SM,
+// where they fill the chip.
 template <bool NEG>   // NEG: y = w - S x
 __global__ void __launch_bounds__(128)
     spmv_rows_kernel(const double *__restrict__ S, const double *__restrict__ x, double *__restrict__ y,

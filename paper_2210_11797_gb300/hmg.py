@@ -268,8 +268,8 @@ class Solver:
     def set_options(self, **kw):
         for k, v in kw.items():
             setattr(self.opts, k, _option_value(k, v))
-        # (hmg_set_options makes the FP32 copies of the operators when the precision becomes
-        # mixed, and rebuilds them with the factors when a relaxation weight changes)
+        # (hmg_set_options forms the operators again and makes their FP32 copies when the precision
+        # becomes mixed, and rebuilds the factors when a relaxation weight changes)
         _check(self.ctx, lib().hmg_set_options(self.ctx, C.byref(self.opts)))
         if self.opts.precision == PRECISION["mixed"]:
             self._fp32_built = True

@@ -59,3 +59,26 @@ def test_degree_p_without_shift_is_refused():
     co.sigma = 0.0
     with pytest.raises(HmgError):
         Solver(hier, co, degree=1)
+
+
+@pytest.mark.parametrize("mesh,n,L,degree", [("plane", 6, 5, 0), ("sphere", 8, 33, 0), ("plane", 4, 3, 2)])
+def test_switching_to_mixed_gives_the_operators_of_a_mixed_context(mesh, n, L, degree):
+    """The FP32 preconditioner amplifies last-bit differences of S, so a context that becomes mixed takes
+    the operators that a context created so has: the same solution, bit for bit."""
+    from paper_2210_11797_gb300.hmg import Solver
+    hier, co = _system(mesh, n, L, degree, 0.0)
+    a, b = (Solver(hier, co, degree=degree, precision=p, tol=1e-6) for p in ("fp64", "mixed"))
+    g = torch.Generator(device="cuda").manual_seed(2)
+    Ru, Rp = (torch.randn(m, generator=g, dtype=torch.float64, device="cuda") for m in (a.nu * a.ncell, a.npr * a.ncell))
+    first = a.solve(Ru, Rp)[0]
+    a.set_options(precision="mixed")
+    want = b.solve(Ru, Rp)[0]
+    assert torch.equal(a.solve(Ru, Rp)[0], want)
+    a.set_options(precision="fp64")
+    assert float((a.solve(Ru, Rp)[0] - first).norm()) <= 1e-4 * float(first.norm())   # both at tol 1e-6
+    a.assemble()
+    assert torch.equal(a.solve(Ru, Rp)[0], first)
+    a.set_options(precision="mixed")   # (FP32 copies of the earlier operators are there by now)
+    assert torch.equal(a.solve(Ru, Rp)[0], want)
+    a.close()
+    b.close()
