@@ -149,12 +149,12 @@ int launch_spmv(Ctx *c, const double *x, double *y, int mode, const double *w, i
   Prof prof(c, kCompApply);
   const int *as = alpha && mode == 1 ? c->state : nullptr;
   // up to four of spmv_kernel's blocks per SM (its last wave of them is uneven: 308 blocks at C24 x 30)
-  if (mode != 0 && g <= 4u * (unsigned)c->num_sms) {
+  if (g <= 4u * (unsigned)c->num_sms) {
     if (mode == 3) y = static_cast<double *>(c->w1);   // (a place for the residual: the preconditioner is idle)
     auto rows = mode == 3 ? spmv_rows_kernel<true> : spmv_rows_kernel<false>;
     rows<<<grid_for(f.ntrace, 128), 128, 0, c->stream>>>(c->S, x, y, w, d, f.edge_stencil, f.col_edges);
     auto dots = mode == 1 ? spmv_dots_kernel<1> : (mode == 2 ? spmv_dots_kernel<2> : spmv_dots_kernel<3>);
-    dots<<<g, kRedThreads, 0, c->stream>>>(y, w, f.ntrace, c->part, slot0, slot1, c->counter, c->scal, as);
+    if (mode != 0) dots<<<g, kRedThreads, 0, c->stream>>>(y, w, f.ntrace, c->part, slot0, slot1, c->counter, c->scal, as);
     HMG_CUDA(c, cudaGetLastError());
     return HMG_OK;
   }
