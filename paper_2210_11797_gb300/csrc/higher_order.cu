@@ -35,6 +35,11 @@ template <int P>
 constexpr int kHoFacets = kHoRowThreads / Ho<P>::NB;   // facets per block
 template <int P>
 constexpr int kHoRows = kHoFacets<P> * Ho<P>::NB;      // rows per block
+// rows per thread (consecutive rows of one facet, which share its x values) and threads per block
+template <int P, typename T>
+constexpr int kHoR = P == 2 ? (sizeof(T) == 4 ? 3 : 1) : 16 / (int)sizeof(T);
+template <int P, typename T>
+constexpr int kHoThreads = (kHoRows<P> / kHoR<P, T> + 31) / 32 * 32;
 
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int NLEFT>
@@ -53,17 +58,35 @@ __device__ __forceinline__ void cp_async(void *smem, const void *gmem) {
 // the couplings inside the smoother's diagonal block D of Algorithm 1 (acc - (S - D) x): on a
 // vertical facet its own nodes, on a horizontal facet the horizontal facets of its column (A's
 // bottom and top, B's bottom).
-// A facet's NB coefficients come through shared memory by cp.async, one facet ahead of the products, into
-// this thread's column of buf ([NB][kHoRowThreads]; no barrier, a thread reads what it copied). With plain
-// loads the compiler keeps 32 or 40 registers, four to eight loads in flight per thread, and a mesh of one
-// wave pays eleven times their latency: at p = 3 on 16 x 16 x 16 cells the FP32 sweep's rows took 46 to 54
-// us and take 32 (118 MB), the FP32 residual's 33 and 31, the FP64 S apply 83 and 79 (FP64 issue alone:
-// 64). In FP32 x is an internal work vector (256-byte aligned), read NT values at a time.
+// A thread takes R consecutive rows of the facet. A facet's coefficients come through shared memory by
+// cp.async, one facet ahead of the products, into this thread's part of buf ([NB][threads][R]; no barrier, a
+// thread reads what it copied): a slot is refilled as soon as it is read. In FP32 x is an internal work
+// vector (256-byte aligned), read NT values at a time. With plain loads the compiler keeps few of them in flight, and a mesh of one wave
+// pays their latency for each facet. p = 3, 16 x 16 x 16 cells: FP32 sweep rows 46-54 us with plain loads and
+// a row per thread, 30 now (118 MB), FP32 residual 33 and 28, FP64 S apply 83 and 79 (FP64 issue alone: 64).
+// R is one 16-byte copy; at p = 2 (nine rows) FP64 takes 1 (S apply on 56 x 56 x 32 cells 470 us, 545 at 3).
+template <int R, typename T>
+__device__ __forceinline__ void ho_copy(T *smem, const T *gmem) {   // R values, 16 bytes at once where they are
+  if constexpr (R * sizeof(T) == 16) cp_async<16>(smem, gmem);
+  else
+#pragma unroll
+    for (int r = 0; r < R; ++r) cp_async<sizeof(T)>(smem + r, gmem + r);
+}
+template <int R, typename T>
+__device__ __forceinline__ void ho_take(T (&v)[R], const T *smem) {
+  if constexpr (R * sizeof(T) == 16) {
+    const int4 u = *reinterpret_cast<const int4 *>(smem);
+    memcpy(v, &u, 16);
+  } else {
+#pragma unroll
+    for (int r = 0; r < R; ++r) v[r] = smem[r];
+  }
+}
 template <int P, bool NEG, bool OFFD, typename TS>
-__device__ __forceinline__ TS ho_row(const TS *__restrict__ S, const TS *__restrict__ x, const HoGeo &g, int64_t T,
-                                     int64_t F, int n, TS acc, TS *buf) {
+__device__ __forceinline__ void ho_row(const TS *__restrict__ S, const TS *__restrict__ x, const HoGeo &g, int64_t T,
+                                       int64_t F, int n, TS (&acc)[kHoR<P, TS>], TS *buf) {
   using H = Ho<P>;
-  constexpr int NB = H::NB, NT = H::NT;
+  constexpr int NB = H::NB, NT = H::NT, R = kHoR<P, TS>, STEP = kHoThreads<P, TS> * R;
   const HoFacet fc = ho_facet(g, F);
   const bool vert = F < g.nhf;
   const TS *s0 = S + (int64_t)NB * F + n;
@@ -75,13 +98,9 @@ __device__ __forceinline__ TS ho_row(const TS *__restrict__ S, const TS *__restr
     }
     return j;
   };
-  auto stage = [&](int j) {
-    const TS *s = s0 + (int64_t)j * NB * T;
+  int nj = next(0);   // (every row takes a facet of its first cell)
 #pragma unroll
-    for (int q = 0; q < NB; ++q) cp_async<sizeof(TS)>(buf + q * kHoRowThreads, s + (int64_t)q * T);
-  };
-  int nj = next(0);
-  stage(nj);   // (every row takes a facet of its first cell)
+  for (int q = 0; q < NB; ++q) ho_copy<R>(buf + q * STEP, s0 + ((int64_t)nj * NB + q) * T);
 #pragma unroll 1
   for (int j = 0; j < 12; ++j) {
     if (j != nj) continue;
@@ -100,7 +119,7 @@ __device__ __forceinline__ TS ho_row(const TS *__restrict__ S, const TS *__restr
     } else {
       xf = x + g.NH + NB * (c * (g.L + 1) + k + (f == 5 ? 1 : 0));
     }
-    TS a[NB], v[NB];
+    TS v[NB];
 #pragma unroll
     for (int q = 0; q < NT; ++q) {
       const TS *xq = xf + q * ds;
@@ -117,15 +136,61 @@ __device__ __forceinline__ TS ho_row(const TS *__restrict__ S, const TS *__restr
     }
     cp_async_commit();
     cp_async_wait<0>();
-#pragma unroll
-    for (int q = 0; q < NB; ++q) a[q] = buf[q * kHoRowThreads];
     nj = next(j + 1);
-    if (nj < 12) stage(nj);
+    const TS *s = s0 + (int64_t)nj * NB * T;
 #pragma unroll
-    for (int q = 0; q < NB; ++q) acc = fma(NEG ? -a[q] : a[q], v[q], acc);
+    for (int q = 0; q < NB; ++q) {
+      TS a[R];
+      ho_take<R>(a, buf + q * STEP);
+      if (nj < 12) ho_copy<R>(buf + q * STEP, s + (int64_t)q * T);
+#pragma unroll
+      for (int r = 0; r < R; ++r) acc[r] = fma(NEG ? -a[r] : a[r], v[q], acc[r]);
+    }
   }
-  return acc;
 }
+
+// The same products, negative, for all NB rows of a facet by one thread, in FP32: a slot's coefficients in
+// 16-byte loads where NB allows, and each x value read once for NB products. It needs a facet for every
+// thread of the chip: kHoFacetRows.
+template <int P, bool OFFD>
+__device__ __forceinline__ void ho_facet_rows(const float *__restrict__ S, const float *__restrict__ x, const HoGeo &g,
+                                              int64_t T, int64_t F, float (&acc)[Ho<P>::NB]) {
+  using H = Ho<P>;
+  constexpr int NB = H::NB, U = P == 1 ? 4 : 2;
+  const HoFacet fc = ho_facet(g, F);
+  const bool vert = F < g.nhf;
+  const float *Sr = S + (int64_t)NB * F;
+  auto cell = [&](int c, int k, int skip) {
+#pragma unroll U
+    for (int q = 0; q < H::NF; ++q) {
+      if (q / NB == skip || (OFFD && !vert && q / NB >= 4)) continue;
+      const float xv = __ldg(x + ho_gid<P>(g, c, k, q));
+      const float *s = Sr + (int64_t)q * T;
+      if constexpr (NB % 4 == 0) {
+#pragma unroll
+        for (int n = 0; n < NB; n += 4) {
+          const float4 v = __ldcs(reinterpret_cast<const float4 *>(s + n));
+          acc[n] = fmaf(-v.x, xv, acc[n]);
+          acc[n + 1] = fmaf(-v.y, xv, acc[n + 1]);
+          acc[n + 2] = fmaf(-v.z, xv, acc[n + 2]);
+          acc[n + 3] = fmaf(-v.w, xv, acc[n + 3]);
+        }
+      } else {
+#pragma unroll
+        for (int n = 0; n < NB; ++n) acc[n] = fmaf(-__ldcs(s + n), xv, acc[n]);
+      }
+    }
+  };
+  cell(fc.cA, fc.kA, OFFD && vert ? fc.fA : -1);
+  Sr += (int64_t)H::NF * T;
+  if (fc.cB >= 0) cell(fc.cB, fc.kB, fc.fB);
+}
+// FP32 rows from which a facet per thread is the faster form (sweep rows and residual of p = 1, 2, 3: 98 /
+// 182 / 237 and 91 / 170 / 227 us against 121 / 254 / 294 and 89 / 219 / 264 with R rows per thread, at
+// 3.6 / 2.8 / 2.5 M rows; at 0.2 M rows of p = 3, 49 blocks, 135 us against 30). The line is where the
+// facet form's 130 us of latency at p = 3 meet the other's 120 us per million rows. Both forms add a row's
+// products in the same order.
+constexpr int64_t kHoFacetRows = 1 << 20;
 
 // ---- assembly -------------------------------------------------------------------------------
 // own[c][f] = 1 where column c owns the edge of its face f (each entry written by one edge)
@@ -315,19 +380,25 @@ __global__ void __launch_bounds__(32 * kHoFacWarps)
 // lowest-order S apply does (3: (b - S x, b - S x), no y): a facet's products are summed in row order by
 // one thread into fs[F] (and fs[nF + F]), which ho_reduce_kernel adds up.
 template <int P, int MODE>
-__global__ void __launch_bounds__(kHoRowThreads)
+__global__ void __launch_bounds__(kHoThreads<P, double>)
     ho_spmv_kernel(const HoGeo g, int64_t T, const double *__restrict__ S, const double *__restrict__ x,
                    double *__restrict__ y, const double *__restrict__ w, double *__restrict__ fs) {
-  constexpr int NB = Ho<P>::NB, FB = kHoFacets<P>;
-  __shared__ double ss[NB * kHoRowThreads];
+  constexpr int NB = Ho<P>::NB, FB = kHoFacets<P>, R = kHoR<P, double>;
+  __shared__ __align__(16) double ss[NB * kHoThreads<P, double> * R];
   __shared__ double sv[MODE ? kHoRows<P> : 1], sw[MODE == 1 || MODE == 2 ? kHoRows<P> : 1];
-  const int i = threadIdx.x;
-  const int64_t row = (int64_t)blockIdx.x * kHoRows<P> + i, F = (int64_t)blockIdx.x * FB + i / NB;
-  if (i < kHoRows<P> && row < T) {
-    const double v = ho_row<P, MODE == 3, false>(S, x, g, T, F, i % NB, MODE == 3 ? __ldg(w + row) : 0.0, ss + i);
-    if (MODE != 3) y[row] = v;
-    if (MODE) sv[i] = v;
-    if (MODE == 1 || MODE == 2) sw[i] = __ldg(w + row);
+  const int i = threadIdx.x, i0 = i * R;
+  const int64_t row = (int64_t)blockIdx.x * kHoRows<P> + i0, F = (int64_t)blockIdx.x * FB + i0 / NB;
+  if (i0 < kHoRows<P> && row < T) {
+    double v[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) v[r] = MODE == 3 ? __ldg(w + row + r) : 0.0;
+    ho_row<P, MODE == 3, false>(S, x, g, T, F, i0 % NB, v, ss + i0);
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      if (MODE != 3) y[row + r] = v[r];
+      if (MODE) sv[i0 + r] = v[r];
+      if (MODE == 1 || MODE == 2) sw[i0 + r] = __ldg(w + row + r);
+    }
   }
   if (MODE) {
     __syncthreads();
@@ -546,44 +617,54 @@ __global__ void ho_rhs_kernel(const HoGeo g, int64_t T, const double *__restrict
 // type (double, or float in the FP32 preconditioner, whose b is the FP64 Krylov residual and
 // whose last sweep writes FP64).
 template <int P, bool ZERO, typename T = double, typename Tb = double, typename Tin = double, typename Tout = double>
-__global__ void __launch_bounds__(kHoRowThreads)
+__global__ void __launch_bounds__(ZERO ? kHoRowThreads : kHoThreads<P, T>)
     ho_sweep_rows_kernel(const HoGeo g, int64_t TT, const T *__restrict__ S, const T *__restrict__ hw,
                          const Tb *__restrict__ b, const Tin *__restrict__ lam_in,
                          Tout *__restrict__ lam_out, double keep) {
-  constexpr int NB = Ho<P>::NB;
-  constexpr bool AHEAD = !ZERO && sizeof(T) == 4;   // (FP64 is bound by its issue rate)
+  constexpr int NB = Ho<P>::NB, R = ZERO ? 1 : kHoR<P, T>, STEP = kHoThreads<P, T> * kHoR<P, T>;
+  constexpr bool AHEAD = !ZERO && sizeof(T) == 4;         // (FP64 is bound by its issue rate)
   __shared__ T sr[kHoRows<P>];
-  __shared__ T sf[AHEAD ? NB * kHoRowThreads : 1];       // the rows of omega D_F^-1, copied behind the products
-  __shared__ T ss[ZERO ? 1 : NB * kHoRowThreads];
-  const int i = threadIdx.x, n = i % NB;
-  const int64_t row = (int64_t)blockIdx.x * kHoRows<P> + i, F = (int64_t)blockIdx.x * kHoFacets<P> + i / NB;
-  const bool act = i < kHoRows<P> && row < (ZERO ? g.NH : TT);
-  T r = (T)0;
+  __shared__ __align__(16) T sf[AHEAD ? NB * STEP : 1];   // the rows of omega D_F^-1, copied behind the products
+  __shared__ __align__(16) T ss[ZERO ? 1 : NB * STEP];
+  const int i0 = threadIdx.x * R, n = i0 % NB;
+  const int64_t row = (int64_t)blockIdx.x * kHoRows<P> + i0, F = (int64_t)blockIdx.x * kHoFacets<P> + i0 / NB;
+  const bool act = i0 < kHoRows<P> && row < (ZERO ? g.NH : TT);
+  const T *f = hw + (int64_t)NB * NB * F + n;
+  T v[R];
   if (act) {
     if (AHEAD && F < g.nhf) {
-      const T *f = hw + (int64_t)NB * NB * F + n;
 #pragma unroll
-      for (int m = 0; m < NB; ++m) cp_async<sizeof(T)>(sf + m * kHoRowThreads + i, f + NB * m);
+      for (int m = 0; m < NB; ++m) ho_copy<R>(sf + m * STEP + i0, f + NB * m);
     }
-    r = (T)__ldg(b + row);
-    if constexpr (!ZERO) r = ho_row<P, true, true>(S, lam_in, g, TT, F, n, r, ss + i);
-    sr[i] = r;
+#pragma unroll
+    for (int r = 0; r < R; ++r) v[r] = (T)__ldg(b + row + r);
+    if constexpr (!ZERO) ho_row<P, true, true>(S, lam_in, g, TT, F, n, v, ss + i0);
+#pragma unroll
+    for (int r = 0; r < R; ++r) sr[i0 + r] = v[r];
   }
   __syncthreads();
   if (!act) return;
   if (F < g.nhf) {
-    const T *f = hw + (int64_t)NB * NB * F + n, *rf = sr + (i - n);
-    T v = ZERO ? (T)0 : (T)keep * (T)lam_in[row];
+    const T *rf = sr + (i0 - n);
+#pragma unroll
+    for (int r = 0; r < R; ++r) v[r] = ZERO ? (T)0 : (T)keep * (T)lam_in[row + r];
     if (AHEAD) {
       cp_async_commit();
       cp_async_wait<0>();
     }
 #pragma unroll
-    for (int m = 0; m < NB; ++m) v = fma(AHEAD ? sf[m * kHoRowThreads + i] : __ldg(f + NB * m), rf[m], v);
-    lam_out[row] = (Tout)v;
-  } else {
-    lam_out[row] = (Tout)r;
+    for (int m = 0; m < NB; ++m) {
+      T a[R];
+      if constexpr (AHEAD) ho_take<R>(a, sf + m * STEP + i0);
+      else
+#pragma unroll
+        for (int r = 0; r < R; ++r) a[r] = __ldg(f + NB * m + r);
+#pragma unroll
+      for (int r = 0; r < R; ++r) v[r] = fma(a[r], rf[m], v[r]);
+    }
   }
+#pragma unroll
+  for (int r = 0; r < R; ++r) lam_out[row + r] = (Tout)v[r];
 }
 
 // Part 2's ring of factor blocks: levels in flight and values per column of a slot (padded by NB, so that
@@ -709,16 +790,76 @@ __global__ void __launch_bounds__(64)
 // R = b - S lam (Algorithm 2 line 3), one thread per row. ZSWEEP: lam is one sweep from zero,
 // lam = omega D^-1 b, so R = (1 - omega) b - (S - D) lam (equal in exact arithmetic).
 template <int P, bool ZSWEEP, typename T = double>
-__global__ void __launch_bounds__(kHoRowThreads)
+__global__ void __launch_bounds__(kHoThreads<P, T>)
     ho_residual_kernel(const HoGeo g, int64_t TT, const T *__restrict__ S, const double *__restrict__ b,
-                       const T *__restrict__ lam, T *__restrict__ R, double keep) {
+                       const T *__restrict__ lam, T *__restrict__ R_out, double keep) {
+  constexpr int NB = Ho<P>::NB, R = kHoR<P, T>;
+  __shared__ __align__(16) T ss[NB * kHoThreads<P, T> * R];
+  const int i0 = threadIdx.x * R;
+  const int64_t row = (int64_t)blockIdx.x * kHoRows<P> + i0, F = (int64_t)blockIdx.x * kHoFacets<P> + i0 / NB;
+  if (i0 >= kHoRows<P> || row >= TT) return;
+  T v[R];
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    const T bv = (T)__ldg(b + row + r);
+    v[r] = ZSWEEP ? (T)keep * bv : bv;
+  }
+  ho_row<P, true, ZSWEEP>(S, lam, g, TT, F, i0 % NB, v, ss + i0);
+#pragma unroll
+  for (int r = 0; r < R; ++r) R_out[row + r] = v[r];
+}
+
+// Part 1 of a sweep and the residual in FP32 with a facet per thread (kHoFacetRows). The Jacobi step goes
+// through shared memory, a thread per row, so that the factors and the results are coalesced.
+template <int P, typename Tout>
+__global__ void __launch_bounds__(kHoRowThreads)
+    ho_sweep_facets_kernel(const HoGeo g, int64_t TT, const float *__restrict__ S, const float *__restrict__ hw,
+                           const double *__restrict__ b, const float *__restrict__ lam_in, Tout *__restrict__ lam_out,
+                           double keep) {
+  constexpr int NB = Ho<P>::NB, LD = NB | 1;
+  __shared__ float sr[kHoRowThreads * LD];
+  const int64_t F0 = (int64_t)blockIdx.x * kHoRowThreads, F = F0 + threadIdx.x, nF = g.nhf + g.nzf;
+  if (F < nF) {
+    float acc[NB];
+#pragma unroll
+    for (int n = 0; n < NB; ++n) acc[n] = (float)__ldg(b + NB * F + n);
+    ho_facet_rows<P, true>(S, lam_in, g, TT, F, acc);
+#pragma unroll
+    for (int n = 0; n < NB; ++n) sr[threadIdx.x * LD + n] = acc[n];
+  }
+  __syncthreads();
+  const int rows = NB * (int)min((int64_t)kHoRowThreads, nF - F0);
+  for (int e = threadIdx.x; e < rows; e += kHoRowThreads) {
+    const int f = e / NB, n = e - f * NB;
+    const float *rf = sr + f * LD;
+    const int64_t row = NB * F0 + e;
+    float v = rf[n];
+    if (F0 + f < g.nhf) {
+      const float *w = hw + (int64_t)NB * NB * (F0 + f) + n;
+      v = (float)keep * lam_in[row];
+#pragma unroll
+      for (int m = 0; m < NB; ++m) v = fmaf(__ldg(w + NB * m), rf[m], v);
+    }
+    lam_out[row] = (Tout)v;
+  }
+}
+
+template <int P, bool ZSWEEP>
+__global__ void __launch_bounds__(kHoRowThreads)
+    ho_residual_facets_kernel(const HoGeo g, int64_t TT, const float *__restrict__ S, const double *__restrict__ b,
+                              const float *__restrict__ lam, float *__restrict__ R, double keep) {
   constexpr int NB = Ho<P>::NB;
-  __shared__ T ss[NB * kHoRowThreads];
-  const int i = threadIdx.x;
-  const int64_t row = (int64_t)blockIdx.x * kHoRows<P> + i, F = (int64_t)blockIdx.x * kHoFacets<P> + i / NB;
-  if (i >= kHoRows<P> || row >= TT) return;
-  const T bv = (T)__ldg(b + row);
-  R[row] = ho_row<P, true, ZSWEEP>(S, lam, g, TT, F, i % NB, ZSWEEP ? (T)keep * bv : bv, ss + i);
+  const int64_t F = (int64_t)blockIdx.x * kHoRowThreads + threadIdx.x;
+  if (F >= g.nhf + g.nzf) return;
+  float acc[NB];
+#pragma unroll
+  for (int n = 0; n < NB; ++n) {
+    const float bv = (float)__ldg(b + NB * F + n);
+    acc[n] = ZSWEEP ? (float)keep * bv : bv;
+  }
+  ho_facet_rows<P, ZSWEEP>(S, lam, g, TT, F, acc);
+#pragma unroll
+  for (int n = 0; n < NB; ++n) R[NB * F + n] = acc[n];
 }
 
 // bbar_K = Gamma_K (P^T R)_K (Algorithm 2 lines 4-5): P is constant on a facet (all its nodes)
@@ -932,10 +1073,10 @@ static int ho_launch_spmv_p(Ctx *c, const double *x, double *y, int mode, const 
   const unsigned grid = grid_for(h.T, kHoRows<P>);
   Prof prof(c, kCompApply);
   switch (mode) {
-    case 0: ho_spmv_kernel<P, 0><<<grid, kHoRowThreads, 0, c->stream>>>(g, h.T, h.S, x, y, w, h.fs); break;
-    case 1: ho_spmv_kernel<P, 1><<<grid, kHoRowThreads, 0, c->stream>>>(g, h.T, h.S, x, y, w, h.fs); break;
-    case 2: ho_spmv_kernel<P, 2><<<grid, kHoRowThreads, 0, c->stream>>>(g, h.T, h.S, x, y, w, h.fs); break;
-    default: ho_spmv_kernel<P, 3><<<grid, kHoRowThreads, 0, c->stream>>>(g, h.T, h.S, x, y, w, h.fs); break;
+    case 0: ho_spmv_kernel<P, 0><<<grid, kHoThreads<P, double>, 0, c->stream>>>(g, h.T, h.S, x, y, w, h.fs); break;
+    case 1: ho_spmv_kernel<P, 1><<<grid, kHoThreads<P, double>, 0, c->stream>>>(g, h.T, h.S, x, y, w, h.fs); break;
+    case 2: ho_spmv_kernel<P, 2><<<grid, kHoThreads<P, double>, 0, c->stream>>>(g, h.T, h.S, x, y, w, h.fs); break;
+    default: ho_spmv_kernel<P, 3><<<grid, kHoThreads<P, double>, 0, c->stream>>>(g, h.T, h.S, x, y, w, h.fs); break;
   }
   const unsigned rg = grid_for(nF, 2048);
   if (mode == 2) ho_reduce_kernel<2><<<rg, 256, 0, c->stream>>>(h.fs, nF, slot0, slot1, c->part, c->counter, c->scal);
@@ -993,9 +1134,15 @@ static int ho_sweep(Ctx *c, const double *b, const Tin *lam_in, Tout *lam_out) {
   const size_t smem = sizeof(T) * (HoLines<P>::DEPTH * H::CPW * HoLines<P>::STRIDE + (size_t)H::NB * cpb * (g.L + 1));
   const double keep = 1.0 - h.factor_omega;
   Prof prof(c, ZERO ? kCompPresmooth : kCompSweep, 2);
-  ho_sweep_rows_kernel<P, ZERO, T, double, Tin, Tout>
-      <<<grid_for(ZERO ? g.NH : h.T, kHoRows<P>), kHoRowThreads, 0, c->stream>>>(
+  if constexpr (!ZERO && sizeof(T) == 4) {
+    if (h.T >= kHoFacetRows)
+      ho_sweep_facets_kernel<P, Tout><<<grid_for(g.nhf + g.nzf, kHoRowThreads), kHoRowThreads, 0, c->stream>>>(
           g, h.T, HoPrec<T>::S(h), HoPrec<T>::hw(h), b, lam_in, lam_out, keep);
+  }
+  if (ZERO || sizeof(T) == 8 || h.T < kHoFacetRows)
+    ho_sweep_rows_kernel<P, ZERO, T, double, Tin, Tout>
+        <<<grid_for(ZERO ? g.NH : h.T, kHoRows<P>), ZERO ? kHoRowThreads : kHoThreads<P, T>, 0, c->stream>>>(
+            g, h.T, HoPrec<T>::S(h), HoPrec<T>::hw(h), b, lam_in, lam_out, keep);
   auto lines = [&](auto kern, const auto *src) {
     const cudaError_t e = smem > 48 * 1024 ? cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)
                                            : cudaSuccess;
@@ -1069,12 +1216,19 @@ static int ho_precond_p(Ctx *c, const double *r, double *z) {
   T *cb = static_cast<T *>(c->cb);
   {
     Prof pr(c, kCompResidual, 2);
-    if (c->opt.n_pre == 1)   // w1 is one sweep from zero                                       // line 3
-      ho_residual_kernel<P, true, T><<<grid_for(TT, kHoRows<P>), kHoRowThreads, 0, c->stream>>>(
-          g, TT, HoPrec<T>::S(h), r, w1, w2, 1.0 - h.factor_omega);
-    else
-      ho_residual_kernel<P, false, T><<<grid_for(TT, kHoRows<P>), kHoRowThreads, 0, c->stream>>>(
-          g, TT, HoPrec<T>::S(h), r, w1, w2, 0.0);
+    const bool zsweep = c->opt.n_pre == 1;   // w1 is one sweep from zero                       // line 3
+    const double rkeep = zsweep ? 1.0 - h.factor_omega : 0.0;
+    bool done = false;
+    if constexpr (sizeof(T) == 4) {
+      if ((done = h.T >= kHoFacetRows)) {
+        auto k = zsweep ? ho_residual_facets_kernel<P, true> : ho_residual_facets_kernel<P, false>;
+        k<<<grid_for(g.nhf + g.nzf, kHoRowThreads), kHoRowThreads, 0, c->stream>>>(g, TT, HoPrec<T>::S(h), r, w1, w2, rkeep);
+      }
+    }
+    if (!done) {
+      auto k = zsweep ? ho_residual_kernel<P, true, T> : ho_residual_kernel<P, false, T>;
+      k<<<grid_for(TT, kHoRows<P>), kHoThreads<P, T>, 0, c->stream>>>(g, TT, HoPrec<T>::S(h), r, w1, w2, rkeep);
+    }
     ho_restrict_kernel<P, T><<<grid_for(C, 64), 64, 0, c->stream>>>(g, C, w2, HoPrec<T>::gamma(h), cb);   // lines 4-5
     HMG_CUDA(c, cudaGetLastError());
   }

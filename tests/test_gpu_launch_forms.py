@@ -116,3 +116,19 @@ def test_degree_p_line_solves_beyond_the_ring(p, n, nlev):
         assert (z32 - z).abs().max() <= 1e-4 * z.abs().max()
     finally:
         s.close()
+
+
+@pytest.mark.parametrize("p,n,nlev", [(1, 64, 24), (2, 44, 20), (3, 30, 26)])
+def test_degree_p_fp32_facet_form_on_large_meshes(p, n, nlev):
+    """Meshes above the 2^20 rows from which the FP32 rows take a facet per thread, the last block of
+    facets ragged: one preconditioner call against the FP64 one, the bound of the test above."""
+    w = I.planar_helmholtz(n=n, nlev=nlev, nmg=2)
+    s = _solver(w, tol=1e-8, degree=p)
+    try:
+        assert s.ntrace >= 1 << 20
+        r = _cuda(np.random.default_rng(9).standard_normal(s.ntrace))
+        z = s.precond(r)
+        s.set_options(precision="mixed")
+        assert (s.precond(r) - z).abs().max() <= 1e-4 * z.abs().max()
+    finally:
+        s.close()
