@@ -25,11 +25,10 @@
 
 namespace hmg {
 
-// Threads of the row kernels: one thread per trace row, whole facets per block (p = 2: 28 facets of nine
-// rows). A row's S coefficients are one value per slot, so the lanes of a warp read consecutive
-// addresses, and the NB rows of a facet read the same x value. One thread per facet with NB
-// accumulators instead spread a warp's loads over 32 lines and left most of the GPU idle on small
-// meshes (16 x 16 x 16 cells at p = 3: 49 blocks on 152 SMs, S apply 266 us).
+// The row kernels take whole facets per block (p = 2: 28 facets of nine rows) and a few rows of one facet
+// per thread: the lanes of a warp read consecutive coefficients of a slot, and the rows of a facet share
+// its x values. One thread per facet with NB accumulators leaves most of the GPU idle on small meshes (16 x
+// 16 x 16 cells at p = 3: 49 blocks on 152 SMs, S apply 266 us); on large ones FP32 takes it (below).
 constexpr int kHoRowThreads = 256;
 template <int P>
 constexpr int kHoFacets = kHoRowThreads / Ho<P>::NB;   // facets per block
