@@ -985,6 +985,7 @@ static int ho_build_fp32(Ctx *c) {
 
 void ho_free(Ctx *c) {
   HoData &h = c->ho;
+  if (h.tab) drop_graph(c);   // captured launches hold these buffers (tab is the first of them to be made)
   double **bufs[] = {&h.tab, &h.gtab, &h.ctab, &h.ltab, &h.S, &h.Ainv, &h.hw, &h.zf, &h.gamma, &h.m, &h.fs};
   for (double **b : bufs) {
     dev_free(c, *b);

@@ -453,8 +453,9 @@ void drop_graph(Ctx *c) {
   drop_batch_graph(c);
 }
 
-// The graph of the loop depends on the options only: a caller's new vectors do not rebuild it (capturing
-// and instantiating it again took 0.18 ms, a fifth of a small solve).
+// The graph of the loop holds the context's buffers and the options it was captured with, no vector of the
+// caller's: new vectors do not rebuild it (capturing and instantiating it again took 0.18 ms, a fifth of a
+// small solve). Whatever frees or replaces one of those buffers calls drop_graph.
 static int ensure_solve_graph(Ctx *c) {
   if (c->graph_exec && std::memcmp(&c->graph_opt, &c->opt, sizeof(c->opt)) == 0) return HMG_OK;
   drop_graph(c);
