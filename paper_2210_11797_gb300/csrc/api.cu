@@ -376,6 +376,7 @@ int hmg_assemble_trace(hmg_ctx *c) {
   const bool need_fp32 = c->opt.precision == HMG_PRECISION_MIXED;
   if (!c->have_mesh || !c->have_coeffs) return fail(c, HMG_ERR_NOT_READY, "mesh or coefficients not set");
   if (c->have_fp32 && need_fp32) c->have_fp32 = false;  // rebuild copies from fresh FP64 data
+  c->assembled = false;   // until all of it is there: a failure below leaves operators and workspace in part
   int st;
   const Level &f = c->lv[0];
   const int64_t T = f.ntrace, C = f.ncell;
@@ -387,24 +388,30 @@ int hmg_assemble_trace(hmg_ctx *c) {
   const int64_t nhost = std::max(7 * C + T, T1 ? (int64_t)(cell_nu_of(c->opt.degree) + cell_np_of(c->opt.degree)) * C + T1 : 0);
   if (c->vec_cap < nvec) {
     double **vecs[] = {&c->B, &c->r, &c->rhat, &c->p, &c->v, &c->s, &c->t, &c->phat, &c->shat};
+    drop_graph(c);   // a cached solve graph holds the old vectors
+    c->vec_cap = 0;
     for (double **v : vecs) {
       dev_free(c, *v);
       *v = nullptr;
-      if ((st = dev_alloc(c, v, (size_t)nvec))) return st;
     }
+    for (double **v : vecs)
+      if ((st = dev_alloc(c, v, (size_t)nvec))) return st;
     c->vec_cap = nvec;
-    drop_graph(c);   // a cached solve graph holds the old vectors
   }
   if (c->work_cap < nwork) {
     void **ws[] = {&c->w1, &c->w2, &c->w3};
+    drop_graph(c);
+    c->work_cap = 0;
     for (void **w : ws) {
       dev_free(c, *w);
+      *w = nullptr;
+    }
+    for (void **w : ws) {
       double *tmp = nullptr;
       if ((st = dev_alloc(c, &tmp, (size_t)nwork))) return st;
       *w = tmp;
     }
     c->work_cap = nwork;
-    drop_graph(c);
   }
   if ((st = assemble_all(c))) return st;   // its per-cell data passes through the Krylov vectors
   if (!c->cb) {
@@ -415,6 +422,7 @@ int hmg_assemble_trace(hmg_ctx *c) {
   if (c->host_cap < nhost) {
     dev_free(c, c->host_in);
     c->host_in = nullptr;
+    c->host_cap = 0;
     if ((st = dev_alloc(c, &c->host_in, (size_t)nhost))) return st;
     c->host_cap = nhost;
   }
@@ -719,7 +727,7 @@ int hmg_get_coarse_model(hmg_ctx *c, float *params, int32_t n) {
   int st = mesh_ready(c);
   if (st) return st;
   if (!params || n != kCoarseParams) return fail(c, HMG_ERR_INVALID_ARG, "params must hold hmg_coarse_model_size() floats");
-  if (!c->nn_w) return fail(c, HMG_ERR_NOT_READY, "no coarse model set");
+  if (!c->nn_diag) return fail(c, HMG_ERR_NOT_READY, "no coarse model set");
   HMG_CUDA(c, cudaMemcpyAsync(params, c->nn_w, sizeof(float) * kCoarseParams, cudaMemcpyDeviceToHost, c->stream));
   return finish(c, HMG_OK);
 }
@@ -728,7 +736,7 @@ int hmg_apply_coarse_model(hmg_ctx *c, const double *bbar, double *out, int32_t 
   int st = ready(c);
   if (st) return st;
   if (!bbar || !out || bbar == out || mode < 0 || mode > 2) return fail(c, HMG_ERR_INVALID_ARG, "bad arguments");
-  if (!c->nn_w) return fail(c, HMG_ERR_NOT_READY, "no coarse model set");
+  if (!c->nn_diag) return fail(c, HMG_ERR_NOT_READY, "no coarse model set");
   if ((st = finish(c, apply_coarse_model(c, bbar, out, mode)))) return st;
   st = check_wait_flag(c);
   if (st == HMG_ERR_TIMEOUT && mode == 0 && !c->nn_tc_off) {   // see hmg_apply_coarse_model
@@ -742,7 +750,7 @@ static int check_patches(hmg_ctx *c, const float *x, const float *t, int32_t nsa
   if (!x || !t) return fail(c, HMG_ERR_INVALID_ARG, "null pointer");
   if (nsamp < 1 || nx < 1 || ny < 1 || (int64_t)nsamp * nx * ny > (1 << 26))
     return fail(c, HMG_ERR_INVALID_ARG, "bad patch batch shape");
-  if (!c->nn_w) return fail(c, HMG_ERR_NOT_READY, "no coarse model set");
+  if (!c->nn_diag) return fail(c, HMG_ERR_NOT_READY, "no coarse model set");
   return HMG_OK;
 }
 

@@ -938,35 +938,31 @@ static int assemble_levels(Ctx *c, double *rec) {
   Level &f = c->lv[0];
   const int64_t C = f.ncell, T = f.ntrace;
   int st;
-  if (!c->S) {
-    if ((st = dev_alloc(c, &c->S, (size_t)kSlots * T))) return st;
-    if ((st = dev_alloc(c, &c->Sz_w, (size_t)f.ntz))) return st;
-    if ((st = dev_alloc(c, &c->Sz_l, (size_t)f.ntz))) return st;
-    if ((st = dev_alloc(c, &c->Sz_cp, (size_t)f.ntz))) return st;
-    if ((st = dev_alloc(c, &c->Sh_w, (size_t)f.nth))) return st;
-    if ((st = dev_alloc(c, &c->Ainv, (size_t)49 * C))) return st;
-    if ((st = dev_alloc(c, &c->kth, (size_t)6 * C))) return st;
-    if ((st = dev_alloc(c, &c->gamma, (size_t)C))) return st;
-    if ((st = dev_alloc(c, &c->asm_flag, 1))) return st;
-  }
+  if ((st = dev_make(c, &c->S, (size_t)kSlots * T))) return st;
+  if ((st = dev_make(c, &c->Sz_w, (size_t)f.ntz))) return st;
+  if ((st = dev_make(c, &c->Sz_l, (size_t)f.ntz))) return st;
+  if ((st = dev_make(c, &c->Sz_cp, (size_t)f.ntz))) return st;
+  if ((st = dev_make(c, &c->Sh_w, (size_t)f.nth))) return st;
+  if ((st = dev_make(c, &c->Ainv, (size_t)49 * C))) return st;
+  if ((st = dev_make(c, &c->kth, (size_t)6 * C))) return st;
+  if ((st = dev_make(c, &c->gamma, (size_t)C))) return st;
+  if ((st = dev_make(c, &c->asm_flag, 1))) return st;
   HMG_CUDA(c, cudaMemsetAsync(c->asm_flag, 0, sizeof(int), c->stream));
   for (int l = 0; l < c->nmg; ++l) {
     Level &lv = c->lv[l];
     const CellArgs a{lv.geometry, lv.ncol, lv.nlev, lv.ncell, lv.radius, lv.corners, lv.z,
                      lv.theta_lev, lv.exner_lev, lv.exner, lv.col_nbr, c->sc};
     if (!lv.geo_ready) {   // the sums depend on the mesh only, which a context keeps
-      if (!lv.ctab && (st = dev_alloc(c, &lv.ctab, (size_t)Col::N * lv.ncol))) return st;
-      if (!lv.ltab && (st = dev_alloc(c, &lv.ltab, (size_t)Lev::N * lv.nlev))) return st;
+      if ((st = dev_make(c, &lv.ctab, (size_t)Col::N * lv.ncol))) return st;
+      if ((st = dev_make(c, &lv.ltab, (size_t)Lev::N * lv.nlev))) return st;
       column_kernel<<<grid_for(lv.ncol, 64) + grid_for(lv.nlev, 64), 64, 0, c->stream>>>(a, lv.ctab, lv.ltab);
       HMG_CUDA(c, cudaGetLastError());
       lv.geo_ready = true;
     }
-    if (!lv.H) {
-      if ((st = dev_alloc(c, &lv.H, (size_t)kHCoef * lv.ncell))) return st;
-      if ((st = dev_alloc(c, &lv.Hz_w, (size_t)lv.ncell))) return st;
-      if ((st = dev_alloc(c, &lv.Hz_l, (size_t)lv.ncell))) return st;
-      if ((st = dev_alloc(c, &lv.Hz_cp, (size_t)lv.ncell))) return st;
-    }
+    if ((st = dev_make(c, &lv.H, (size_t)kHCoef * lv.ncell))) return st;
+    if ((st = dev_make(c, &lv.Hz_w, (size_t)lv.ncell))) return st;
+    if ((st = dev_make(c, &lv.Hz_l, (size_t)lv.ncell))) return st;
+    if ((st = dev_make(c, &lv.Hz_cp, (size_t)lv.ncell))) return st;
     const CellOut q = cell_buffers(c, l);
     if (rec) {
       if ((st = gauss_cells(c, a, q, rec, l == 0 ? c->Ainv : nullptr))) return st;

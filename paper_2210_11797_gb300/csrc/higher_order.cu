@@ -946,7 +946,7 @@ static int ho_build_factors(Ctx *c) {
   ho_zfactor_kernel<P><<<grid_for(g.ncol, kHoFacWarps), 32 * kHoFacWarps, zsmem, c->stream>>>(
       g, h.T, h.S, c->opt.omega, h.zf, sing);
   HMG_CUDA(c, cudaGetLastError());
-  if (h.S32) {   // the FP32 preconditioner's copies of the factors follow them
+  if (h.gamma32) {   // the FP32 preconditioner's copies of the factors follow them (gamma32: the last made)
     const int64_t nh = (int64_t)NB * NB * g.nhf, nz = (int64_t)3 * NB * NB * g.nzf;
     ho_convert_kernel<double, float><<<grid_for(nh, 256), 256, 0, c->stream>>>(h.hw, h.hw32, nh);
     ho_convert_kernel<double, float><<<grid_for(nz, 256), 256, 0, c->stream>>>(h.zf, h.zf32, nz);
@@ -969,12 +969,10 @@ static int ho_build_fp32(Ctx *c) {
   const int64_t C = c->lv[0].ncell, nS = (int64_t)H::SLOTS * h.T;
   const int64_t nh = (int64_t)H::NB * H::NB * g.nhf, nz = (int64_t)3 * H::NB * H::NB * g.nzf;
   int st;
-  if (!h.S32) {
-    if ((st = dev_alloc(c, &h.S32, (size_t)nS))) return st;
-    if ((st = dev_alloc(c, &h.hw32, (size_t)nh))) return st;
-    if ((st = dev_alloc(c, &h.zf32, (size_t)nz))) return st;
-    if ((st = dev_alloc(c, &h.gamma32, (size_t)C))) return st;
-  }
+  if ((st = dev_make(c, &h.S32, (size_t)nS))) return st;
+  if ((st = dev_make(c, &h.hw32, (size_t)nh))) return st;
+  if ((st = dev_make(c, &h.zf32, (size_t)nz))) return st;
+  if ((st = dev_make(c, &h.gamma32, (size_t)C))) return st;
   ho_convert_kernel<double, float><<<grid_for(nS, 256), 256, 0, c->stream>>>(h.S, h.S32, nS);
   ho_convert_kernel<double, float><<<grid_for(nh, 256), 256, 0, c->stream>>>(h.hw, h.hw32, nh);
   ho_convert_kernel<double, float><<<grid_for(nz, 256), 256, 0, c->stream>>>(h.zf, h.zf32, nz);
@@ -1181,7 +1179,7 @@ static int ho_precond_p(Ctx *c, const double *r, double *z) {
   const HoGeo g = ho_geo<P>(c);
   const int64_t TT = h.T, C = c->lv[0].ncell;
   int st;
-  if (!HoPrec<T>::S(h)) return fail(c, HMG_ERR_NOT_READY, "the FP32 copies of the degree-p operator are missing");
+  if (!HoPrec<T>::gamma(h)) return fail(c, HMG_ERR_NOT_READY, "the FP32 copies of the degree-p operator are missing");
   T *w1 = static_cast<T *>(c->w1), *w2 = static_cast<T *>(c->w2), *w3 = static_cast<T *>(c->w3);
   if (c->opt.precond == HMG_PRECOND_NONE) {
     HMG_CUDA(c, cudaMemcpyAsync(z, r, sizeof(double) * TT, cudaMemcpyDeviceToDevice, c->stream));
@@ -1272,7 +1270,7 @@ int ho_assemble(Ctx *c) {
 }
 
 int ho_refactor_if_needed(Ctx *c) {
-  if (c->opt.precision == HMG_PRECISION_MIXED && !c->ho.S32) {   // switched to the FP32 preconditioner
+  if (c->opt.precision == HMG_PRECISION_MIXED && !c->ho.gamma32) {   // switched to the FP32 preconditioner
     int st = HMG_OK;
     switch (c->degree) {
       case 1: st = ho_build_fp32<1>(c); break;

@@ -254,11 +254,18 @@ int dev_alloc(Ctx *c, T **p, size_t n) {
   cudaError_t e = cudaMalloc(&q, n * sizeof(T) > 0 ? n * sizeof(T) : 16);
   if (e != cudaSuccess) {
     *p = nullptr;
+    cudaGetLastError();   // reported here: the next launch check must not find it
     return fail(c, HMG_ERR_OUT_OF_MEMORY, std::string("cudaMalloc: ") + cudaGetErrorString(e));
   }
   c->owned.push_back(q);
   *p = static_cast<T *>(q);
   return HMG_OK;
+}
+
+// The same where *p is not there yet (a group of buffers made this way can be completed after one failed).
+template <typename T>
+int dev_make(Ctx *c, T **p, size_t n) {
+  return *p ? HMG_OK : dev_alloc(c, p, n);
 }
 
 // Releases one device allocation of the context (and forgets it).

@@ -823,11 +823,9 @@ static int gm_buffers(Ctx *c, int m) {
   int s;
   if ((s = dev_alloc(c, &c->gm_V, (size_t)(m + 1) * n))) return s;
   if ((s = dev_alloc(c, &c->gm_Z, (size_t)m * n))) return s;
-  if (!c->gm_h) {
-    if ((s = dev_alloc(c, &c->gm_h, (size_t)3 * (kMaxRestart + 2)))) return s;
-    if ((s = dev_alloc(c, &c->gm_part, (size_t)(kMaxRestart + 1) * kGmBlocks))) return s;
-    if ((s = dev_alloc(c, &c->gm_y, (size_t)kMaxRestart))) return s;
-  }
+  if ((s = dev_make(c, &c->gm_h, (size_t)3 * (kMaxRestart + 2)))) return s;
+  if ((s = dev_make(c, &c->gm_part, (size_t)(kMaxRestart + 1) * kGmBlocks))) return s;
+  if ((s = dev_make(c, &c->gm_y, (size_t)kMaxRestart))) return s;
   c->gm_restart = m;
   c->gm_n = n;
   return HMG_OK;

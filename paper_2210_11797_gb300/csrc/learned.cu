@@ -1235,7 +1235,7 @@ int nn_pack_weights(Ctx *c) {
 // dPi = D^-1/2 f(D^-1/2 bbar) on the finest mesh, in the preconditioner's precision.
 template <typename T>
 int learned_coarse(Ctx *c, const T *bbar, T *out) {
-  if (!c->nn_w) return fail(c, HMG_ERR_NOT_READY, "no coarse model set");
+  if (!c->nn_diag) return fail(c, HMG_ERR_NOT_READY, "no coarse model set");
   const double *dH = nullptr;
   const float *dH32 = nullptr;
   if (sizeof(T) == 8) dH = c->lv[0].H; else dH32 = c->lv[0].H32;   // row 0 of H = its diagonal
@@ -1247,7 +1247,7 @@ template int learned_coarse<double>(Ctx *, const double *, double *);
 template int learned_coarse<float>(Ctx *, const float *, float *);
 
 int nn_setup(Ctx *c) {
-  if (c->nn_w) return HMG_OK;
+  if (c->nn_diag) return HMG_OK;   // (the last of its buffers)
   const Level &f = c->lv[0];
   if (f.nlev > kMaxL) return fail(c, HMG_ERR_INVALID_ARG, "the network kernels take at most 128 levels");
   int st;
@@ -1262,17 +1262,10 @@ int nn_setup(Ctx *c) {
                                    kTcSmem));
   HMG_CUDA(c, cudaFuncSetAttribute(nn_bwd1_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kBwSmem));
   HMG_CUDA(c, cudaFuncSetAttribute(nn_bwd1_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024));
-  if ((st = dev_alloc(c, &c->nn_w, kNParams))) return st;
-  {
-    __nv_bfloat16 *bimg;
-    if ((st = dev_alloc(c, &bimg, (size_t)32 * 96))) return st;   // cudaMalloc: 256-B aligned
-    c->nn_bimg = bimg;
-    if ((st = dev_alloc(c, &bimg, (size_t)32 * 96))) return st;
-    c->nn_bimg_t = bimg;
-  }
-  float *tmp;
-  if ((st = dev_alloc(c, &tmp, (size_t)kCh * f.ncell))) return st;   // BF16 h2 fits in half
-  c->nn_act = tmp;
+  if ((st = dev_make(c, &c->nn_w, kNParams))) return st;
+  for (void **image : {&c->nn_bimg, &c->nn_bimg_t})
+    if ((st = dev_make(c, reinterpret_cast<__nv_bfloat16 **>(image), (size_t)32 * 96))) return st;   // cudaMalloc: 256-B aligned
+  if ((st = dev_make(c, reinterpret_cast<float **>(&c->nn_act), (size_t)kCh * f.ncell))) return st;   // BF16 h2 fits in half
   // corner neighbours: across face f to n, then across the face of n after the shared one
   std::vector<int32_t> nbr(4 * (size_t)f.ncol), nbf(4 * (size_t)f.ncol), diag(4 * (size_t)f.ncol);
   HMG_CUDA(c, cudaMemcpy(nbr.data(), f.col_nbr, nbr.size() * 4, cudaMemcpyDeviceToHost));
@@ -1354,39 +1347,34 @@ int train_buffers(Ctx *c, int64_t cells, int nblocks_max) {
   TrainBufs &tb = c->train;
   int st;
   if (tb.cap_cells < cells) {
-    void **acts[] = {&tb.h1, &tb.h2};
-    for (void **a : acts) {   // storage for FP32 activations (BF16 uses half of it)
-      dev_free(c, *a);
-      float *f;
-      if ((st = dev_alloc(c, &f, (size_t)kCh * cells))) return st;
-      *a = f;
+    // (h1, h2: storage for FP32 activations, BF16 uses half of it)
+    float **bufs[] = {reinterpret_cast<float **>(&tb.h1), reinterpret_cast<float **>(&tb.h2), &tb.ga3, &tb.ga2};
+    tb.cap_cells = 0;
+    for (float **b : bufs) {
+      dev_free(c, *b);
+      *b = nullptr;
     }
-    float **grads[] = {&tb.ga3, &tb.ga2};
-    for (float **g : grads) {
-      dev_free(c, *g);
-      if ((st = dev_alloc(c, g, (size_t)kCh * cells))) return st;
-    }
+    for (float **b : bufs)
+      if ((st = dev_alloc(c, b, (size_t)kCh * cells))) return st;
     tb.cap_cells = cells;
   }
   if (tb.cap_blocks < nblocks_max) {
+    float **parts[] = {&tb.part3, &tb.partM, &tb.part1, &tb.part2};
+    tb.cap_blocks = 0;
     dev_free(c, tb.loss_part);
-    if ((st = dev_alloc(c, &tb.loss_part, (size_t)nblocks_max))) return st;
-    float **parts[] = {&tb.part3, &tb.partM, &tb.part1};
+    tb.loss_part = nullptr;
     for (float **q : parts) {
       dev_free(c, *q);
-      if ((st = dev_alloc(c, q, (size_t)nblocks_max * 96))) return st;
+      *q = nullptr;
     }
-    dev_free(c, tb.part2);
-    if ((st = dev_alloc(c, &tb.part2, (size_t)nblocks_max * 3072))) return st;
+    if ((st = dev_alloc(c, &tb.loss_part, (size_t)nblocks_max))) return st;
+    for (float **q : parts)
+      if ((st = dev_alloc(c, q, (size_t)nblocks_max * (q == &tb.part2 ? 3072 : 96)))) return st;
     tb.cap_blocks = nblocks_max;
   }
-  if (!tb.grad) {
-    if ((st = dev_alloc(c, &tb.grad, (size_t)kNParams))) return st;
-    if ((st = dev_alloc(c, &tb.m, (size_t)kNParams))) return st;
-    if ((st = dev_alloc(c, &tb.v, (size_t)kNParams))) return st;
-    if ((st = dev_alloc(c, &tb.loss, 1))) return st;
-  }
-  return HMG_OK;
+  for (float **p : {&tb.grad, &tb.m, &tb.v})
+    if ((st = dev_make(c, p, (size_t)kNParams))) return st;
+  return dev_make(c, &tb.loss, 1);
 }
 
 int coarse_model_grad(Ctx *c, const float *x, const float *t, int nsamp, int nx, int ny, int fp32,
@@ -1524,10 +1512,8 @@ int collect_pair(Ctx *c, const double *bbar) {
   const Level &f = c->lv[0];
   const int64_t C = f.ncell;
   int st;
-  if (!c->collect_r) {
-    if ((st = dev_alloc(c, &c->collect_r, (size_t)C))) return st;
-    if ((st = dev_alloc(c, &c->collect_y, (size_t)C))) return st;
-  }
+  if ((st = dev_make(c, &c->collect_r, (size_t)C))) return st;
+  if ((st = dev_make(c, &c->collect_y, (size_t)C))) return st;
   const double *dH = f.H;   // row 0 of H: its diagonal
   scale_to_float_kernel<<<grid_for(C, 256), 256, 0, c->stream>>>(bbar, dH, false, c->collect_x + c->collect_n * C, C);
   HMG_CUDA(c, cudaMemsetAsync(c->collect_y, 0, sizeof(double) * C, c->stream));

@@ -257,14 +257,12 @@ int build_mixed(Ctx *c, const double *rec0) {
   const Level &f = c->lv[0];
   const int64_t T = f.ntrace, C = f.ncell;
   int st;
-  if (!c->mx_Mu) {
-    if ((st = dev_alloc(c, &c->mx_Mu, (size_t)kSlots * T))) return st;
-    if ((st = dev_alloc(c, &c->mx_Gx, (size_t)2 * T))) return st;
-    if ((st = dev_alloc(c, &c->mx_Bx, (size_t)7 * C))) return st;
-    if ((st = dev_alloc(c, &c->mx_ilump, (size_t)T))) return st;
-    if ((st = dev_alloc(c, &c->mx_x, (size_t)(T + C)))) return st;
-    if ((st = dev_alloc(c, &c->mx_bp, (size_t)C))) return st;
-  }
+  if ((st = dev_make(c, &c->mx_Mu, (size_t)kSlots * T))) return st;
+  if ((st = dev_make(c, &c->mx_Gx, (size_t)2 * T))) return st;
+  if ((st = dev_make(c, &c->mx_Bx, (size_t)7 * C))) return st;
+  if ((st = dev_make(c, &c->mx_ilump, (size_t)T))) return st;
+  if ((st = dev_make(c, &c->mx_x, (size_t)(T + C)))) return st;
+  if ((st = dev_make(c, &c->mx_bp, (size_t)C))) return st;
   const MixedArgs a = mixed_args(c);
   mixed_rows_kernel<<<grid_for(T, 256), 256, 0, c->stream>>>(a, rec0, c->mx_Mu, c->mx_Gx, c->mx_ilump);
   mixed_cell_rows_kernel<<<grid_for(C, 256), 256, 0, c->stream>>>(a, rec0, c->mx_Bx);
