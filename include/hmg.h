@@ -214,12 +214,16 @@ int hmg_default_options(hmg_options *opt);
  * cuda_stream: a cudaStream_t owned by the caller (NULL = the legacy default stream). */
 int hmg_create(hmg_ctx **out, const hmg_options *opt, void *cuda_stream);
 
-/* Replace the options (e.g. the tolerance or a relaxation weight). On an assembled context, the first
- * switch to HMG_PRECISION_MIXED forms the operators again, by the direct Gauss sums that contexts
- * created with this precision use (equal to rounding, which the FP32 preconditioner amplifies), and
- * makes their FP32 copies (device memory for them is allocated here, once; synchronises; where the
- * sums' scratch does not fit, the copies are made from the operators there are). A change of degree
- * needs hmg_assemble_trace. */
+/* Replace the options (e.g. the tolerance or a relaxation weight). On a context assembled in FP64, the
+ * first switch to HMG_PRECISION_MIXED forms a second set of operators, by the direct Gauss sums that
+ * contexts created with this precision use (equal to rounding, which the FP32 preconditioner amplifies),
+ * with their FP32 copies. It takes as long as the assembly of such a context and as much device memory
+ * as the operators again; both sets are kept until the next hmg_assemble_trace, so that further switches
+ * cost nothing and FP64 results after a switch back are those from before it. Where the second set does
+ * not fit, the copies are made from the operators there are; where these do not fit either, the call
+ * returns HMG_ERR_OUT_OF_MEMORY. A context assembled with precision mixed keeps its operators in FP64.
+ * After an error the options are the ones from before the call. A change of degree needs
+ * hmg_assemble_trace. */
 int hmg_set_options(hmg_ctx *ctx, const hmg_options *opt);
 
 /* Set the mesh hierarchy: levels[0] finest ... levels[nmg-1] coarsest; every level has

@@ -5,8 +5,10 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <initializer_list>
 #include <new>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include <nvtx3/nvToolsExt.h>
@@ -88,6 +90,87 @@ Prof::~Prof() {
   if (e1 < 0) return;
   cudaEventRecord(c_->ev_pool[e1], c_->stream);
   c_->marks.push_back({comp_, e0_, e1, launches_});
+}
+
+// The operators and the set beside them exchanged. (Captured launches hold the set they were captured with.)
+static void swap_operators(Ctx *c) {
+  drop_graph(c);
+  std::swap(static_cast<OperatorSet &>(*c), c->other);
+  for (int l = 0; l < c->nmg; ++l) std::swap(static_cast<LevelOperators &>(c->lv[l]), c->other_lv[l]);
+}
+
+static void free_operators(Ctx *c) {
+  drop_graph(c);
+  ho_free(c);
+  auto release = [c](std::initializer_list<void *> ps) {
+    for (void *p : ps) dev_free(c, p);
+  };
+  release({c->S, c->Sz_w, c->Sz_l, c->Sz_cp, c->Sh_w, c->Ainv, c->kth, c->gamma});
+  release({c->S32, c->Sz_w32, c->Sz_l32, c->Sz_cp32, c->Sh_w32, c->gamma32});
+  static_cast<OperatorSet &>(*c) = OperatorSet{};
+  for (int l = 0; l < c->nmg; ++l) {
+    LevelOperators &o = c->lv[l];
+    release({o.H, o.Hz_w, o.Hz_l, o.Hz_cp, o.H32, o.Hz_w32, o.Hz_l32, o.Hz_cp32});
+    o = LevelOperators{};
+  }
+}
+
+static void free_other(Ctx *c) {
+  if (!c->have_other) return;
+  swap_operators(c);
+  free_operators(c);
+  swap_operators(c);
+  c->have_other = false;
+}
+
+static int assemble_operators(Ctx *c) {
+  int st;
+  c->have_fp32 = false;
+  if ((st = assemble_all(c))) return st;
+  if (c->degree >= 1 && (st = ho_assemble(c))) return st;
+  c->direct_sums = c->opt.precision == HMG_PRECISION_MIXED;
+  return HMG_OK;
+}
+
+// The operators in the form of the precision that was switched to. Contexts with the FP32 preconditioner
+// have the direct sums' (gauss_cells.cu says why), so the first switch to it forms these, beside the
+// others, which stay as they are: nothing is lost where it fails, and switching back gives the earlier
+// results, bit for bit. Where they do not fit, the preconditioner takes FP32 copies of the operators there
+// are (follow_options). Operators assembled by direct sums serve FP64 as well.
+static int switch_precision(Ctx *c) {
+  const bool mixed = c->opt.precision == HMG_PRECISION_MIXED;
+  if (mixed == c->direct_sums) return HMG_OK;
+  if (c->have_other) {
+    swap_operators(c);
+    return HMG_OK;
+  }
+  if (!mixed) return HMG_OK;
+  swap_operators(c);
+  const int st = assemble_operators(c);
+  c->have_other = true;
+  if (!st) return HMG_OK;
+  swap_operators(c);
+  free_other(c);
+  return st == HMG_ERR_OUT_OF_MEMORY ? HMG_OK : st;
+}
+
+static int follow_options(Ctx *c, const hmg_options &old) {
+  int st;
+  if (c->assembled && c->opt.degree != c->degree) c->assembled = false;   // a new discretisation
+  if (!c->assembled) return HMG_OK;
+  HMG_CUDA(c, cudaSetDevice(c->device));
+  if (c->opt.precision != old.precision && (st = switch_precision(c))) return st;
+  if (c->opt.precision == HMG_PRECISION_MIXED && !c->have_fp32) {
+    // the FP32 copies from the assembled FP64 operators (the degree-p ones below)
+    if ((st = make_fp32(c))) return st;
+    HMG_CUDA(c, cudaStreamSynchronize(c->stream));
+  }
+  if (c->opt.omega != c->factor_omega || c->opt.mg_omega != c->factor_mg_omega) {
+    if ((st = build_factors(c))) return st;
+    HMG_CUDA(c, cudaStreamSynchronize(c->stream));
+  }
+  // (outside any stream capture: the solve graph replays them)
+  return c->degree >= 1 ? ho_refactor_if_needed(c) : HMG_OK;
 }
 
 static void free_all(Ctx *c) {
@@ -198,30 +281,10 @@ int hmg_set_options(hmg_ctx *c, const hmg_options *opt) {
   if (!c || !opt) return HMG_ERR_INVALID_ARG;
   int st = check_options(c, *opt);
   if (st) return st;
+  const hmg_options old = c->opt;
   c->opt = *opt;
-  if (c->assembled && c->opt.degree != c->degree) c->assembled = false;   // a new discretisation
-  if (c->assembled && c->opt.precision == HMG_PRECISION_MIXED && !c->direct_sums) {
-    // the operators in the form that contexts created with this precision have (gauss_cells.cu says why);
-    // where their scratch does not fit any more, the FP32 copies of the operators there are
-    st = hmg_assemble_trace(c);
-    if (st != HMG_ERR_OUT_OF_MEMORY || c->degree != c->opt.degree) return st;
-  }
-  if (c->assembled && c->opt.precision == HMG_PRECISION_MIXED && !c->have_fp32) {
-    // the FP32 copies from the assembled FP64 operators (the degree-p ones below)
-    HMG_CUDA(c, cudaSetDevice(c->device));
-    if ((st = make_fp32(c))) return st;
-    HMG_CUDA(c, cudaStreamSynchronize(c->stream));
-  }
-  if (c->assembled && (c->opt.omega != c->factor_omega || c->opt.mg_omega != c->factor_mg_omega)) {
-    HMG_CUDA(c, cudaSetDevice(c->device));
-    if ((st = build_factors(c))) return st;
-    HMG_CUDA(c, cudaStreamSynchronize(c->stream));
-  }
-  if (c->assembled && c->degree >= 1) {   // (outside any stream capture: the solve graph replays them)
-    HMG_CUDA(c, cudaSetDevice(c->device));
-    if ((st = ho_refactor_if_needed(c))) return st;
-  }
-  return HMG_OK;
+  if ((st = follow_options(c, old))) c->opt = old;
+  return st;
 }
 
 int hmg_set_mesh(hmg_ctx *c, int32_t nmg, const hmg_mesh_level *levels) {
@@ -373,9 +436,8 @@ int hmg_set_coefficients(hmg_ctx *c, const hmg_scalars *sc, const hmg_background
 int hmg_assemble_trace(hmg_ctx *c) {
   if (!c) return HMG_ERR_INVALID_ARG;
   HMG_CUDA(c, cudaSetDevice(c->device));
-  const bool need_fp32 = c->opt.precision == HMG_PRECISION_MIXED;
   if (!c->have_mesh || !c->have_coeffs) return fail(c, HMG_ERR_NOT_READY, "mesh or coefficients not set");
-  if (c->have_fp32 && need_fp32) c->have_fp32 = false;  // rebuild copies from fresh FP64 data
+  free_other(c);
   c->assembled = false;   // until all of it is there: a failure below leaves operators and workspace in part
   int st;
   const Level &f = c->lv[0];
@@ -413,7 +475,6 @@ int hmg_assemble_trace(hmg_ctx *c) {
     }
     c->work_cap = nwork;
   }
-  if ((st = assemble_all(c))) return st;   // its per-cell data passes through the Krylov vectors
   if (!c->cb) {
     double *tmp;
     if ((st = dev_alloc(c, &tmp, (size_t)C))) return st;
@@ -427,14 +488,13 @@ int hmg_assemble_trace(hmg_ctx *c) {
     c->host_cap = nhost;
   }
   c->degree = c->opt.degree;
-  if (c->degree >= 1 && (st = ho_assemble(c))) {
+  if ((st = assemble_operators(c))) {   // (its per-cell data passes through the Krylov vectors)
+    if (c->degree >= 1) ho_free(c);
     c->degree = 0;
-    ho_free(c);
     return st;
   }
   if (c->degree == 0 && c->ho.degree != 0) ho_free(c);   // the degree-p system is no longer in use
   if (!c->noalloc_scratch && (st = noalloc_setup(c))) return st;
-  c->direct_sums = need_fp32;
   c->assembled = true;
   return HMG_OK;
 }

@@ -853,7 +853,7 @@ static int to_float(Ctx *c, const double *in, float **out, int64_t n) {
 
 // The FP32 preconditioner's copies of the assembled lowest-order operators (S, Gamma, H on every
 // level, then the factors with their copies through build_factors), made from the FP64 data on
-// the device when a context switches to precision mixed: no reassembly.
+// the device: for a context that switches to precision mixed without room for the direct sums' operators.
 int make_fp32(Ctx *c) {
   const Level &f = c->lv[0];
   int st;
@@ -864,7 +864,8 @@ int make_fp32(Ctx *c) {
     if ((st = to_float(c, lv.H, &lv.H32, (int64_t)kHCoef * lv.ncell))) return st;
   }
   c->have_fp32 = true;
-  return build_factors(c);
+  if ((st = build_factors(c))) c->have_fp32 = false;
+  return st;
 }
 
 // Relaxation-weighted Thomas factors of S^zz, 1/diag S^hh and H_z on every level for the

@@ -946,7 +946,7 @@ static int ho_build_factors(Ctx *c) {
   ho_zfactor_kernel<P><<<grid_for(g.ncol, kHoFacWarps), 32 * kHoFacWarps, zsmem, c->stream>>>(
       g, h.T, h.S, c->opt.omega, h.zf, sing);
   HMG_CUDA(c, cudaGetLastError());
-  if (h.gamma32) {   // the FP32 preconditioner's copies of the factors follow them (gamma32: the last made)
+  if (h.have_fp32) {   // the FP32 preconditioner's copies of the factors follow them
     const int64_t nh = (int64_t)NB * NB * g.nhf, nz = (int64_t)3 * NB * NB * g.nzf;
     ho_convert_kernel<double, float><<<grid_for(nh, 256), 256, 0, c->stream>>>(h.hw, h.hw32, nh);
     ho_convert_kernel<double, float><<<grid_for(nz, 256), 256, 0, c->stream>>>(h.zf, h.zf32, nz);
@@ -978,6 +978,7 @@ static int ho_build_fp32(Ctx *c) {
   ho_convert_kernel<double, float><<<grid_for(nz, 256), 256, 0, c->stream>>>(h.zf, h.zf32, nz);
   ho_convert_kernel<double, float><<<grid_for(C, 256), 256, 0, c->stream>>>(h.gamma, h.gamma32, C);
   HMG_CUDA(c, cudaGetLastError());
+  h.have_fp32 = true;
   return HMG_OK;
 }
 
@@ -1000,6 +1001,7 @@ void ho_free(Ctx *c) {
     dev_free(c, *b);
     *b = nullptr;
   }
+  h.have_fp32 = false;
   h.degree = 0;
   h.ncell = 0;
   h.T = 0;
@@ -1033,6 +1035,7 @@ static int ho_assemble_p(Ctx *c) {
     h.T = T;
   }
   h.factor_omega = 0.0;
+  h.have_fp32 = false;
   HMG_CUDA(c, cudaMemsetAsync(h.own, 0, 4 * (size_t)f.ncol, c->stream));
   ho_own_kernel<<<grid_for(f.nedge, 256), 256, 0, c->stream>>>(f.edge_stencil, f.edge_fc, f.nedge, h.own);
   HMG_CUDA(c, cudaMemsetAsync(h.flag, 0, sizeof(int), c->stream));
@@ -1179,7 +1182,7 @@ static int ho_precond_p(Ctx *c, const double *r, double *z) {
   const HoGeo g = ho_geo<P>(c);
   const int64_t TT = h.T, C = c->lv[0].ncell;
   int st;
-  if (!HoPrec<T>::gamma(h)) return fail(c, HMG_ERR_NOT_READY, "the FP32 copies of the degree-p operator are missing");
+  if (sizeof(T) == 4 && !h.have_fp32) return fail(c, HMG_ERR_NOT_READY, "the FP32 copies of the degree-p operator are missing");
   T *w1 = static_cast<T *>(c->w1), *w2 = static_cast<T *>(c->w2), *w3 = static_cast<T *>(c->w3);
   if (c->opt.precond == HMG_PRECOND_NONE) {
     HMG_CUDA(c, cudaMemcpyAsync(z, r, sizeof(double) * TT, cudaMemcpyDeviceToDevice, c->stream));
@@ -1270,7 +1273,7 @@ int ho_assemble(Ctx *c) {
 }
 
 int ho_refactor_if_needed(Ctx *c) {
-  if (c->opt.precision == HMG_PRECISION_MIXED && !c->ho.gamma32) {   // switched to the FP32 preconditioner
+  if (c->opt.precision == HMG_PRECISION_MIXED && !c->ho.have_fp32) {   // switched to the FP32 preconditioner
     int st = HMG_OK;
     switch (c->degree) {
       case 1: st = ho_build_fp32<1>(c); break;

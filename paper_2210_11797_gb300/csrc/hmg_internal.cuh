@@ -45,7 +45,16 @@ struct Scal {
 };
 
 // Device-side description of one multigrid level.
-struct Level {
+// The assembled pressure operator of one level (device).
+struct LevelOperators {
+  double *H = nullptr;              // [7][ncell]
+  // Thomas factors of H_z with the relaxation mg_omega folded in (pivot p_k): omega / p_k,
+  // sub_k / p_k and sup_k / p_k, [ncell] each
+  double *Hz_w = nullptr, *Hz_l = nullptr, *Hz_cp = nullptr;
+  float *H32 = nullptr, *Hz_w32 = nullptr, *Hz_l32 = nullptr, *Hz_cp32 = nullptr;
+};
+
+struct Level : LevelOperators {
   int geometry = 0;
   int ncol = 0, nlev = 0, nedge = 0;
   int64_t ncell = 0, nth = 0, ntz = 0, ntrace = 0;
@@ -63,12 +72,6 @@ struct Level {
   double *theta_lev = nullptr, *exner_lev = nullptr, *exner = nullptr;
   double *ctab = nullptr, *ltab = nullptr;   // geometry sums per column and per level (assembly)
   bool geo_ready = false;                    // they have been made (they depend on the mesh only)
-  // assembled pressure operator (device)
-  double *H = nullptr;              // [7][ncell]
-  // Thomas factors of H_z with the relaxation mg_omega folded in (pivot p_k): omega / p_k,
-  // sub_k / p_k and sup_k / p_k, [ncell] each
-  double *Hz_w = nullptr, *Hz_l = nullptr, *Hz_cp = nullptr;
-  float *H32 = nullptr, *Hz_w32 = nullptr, *Hz_l32 = nullptr, *Hz_cp32 = nullptr;
   // multigrid work vectors, sized for doubles (used as float in the mixed path)
   void *vb = nullptr, *vx = nullptr, *vy = nullptr;
 };
@@ -109,23 +112,11 @@ struct HoData {
   double factor_omega = 0.0;   // the omega the smoother factors hold
   // FP32 copies for the FP32 preconditioner (precision mixed): S, the smoother factors, Gamma
   float *S32 = nullptr, *hw32 = nullptr, *zf32 = nullptr, *gamma32 = nullptr;
+  bool have_fp32 = false;      // they are there and hold the present operators
 };
 
-// A process-wide counter: a context takes a new value when it is created and whenever its
-// captured launches go stale, so (context address, generation) never names two states.
-uint64_t next_graph_gen();
-
-struct Ctx {
-  int device = 0;
-  cudaStream_t stream = nullptr;
-  hmg_options opt{};
-  hmg_scalars sc{};
-  std::string err;
-  int nmg = 0;
-  Level lv[kMaxLevels];
-  bool have_mesh = false, have_coeffs = false, assembled = false, have_fp32 = false;
-  bool direct_sums = false;   // the operators come from direct Gauss sums (gauss_cells.cu)
-  int degree = 0;              // polynomial degree of the assembled system (0 .. 3)
+// What an assembly makes of the mesh and the coefficients (with the LevelOperators of every level).
+struct OperatorSet {
   HoData ho;
   // finest-level trace system (device)
   double *S = nullptr;        // [11][ntrace]
@@ -136,9 +127,32 @@ struct Ctx {
   double *Ainv = nullptr;     // [49][ncell] A_K^-1, entry (i, j) at (7 i + j) * ncell + K
   double *kth = nullptr;      // [6][ncell] diagonal of K_K (k theta on each local face)
   double *gamma = nullptr;    // [ncell]
-  int *asm_flag = nullptr;    // set by the assembly when a cell matrix is singular
   float *S32 = nullptr, *Sz_w32 = nullptr, *Sz_l32 = nullptr, *Sz_cp32 = nullptr, *Sh_w32 = nullptr,
         *gamma32 = nullptr;
+  bool have_fp32 = false;     // the FP32 copies are there and hold the present operators
+  bool direct_sums = false;   // the operators come from direct Gauss sums (gauss_cells.cu)
+};
+
+// A process-wide counter: a context takes a new value when it is created and whenever its
+// captured launches go stale, so (context address, generation) never names two states.
+uint64_t next_graph_gen();
+
+struct Ctx : OperatorSet {
+  int device = 0;
+  cudaStream_t stream = nullptr;
+  hmg_options opt{};
+  hmg_scalars sc{};
+  std::string err;
+  int nmg = 0;
+  Level lv[kMaxLevels];
+  bool have_mesh = false, have_coeffs = false, assembled = false;
+  int degree = 0;              // polynomial degree of the assembled system (0 .. 3)
+  int *asm_flag = nullptr;     // set by the assembly when a cell matrix is singular
+  // The same operators in the other precision's form, once the precision was switched after an assembly
+  // (have_other; until the next assembly): switching back exchanges the two.
+  OperatorSet other;
+  LevelOperators other_lv[kMaxLevels];
+  bool have_other = false;
   // Krylov workspace (FP64, [ntrace] each)
   double *B = nullptr, *r = nullptr, *rhat = nullptr, *p = nullptr, *v = nullptr,
          *s = nullptr, *t = nullptr, *phat = nullptr, *shat = nullptr;

@@ -266,11 +266,16 @@ class Solver:
         return self.torch.empty(n, dtype=self.torch.float64, device=self.device)
 
     def set_options(self, **kw):
+        old = Options.from_buffer_copy(self.opts)
         for k, v in kw.items():
             setattr(self.opts, k, _option_value(k, v))
-        # (hmg_set_options forms the operators again and makes their FP32 copies when the precision
-        # becomes mixed, and rebuilds the factors when a relaxation weight changes)
-        _check(self.ctx, lib().hmg_set_options(self.ctx, C.byref(self.opts)))
+        # (hmg_set_options forms a second set of operators with its FP32 copies when the precision of an
+        # FP64 context becomes mixed, and rebuilds the factors when a relaxation weight changes)
+        try:
+            _check(self.ctx, lib().hmg_set_options(self.ctx, C.byref(self.opts)))
+        except HmgError:   # the library has kept its options
+            self.opts = old
+            raise
         if self.opts.precision == PRECISION["mixed"]:
             self._fp32_built = True
         if self.opts.degree != self.degree:       # a new discretisation: assemble it

@@ -1,6 +1,6 @@
 """What a context keeps between calls: the solve graph across changes of the degree, its buffers and
-readiness after an allocation that failed. A context that has been through other states gives what a new
-context gives, bit for bit."""
+readiness after an allocation that failed, the operators across changes of the precision. A context that
+has been through other states gives what a new context gives, bit for bit."""
 import contextlib
 
 import numpy as np
@@ -111,3 +111,85 @@ def test_failed_training_batch_leaves_the_buffers_whole():
         got = s.coarse_model_grad(*batch, 8, 8)
     assert got[0] == want[0] and np.array_equal(got[1], want[1])
     s.close()
+
+
+def _system(degree):
+    """(a workload, MB for the FP32 copies but not for the second set of operators, MB for neither)"""
+    if degree == 0:
+        return I.cubed_sphere(24, 30), 70, 8
+    return I.planar_helmholtz(n=16, nlev=16, nmg=2), 500, 100   # (S in FP32: 147)
+
+
+@pytest.mark.parametrize("degree", [0, 1, 3])
+def test_precision_switch_and_back(degree):
+    """FP64 -> mixed -> FP64 -> mixed: each precision's results are those of its first solve and of a new
+    context, also with a relaxation weight changed in between."""
+    w = I.planar_helmholtz(n=8, nlev=5, nmg=2) if degree else I.cubed_sphere(6, 11)
+    s = _solver(w, degree=degree, tol=1e-9)
+    new = {p: _solver(w, degree=degree, tol=1e-9, precision=p) for p in ("fp64", "mixed")}
+    rhs = _rhs(s, 1)
+
+    def values(x):
+        lam = x.solve(*rhs)[0]
+        return [lam, *x.reconstruct(lam, *rhs), x.gamma(), x.precond(lam), x.line_smooth(lam, lam.clone(), 2)]
+
+    for omega in (0.6, 0.6, 0.7, 0.6):
+        for p in ("fp64", "mixed"):
+            s.set_options(precision=p)
+            for x in (s, new[p]):
+                x.set_options(omega=omega)
+            for got, want in zip(values(s), values(new[p])):
+                assert torch.equal(got, want), (p, omega)
+    s.set_options(precision="fp64")
+    s.assemble()
+    assert all(torch.equal(a, b) for a, b in zip(values(s), values(new["fp64"])))
+    for x in (s, *new.values()):
+        x.close()
+
+
+@pytest.mark.parametrize("degree", [0, 3])
+def test_precision_switch_without_room(degree):
+    """Where neither the second set nor FP32 copies of the first fit, the switch fails and the context goes
+    on in FP64 as before; with room it then gives a mixed context's results."""
+    from paper_2210_11797_gb300.hmg import HmgError
+    w, _, leave = _system(degree)
+    s = _solver(w, degree=degree)
+    rhs = _rhs(s, 1)
+    lam = s.solve(*rhs)[0]
+    for _ in range(2):
+        with _full(leave), pytest.raises(HmgError) as e:
+            s.set_options(precision="mixed")
+        assert e.value.status == 8
+        assert torch.equal(s.solve(*rhs)[0], lam)
+        s.set_options(tol=1e-6)
+        assert torch.equal(s.solve(*rhs)[0], lam)
+    s.set_options(precision="mixed")
+    new = _solver(w, degree=degree, precision="mixed")
+    assert torch.equal(s.solve(*rhs)[0], new.solve(*rhs)[0])
+    s.close()
+    new.close()
+
+
+@pytest.mark.parametrize("degree", [0, 3])
+def test_precision_switch_without_room_for_a_second_set(degree):
+    """The FP32 preconditioner then takes copies of the operators there are: the solve meets its tolerance
+    in the FP64 operator, FP64 is as before, and a later switch with room makes the second set."""
+    w, leave, _ = _system(degree)
+    s = _solver(w, degree=degree)
+    rhs = _rhs(s, 1)
+    lam, st = s.solve(*rhs)
+    b = s.trace_rhs(*rhs)
+    with _full(leave):
+        s.set_options(precision="mixed")
+    lam32, st32 = s.solve(*rhs)
+    assert not torch.equal(lam32, lam) and abs(st32["iterations"] - st["iterations"]) <= 2
+    assert (b - s.apply_trace(lam32)).norm() <= 1.05e-6 * b.norm()
+    s.set_options(tol=1e-6)   # (not tried again here)
+    assert torch.equal(s.solve(*rhs)[0], lam32)
+    s.set_options(precision="fp64")
+    assert torch.equal(s.solve(*rhs)[0], lam)
+    s.set_options(precision="mixed")
+    new = _solver(w, degree=degree, precision="mixed")
+    assert torch.equal(s.solve(*rhs)[0], new.solve(*rhs)[0])
+    s.close()
+    new.close()
