@@ -670,10 +670,7 @@ int ho_gauss_cell_matrices(Ctx *c) {
     if ((st = dev_alloc(c, &h.gtab, tab.size()))) return st;
     HMG_CUDA(c, cudaMemcpy(h.gtab, tab.data(), sizeof(double) * tab.size(), cudaMemcpyHostToDevice));
   }
-  // the facet weights with this file's bits too (host compilers may contract the quadrature rule's sums
-  // differently in another file)
-  HMG_CUDA(c, cudaMemcpyAsync(h.tab + Ho<P>::TC, h.gtab + HoGauss<P>::TC, sizeof(double) * Ho<P>::NB,
-                              cudaMemcpyDeviceToDevice, c->stream));
+  h.cw = h.gtab + HoGauss<P>::TC;   // (host compilers may contract the quadrature rule's sums differently in another file)
   const HoGaussArgs a{f.geometry, f.ncol, f.nlev, f.ncell, f.radius, c->sc.sigma, f.corners, f.z};
   const size_t smem = HoGaussSmem<P>::BYTES;
   HMG_CUDA(c, cudaFuncSetAttribute(ho_gauss_cell_kernel<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));

@@ -206,7 +206,7 @@ __global__ void ho_own_kernel(const int32_t *__restrict__ stencil, const int32_t
 // the node's local index in A), and in slots NF .. 2 NF - 1 the same of cell B, whose
 // shared-facet entries are added into A's slots (and stored as 0).
 template <int P>
-__global__ void ho_rows_kernel(const HoGeo g, int64_t T, const double *__restrict__ tab,
+__global__ void ho_rows_kernel(const HoGeo g, int64_t T, const double *__restrict__ Cw,
                                const double *__restrict__ Ainv, double *__restrict__ S) {
   using H = Ho<P>;
   constexpr int N = H::N;
@@ -214,7 +214,6 @@ __global__ void ho_rows_kernel(const HoGeo g, int64_t T, const double *__restric
   if (row >= T) return;
   const int64_t F = row / H::NB;
   const int n = (int)(row - F * H::NB), s = n / H::NT, t = n - s * H::NT;
-  const double *Cw = tab + H::TC;
   const HoFacet fc = ho_facet(g, F);
   const int qa = H::NB * fc.fA + n;
   const double *IA = Ainv + ((int64_t)fc.cA * g.L + fc.kA) * (int64_t)(N * N) + (int64_t)qa * N;
@@ -498,7 +497,7 @@ struct HoDot {
 // (A_K^-1 R_K)_q on the facet dofs q < NF, into o0 (q < NF / 2) and o1, NF / 2 per cell each.
 template <int P, bool REC>
 __global__ void __launch_bounds__(kHoDotThreads)
-    ho_dot_kernel(const HoGeo g, int64_t ncell, const double *__restrict__ tab, const double *__restrict__ Ainv,
+    ho_dot_kernel(const HoGeo g, int64_t ncell, const double *__restrict__ cw, const double *__restrict__ Ainv,
                   const double *__restrict__ lam, const double *__restrict__ Ru, const double *__restrict__ Rp,
                   double *__restrict__ o0, double *__restrict__ o1) {
   using H = Ho<P>;
@@ -518,7 +517,7 @@ __global__ void __launch_bounds__(kHoDotThreads)
     double v = j < H::NU ? Ru[K * H::NU + j] : Rp[K * H::NP + (j - H::NU)];
     if (REC && j < H::NF) {
       const int c = (int)((unsigned)K / (unsigned)g.L), k = (int)((unsigned)K - (unsigned)c * (unsigned)g.L);
-      v = fma(-tab[H::TC + j % H::NB], lam[ho_gid<P>(g, c, k, j)], v);
+      v = fma(-cw[j % H::NB], lam[ho_gid<P>(g, c, k, j)], v);
     }
     r[e] = v;
   }
@@ -577,14 +576,14 @@ static int ho_launch_dot(Ctx *c, const double *lam, const double *Ru, const doub
   const int64_t C = c->lv[0].ncell;
   HMG_CUDA(c, cudaFuncSetAttribute(ho_dot_kernel<P, REC>, cudaFuncAttributeMaxDynamicSharedMemorySize, D::SMEM));
   ho_dot_kernel<P, REC><<<grid_for(C * D::ROWS, kHoDotThreads), kHoDotThreads, D::SMEM, c->stream>>>(
-      ho_geo<P>(c), C, c->ho.tab, c->ho.Ainv, lam, Ru, Rp, o0, o1);
+      ho_geo<P>(c), C, c->ho.cw, c->ho.Ainv, lam, Ru, Rp, o0, o1);
   HMG_CUDA(c, cudaGetLastError());
   return HMG_OK;
 }
 
 // B_lambda row NB F + n: the sum over the facet's cells of C_K (A_K^-1 R_K) at the node's local dof
 template <int P>
-__global__ void ho_rhs_kernel(const HoGeo g, int64_t T, const double *__restrict__ tab, const double *__restrict__ d0,
+__global__ void ho_rhs_kernel(const HoGeo g, int64_t T, const double *__restrict__ cw, const double *__restrict__ d0,
                               const double *__restrict__ d1, double *__restrict__ B) {
   using H = Ho<P>;
   constexpr int HF = H::NF / 2;
@@ -599,7 +598,7 @@ __global__ void ho_rhs_kernel(const HoGeo g, int64_t T, const double *__restrict
   };
   double v = cell(fc.cA, fc.kA, H::NB * fc.fA + n);
   if (fc.cB >= 0) v += cell(fc.cB, fc.kB, H::NB * fc.fB + H::NT * (fc.flipB ? P - s : s) + t);
-  B[row] = tab[H::TC + n] * v;
+  B[row] = cw[n] * v;
 }
 
 // ---- Algorithm 1 at p >= 1 ------------------------------------------------------------------------
@@ -1001,6 +1000,7 @@ void ho_free(Ctx *c) {
     dev_free(c, *b);
     *b = nullptr;
   }
+  h.cw = nullptr;
   h.have_fp32 = false;
   h.degree = 0;
   h.ncell = 0;
@@ -1047,7 +1047,7 @@ static int ho_assemble_p(Ctx *c) {
   HMG_CUDA(c, cudaStreamSynchronize(c->stream));
   if (sing) return fail(c, HMG_ERR_INVALID_ARG, "a degree-p cell matrix A_K is singular");
   const HoGeo g = ho_geo<P>(c);
-  ho_rows_kernel<P><<<grid_for(h.T, 256), 256, 0, c->stream>>>(g, h.T, h.tab, h.Ainv, h.S);
+  ho_rows_kernel<P><<<grid_for(h.T, 256), 256, 0, c->stream>>>(g, h.T, h.cw, h.Ainv, h.S);
   HMG_CUDA(c, cudaGetLastError());
   if (gauss) {   // P^T S P 1 by the operator itself (P 1 = 1)
     double *ones = sk1, *s1 = static_cast<double *>(c->w2);
@@ -1094,7 +1094,7 @@ static int ho_trace_rhs_p(Ctx *c, const double *Ru, const double *Rp, double *B)
   double *d0 = static_cast<double *>(c->w1), *d1 = static_cast<double *>(c->w2);
   int st;
   if ((st = ho_launch_dot<P, false>(c, nullptr, Ru, Rp, d0, d1))) return st;
-  ho_rhs_kernel<P><<<grid_for(h.T, 256), 256, 0, c->stream>>>(ho_geo<P>(c), h.T, h.tab, d0, d1, B);
+  ho_rhs_kernel<P><<<grid_for(h.T, 256), 256, 0, c->stream>>>(ho_geo<P>(c), h.T, h.cw, d0, d1, B);
   HMG_CUDA(c, cudaGetLastError());
   return HMG_OK;
 }

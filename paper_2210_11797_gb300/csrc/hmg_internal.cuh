@@ -107,6 +107,7 @@ struct HoData {
   double *tab = nullptr;       // reference-element tables
   int *itab = nullptr;         // and their integer part
   double *gtab = nullptr;      // tables of the direct Gauss sums (contexts with the FP32 preconditioner)
+  const double *cw = nullptr;  // [NB] facet weights of C_K, in the tables that the cell matrices were formed from
   double *ctab = nullptr, *ltab = nullptr;   // geometry sums per column and per level
   int *flag = nullptr;         // singular-matrix flag of the assembly
   double factor_omega = 0.0;   // the omega the smoother factors hold

@@ -492,6 +492,7 @@ int ho_cell_matrices(Ctx *c, double *sk1) {
   ho_cell_kernel<P><<<(unsigned)f.ncell, SH::THREADS, smem, c->stream>>>(ho_cell_args(c), f.ncell, h.Ainv, h.m, sk1,
                                                                         h.flag);
   HMG_CUDA(c, cudaGetLastError());
+  h.cw = h.tab + Ho<P>::TC;
   return HMG_OK;
 }
 

@@ -193,3 +193,23 @@ def test_precision_switch_without_room_for_a_second_set(degree):
     assert torch.equal(s.solve(*rhs)[0], new.solve(*rhs)[0])
     s.close()
     new.close()
+
+
+@pytest.mark.parametrize("degree", [0, 1, 2, 3])
+def test_assembly_in_the_other_precision(degree):
+    """A context assembled for the FP32 preconditioner, switched to FP64 and assembled again has the
+    operators, right-hand side and recovery of an FP64 context, and the other way round."""
+    w = I.planar_helmholtz(n=6, nlev=3, nmg=1)
+    new = {p: _solver(w, degree=degree, precision=p) for p in ("fp64", "mixed")}
+    s = _solver(w, degree=degree, precision="mixed")
+    rhs = _rhs(s, 1)
+    x = torch.randn(s.ntrace, generator=torch.Generator(device="cuda").manual_seed(3), dtype=torch.float64,
+                    device="cuda")
+    for p in ("fp64", "mixed", "fp64"):
+        s.set_options(precision=p)
+        s.assemble()
+        for got, want in zip(*([y.trace_rhs(*rhs), y.apply_trace(x), *y.reconstruct(x, *rhs), y.gamma(),
+                                y.precond(x)] for y in (s, new[p]))):
+            assert torch.equal(got, want), p
+    for y in (s, *new.values()):
+        y.close()
