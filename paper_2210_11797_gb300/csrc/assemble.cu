@@ -953,7 +953,7 @@ static int assemble_levels(Ctx *c, double *rec) {
     Level &lv = c->lv[l];
     const CellArgs a{lv.geometry, lv.ncol, lv.nlev, lv.ncell, lv.radius, lv.corners, lv.z,
                      lv.theta_lev, lv.exner_lev, lv.exner, lv.col_nbr, c->sc};
-    if (!lv.geo_ready) {   // the sums depend on the mesh only, which a context keeps
+    if (!rec && !lv.geo_ready) {   // the sums depend on the mesh only, which a context keeps
       if ((st = dev_make(c, &lv.ctab, (size_t)Col::N * lv.ncol))) return st;
       if ((st = dev_make(c, &lv.ltab, (size_t)Lev::N * lv.nlev))) return st;
       column_kernel<<<grid_for(lv.ncol, 64) + grid_for(lv.nlev, 64), 64, 0, c->stream>>>(a, lv.ctab, lv.ltab);

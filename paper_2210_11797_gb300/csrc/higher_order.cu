@@ -983,7 +983,7 @@ static int ho_build_fp32(Ctx *c) {
 
 void ho_free(Ctx *c) {
   HoData &h = c->ho;
-  if (h.tab) drop_graph(c);   // captured launches hold these buffers (tab is the first of them to be made)
+  if (h.flag) drop_graph(c);   // captured launches hold these buffers (flag is the first of them to be made)
   double **bufs[] = {&h.tab, &h.gtab, &h.ctab, &h.ltab, &h.S, &h.Ainv, &h.hw, &h.zf, &h.gamma, &h.m, &h.fs};
   for (double **b : bufs) {
     dev_free(c, *b);
@@ -1020,7 +1020,7 @@ static int ho_assemble_p(Ctx *c) {
   if (C > 0x7fffffff) return fail(c, HMG_ERR_INVALID_ARG, "too many cells for one launch");
   if (h.degree != P || h.ncell != C || h.T != ho_trace_size(c, P)) {   // (re)allocate for this degree and mesh
     ho_free(c);
-    if ((st = ho_make_tables<P>(c))) return st;
+    if ((st = dev_alloc(c, &h.flag, 1))) return st;
     const int64_t T = ho_trace_size(c, P);
     if ((st = dev_alloc(c, &h.S, (size_t)H::SLOTS * T))) return st;
     if ((st = dev_alloc(c, &h.Ainv, (size_t)H::N * H::N * C))) return st;

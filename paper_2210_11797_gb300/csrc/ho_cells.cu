@@ -455,7 +455,7 @@ static HoCellArgs ho_cell_args(const Ctx *c) {
 }
 
 template <int P>
-int ho_make_tables(Ctx *c) {
+static int ho_make_tables(Ctx *c) {
   using H = Ho<P>;
   const Level &f = c->lv[0];
   HoData &h = c->ho;
@@ -467,10 +467,8 @@ int ho_make_tables(Ctx *c) {
   if ((st = dev_alloc(c, &h.itab, itab.size()))) return st;
   if ((st = dev_alloc(c, &h.ctab, (size_t)H::CTAB * f.ncol))) return st;
   if ((st = dev_alloc(c, &h.ltab, (size_t)H::LTAB * f.nlev))) return st;
-  if ((st = dev_alloc(c, &h.flag, 1))) return st;
   HMG_CUDA(c, cudaMemcpy(h.tab, tab.data(), sizeof(double) * tab.size(), cudaMemcpyHostToDevice));
   HMG_CUDA(c, cudaMemcpy(h.itab, itab.data(), sizeof(int) * itab.size(), cudaMemcpyHostToDevice));
-  HMG_CUDA(c, cudaMemsetAsync(h.flag, 0, sizeof(int), c->stream));
   const HoCellArgs a = ho_cell_args(c);
   ho_column_kernel<P><<<f.ncol, kHoColThreads, sizeof(double) * kHoColSmem<P>, c->stream>>>(a, h.flag);
   ho_level_kernel<P><<<grid_for(f.nlev, 32), 32, 0, c->stream>>>(a);
@@ -487,6 +485,8 @@ int ho_cell_matrices(Ctx *c, double *sk1) {
   using SH = HoCellShape<P>;
   const Level &f = c->lv[0];
   HoData &h = c->ho;
+  int st;
+  if (!h.tab && (st = ho_make_tables<P>(c))) return st;   // (a failure here frees the layout)
   const int smem = (int)sizeof(double) * SH::doubles(f.geometry == 1);
   HMG_CUDA(c, cudaFuncSetAttribute(ho_cell_kernel<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
   ho_cell_kernel<P><<<(unsigned)f.ncell, SH::THREADS, smem, c->stream>>>(ho_cell_args(c), f.ncell, h.Ainv, h.m, sk1,
@@ -496,9 +496,6 @@ int ho_cell_matrices(Ctx *c, double *sk1) {
   return HMG_OK;
 }
 
-template int ho_make_tables<1>(Ctx *);
-template int ho_make_tables<2>(Ctx *);
-template int ho_make_tables<3>(Ctx *);
 template int ho_cell_matrices<1>(Ctx *, double *);
 template int ho_cell_matrices<2>(Ctx *, double *);
 template int ho_cell_matrices<3>(Ctx *, double *);

@@ -106,11 +106,9 @@ __device__ __forceinline__ HoFacet ho_facet(const HoGeo &g, int64_t F) {
   return r;
 }
 
-// ho_cells.cu: the reference tables and the mesh's geometry sums (once per layout); A_K^-1 of every
-// cell into ho.Ainv, (H 1)_K into ho.m and S_K 1 summed over each facet into sk1 [6][ncell];
-// *ho.flag set when a cell is singular
-template <int P>
-int ho_make_tables(Ctx *c);
+// ho_cells.cu: A_K^-1 of every cell into ho.Ainv, (H 1)_K into ho.m and S_K 1 summed over each facet into
+// sk1 [6][ncell], from the reference tables and the mesh's geometry sums (made on the first call of a
+// layout); *ho.flag set when a cell is singular
 template <int P>
 int ho_cell_matrices(Ctx *c, double *sk1);
 // gauss_cells.cu: A_K^-1 and (H 1)_K by direct Gauss sums and a pivoted elimination

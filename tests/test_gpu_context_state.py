@@ -213,3 +213,23 @@ def test_assembly_in_the_other_precision(degree):
             assert torch.equal(got, want), p
     for y in (s, *new.values()):
         y.close()
+
+
+def test_mixed_context_holds_no_geometry_sums():
+    """The column sums of the factorised set-up (832 bytes per column) are for FP64 assemblies only: a mixed
+    context takes an FP64 one's memory and its FP32 copies, less these."""
+    w = I.planar_helmholtz(n=512, nlev=1, nmg=1)
+
+    def memory(precision):
+        torch.cuda.synchronize()
+        free = torch.cuda.mem_get_info()[0]
+        s = _solver(w, precision=precision)
+        torch.cuda.synchronize()
+        n = free - torch.cuda.mem_get_info()[0]
+        s.close()
+        return n
+
+    memory("fp64")   # (the library's own allocations of a first context)
+    C, T = 512 * 512, 4 * 512 * 512
+    fp32 = 4 * (11 * T + 3 * 2 * C + 2 * C + C + 7 * C + 3 * C)   # S, factors, Gamma, H, its factors
+    assert memory("mixed") <= memory("fp64") + fp32 - 832 * C + (32 << 20)   # (2 MB pages of 14 buffers)
