@@ -726,9 +726,8 @@ static bool fuse_level(const Ctx *c, int l) { return c->lv[l].ncell <= (int64_t)
 int vcycle_launches(const Ctx *c) {
   const int nmg = c->nmg, npre = c->opt.mg_npre, npost = c->opt.mg_npost;
   if (nmg == 1) return c->opt.mg_ncoarse;
-  // finest level: pre-sweeps, restriction, injection and post-sweeps; the coarse levels one launch
-  if (c->opt.mg_fused) return npre + 1 + 1 + 1 + npost;
   int n = npre + (fuse_level(c, 0) ? 0 : 1) + npost;   // finest level: pre-sweeps, (injection,) post-sweeps
+  if (c->opt.mg_fused) return n + 1 + 1;               // its restriction, the coarse levels in one launch
   for (int l = 1; l < nmg; ++l) {
     const bool f = fuse_level(c, l);
     n += (l == nmg - 1 ? c->opt.mg_ncoarse : npre) + (f ? 0 : 1);   // sweeps (+ restriction)

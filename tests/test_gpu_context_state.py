@@ -233,3 +233,18 @@ def test_mixed_context_holds_no_geometry_sums():
     C, T = 512 * 512, 4 * 512 * 512
     fp32 = 4 * (11 * T + 3 * 2 * C + 2 * C + C + 7 * C + 3 * C)   # S, factors, Gamma, H, its factors
     assert memory("mixed") <= memory("fp64") + fp32 - 832 * C + (32 << 20)   # (2 MB pages of 14 buffers)
+
+
+@pytest.mark.parametrize("nmg", [2, 3])
+def test_launch_count_of_the_cooperative_vcycle(nmg):
+    """mg_fused: the finest level's injection is a launch of its own only where it does not ride in the
+    first post-sweep."""
+    w = I.planar_helmholtz(n=16, nlev=8, nmg=nmg)
+    s = _solver(w, tol=1e-8, mg_fused=1, profile=1)
+    rhs = _rhs(s, 1)
+    for cells, injection in ((1 << 18, 0), (0, 1)):
+        s.set_options(mg_fuse_cells=cells)
+        st = s.solve(*rhs)[1]
+        # per V-cycle: 1 pre-sweep, restriction, the coarse levels, (injection,) 2 post-sweeps
+        assert st["components"]["pressure_vcycle"]["launches"] == 2 * st["iterations"] * (5 + injection)
+    s.close()
