@@ -40,7 +40,8 @@ struct Scal {
   static constexpr int BB = 6;              // (B, B)
   static constexpr int ALPHA = 7, OMEGA = 8;
   static constexpr int AUX = 9;             // scratch for tests / true residual
-  static constexpr int BETA = 10;           // (rho_i / rho_{i-1}) (alpha / omega) of the next iteration
+  // 10 and 11: pair collection's dots, 12: the Krylov coarse solve's (both run inside the preconditioner)
+  static constexpr int BETA = 13;           // (rho_i / rho_{i-1}) (alpha / omega) of the next iteration
   static constexpr int N = 16;
 };
 
