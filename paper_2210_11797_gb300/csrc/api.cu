@@ -706,6 +706,13 @@ int hmg_autotune(hmg_ctx *c) {
   return finish(c, autotune(c));
 }
 
+int hmg_test_forms(Ctx *c, int32_t forms) {
+  if (!c || forms < 0 || forms > 2) return HMG_ERR_INVALID_ARG;
+  drop_graph(c);   // captured launches have the other form
+  c->forms = forms;
+  return HMG_OK;
+}
+
 int hmg_get_launch_shapes(hmg_ctx *c, int32_t *sweep, int32_t *mg, int32_t nmg) {
   if (!c || !sweep || (nmg > 0 && !mg)) return HMG_ERR_INVALID_ARG;
   if (!c->have_mesh || nmg != c->nmg) return fail(c, HMG_ERR_INVALID_ARG, "nmg must equal the mesh's levels");

@@ -18,6 +18,8 @@
 // interface k) at NH + NB (c (L + 1) + k), node (s, t) at + NT s + t; on a vertical facet s
 // counts along the edge in the traversal of its owner column (the other column's local s is
 // p - s).
+#include <type_traits>
+
 #include "device_common.cuh"
 #include "hmg_internal.cuh"
 #include "ho_common.cuh"
@@ -25,7 +27,7 @@
 
 namespace hmg {
 
-// The row kernels take whole facets per block (p = 2: 28 facets of nine rows) and a few rows of one facet
+// The row kernels take whole facets per block (p = 2: 28 facets of nine rows) and kHoR rows of one facet
 // per thread: the lanes of a warp read consecutive coefficients of a slot, and the rows of a facet share
 // its x values. One thread per facet with NB accumulators leaves most of the GPU idle on small meshes (16 x
 // 16 x 16 cells at p = 3: 49 blocks on 152 SMs, S apply 266 us); on large ones FP32 takes it (below).
@@ -184,12 +186,14 @@ __device__ __forceinline__ void ho_facet_rows(const float *__restrict__ S, const
   Sr += (int64_t)H::NF * T;
   if (fc.cB >= 0) cell(fc.cB, fc.kB, fc.fB);
 }
-// FP32 rows from which a facet per thread is the faster form (sweep rows and residual of p = 1, 2, 3: 98 /
-// 182 / 237 and 91 / 170 / 227 us against 121 / 254 / 294 and 89 / 219 / 264 with R rows per thread, at
-// 3.6 / 2.8 / 2.5 M rows; at 0.2 M rows of p = 3, 49 blocks, 135 us against 30). The line is where the
-// facet form's 130 us of latency at p = 3 meet the other's 120 us per million rows. Both forms add a row's
-// products in the same order.
-constexpr int64_t kHoFacetRows = 1 << 20;
+// FP32 rows from which a facet per thread is the faster form: where the facet form's latency (2 NF times NB
+// products of one thread) meets the other's time per row. Measured as sweeps (us each with their line
+// solves, by rows / by facets) and residuals: p = 1 sweeps 42 / 46 at 0.61 M rows, 51 / 49 at 0.80 M, 271 / 239
+// at 6.4 M, its residual always by rows (34 / 43 at 0.80 M, 173 / 186 at 6.4 M); p = 2 two sweeps and a
+// residual 284 / 290 at 0.71 M, 322 / 310 at 0.85 M; p = 3 773 / 778 at 1.89 M, 969 / 824 at 2.48 M. Both
+// forms add a row's products in the same order.
+template <int P>
+constexpr int64_t kHoFacetRows = P == 1 ? 700'000 : (P == 2 ? 780'000 : 1'950'000);
 
 // ---- assembly -------------------------------------------------------------------------------
 // own[c][f] = 1 where column c owns the edge of its face f (each entry written by one edge)
@@ -374,7 +378,7 @@ __global__ void __launch_bounds__(32 * kHoFacWarps)
 }
 
 // ---- the operator, the right-hand side and the recovery --------------------------------------
-// y = S x, one thread per row; MODE 1, 2, 3 fuse the inner products of the Krylov loop as the
+// y = S x, kHoR rows per thread; MODE 1, 2, 3 fuse the inner products of the Krylov loop as the
 // lowest-order S apply does (3: (b - S x, b - S x), no y): a facet's products are summed in row order by
 // one thread into fs[F] (and fs[nF + F]), which ho_reduce_kernel adds up.
 template <int P, int MODE>
@@ -604,8 +608,8 @@ __global__ void ho_rhs_kernel(const HoGeo g, int64_t T, const double *__restrict
 // ---- Algorithm 1 at p >= 1 ------------------------------------------------------------------------
 // lam_out = lam_in + omega D^-1 (b - S lam_in) (ZERO: lam_in = 0), evaluated as
 // (1 - omega) lam_in + omega D^-1 (b - (S - D) lam_in): equal in exact arithmetic, without the
-// couplings of a row inside D. Two launches per sweep. Part 1, one thread per row (as parallel as the
-// S apply): the residual rows r = b - (S - D) lam_in; on a vertical facet the NB x NB block Jacobi step
+// couplings of a row inside D. Two launches per sweep. Part 1, kHoR rows per thread as the S apply (in
+// FP32 a facet from kHoFacetRows on): the residual rows r = b - (S - D) lam_in; on a vertical facet the NB x NB block Jacobi step
 // lam_out = keep lam_in + (omega D_F^-1) r at once (the facet's r in shared memory), on a horizontal
 // facet r is parked in lam_out's rows (ZERO: vertical facets only, r = b). Part 2, the line
 // solves: each column's r staged in shared memory, the block Thomas recurrences with LPC lanes
@@ -785,7 +789,71 @@ __global__ void __launch_bounds__(64)
     lam_out[base + i] = (Tout)(ZERO ? sr[i] : fma((T)keep, (T)lam_in[base + i], sr[i]));
 }
 
-// R = b - S lam (Algorithm 2 line 3), one thread per row. ZSWEEP: lam is one sweep from zero,
+// Part 2 at p = 2 in FP32: one warp per block, each lane's factor rows loaded one step ahead into
+// registers. A block of 81 floats is aligned to four bytes only, so that the ring's copies and its reads
+// are three times the instructions of these loads. 88 x 88 x 32 cells: a zero-start sweep 153 us with the
+// ring and 108 so, 56 x 56 x 32: 75 and 69, 16 x 16 x 16: 31 and 29; one warp per block against four
+// (few columns then leave SMs without a block) 69 and 74 us on 56 x 56 x 32.
+template <int P, bool ZERO, typename T, typename Ts, typename Tout>
+__global__ void __launch_bounds__(32)
+    ho_sweep_lines_regs_kernel(const HoGeo g, int cpb, const T *__restrict__ zf, const Ts *src,
+                               const T *__restrict__ lam_in, Tout *lam_out, double keep) {
+  using H = Ho<P>;
+  constexpr int NB = H::NB, NB2 = NB * NB, LPC = H::LPC;
+  extern __shared__ __align__(16) unsigned char ho_lines_smem[];
+  T *sr = reinterpret_cast<T *>(ho_lines_smem);   // [cpb][L+1][NB]
+  const int L1 = g.L + 1, lane = threadIdx.x, c0 = blockIdx.x * cpb, nc = min(cpb, g.ncol - c0);
+  const int64_t base = g.NH + (int64_t)NB * c0 * L1;
+#pragma unroll 4
+  for (int i = lane; i < nc * L1 * NB; i += 32) sr[i] = (T)src[base + i];
+  __syncwarp();
+  const int cc = lane / LPC, n = lane - cc * LPC;
+  const bool act = cc < nc && n < NB;   // (the other lanes follow the first column)
+  T *r = sr + NB * (act ? cc : 0) * L1;
+  const T *f0 = zf + 3 * NB2 * ((int64_t)(c0 + (act ? cc : 0)) * L1) + (act ? n : 0);   // this lane's rows (transposed)
+  // forward: y_k = (omega G_k^-1) r_k - (G_k^-1 L_k) y_{k-1}, y written over r
+  T fa[NB], fb[NB];
+#pragma unroll
+  for (int m = 0; m < NB; ++m) { fa[m] = __ldg(f0 + NB * m); fb[m] = __ldg(f0 + NB2 + NB * m); }
+  for (int k = 0; k < L1; ++k) {
+    const T *f = f0 + 3 * NB2 * min(k + 1, L1 - 1);
+    T na[NB], nb[NB], v = (T)0, u = (T)0;
+#pragma unroll
+    for (int m = 0; m < NB; ++m) { na[m] = __ldg(f + NB * m); nb[m] = __ldg(f + NB2 + NB * m); }
+#pragma unroll
+    for (int m = 0; m < NB; ++m) v = fma(fa[m], r[NB * k + m], v);
+    if (k > 0) {
+#pragma unroll
+      for (int m = 0; m < NB; ++m) u = fma(-fb[m], r[NB * (k - 1) + m], u);
+    }
+    __syncwarp();
+    if (act) r[NB * k + n] = v + u;
+    __syncwarp();
+#pragma unroll
+    for (int m = 0; m < NB; ++m) { fa[m] = na[m]; fb[m] = nb[m]; }
+  }
+  // backward: x_k = y_k - (G_k^-1 U_k) x_{k+1}, x written over y (row k only by its own lane)
+  const T *fu = f0 + 2 * NB2;
+#pragma unroll
+  for (int m = 0; m < NB; ++m) fa[m] = __ldg(fu + 3 * NB2 * max(L1 - 2, 0) + NB * m);
+  for (int k = L1 - 2; k >= 0; --k) {
+    const T *f = fu + 3 * NB2 * max(k - 1, 0);
+    T na[NB], v = act ? r[NB * k + n] : (T)0;
+#pragma unroll
+    for (int m = 0; m < NB; ++m) na[m] = __ldg(f + NB * m);
+#pragma unroll
+    for (int m = 0; m < NB; ++m) v = fma(-fa[m], r[NB * (k + 1) + m], v);
+    if (act) r[NB * k + n] = v;
+    __syncwarp();
+#pragma unroll
+    for (int m = 0; m < NB; ++m) fa[m] = na[m];
+  }
+#pragma unroll 4
+  for (int i = lane; i < nc * L1 * NB; i += 32)
+    lam_out[base + i] = (Tout)(ZERO ? sr[i] : fma((T)keep, (T)lam_in[base + i], sr[i]));
+}
+
+// R = b - S lam (Algorithm 2 line 3), kHoR rows per thread. ZSWEEP: lam is one sweep from zero,
 // lam = omega D^-1 b, so R = (1 - omega) b - (S - D) lam (equal in exact arithmetic).
 template <int P, bool ZSWEEP, typename T = double>
 __global__ void __launch_bounds__(kHoThreads<P, T>)
@@ -808,23 +876,45 @@ __global__ void __launch_bounds__(kHoThreads<P, T>)
 }
 
 // Part 1 of a sweep and the residual in FP32 with a facet per thread (kHoFacetRows). The Jacobi step goes
-// through shared memory, a thread per row, so that the factors and the results are coalesced.
+// through shared memory, a thread per row, so that the factors and the results are coalesced; at p = 1 a
+// thread takes its facet's four rows in 16-byte loads instead (128 x 128 x 32 cells: the sweep 261 us
+// through shared memory, 240 so).
 template <int P, typename Tout>
 __global__ void __launch_bounds__(kHoRowThreads)
     ho_sweep_facets_kernel(const HoGeo g, int64_t TT, const float *__restrict__ S, const float *__restrict__ hw,
                            const double *__restrict__ b, const float *__restrict__ lam_in, Tout *__restrict__ lam_out,
                            double keep) {
   constexpr int NB = Ho<P>::NB, LD = NB | 1;
-  __shared__ float sr[kHoRowThreads * LD];
+  __shared__ float sr[P == 1 ? 1 : kHoRowThreads * LD];
   const int64_t F0 = (int64_t)blockIdx.x * kHoRowThreads, F = F0 + threadIdx.x, nF = g.nhf + g.nzf;
   if (F < nF) {
     float acc[NB];
 #pragma unroll
     for (int n = 0; n < NB; ++n) acc[n] = (float)__ldg(b + NB * F + n);
     ho_facet_rows<P, true>(S, lam_in, g, TT, F, acc);
+    if constexpr (P == 1) {
+      if (F < g.nhf) {
+        const float4 l = __ldg(reinterpret_cast<const float4 *>(lam_in + NB * F));
+        float v[4] = {(float)keep * l.x, (float)keep * l.y, (float)keep * l.z, (float)keep * l.w};
 #pragma unroll
-    for (int n = 0; n < NB; ++n) sr[threadIdx.x * LD + n] = acc[n];
+        for (int m = 0; m < 4; ++m) {
+          const float4 w = __ldg(reinterpret_cast<const float4 *>(hw + NB * NB * F) + m);
+          v[0] = fmaf(w.x, acc[m], v[0]);
+          v[1] = fmaf(w.y, acc[m], v[1]);
+          v[2] = fmaf(w.z, acc[m], v[2]);
+          v[3] = fmaf(w.w, acc[m], v[3]);
+        }
+#pragma unroll
+        for (int n = 0; n < 4; ++n) acc[n] = v[n];
+      }
+#pragma unroll
+      for (int n = 0; n < NB; ++n) lam_out[NB * F + n] = (Tout)acc[n];
+    } else {
+#pragma unroll
+      for (int n = 0; n < NB; ++n) sr[threadIdx.x * LD + n] = acc[n];
+    }
   }
+  if constexpr (P == 1) return;
   __syncthreads();
   const int rows = NB * (int)min((int64_t)kHoRowThreads, nF - F0);
   for (int e = threadIdx.x; e < rows; e += kHoRowThreads) {
@@ -1132,26 +1222,34 @@ static int ho_sweep(Ctx *c, const double *b, const Tin *lam_in, Tout *lam_out) {
   if (cap < 1) return fail(c, HMG_ERR_INVALID_ARG, "too many layers for the degree-p line smoother");
   const int cpb = cap < H::CPW ? cap : H::CPW;
   const unsigned nzb = (unsigned)((g.ncol + cpb - 1) / cpb);
-  const size_t smem = sizeof(T) * (HoLines<P>::DEPTH * H::CPW * HoLines<P>::STRIDE + (size_t)H::NB * cpb * (g.L + 1));
+  const size_t rows = sizeof(T) * H::NB * cpb * (g.L + 1), ring = sizeof(T) * HoLines<P>::DEPTH * H::CPW * HoLines<P>::STRIDE;
   const double keep = 1.0 - h.factor_omega;
   Prof prof(c, ZERO ? kCompPresmooth : kCompSweep, 2);
+  bool by_row = true;
   if constexpr (!ZERO && sizeof(T) == 4) {
-    if (h.T >= kHoFacetRows)
+    by_row = first_form(c, h.T < kHoFacetRows<P>);
+    if (!by_row)
       ho_sweep_facets_kernel<P, Tout><<<grid_for(g.nhf + g.nzf, kHoRowThreads), kHoRowThreads, 0, c->stream>>>(
           g, h.T, HoPrec<T>::S(h), HoPrec<T>::hw(h), b, lam_in, lam_out, keep);
   }
-  if (ZERO || sizeof(T) == 8 || h.T < kHoFacetRows)
+  if (by_row)
     ho_sweep_rows_kernel<P, ZERO, T, double, Tin, Tout>
         <<<grid_for(ZERO ? g.NH : h.T, kHoRows<P>), ZERO ? kHoRowThreads : kHoThreads<P, T>, 0, c->stream>>>(
             g, h.T, HoPrec<T>::S(h), HoPrec<T>::hw(h), b, lam_in, lam_out, keep);
-  auto lines = [&](auto kern, const auto *src) {
+  auto lines = [&](auto kern, int threads, size_t smem, const auto *src) {
     const cudaError_t e = smem > 48 * 1024 ? cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)
                                            : cudaSuccess;
-    if (e == cudaSuccess) kern<<<nzb, 64, smem, c->stream>>>(g, cpb, HoPrec<T>::zf(h), src, lam_in, lam_out, keep);
+    if (e == cudaSuccess) kern<<<nzb, threads, smem, c->stream>>>(g, cpb, HoPrec<T>::zf(h), src, lam_in, lam_out, keep);
     return e;
   };
-  if constexpr (ZERO) HMG_CUDA(c, lines(ho_sweep_lines_kernel<P, ZERO, T, double, Tin, Tout>, b));
-  else HMG_CUDA(c, lines(ho_sweep_lines_kernel<P, ZERO, T, Tout, Tin, Tout>, lam_out));
+  using Ts = std::conditional_t<ZERO, double, Tout>;
+  const Ts *src;
+  if constexpr (ZERO) src = b;
+  else src = lam_out;
+  if constexpr (P == 2 && sizeof(T) == 4)
+    HMG_CUDA(c, lines(ho_sweep_lines_regs_kernel<P, ZERO, T, Ts, Tout>, 32, rows, src));
+  else
+    HMG_CUDA(c, lines(ho_sweep_lines_kernel<P, ZERO, T, Ts, Tin, Tout>, 64, ring + rows, src));
   HMG_CUDA(c, cudaGetLastError());
   return HMG_OK;
 }
@@ -1219,14 +1317,15 @@ static int ho_precond_p(Ctx *c, const double *r, double *z) {
     Prof pr(c, kCompResidual, 2);
     const bool zsweep = c->opt.n_pre == 1;   // w1 is one sweep from zero                       // line 3
     const double rkeep = zsweep ? 1.0 - h.factor_omega : 0.0;
-    bool done = false;
-    if constexpr (sizeof(T) == 4) {
-      if ((done = h.T >= kHoFacetRows)) {
+    bool by_row = true;
+    if constexpr (sizeof(T) == 4 && P > 1) {
+      by_row = first_form(c, h.T < kHoFacetRows<P>);
+      if (!by_row) {
         auto k = zsweep ? ho_residual_facets_kernel<P, true> : ho_residual_facets_kernel<P, false>;
         k<<<grid_for(g.nhf + g.nzf, kHoRowThreads), kHoRowThreads, 0, c->stream>>>(g, TT, HoPrec<T>::S(h), r, w1, w2, rkeep);
       }
     }
-    if (!done) {
+    if (by_row) {
       auto k = zsweep ? ho_residual_kernel<P, true, T> : ho_residual_kernel<P, false, T>;
       k<<<grid_for(TT, kHoRows<P>), kHoThreads<P, T>, 0, c->stream>>>(g, TT, HoPrec<T>::S(h), r, w1, w2, rkeep);
     }

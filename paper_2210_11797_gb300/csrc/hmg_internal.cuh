@@ -223,6 +223,7 @@ struct Ctx : OperatorSet {
   // looked up once by hmg_assemble_trace
   double *noalloc_scratch = nullptr;
   int num_sms = 0;
+  int forms = 0;                    // hmg_test_forms
   int wave_blocks[2] = {0, 0};   // resident blocks (all SMs) of the BiCGStab vector kernels
   // configuration 1 (mixed.cu): the 2x2 operator (velocity block in the 11-slot layout of S,
   // G couplings [2][ntrace], B couplings and M3^Pi [7][ncell]), 1 / lumped mass [ntrace], the
@@ -242,6 +243,10 @@ struct Ctx : OperatorSet {
   std::vector<Mark> marks;
   int ev_next = 0;
 };
+
+// Kernels with two forms, chosen by the size of the mesh: whether to take the first one (the form of small
+// meshes).
+inline bool first_form(const Ctx *c, bool by_size) { return c->forms == 0 ? by_size : c->forms == 1; }
 
 // Records CUDA events around one solver component when profiling is on (no-op otherwise).
 class Prof {
@@ -424,6 +429,9 @@ int vcycle_launches(const Ctx *c);
 int coarse_krylov(Ctx *c, const double *b, double *x, double tol, int maxit);
 // flexible GMRES(restart) driver (krylov.cu)
 int fgmres_solve(Ctx *c, const double *Rub, const double *Rpi, double *lambda, hmg_solve_stats *st);
+// Not part of the ABI: forms = 1 or 2 makes this context take the first or the second form of the kernels
+// that have two (first_form) on any mesh, 0 by size as always. For the tests that compare the two.
+extern "C" int hmg_test_forms(Ctx *c, int32_t forms);
 // Launch-shape autotuning of one context (columns per block of the sweep and MG smoother).
 int autotune(Ctx *c);
 // Sweep / smoother launches with explicit columns and threads per block (autotuner).
