@@ -149,7 +149,7 @@ int launch_spmv(Ctx *c, const double *x, double *y, int mode, const double *w, i
   Prof prof(c, kCompApply);
   const int *as = alpha && mode == 1 ? c->state : nullptr;
   // up to four of spmv_kernel's blocks per SM (its last wave of them is uneven: 308 blocks at C24 x 30)
-  if (g <= 4u * (unsigned)c->num_sms) {
+  if (first_form(c, g <= 4u * (unsigned)c->num_sms)) {
     if (mode == 3) y = static_cast<double *>(c->w1);   // (a place for the residual: the preconditioner is idle)
     auto rows = mode == 3 ? spmv_rows_kernel<true> : spmv_rows_kernel<false>;
     rows<<<grid_for(f.ntrace, 128), 128, 0, c->stream>>>(c->S, x, y, w, d, f.edge_stencil, f.col_edges);
@@ -619,10 +619,10 @@ static int two_level(Ctx *c, const double *r, double *z, const FusedVector *fv) 
   {
     Prof pp(c, kCompProlong);
     // four rows per thread where that still gives every SM two blocks of 256
-    if (f.ntrace >= (int64_t)4 * 256 * 2 * c->num_sms)
-      prolong_kernel<T, 4><<<grid_for(f.ntrace, 256 * 4), 256, 0, c->stream>>>(w1, dpi, w2, d, f.edge_stencil);
-    else
+    if (first_form(c, f.ntrace < (int64_t)4 * 256 * 2 * c->num_sms))
       prolong_kernel<T, 1><<<grid_for(f.ntrace, 128), 128, 0, c->stream>>>(w1, dpi, w2, d, f.edge_stencil);
+    else
+      prolong_kernel<T, 4><<<grid_for(f.ntrace, 256 * 4), 256, 0, c->stream>>>(w1, dpi, w2, d, f.edge_stencil);
   }
   HMG_CUDA(c, cudaGetLastError());
   // line 8: postsmooth

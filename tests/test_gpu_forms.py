@@ -1,5 +1,6 @@
-"""Kernels with two forms chosen by the size of the mesh, both run on the same mesh: the FP32 rows of degree
-p. They add in the same order, so everything is compared bit for bit."""
+"""Kernels with two forms chosen by the size of the mesh, both run on the same mesh: the S apply with its
+inner products and the prolongation at degree 0, the FP32 rows of degree p. They add in the same order, so
+everything is compared bit for bit."""
 import ctypes
 
 import pytest
@@ -28,6 +29,25 @@ def _both(s, call):
         out.append(call())
     _forms(s, 0)
     return out
+
+
+# 45 rows (less than a warp pair), 1,000 to 80,000: below, at and above whole blocks of 128, 256 and 1,024
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+@pytest.mark.parametrize("mesh,n,nlev,nmg", [("plane", 3, 2, 1), ("plane", 8, 5, 2), ("plane", 32, 8, 3),
+                                             ("sphere", 9, 17, 1), ("sphere", 24, 7, 3)])
+def test_lowest_order_forms(mesh, n, nlev, nmg, precision):
+    from paper_2210_11797_gb300.hmg import Solver
+    w = I.planar_helmholtz(n=n, nlev=nlev, nmg=nmg) if mesh == "plane" else I.cubed_sphere(n, nlev, nmg=nmg)
+    s = Solver(w.hier, w.coeffs, tol=1e-8, precision=precision)
+    Ru, Rp, x = _rand(1, 6 * s.ncell, s.ncell, s.ntrace)
+
+    def call():
+        lam, st = s.solve(Ru, Rp, check=False)
+        return (s.apply_trace(x), s.precond(x), lam), (st["iterations"], st["history"], st["true_rel_residual"])
+
+    (a, sa), (b, sb) = _both(s, call)
+    assert all(torch.equal(p, q) for p, q in zip(a, b)) and sa == sb
+    s.close()
 
 
 # facets below, at and above whole blocks of both forms; columns that leave a ragged warp of line solves
