@@ -584,26 +584,35 @@ __global__ void __launch_bounds__(128)
 // field, where a thread per cell made nine, which bounded it (the loads of 30-level columns straddle
 // lines: about two cycles of the load unit each). Consecutive threads are on consecutive levels, so the
 // loads and stores are coalesced. 64 patches of 16 x 16 x 30 in BF16: 126 -> 64 us. blockIdx.y picks
-// two of the 32 channels; block x writes entries 6 y .. 6 y + 5 of partial row x.
+// two of the 32 channels; block x writes entries 6 y .. 6 y + 5 of partial row x. A batch of few rows (few
+// patches, narrow and long) is cut into nseg segments along y, which load the row before and after theirs.
 constexpr int kBw2Ch = 2;
-template <typename A>
+// Segments that give each of the 6 resident blocks of an SM its rows, of at least 16 cells (two halo rows
+// cost a tenth then; shorter patches are taken whole). One patch of 1 x 1024 columns x 30: the gradient took
+// 446 us in one segment, of which this kernel was 340 (a thread per cell: 188).
+static int bw2_segments(const Ctx *c, int64_t rows, int ny) {   // rows: threads of one segment per channel pair
+  const int64_t want = ((int64_t)6 * 128 * c->num_sms * kBw2Ch / kCh + rows - 1) / rows, most = ny / 16;
+  return (int)(want < most ? want : (most > 1 ? most : 1));
+}
+template <typename A, bool SEG>   // SEG: nseg > 1
 __global__ void __launch_bounds__(128, 6)
     nn_bwd2_kernel(const float *__restrict__ wts, const A *__restrict__ h2, const float *__restrict__ ga3,
-                   int nsamp, int nx, int ny, int L, float *__restrict__ ga2, float *__restrict__ part) {
+                   int nsamp, int nx, int ny, int L, int nseg, float *__restrict__ ga2, float *__restrict__ part) {
   __shared__ float Mw[3 * kBw2Ch], red[4][3 * kBw2Ch];
   const int ch0 = blockIdx.y * kBw2Ch;
   if (threadIdx.x < 3 * kBw2Ch) Mw[threadIdx.x] = rnd<A>(wts[kOffM + 3 * ch0 + threadIdx.x]);
   __syncthreads();
-  const int64_t P = (int64_t)nx * ny, C = (int64_t)nsamp * P * L, row = (int64_t)nx * L, units = (int64_t)nsamp * row;
+  const int64_t P = (int64_t)nx * ny, C = (int64_t)nsamp * P * L, row = (int64_t)nx * L, units = (int64_t)nsamp * (SEG ? nseg : 1) * row;
   float acc[3 * kBw2Ch];
 #pragma unroll
   for (int q = 0; q < 3 * kBw2Ch; ++q) acc[q] = 0.f;
   for (int64_t U = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; U < units; U += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t sm = U / row;
-    const int ik = (int)(U - sm * row), i = ik / L;
+    const int64_t ss = U / row, sm = SEG ? ss / nseg : ss;   // sample and segment, sample
+    const int ik = (int)(U - ss * row), i = ik / L, sg = SEG ? (int)(ss - sm * nseg) : 0;
+    const int j0 = SEG ? (int)((int64_t)ny * sg / nseg) : 0, j1 = SEG ? (int)((int64_t)ny * (sg + 1) / nseg) : ny;
     const bool left = i > 0, right = i < nx - 1;
     const int ol = left ? -L : 0, orr = right ? L : 0;   // 0: a load that is not used
-    int64_t K = (int64_t)ch0 * C + sm * P * L + ik;
+    int64_t K = (int64_t)ch0 * C + sm * P * L + j0 * row + ik;
     float gp[kBw2Ch][3], gc[kBw2Ch][3], hp[kBw2Ch][3], hc[kBw2Ch][3];   // (left, centre, right) of rows j - 1, j
     auto load = [&](int64_t at, float (&g)[kBw2Ch][3], float (&h)[kBw2Ch][3]) {
 #pragma unroll
@@ -619,9 +628,10 @@ __global__ void __launch_bounds__(128, 6)
     for (int c = 0; c < kBw2Ch; ++c)
 #pragma unroll
       for (int q = 0; q < 3; ++q) gp[c][q] = hp[c][q] = 0.f;
+    if (SEG && j0 > 0) load(K - row, gp, hp);
     load(K, gc, hc);
 #pragma unroll 2
-    for (int j = 0; j < ny; ++j, K += row) {
+    for (int j = j0; j < j1; ++j, K += row) {
       float gn[kBw2Ch][3] = {}, hn[kBw2Ch][3] = {};
       if (j + 1 < ny) load(K + row, gn, hn);
 #pragma unroll
@@ -1304,9 +1314,11 @@ static int nn_batch_grad(Ctx *c, const float *x, const float *t, const float *tn
   nn_back_kernel<A, float, true><<<g, 128, back_smem(kNnCpb, L, true), c->stream>>>(
       c->nn_w, h2, nb, ncol, L, kNnCpb, nullptr, nullptr, nullptr, t, tn, P, 1.f / (float)nsamp, tb.loss_part,
       tb.ga3, tb.part3);
-  const int64_t g2max = (int64_t)2 * c->num_sms, g2need = ((int64_t)nsamp * nx * L + 127) / 128;   // partial rows: at most 2 per SM
+  const int nseg = bw2_segments(c, (int64_t)nsamp * nx * L, ny);
+  const int64_t g2max = (int64_t)2 * c->num_sms, g2need = ((int64_t)nsamp * nseg * nx * L + 127) / 128;   // partial rows: at most 2 per SM
   const unsigned g2 = (unsigned)(g2need < g2max ? g2need : g2max);
-  nn_bwd2_kernel<A><<<dim3(g2, kCh / kBw2Ch), 128, 0, c->stream>>>(c->nn_w, h2, tb.ga3, nsamp, nx, ny, L, tb.ga2,
+  auto bwd2 = nseg > 1 ? nn_bwd2_kernel<A, true> : nn_bwd2_kernel<A, false>;
+  bwd2<<<dim3(g2, kCh / kBw2Ch), 128, 0, c->stream>>>(c->nn_w, h2, tb.ga3, nsamp, nx, ny, L, nseg, tb.ga2,
                                                                    tb.partM);
   unsigned g1;
   if (sizeof(A) == 2) {   // BF16 storage: the 32 -> 32 convolution's dX and dW on the tensor cores
