@@ -574,6 +574,34 @@ __global__ void __launch_bounds__(kHoDotThreads)
   }
 }
 
+// The recovery at p = 1 on small meshes: a thread per row that reads its row of A_K^-1 itself. Its short
+// rows (44 columns) cost less there than the staging, whose shared memory leaves three blocks per SM: 28 x
+// 28 x 16 cells 86 us (staged 91), 40 x 40 x 16 149 (152), 64 x 64 x 16 344 (332).
+constexpr int64_t kHoDirectCells = 40'000;
+template <int P>
+__global__ void ho_recover_direct_kernel(const HoGeo g, int64_t ncell, const double *__restrict__ cw,
+                                         const double *__restrict__ Ainv, const double *__restrict__ lam,
+                                         const double *__restrict__ Ru, const double *__restrict__ Rp,
+                                         double *__restrict__ u, double *__restrict__ pi) {
+  using H = Ho<P>;
+  constexpr int N = H::N;
+  const int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (idx >= ncell * N) return;
+  const int64_t K = idx / N;
+  const int i = (int)(idx - K * N);
+  const int c = (int)((unsigned)K / (unsigned)g.L), k = (int)((unsigned)K - (unsigned)c * (unsigned)g.L);
+  const double *I = Ainv + K * (int64_t)(N * N) + (int64_t)i * N;
+  double v = 0.0;
+  for (int j = 0; j < H::NU; ++j) {
+    double r = Ru[K * H::NU + j];
+    if (j < H::NF) r = fma(-cw[j % H::NB], lam[ho_gid<P>(g, c, k, j)], r);
+    v = fma(I[j], r, v);
+  }
+  for (int j = 0; j < H::NP; ++j) v = fma(I[H::NU + j], Rp[K * H::NP + j], v);
+  if (i < H::NU) u[K * H::NU + i] = v;
+  else pi[K * H::NP + (i - H::NU)] = v;
+}
+
 template <int P, bool REC>
 static int ho_launch_dot(Ctx *c, const double *lam, const double *Ru, const double *Rp, double *o0, double *o1) {
   using D = HoDot<P, REC>;
@@ -585,7 +613,35 @@ static int ho_launch_dot(Ctx *c, const double *lam, const double *Ru, const doub
   return HMG_OK;
 }
 
-// B_lambda row NB F + n: the sum over the facet's cells of C_K (A_K^-1 R_K) at the node's local dof
+// B_lambda row NB F + n: the sum over the facet's cells of C_K (A_K^-1 R_K) at the node's local dof, from the
+// products of ho_dot_kernel, or (p = 1) by a thread per row that reads its rows of A_K^-1 itself: with 44
+// columns the second launch and the products' way through memory cost more than the staging saves (24 x 24
+// x 10 cells 31 us, 41 staged; 128 x 128 x 32 1.25 and 1.32 ms; p = 2 and 3 gain from 16 x 16 x 16 on, 96
+// and 92 us, 465 and 274).
+template <int P>
+__global__ void ho_rhs_direct_kernel(const HoGeo g, int64_t T, const double *__restrict__ cw,
+                                     const double *__restrict__ Ainv, const double *__restrict__ Ru,
+                                     const double *__restrict__ Rp, double *__restrict__ B) {
+  using H = Ho<P>;
+  constexpr int N = H::N;
+  const int64_t row = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (row >= T) return;
+  const int64_t F = row / H::NB;
+  const int n = (int)(row - F * H::NB), s = n / H::NT, t = n - s * H::NT;
+  const HoFacet fc = ho_facet(g, F);
+  auto cell = [&](int cc, int kk, int q) {
+    const int64_t K = (int64_t)cc * g.L + kk;
+    const double *I = Ainv + K * (int64_t)(N * N) + (int64_t)q * N;
+    double v = 0.0;
+    for (int j = 0; j < H::NU; ++j) v = fma(I[j], Ru[K * H::NU + j], v);
+    for (int j = 0; j < H::NP; ++j) v = fma(I[H::NU + j], Rp[K * H::NP + j], v);
+    return v;
+  };
+  double v = cell(fc.cA, fc.kA, H::NB * fc.fA + n);
+  if (fc.cB >= 0) v += cell(fc.cB, fc.kB, H::NB * fc.fB + H::NT * (fc.flipB ? P - s : s) + t);
+  B[row] = cw[n] * v;
+}
+
 template <int P>
 __global__ void ho_rhs_kernel(const HoGeo g, int64_t T, const double *__restrict__ cw, const double *__restrict__ d0,
                               const double *__restrict__ d1, double *__restrict__ B) {
@@ -1180,6 +1236,11 @@ template <int P>
 static int ho_trace_rhs_p(Ctx *c, const double *Ru, const double *Rp, double *B) {
   const HoData &h = c->ho;
   Prof prof(c, kCompRhs);
+  if constexpr (P == 1) {
+    ho_rhs_direct_kernel<P><<<grid_for(h.T, 128), 128, 0, c->stream>>>(ho_geo<P>(c), h.T, h.cw, h.Ainv, Ru, Rp, B);
+    HMG_CUDA(c, cudaGetLastError());
+    return HMG_OK;
+  }
   // the cells' products pass through the preconditioner's work vectors (T >= 3 NB C = NF / 2 C doubles each)
   double *d0 = static_cast<double *>(c->w1), *d1 = static_cast<double *>(c->w2);
   int st;
@@ -1191,6 +1252,15 @@ static int ho_trace_rhs_p(Ctx *c, const double *Ru, const double *Rp, double *B)
 
 template <int P>
 static int ho_reconstruct_p(Ctx *c, const double *lam, const double *Ru, const double *Rp, double *u, double *pi) {
+  const int64_t C = c->lv[0].ncell;
+  if constexpr (P == 1) {
+    if (first_form(c, C < kHoDirectCells)) {
+      ho_recover_direct_kernel<P><<<grid_for(C * Ho<P>::N, 128), 128, 0, c->stream>>>(ho_geo<P>(c), C, c->ho.cw, c->ho.Ainv,
+                                                                                       lam, Ru, Rp, u, pi);
+      HMG_CUDA(c, cudaGetLastError());
+      return HMG_OK;
+    }
+  }
   return ho_launch_dot<P, true>(c, lam, Ru, Rp, u, pi);
 }
 

@@ -1,5 +1,5 @@
 """Kernels with two forms chosen by the size of the mesh, both run on the same mesh: the S apply with its
-inner products and the prolongation at degree 0, the FP32 rows of degree p. They add in the same order, so
+inner products and the prolongation at degree 0, the FP32 rows of degree p, the recovery of degree 1. They add in the same order, so
 everything is compared bit for bit."""
 import ctypes
 
@@ -64,4 +64,15 @@ def test_degree_p_fp32_forms(p, n, nlev, n_pre):
     a, b = _both(s, lambda: s.precond(x))
     assert torch.equal(a, b)
     assert (a - z).abs().max() <= 1e-4 * z.abs().max()   # FP32 rounding; a wrong term is of the result's size
+    s.close()
+
+
+@pytest.mark.parametrize("n,nlev", [(2, 1), (5, 3), (9, 7), (24, 10)])
+def test_degree_1_recovery_forms(n, nlev):
+    from paper_2210_11797_gb300.hmg import Solver
+    w = I.planar_helmholtz(n=n, nlev=nlev, nmg=1)
+    s = Solver(w.hier, w.coeffs, degree=1)
+    Ru, Rp, x = _rand(3, s.nu * s.ncell, s.npr * s.ncell, s.ntrace)
+    a, b = _both(s, lambda: s.reconstruct(x, Ru, Rp))
+    assert torch.equal(a[0], b[0]) and torch.equal(a[1], b[1])
     s.close()
