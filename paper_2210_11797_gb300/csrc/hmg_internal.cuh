@@ -449,10 +449,12 @@ constexpr int kMaxLayers = 2045;
 // phase, which occupies the FP64 pipe per warp), fewer where that would leave SMs without a block: a
 // level of few columns waits on latency, and a small block takes its cells in one pass. C12 x 30 (864
 // columns, FP64, cold caches): a smoothing sweep 13.7 us at 32 columns (27 blocks), 8 us at 4 (216); its
-// fused restriction and sweep 31 and 13 us.
-inline int default_columns(const Ctx *c, int ncol, int limit) {
+// fused restriction and sweep 31 and 13 us. Below 128 cells a block gets no faster: a V-cycle of a plane
+// of 8 x 8 x 8 cells takes 59 us so and 66 at one column per block, of 12 x 20 x 3 levels 69 and 70, at 256
+// cells a solve of C8 x 30 1,955 us (1,927 at 128, 1,978 at one column).
+inline int default_columns(const Ctx *c, int ncol, int nlev, int limit) {
   int n = limit < 32 ? limit : 32;
-  while (n > 1 && (int64_t)n * c->num_sms > ncol) n >>= 1;
+  while (n > 1 && (int64_t)n * c->num_sms > ncol && n * nlev > 128) n >>= 1;
   return n;
 }
 

@@ -483,7 +483,7 @@ static MGArgs mg_args(const Ctx *c, int l, int pm = 0) {
   MGArgs a;
   a.L = lv.nlev;
   a.ncol = lv.ncol;
-  const int cdef = default_columns(c, lv.ncol, mg_cpb_limit(lv.nlev));
+  const int cdef = default_columns(c, lv.ncol, lv.nlev, mg_cpb_limit(lv.nlev));
   const int tc = c->tune_mg_cpb[pm][l];
   a.cpb = tc > 0 && tc <= mg_cpb_limit(lv.nlev) ? tc : cdef;
   a.ncell = lv.ncell;

@@ -411,7 +411,7 @@ static int launch_sweep(Ctx *c, const Tb *b, const T *lam_in, Tout *lam_out, int
   a.d = dims_of(f);
   a.ncol = f.ncol;
   const int cpb_max = sweep_cpb_limit(f.nlev);
-  const int cpb_def = default_columns(c, f.ncol, cpb_max);
+  const int cpb_def = default_columns(c, f.ncol, f.nlev, cpb_max);
   const int pm = sizeof(T) == 4 ? 1 : 0;   // FP32 preconditioner kernels have their own tuned shape
   if constexpr (sizeof(T) == 4) {
     // columns per block -1 (given or tuned): one warp per lambda^z column
