@@ -235,8 +235,9 @@ int hmg_set_mesh(hmg_ctx *ctx, int32_t nmg, const hmg_mesh_level *levels);
 int hmg_set_coefficients(hmg_ctx *ctx, const hmg_scalars *scalars, const hmg_background *levels);
 
 /* Build everything a solve needs (Eqs. bilinear_forms, hybrid-S, elliptic_pressure_system,
- * scaling_matrix): per cell the 7x7 A_K by 3x3x3 Gauss quadrature, its LU with partial
- * pivoting and inverse, S_K = (A_K^-1)_uu K_K; the rows of S (11 coefficients each); the
+ * scaling_matrix): per cell the 7x7 A_K by 3x3x3 Gauss quadrature (its sums factorised per column
+ * and level, or taken point by point with precision mixed) and its inverse by block elimination,
+ * S_K = (A_K^-1)_uu K_K; the rows of S (11 coefficients each); the
  * Thomas factors of S^zz and 1/diag(S^hh); H and the Thomas factors of H_z on every level;
  * Gamma = (H 1) / (P^T S P 1). Allocates the solver workspace. After a failure the context is not
  * assembled (HMG_ERR_NOT_READY from the calls that need it) until an assembly succeeds. */

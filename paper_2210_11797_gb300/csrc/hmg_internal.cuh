@@ -175,11 +175,12 @@ struct Ctx : OperatorSet {
   int *state_host = nullptr;   // pinned [4]
   double *hist_host = nullptr; // pinned [HMG_MAX_HISTORY]
   cudaEvent_t as_e0 = nullptr, as_e1 = nullptr;   // start / end of an enqueued (async) solve
-  cudaEvent_t loop_done = nullptr;   // recorded by the solve graph when its Krylov loop ends
+  cudaEvent_t loop_done = nullptr;   // recorded behind the loop's graph, before the final residual
   cudaEvent_t copy_done = nullptr;   // end of the copy of lambda to the host
   cudaStream_t copy_stream = nullptr;   // that copy, overlapping the final residual
   bool stats_pending = false;  // an async solve's results are on their way to the host
-  // whole-solve CUDA graph (B_lambda, a WHILE node over BiCGStab iterations, final residual)
+  // the CUDA graph of a solve's loop (its start and a WHILE node over BiCGStab iterations; the right-hand
+  // side and the final residual are launched around it)
   cudaStream_t cap_stream = nullptr;
   cudaGraphExec_t graph_exec = nullptr;
   cudaGraph_t graph = nullptr;
@@ -378,7 +379,8 @@ inline int64_t sys_n(const Ctx *c) {
 // Batched solves: one CUDA graph with one branch per context (contexts on one device).
 int krylov_solve_batched(hmg_ctx *const *ctxs, int n, const double *const *Rub,
                          const double *const *Rpi, double *const *lambda, hmg_solve_stats *st);
-// Releases the context's cached solve graph.
+// Releases the context's cached graphs. Called by whatever frees or replaces a buffer that captured launches
+// hold, or changes what they would launch.
 void drop_graph(Ctx *c);
 
 // ---- degree p = 1, 2, 3 (higher_order.cu) -----------------------------------------------------

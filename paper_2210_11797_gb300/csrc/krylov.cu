@@ -4,12 +4,13 @@
 // 2210.11797: BiCGStab reducing the residual two-norm by the tolerance).
 //
 // Everything the loop decides lives on the device: the inner products are deterministic
-// reductions into ctx->scal, the vector kernels compute alpha, beta and omega from them,
-// and a check kernel appends ||r_i|| / ||B|| to a history array and decides whether to go
-// on. With hmg_options.graph the whole solve is one CUDA graph in which a WHILE conditional
-// node repeats the iteration body until the check kernel clears its condition, so a solve
-// costs one graph launch and one synchronisation. Batched solves put one such branch per
-// context into a single graph. With graph = 0 (or profile = 1) the host drives the loop.
+// reductions into ctx->scal, the kernels that finish them form alpha, beta and omega, and the last
+// of an iteration appends ||r_i|| / ||B|| to a history array and decides whether to go on. With
+// hmg_options.graph the loop is one CUDA graph in which a WHILE conditional node repeats the
+// iteration body until that kernel clears its condition; the right-hand side and the final
+// residual are launched before and after it, and a solve synchronises once. Batched solves put one
+// branch per context, with both, into a single graph. With graph = 0 (or profile = 1) the host
+// drives the loop.
 #include <algorithm>
 #include <atomic>
 #include <cmath>

@@ -183,7 +183,7 @@ __device__ __forceinline__ void smooth_block_src(const MGArgs &a, const T *__res
   const int n = nc * a.L;
   const int64_t base = (int64_t)c0 * a.L;
   // all threads: r omega / pivot and the factors, so that the serial Thomas recurrences
-  // below are one FMA per row each (factors from pressure_factor_kernel)
+  // below are one FMA per row each (factors from factor_kernel)
   for (int i = threadIdx.x; i < n; i += blockDim.x) {
     const int c = c0 + i / a.L, k = i % a.L;
     const int64_t K = base + i;
