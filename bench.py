@@ -31,9 +31,9 @@ UNIT = "trace unknowns/s"
 # DRAM traffic per launch of the dominant kernel from an ncu capture (see profiles/), keyed
 # by the sha256 of the kernel sources it was taken on; a changed source makes it stale (null).
 # C96: dram__bytes_read.sum + dram__bytes_write.sum of the full sweep, captured at full size
-# (a one-pass metric set), mean of two launches (585.7 + 24.3 and 584.1 + 24.4 MB).
+# (a one-pass metric set), mean of two launches (584.8 + 23.8 and 583.6 + 24.3 MB).
 TRAFFIC = {
-    "line_sweep:c96:fp64:bbd86f2c8e64b6de": 609226240,
+    "line_sweep:c96:fp64:2e4600e1acd1b284": 608252928,
 }
 
 
