@@ -846,8 +846,8 @@ __global__ void __launch_bounds__(64)
 }
 
 // Part 2 at p = 2 in FP32: one warp per block, each lane's factor rows loaded one step ahead into
-// registers. A block of 81 floats is aligned to four bytes only, so that the ring's copies and its reads
-// are three times the instructions of these loads. 88 x 88 x 32 cells: a zero-start sweep 153 us with the
+// registers. A block of 81 floats is aligned to four bytes only, so that the ring takes a 4-byte copy and a
+// shared-memory read per factor. 88 x 88 x 32 cells: a zero-start sweep 153 us with the
 // ring and 108 so, 56 x 56 x 32: 75 and 69, 16 x 16 x 16: 31 and 29; one warp per block against four
 // (few columns then leave SMs without a block) 69 and 74 us on 56 x 56 x 32.
 template <int P, bool ZERO, typename T, typename Ts, typename Tout>

@@ -80,7 +80,7 @@ struct Level : LevelOperators {
 // Work buffers of the coarse-model training (learned.cu), grown on demand and reused.
 struct TrainBufs {
   int64_t cap_cells = 0, cap_blocks = 0;
-  void *h1 = nullptr, *h2 = nullptr;   // activations (BF16 or FP32)
+  float *h1 = nullptr, *h2 = nullptr;   // activations (as BF16 or FP32)
   float *ga3 = nullptr, *ga2 = nullptr;
   double *loss_part = nullptr, *loss = nullptr;
   float *part3 = nullptr, *partM = nullptr, *part2 = nullptr, *part1 = nullptr;
@@ -288,6 +288,12 @@ int dev_alloc(Ctx *c, T **p, size_t n) {
 template <typename T>
 int dev_make(Ctx *c, T **p, size_t n) {
   return *p ? HMG_OK : dev_alloc(c, p, n);
+}
+inline int dev_make(Ctx *c, void **p, size_t bytes) {
+  unsigned char *q = static_cast<unsigned char *>(*p);
+  const int st = dev_make(c, &q, bytes);
+  *p = q;
+  return st;
 }
 
 // Releases one device allocation of the context (and forgets it).

@@ -588,8 +588,8 @@ __global__ void __launch_bounds__(128)
 // patches, narrow and long) is cut into nseg segments along y, which load the row before and after theirs.
 constexpr int kBw2Ch = 2;
 // Segments that give each of the 6 resident blocks of an SM its rows, of at least 16 cells (two halo rows
-// cost a tenth then; shorter patches are taken whole). One patch of 1 x 1024 columns x 30: the gradient took
-// 446 us in one segment, of which this kernel was 340 (a thread per cell: 188).
+// cost a tenth then; shorter patches are taken whole). One patch of 1 x 1024 columns x 30: the gradient takes
+// 438 us with one segment, 128 with 64 (186 with a thread per cell).
 static int bw2_segments(const Ctx *c, int64_t rows, int ny) {   // rows: threads of one segment per channel pair
   const int64_t want = ((int64_t)6 * 128 * c->num_sms * kBw2Ch / kCh + rows - 1) / rows, most = ny / 16;
   return (int)(want < most ? want : (most > 1 ? most : 1));
@@ -1274,8 +1274,8 @@ int nn_setup(Ctx *c) {
   HMG_CUDA(c, cudaFuncSetAttribute(nn_bwd1_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024));
   if ((st = dev_make(c, &c->nn_w, kNParams))) return st;
   for (void **image : {&c->nn_bimg, &c->nn_bimg_t})
-    if ((st = dev_make(c, reinterpret_cast<__nv_bfloat16 **>(image), (size_t)32 * 96))) return st;   // cudaMalloc: 256-B aligned
-  if ((st = dev_make(c, reinterpret_cast<float **>(&c->nn_act), (size_t)kCh * f.ncell))) return st;   // BF16 h2 fits in half
+    if ((st = dev_make(c, image, sizeof(__nv_bfloat16) * 32 * 96))) return st;   // cudaMalloc: 256-B aligned
+  if ((st = dev_make(c, &c->nn_act, sizeof(float) * kCh * f.ncell))) return st;   // BF16 h2 fits in half
   // corner neighbours: across face f to n, then across the face of n after the shared one
   std::vector<int32_t> nbr(4 * (size_t)f.ncol), nbf(4 * (size_t)f.ncol), diag(4 * (size_t)f.ncol);
   HMG_CUDA(c, cudaMemcpy(nbr.data(), f.col_nbr, nbr.size() * 4, cudaMemcpyDeviceToHost));
@@ -1360,7 +1360,7 @@ int train_buffers(Ctx *c, int64_t cells, int nblocks_max) {
   int st;
   if (tb.cap_cells < cells) {
     // (h1, h2: storage for FP32 activations, BF16 uses half of it)
-    float **bufs[] = {reinterpret_cast<float **>(&tb.h1), reinterpret_cast<float **>(&tb.h2), &tb.ga3, &tb.ga2};
+    float **bufs[] = {&tb.h1, &tb.h2, &tb.ga3, &tb.ga2};
     tb.cap_cells = 0;
     for (float **b : bufs) {
       dev_free(c, *b);
