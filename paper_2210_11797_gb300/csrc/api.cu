@@ -283,7 +283,10 @@ int hmg_set_options(hmg_ctx *c, const hmg_options *opt) {
   if (st) return st;
   const hmg_options old = c->opt;
   c->opt = *opt;
-  if ((st = follow_options(c, old))) c->opt = old;
+  if ((st = follow_options(c, old))) {
+    c->opt = old;
+    if (c->assembled && c->have_other && c->direct_sums != (old.precision == HMG_PRECISION_MIXED)) swap_operators(c);
+  }
   return st;
 }
 
